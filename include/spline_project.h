@@ -168,18 +168,16 @@ sp_status spline_visited(const sp_grid *grid, const sp_lines *lines, int32_t *co
  *   spline_plan_prepare  line setup (eq. rayparam) and footprint tables
  *                        (Prop. 1, eq. xsa), for THETA_Y and POINTS lists
  *                        the strip kernels' line order, and, where the plan keeps
- *                        them, the row records: for every major-axis row of
- *                        every line, the position of its run of nodes and
- *                        the argument of its footprint polynomials (the
- *                        traversal of Algorithm 2), sorted by polynomial;
+ *                        them, the row records: where each line's rows start
+ *                        in their runs of nodes and how that moves from row to
+ *                        row (the traversal of Algorithm 2 in fixed point);
  *   spline_plan_fwd      forward projection (Algorithms 1-2);
  *   spline_plan_adj      adjoint.
  * Row records (spline_plan_set_records) are for plans that project many
  * times per prepare (iterative reconstruction): the projections then read
- * them instead of recomputing the rows, with the same results (the forward
- * bit for bit), at the price of a longer prepare and about 8 bytes per line
- * and row of device memory (2.7 GB for 720 x 768 lines on a 512 x 512
- * grid).  New plans keep none.
+ * them instead of deriving them from the line records, with the same results
+ * (the forward bit for bit), for 16 bytes of device memory per line.  New
+ * plans keep none.
  * spline_plan_create allocates (cudaMalloc on the current device) and copies
  * the descriptors but enqueues no work; the device arrays that `lines` points
  * to must stay valid until the last spline_plan_prepare on the plan has run.
@@ -290,8 +288,8 @@ sp_status spline_batch_destroy(sp_batch *batch);
 
 /* Number of lines of the plan (-1 if plan is NULL). */
 int64_t spline_plan_lines(const sp_plan *plan);
-/* Device bytes of the plan's row records (0: the plan keeps none and its
- * projections traverse the rows themselves; -1 if plan is NULL). */
+/* Device bytes of the plan's row records (0: the plan keeps none; -1 if plan
+ * is NULL). */
 int64_t spline_plan_record_bytes(const sp_plan *plan);
 /*
  * keep = 1: the plan keeps row records, written by every later
@@ -302,10 +300,11 @@ int64_t spline_plan_record_bytes(const sp_plan *plan);
  */
 sp_status spline_plan_set_records(sp_plan *plan, int32_t keep);
 /*
- * Diagnostics of the plan's forward projections so far (synchronises):
- * slow_rows = rows whose run of nodes fell outside the shared-memory window
- * staged for their group of lines and were read from global memory instead
- * (results are the same; only speed differs).
+ * Diagnostics of the plan's projections so far (synchronises): slow_rows =
+ * rows whose run of nodes fell outside the shared-memory window staged for
+ * their group of lines and were read from global memory instead.  The strip
+ * kernels size every window so that it holds the runs of all its lines, so the
+ * count is 0.
  */
 sp_status spline_plan_stats(const sp_plan *plan, int64_t *slow_rows);
 /* Free the plan and its device memory (synchronises the device first). */

@@ -391,7 +391,7 @@ class Plan:
         return int(load().spline_plan_record_bytes(self._h))
 
     def slow_rows(self) -> int:
-        """Rows read from global memory because they fell outside the staged window."""
+        """Rows read from global memory because they fell outside the staged window (0: windows hold every run)."""
         v = ctypes.c_int64(0)
         _check(load().spline_plan_stats(self._h, ctypes.byref(v)))
         return int(v.value)

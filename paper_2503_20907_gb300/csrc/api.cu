@@ -170,10 +170,8 @@ void *order_area(const spx::GridDev &g, const spx::LinesDev &L, void *extra)
     return static_cast<char *>(extra) + align_up(spx::strip_scratch_bytes(g)) + 256;
 }
 
-// Kernel paths: strip kernels (structured geometries, any degree) or the
-// general warp-per-line kernels.  kPathAuto takes the strip kernels for degree
-// >= 1 (at degree 0 a row has at most two candidates, too few to repay the
-// row records and their sort; the strip kernels run it when asked).
+// Kernel paths: strip kernels or the general warp-per-line kernels.  kPathAuto
+// takes the strip kernels for degree >= 1.
 // kPathGather (adjoint only): the pixel-driven gather where it applies.
 enum KernelPath { kPathAuto = 0, kPathStrip = 1, kPathGeneral = 2, kPathGather = 3 };
 
@@ -185,35 +183,36 @@ bool use_strip(const spx::GridDev &g, const spx::LinesDev &L, void *extra, int p
 // Forward projection (rec: the plan's row records, or NULL).
 cudaError_t run_fwd(const spx::GridDev &g, const spx::LinesDev &L, const spx::LineHdr *hdr, const float *tabs,
                     void *extra, const float *coef, float *sino, cudaStream_t s, int path = kPathAuto,
-                    const spx::StripRec *rec = nullptr)
+                    const longlong2 *rec = nullptr)
 {
     if (use_strip(g, L, extra, path))
-        return spx::launch_fwd_strip(g, L, hdr, tabs, coef, extra, sino, slow_counter(g, extra), s, rec);
+        return spx::launch_fwd_strip(g, L, hdr, tabs, coef, extra, sino, s, rec);
     return spx::launch_fwd(g, hdr, tabs, L.m, coef, sino, s);
 }
 
 // Adjoint (coef_out overwritten).
 cudaError_t run_adj(const spx::GridDev &g, const spx::LinesDev &L, const spx::LineHdr *hdr, const float *tabs,
                     void *extra, const float *sino, float *coef_out, cudaStream_t s, int path = kPathAuto,
-                    const spx::StripRec *rec = nullptr)
+                    const longlong2 *rec = nullptr)
 {
     if (path == kPathGather && spx::gather_supported(g, L))
         return spx::launch_adj_gather(g, L, hdr, tabs, sino, coef_out, s);
     if (use_strip(g, L, extra, path))
-        return spx::launch_adj_strip(g, L, hdr, tabs, sino, extra, coef_out, slow_counter(g, extra), s, rec,
+        return spx::launch_adj_strip(g, L, hdr, tabs, sino, extra, coef_out, s, rec,
                                      defer_area(g, L, extra));
     return spx::launch_adj(g, hdr, tabs, L.m, sino, coef_out, s);
 }
 
-// Row records a plan keeps: strip-path geometries of degree >= 1 (where the
-// strip kernels are the automatic choice), if they fit in a quarter of the
-// device's free memory and kRecMaxBytes.
+// Row records a plan keeps (W of row 0 and its step, per line): strip-path
+// geometries of degree >= 1 (where the strip kernels are the automatic
+// choice), if they fit in a quarter of the device's free memory and
+// kRecMaxBytes.
 constexpr size_t kRecMaxBytes = size_t(16) << 30;
 
 size_t rec_bytes_wanted(const spx::GridDev &g, const spx::LinesDev &L)
 {
     if (!spx::strip_supported(g, L) || g.kdeg < 1 || L.m == 0) return 0;
-    return (size_t)L.m * (size_t)spx::strip_rec_line_bytes(g);
+    return (size_t)L.m * sizeof(longlong2);
 }
 
 sp_status prepare(const spx::GridDev &g, spx::LinesDev &L, cudaStream_t s,
@@ -363,7 +362,7 @@ struct sp_plan {
     spx::LineHdr *hdr;
     float *tabs;
     void *extra;       // strip scratch (transposed coefficients, slow-row counter) or NULL
-    spx::StripRec rec; // row records written by prepare (base NULL: none)
+    longlong2 *rec;    // row records written by prepare (NULL: none)
     bool prepared;
     void *cg_ws;       // CGLS vectors and scalars, allocated on first use
     size_t cg_bytes;
@@ -377,7 +376,7 @@ namespace {
 // if it keeps none (the projections then traverse the rows themselves).
 bool plan_alloc_records(sp_plan *p)
 {
-    if (p->rec.base) return true;
+    if (p->rec) return true;
     const size_t rb = rec_bytes_wanted(p->g, p->L);
     if (rb == 0) return false;
     size_t fr = 0, tot = 0;
@@ -390,7 +389,7 @@ bool plan_alloc_records(sp_plan *p)
         cudaGetLastError();
         return false;
     }
-    p->rec = spx::StripRec{static_cast<unsigned char *>(r), spx::strip_rec_line_bytes(p->g)};
+    p->rec = static_cast<longlong2 *>(r);
     return true;
 }
 
@@ -431,7 +430,7 @@ sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan
     p->cg_ws = nullptr;
     p->cg_bytes = 0;
     p->path_fwd = p->path_adj = kPathAuto;
-    p->rec = spx::StripRec{nullptr, 0};
+    p->rec = nullptr;
     if (p->extra) {
         e = cudaMemset(slow_counter(g, p->extra), 0, sizeof(int));
         if (e != cudaSuccess) {
@@ -445,8 +444,6 @@ sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan
     return SP_OK;
 }
 
-// The plan's row records, if it keeps them (written by every prepare).
-const spx::StripRec *plan_rec(const sp_plan *p) { return p->rec.base ? &p->rec : nullptr; }
 }  // namespace
 
 extern "C" {
@@ -462,15 +459,15 @@ sp_status spline_plan_set_records(sp_plan *plan, int32_t keep)
     if (!plan) return fail(SP_EINVAL, "plan is NULL");
     if (keep != 0 && keep != 1) return fail(SP_EINVAL, "keep must be 0 or 1");
     if (keep == 0) {
-        if (plan->rec.base) {
+        if (plan->rec) {
             cudaError_t e = cudaDeviceSynchronize();
             if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
-            cudaFree(plan->rec.base);
-            plan->rec = spx::StripRec{nullptr, 0};
+            cudaFree(plan->rec);
+            plan->rec = nullptr;
         }
         return SP_OK;
     }
-    if (plan->rec.base) return SP_OK;
+    if (plan->rec) return SP_OK;
     if (rec_bytes_wanted(plan->g, plan->L) == 0)
         return fail(SP_EUNSUPPORTED, "row records exist only for B-spline or box-spline grids of degree >= 1");
     if (!plan_alloc_records(plan)) return fail(SP_ENOMEM, "row records do not fit in device memory");
@@ -490,8 +487,8 @@ sp_status spline_plan_prepare(sp_plan *plan, void *stream)
         e = spx::launch_line_order(plan->g, plan->L, plan->hdr, const_cast<int *>(plan->L.order), s);
         if (e != cudaSuccess) return cuda_fail(e, "line order");
     }
-    if (plan->rec.base) {
-        e = spx::launch_strip_record(plan->g, plan->L, plan->hdr, plan->tabs, plan->rec, s);
+    if (plan->rec) {
+        e = spx::launch_row_records(plan->hdr, plan->L.m, plan->rec, s);
         if (e != cudaSuccess) return cuda_fail(e, "row records");
     }
     plan->prepared = true;
@@ -506,7 +503,7 @@ sp_status spline_plan_fwd(const sp_plan *plan, const float *coef, float *sino, v
     if (plan->L.m == 0) return SP_OK;
     if (!coef || !sino) return fail(SP_EINVAL, "coef/sino pointers are NULL");
     cudaError_t e = run_fwd(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, coef, sino,
-                            static_cast<cudaStream_t>(stream), plan->path_fwd, plan_rec(plan));
+                            static_cast<cudaStream_t>(stream), plan->path_fwd, plan->rec);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "forward projection");
 }
 
@@ -518,7 +515,7 @@ sp_status spline_plan_adj(const sp_plan *plan, const float *sino, float *coef_ou
     if (!coef_out) return fail(SP_EINVAL, "coef_out pointer is NULL");
     if (plan->L.m > 0 && !sino) return fail(SP_EINVAL, "sino pointer is NULL");
     cudaError_t e = run_adj(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, sino, coef_out,
-                            static_cast<cudaStream_t>(stream), plan->path_adj, plan_rec(plan));
+                            static_cast<cudaStream_t>(stream), plan->path_adj, plan->rec);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "adjoint projection");
 }
 
@@ -526,12 +523,12 @@ namespace {
 cudaError_t plan_fwd_cb(void *ctx, const float *coef, float *sino, cudaStream_t s)
 {
     const sp_plan *p = static_cast<const sp_plan *>(ctx);
-    return run_fwd(p->g, p->L, p->hdr, p->tabs, p->extra, coef, sino, s, p->path_fwd, plan_rec(p));
+    return run_fwd(p->g, p->L, p->hdr, p->tabs, p->extra, coef, sino, s, p->path_fwd, p->rec);
 }
 cudaError_t plan_adj_cb(void *ctx, const float *sino, float *coef_out, cudaStream_t s)
 {
     const sp_plan *p = static_cast<const sp_plan *>(ctx);
-    return run_adj(p->g, p->L, p->hdr, p->tabs, p->extra, sino, coef_out, s, p->path_adj, plan_rec(p));
+    return run_adj(p->g, p->L, p->hdr, p->tabs, p->extra, sino, coef_out, s, p->path_adj, p->rec);
 }
 }  // namespace
 
@@ -572,7 +569,7 @@ int64_t spline_plan_lines(const sp_plan *plan) { return plan ? plan->L.m : -1; }
 int64_t spline_plan_record_bytes(const sp_plan *plan)
 {
     if (!plan) return -1;
-    return plan->rec.base ? plan->L.m * (int64_t)plan->rec.line_bytes : 0;
+    return plan->rec ? plan->L.m * (int64_t)sizeof(longlong2) : 0;
 }
 
 }  // extern "C"
@@ -630,16 +627,15 @@ sp_status spline_plan_autotune(sp_plan *plan, const float *coef, const float *si
         float *tmp_s = nullptr, *tmp_c = nullptr;
         cudaError_t e = cudaMalloc(&tmp_s, sizeof(float) * (size_t)m);
         if (e == cudaSuccess) e = cudaMalloc(&tmp_c, sizeof(float) * (size_t)n);
-        const spx::StripRec *rec = plan_rec(plan);
         for (int k = 0; k < (gather ? 5 : 4) && e == cudaSuccess; ++k) {
             const int path = k == 4 ? kPathGather : ((k & 1) ? kPathGeneral : kPathStrip);
             if (k < 2)
                 e = time_runs([&] { return run_fwd(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, coef, tmp_s, s,
-                                                   path, rec); },
+                                                   path, plan->rec); },
                               3, s, &t[k]);
             else
                 e = time_runs([&] { return run_adj(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, sino, tmp_c, s,
-                                                   path, rec); },
+                                                   path, plan->rec); },
                               3, s, &t[k]);
         }
         cudaError_t e2 = cudaStreamSynchronize(s);
@@ -692,11 +688,11 @@ struct sp_batch {
     spx::StripJob *jobs_dev[2] = {nullptr, nullptr};   // forward, adjoint
     std::vector<spx::StripJob> jobs_host[2];
     int64_t chunks[2] = {0, 0};
-    // jobs grouped by kernel degree (one queue launch per degree):
+    // jobs grouped by kind (one queue launch per B-spline degree and basis):
     // jobs [gjob0, gjob0 + gnjob) of group deg own gtotal chunks
-    int gjob0[2][4] = {}, gnjob[2][4] = {};
-    int64_t gtotal[2][4] = {};
-    unsigned long long *counter = nullptr;              // [2][4 degrees][3]: queue counters
+    int gjob0[2][spx::kQueueKinds] = {}, gnjob[2][spx::kQueueKinds] = {};
+    int64_t gtotal[2][spx::kQueueKinds] = {};
+    unsigned long long *counter = nullptr;              // [2][kinds][3]: queue counters
     long long *defer = nullptr;                          // adjoint chunks deferred to float strips
     int64_t defer_cap = 0;
 };
@@ -779,19 +775,18 @@ cudaError_t upload_jobs(sp_batch *b, int d, In in, Out outp, std::vector<char> &
     hj.clear();
     queued.assign(b->plans.size(), 0);
     int64_t all = 0;
-    for (int deg = 0; deg <= 3; ++deg) {
+    for (int deg = 0; deg < spx::kQueueKinds; ++deg) {
         b->gjob0[d][deg] = (int)hj.size();
         int64_t c0 = 0;   // chunk indices count within the degree's group
         for (size_t i = 0; i < b->plans.size(); ++i) {
             const sp_plan *p = b->plans[i];
             const int path = d ? p->path_adj : p->path_fwd;
             // (degree 0 takes the strip kernels when set or tuned to them)
-            if (p->g.kdeg != deg || p->L.m == 0 || !use_strip(p->g, p->L, p->extra, path)) continue;
+            if (spx::strip_queue_kind(p->g) != deg || p->L.m == 0 || !use_strip(p->g, p->L, p->extra, path)) continue;
             spx::StripJob J = d ? spx::make_strip_job(p->g, p->L, p->hdr, p->tabs, true, nullptr,
-                                                      const_cast<float *>(in[i]), outp[i], p->extra,
-                                                      slow_counter(p->g, p->extra))
+                                                      const_cast<float *>(in[i]), outp[i], p->extra)
                                 : spx::make_strip_job(p->g, p->L, p->hdr, p->tabs, false, in[i], outp[i], nullptr,
-                                                      p->extra, slow_counter(p->g, p->extra));
+                                                      p->extra);
             J.chunk0 = c0;
             c0 += spx::strip_job_chunks(J);
             hj.push_back(J);
@@ -824,10 +819,10 @@ cudaError_t run_queue(sp_batch *b, int d, cudaStream_t s)
     cudaError_t e = cudaSuccess;
     for (size_t k = 0; k < hj.size() && e == cudaSuccess; ++k) e = spx::launch_strip_pre(hj[k], d == 1, s);
     int64_t defer0 = 0;   // each degree's deferred chunks in its own part of the list
-    for (int deg = 0; deg <= 3 && e == cudaSuccess; ++deg) {
+    for (int deg = 0; deg < spx::kQueueKinds && e == cudaSuccess; ++deg) {
         if (b->gnjob[d][deg] == 0) continue;
         e = spx::launch_strip_queue(deg, d == 1, b->jobs_dev[d] + b->gjob0[d][deg], b->gnjob[d][deg],
-                                    b->gtotal[d][deg], b->counter + 12 * d + 3 * deg,
+                                    b->gtotal[d][deg], b->counter + 3 * spx::kQueueKinds * d + 3 * deg,
                                     d == 1 ? b->defer + defer0 : nullptr, s);
         defer0 += b->gtotal[d][deg];
     }
@@ -859,7 +854,7 @@ sp_status spline_batch_create(int32_t count, const sp_grid *grids, const sp_line
     cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     for (int d = 0; d < 2 && e == cudaSuccess; ++d) e = cudaMalloc(&b->jobs_dev[d], sizeof(spx::StripJob) * (size_t)count);
-    if (e == cudaSuccess) e = cudaMalloc(&b->counter, 24 * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMalloc(&b->counter, 6 * spx::kQueueKinds * sizeof(unsigned long long));
     for (int k = 0; k < kBatchStreams && e == cudaSuccess; ++k) {
         e = cudaStreamCreateWithFlags(&b->streams[k], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming);
@@ -1053,12 +1048,12 @@ sp_status spline_plan_destroy(sp_plan *plan)
     g_err.clear();
     if (!plan) return SP_OK;
     sp_status st = SP_OK;
-    if (plan->mem || plan->cg_ws || plan->rec.base) {
+    if (plan->mem || plan->cg_ws || plan->rec) {
         cudaError_t e = cudaDeviceSynchronize();
         if (e != cudaSuccess) st = cuda_fail(e, "cudaDeviceSynchronize");
         if (plan->mem) cudaFree(plan->mem);
         if (plan->cg_ws) cudaFree(plan->cg_ws);
-        if (plan->rec.base) cudaFree(plan->rec.base);
+        if (plan->rec) cudaFree(plan->rec);
     }
     delete plan;
     return st;

@@ -67,13 +67,12 @@ enum TabMode : int {
 
 enum LineFlags : int {
     kVert = 1,        // rows are x2 (index j), columns x1 (index i)
-    kKapNeg = 2,      // u decreases with the column index
     kDeg0Axis = 4,    // degree 0 and b == 0: rectangle, midpoint value at its edges
     kEmpty = 8,       // the line meets no support
 };
 
 // Per-line record (64 bytes).  u(r, q) = U0 + (r - r_ref) rho + (q - q_ref) kappa,
-// kappa = +-a; rho and a are carried as hi + lo pairs whose hi parts make the
+// kappa = a (lines are oriented so that u grows with the column); rho and a are carried as hi + lo pairs whose hi parts make the
 // products with row and step counts exact.
 struct __align__(16) LineHdr {
     float U0;              // u at (r_ref, q_ref), in (0, a]
@@ -212,7 +211,7 @@ struct RowEval {
 };
 
 template <int DEG>
-__device__ __forceinline__ RowEval row_eval(const LineHdr &H, const float *s, float inv_a, int sgn, int r)
+__device__ __forceinline__ RowEval row_eval(const LineHdr &H, const float *s, float inv_a, int r)
 {
     RowEval e;
     int k;
@@ -233,7 +232,7 @@ __device__ __forceinline__ RowEval row_eval(const LineHdr &H, const float *s, fl
         e.uhi = u0;
         e.ulo = 0.f;
     }
-    e.q0 = H.q_ref - sgn * k;
+    e.q0 = H.q_ref - k;
     return e;
 }
 
@@ -262,13 +261,6 @@ cudaError_t launch_visited(const GridDev &g, const LineHdr *hdr, const float *ta
                            cudaStream_t s);
 cudaError_t launch_expand(const LinesDev &L, float *theta_out, float *y_out, cudaStream_t s);
 
-// Sorted row records of every line, kept by a plan so that its projections
-// skip the per-row traversal (strip.cu): line_bytes per line, line-major.
-struct StripRec {
-    unsigned char *base;
-    long long line_bytes;
-};
-
 // Free line lists in strip-kernel order (order.cu): the key of every line
 // (major axis, then direction, then the position of its run at the grid's
 // middle row) and a stable radix sort of the line indices by it.  `area`
@@ -281,31 +273,25 @@ inline bool strip_needs_order(const LinesDev &L) { return L.kind == SP_LINES_THE
 
 // Forward projection with coefficient strips in shared memory (strip.cu), for
 // parallel and fan beams and sorted free line lists (any degree; L.order set
-// for the latter).  `scratch` holds strip_scratch_bytes;
-// `slow_rows` counts rows whose run fell outside the staged window.  With
-// `rec` (written by launch_strip_record for the same lines) the row records
-// are read instead of recomputed.
+// for the latter).  `scratch` holds strip_scratch_bytes; `rec`: the plan's row
+// records, or NULL (the kernels then take the rows from the line records).
 bool strip_supported(const GridDev &g, const LinesDev &L);
 size_t strip_scratch_bytes(const GridDev &g);
-long long strip_rec_line_bytes(const GridDev &g);
 cudaError_t launch_fwd_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *coef, void *scratch, float *sino, int *slow_rows, cudaStream_t s,
-                             const StripRec *rec = nullptr);
+                             const float *coef, void *scratch, float *sino, cudaStream_t s, const longlong2 *rec);
+// The row records of lines of degree >= 1 (W of row 0 and its step, per line), after line setup.
+cudaError_t launch_row_records(const LineHdr *hdr, int64_t m, longlong2 *rec, cudaStream_t s);
 // Adjoint with strip accumulators; coef_out is overwritten.  `defer` holds
 // 2 + strip_chunk_count(L) words (chunks deferred to float strips).
 int64_t strip_chunk_count(const LinesDev &L);
 cudaError_t launch_adj_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *sino, void *scratch, float *coef_out, int *slow_rows, cudaStream_t s,
-                             const StripRec *rec, unsigned *defer);
+                             const float *sino, void *scratch, float *coef_out, cudaStream_t s, const longlong2 *rec,
+                             unsigned *defer);
 // Pixel-driven adjoint (gather.cu): thread per node over all views, no
 // atomics; parallel and fan beams of degree >= 1.  coef_out is overwritten.
 bool gather_supported(const GridDev &g, const LinesDev &L);
 cudaError_t launch_adj_gather(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
                               const float *sino, float *coef_out, cudaStream_t s);
-// The row records of every line of (g, L) into rec (after line setup and tables).
-cudaError_t launch_strip_record(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                                const StripRec &rec, cudaStream_t s);
-
 // One instance of the persistent strip kernel's work queue: the arguments of
 // one strip projection and the index of its first chunk in the queue.
 struct StripJob {
@@ -317,7 +303,6 @@ struct StripJob {
     float *coefT;          // scratch: transposed input (forward) ...
     float *sino;
     float *out, *outT;     // ... or output and transposed output (adjoint)
-    int *err;
     int cpv;               // chunks per view
     int vec;               // 16-byte staging and flushing
     long long chunk0;
@@ -325,18 +310,20 @@ struct StripJob {
 // The job of one strip projection (adj: img_out receives the adjoint of sino;
 // forward: sino receives the projection of img_in).  chunk0 is left 0.
 StripJob make_strip_job(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs, bool adj,
-                        const float *img_in, float *sino, float *img_out, void *scratch, int *err);
+                        const float *img_in, float *sino, float *img_out, void *scratch);
 int64_t strip_job_chunks(const StripJob &J);
 // Before the queue kernel: transposed copy of the input (forward) or cleared
 // outputs (adjoint); after it: the transposed output added in (adjoint).
 cudaError_t launch_strip_pre(const StripJob &J, bool adj, cudaStream_t s);
 cudaError_t launch_strip_post(const StripJob &J, bool adj, cudaStream_t s);
 // The persistent kernel over jobs[0..njobs) (device array, chunk0 ascending,
-// `total` chunks in all, every job of kernel degree deg in 0..3); counter is
+// `total` chunks in all, every job of kind `kind`); counter is
 // three device words, reset here.  The adjoint defers chunks that need float
 // strips to `defer` (device, room for `total` chunk indices) and runs them in
 // a second launch.
-cudaError_t launch_strip_queue(int deg, bool adj, const StripJob *jobs, int njobs, int64_t total,
+constexpr int kQueueKinds = 5;   // B-spline degrees 0..3 and the box-spline
+int strip_queue_kind(const GridDev &g);
+cudaError_t launch_strip_queue(int kind, bool adj, const StripJob *jobs, int njobs, int64_t total,
                                unsigned long long *counter, long long *defer, cudaStream_t s);
 cudaError_t launch_footprint_eval(const GridDev &g, int64_t count, const float *theta, const float *yt,
                                   float *out, float *scratch, cudaStream_t s);

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreads) gather_adj_kernel(GridDev g, LinesDe
                         // the stepping of the strip kernels (row_u0) with the
                         // step count k = -+(q - q_ref), hi products exact
                         const float fr = (float)(r - H.r_ref);
-                        const float fk = (float)((H.flags & kKapNeg) ? (q - H.q_ref) : (H.q_ref - q));
+                        const float fk = (float)(H.q_ref - q);
                         const float big = __fsub_rn(__fmul_rn(fr, H.rho_hi), __fmul_rn(fk, H.a_hi));
                         const float small = __fmaf_rn(fr, H.rho_lo, __fmul_rn(-fk, H.a_lo));
                         const float u = __fadd_rn(__fadd_rn(H.U0, small), big);

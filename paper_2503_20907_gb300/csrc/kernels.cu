@@ -171,15 +171,17 @@ __device__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineH
     const double A = fmax(fabs(dx), fabs(dy));
     const double B = fmin(fabs(dx), fabs(dy));
     const double h = (double)g.h;
-    const double Yhat = ((px - (double)g.cx) * dy - (py - (double)g.cy) * dx) / h;
+    double Yhat = ((px - (double)g.cx) * dy - (py - (double)g.cy) * dx) / h;
     const double ic = 0.5 * (g.nx - 1), jc = 0.5 * (g.ny - 1);
     double kap, rho, rc, qc;
     int Nr, Nq;
     if (vert) { kap = -dy; rho = dx; rc = jc; qc = ic; Nr = g.ny; Nq = g.nx; }
     else { kap = dx; rho = -dy; rc = ic; qc = jc; Nr = g.nx; Nq = g.ny; }
-    const int sgn = kap > 0.0 ? 1 : -1;
+    // a line and its reverse are one line, and phi is even: take the direction
+    // in which u grows with the column
+    if (kap < 0.0) { kap = -kap; rho = -rho; Yhat = -Yhat; }
     // w as the table sees it (support_params, with the table's a and b)
-    int flags = (vert ? kVert : 0) | (sgn < 0 ? kKapNeg : 0);
+    int flags = vert ? kVert : 0;
     if (g.degree == 0 && B == 0.0) flags |= kDeg0Axis;
 
     // Rows whose support run meets the columns [0, Nq): the column of the
@@ -208,10 +210,10 @@ __device__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineH
     const int r_ref = (rb + re) / 2;
     // u at (r_ref, q = 0), then the reference column with U0 in (0, a].
     const double Ur = Yhat + w + ((double)r_ref - rc) * rho - qc * kap;
-    double qr = (sgn > 0) ? floor(-Ur / A) + 1.0 : ceil(Ur / A) - 1.0;
+    double qr = floor(-Ur / A) + 1.0;
     double U0 = Ur + qr * kap;
-    if (U0 <= 0.0) { qr += sgn; U0 = Ur + qr * kap; }
-    else if (U0 > A) { qr -= sgn; U0 = Ur + qr * kap; }
+    if (U0 <= 0.0) { qr += 1.0; U0 = Ur + qr * kap; }
+    else if (U0 > A) { qr -= 1.0; U0 = Ur + qr * kap; }
     // hi parts exact against |row offset| and |step count|, both < maxc
     int maxc = (re - rb) + 8;
     int nb = 0;
@@ -767,16 +769,15 @@ __device__ __forceinline__ void walk_line(const LineHdr &H, const float *tab, co
                                           int lane, Op op)
 {
     const bool vert = H.flags & kVert;
-    const int sgn = (H.flags & kKapNeg) ? -1 : 1;
     const int Nq = vert ? g.nx : g.ny;
     const float inv_a = 1.0f / H.a;
     float s[DEG + 1];
 #pragma unroll
     for (int q = 0; q <= DEG; ++q) s[q] = tab[q];
     for (int r = H.r_begin + lane; r < H.r_end; r += 32) {
-        const RowEval e = row_eval<DEG>(H, s, inv_a, sgn, r);
+        const RowEval e = row_eval<DEG>(H, s, inv_a, r);
         for (int i = 0; i < H.K; ++i) {
-            int q = e.q0 + sgn * i;
+            int q = e.q0 + i;
             if ((unsigned)q < (unsigned)Nq) {
                 float ti = (DEG == 0) ? __fmaf_rn((float)i, H.a_corr, e.t) : e.t;
                 float phi = horner<DEG>(tab + tab_poly(e.sg, i), ti);
@@ -787,7 +788,7 @@ __device__ __forceinline__ void walk_line(const LineHdr &H, const float *tab, co
         }
         if (DEG == 0 && e.tie) {
             // the run also starts at u = 0: midpoint value on that edge too
-            int q = e.q0 - sgn;
+            int q = e.q0 - 1;
             if ((unsigned)q < (unsigned)Nq) {
                 int node = vert ? r * g.nx + q : q * g.nx + r;
                 op(node, 0.5f * inv_a);
@@ -871,8 +872,7 @@ __global__ void visited_kernel(GridDev g, const LineHdr *__restrict__ hdr,
         if (!(H.flags & kEmpty)) {
             const float *tab = tabs + (int64_t)H.tab * kTabFloats;
             const bool vert = H.flags & kVert;
-            const int sgn = (H.flags & kKapNeg) ? -1 : 1;
-            const int Nq = vert ? g.nx : g.ny;
+                    const int Nq = vert ? g.nx : g.ny;
             const float inv_a = 1.0f / H.a;
             // b of the table: 2w = m (a + b)
             const float bf = tab[kTabB];   // b the table was built with
@@ -886,12 +886,12 @@ __global__ void visited_kernel(GridDev g, const LineHdr *__restrict__ hdr,
                 int cnt = 0;
                 RowEval e{0, 0, 0.f, false, 0.f, 0.f};
                 if (r < H.r_end) {
-                    e = row_eval<DEG>(H, s, inv_a, sgn, r);
+                    e = row_eval<DEG>(H, s, inv_a, r);
                     for (int i = 0; i < H.K; ++i) {
-                        int q = e.q0 + sgn * i;
+                        int q = e.q0 + i;
                         if ((unsigned)q < (unsigned)Nq && candidate_in<DEG>(H, s, e, i, bf)) ++cnt;
                     }
-                    if (e.tie && (unsigned)(e.q0 - sgn) < (unsigned)Nq) ++cnt;
+                    if (e.tie && (unsigned)(e.q0 - 1) < (unsigned)Nq) ++cnt;
                 }
                 int incl = cnt;
 #pragma unroll
@@ -904,12 +904,12 @@ __global__ void visited_kernel(GridDev g, const LineHdr *__restrict__ hdr,
                 if (nodes && offsets && cnt > 0) {
                     int64_t pos = base + total + excl;
                     for (int i = 0; i < H.K; ++i) {
-                        int q = e.q0 + sgn * i;
+                        int q = e.q0 + i;
                         if ((unsigned)q < (unsigned)Nq && candidate_in<DEG>(H, s, e, i, bf))
                             nodes[pos++] = vert ? r * g.nx + q : q * g.nx + r;
                     }
-                    if (e.tie && (unsigned)(e.q0 - sgn) < (unsigned)Nq) {
-                        int q = e.q0 - sgn;
+                    if (e.tie && (unsigned)(e.q0 - 1) < (unsigned)Nq) {
+                        int q = e.q0 - 1;
                         nodes[pos++] = vert ? r * g.nx + q : q * g.nx + r;
                     }
                 }

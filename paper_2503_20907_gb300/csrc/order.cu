@@ -46,12 +46,11 @@ __global__ void order_keys_kernel(GridDev g, const LineHdr *__restrict__ hdr, in
     if (!(H.flags & kEmpty) && H.r_end > H.r_begin) {
         const bool vert = (H.flags & kVert) != 0;
         const int Nr = vert ? g.ny : g.nx, Nq = vert ? g.nx : g.ny;
-        const float sgn = (H.flags & kKapNeg) ? -1.f : 1.f;
         // column where u(r, q) = U0 + (r - r_ref) rho + (q - q_ref) kappa
-        // reaches the support's centre w, kappa = sgn a: the run's centre
+        // reaches the support's centre w, kappa = a: the run's centre
         const float rho = H.rho_hi + H.rho_lo;
         const float w = 0.5f * H.two_w;
-        auto centre = [&](float r) { return (float)H.q_ref + sgn * (w - H.U0 - (r - (float)H.r_ref) * rho) / H.a; };
+        auto centre = [&](float r) { return (float)H.q_ref + (w - H.U0 - (r - (float)H.r_ref) * rho) / H.a; };
         const float qa = centre(0.f), qb = centre((float)(Nr - 1));
         const float slope = Nr > 1 ? (qb - qa) / (float)(Nr - 1) : 0.f;
         const float c = 0.5f * (qa + qb);

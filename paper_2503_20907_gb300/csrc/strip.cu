@@ -4,25 +4,52 @@
 //
 // One CTA takes a chunk of up to kChunk neighbouring lines of one view
 // (consecutive detector bins, or consecutive lines of a sorted free list).
-// Such lines are nearly parallel and adjacent,
-// so in every major-axis row their runs of nonzero nodes fall inside a short
-// window; the CTA keeps those windows (a skewed strip, one row per major-axis
-// row) in shared memory: staged from the coefficients for the forward
-// projection, accumulated and then added to the output for the adjoint.
-// Lines whose major axis is x1 use transposed images so that strip rows stay
-// contiguous in global memory.
+// Such lines are nearly parallel and adjacent, so in every major-axis row
+// their runs of nonzero nodes fall inside a short window; the CTA keeps those
+// windows (a skewed strip, one row per major-axis row) in shared memory:
+// staged from the coefficients for the forward projection, accumulated and
+// then added to the output for the adjoint.  Lines whose major axis is x1 use
+// transposed images so that strip rows stay contiguous in global memory.
 //
-// One warp takes one line at a time, in batches of up to kBatch rows:
-//   A. lane per row: u_0 (stepped from row to row in 64-bit fixed point),
-//      its interval sigma, t = u_0 - s_sigma and the strip offset of the
-//      row's first candidate; the rows are then ordered by sigma (counting
-//      sort, in the warp's shared memory);
-//   B. lane per (candidate i, row slot): for each interval sigma the lane
-//      holds the polynomial T[sigma][i] in registers and runs it over the
-//      rows of that interval, two rows per packed FP32 FMA (fma.rn.f32x2).
-// Polynomial coefficients are then read once per interval and batch instead
-// of once per row, which keeps shared-memory traffic to the row records and
-// the coefficients (or strip accumulators) themselves.
+// Lane = line, and the lanes of a warp walk the rows together.  Which
+// polynomial a candidate takes depends on where the row's u_0 lies among the
+// breakpoints s_q of the line's direction, which differs from lane to lane
+// and row to row.  So the kernels do not select polynomials at all.  The
+// footprint of degree n is a spline of degree 2n+1 with simple knots: across
+// the knot p a + q b only its (2n+1)-th derivative jumps, by
+// (-1)^(p+q) C(n+1,p) C(n+1,q) / (a b)^(n+1).  With the polynomials B_i of one
+// base interval of u_0, every candidate i is, for any u_0 in (0, a],
+//
+//   phi(u_0 + i a) = B_i(u_0 - s_base) + sum_q J_{p q} z_q,   p = i - floor(q b / a),
+//   J_{p q} = (-1)^(p+q) C(n+1,p) C(n+1,q) / ((2n+1)! (a b)^(n+1)),
+//   z_q = |u_0 - s_q|^(2n+1) beyond s_q as seen from the base interval, else 0.
+//
+// The sum over q depends on the candidate only through p, so breakpoints with
+// the same floor(q b / a) share one number Z_f = sum_q g_{qf} z_q, and a
+// candidate adds C(n+1, i - f) (-1)^(i - f) Z_f for each of the D = 1 + max f
+// values of f: integer weights known at compile time.  A lane holds its
+// line's B_i in registers (two candidates per packed FMA, fma.rn.f32x2) for
+// the whole strip: no table look-ups, no sorting and no branches per row.
+// The base interval is the one that leaves u_0 the shortest way to go
+// (its distance to the ends of (0, a]); the terms J z then stay below a few
+// tenths, and the FP32 evaluation of phi is about as accurate as one from
+// the interval's own polynomial (rms over random directions 1.4e-8 against
+// 1.2e-8 at degree 3).
+//
+// u_0 is stepped from row to row in 64-bit fixed point: with W(r) =
+// 2^32 u(r)/a - 1 (u(r) the line's offset in row r at its reference column)
+// the high word of W is the row's step count and the low word its u_0.
+//
+// Sums.  Rows are taken in blocks of kRowBlock whose bounds are fixed in the
+// image.  A block's sum is one FP32 chain; block sums are added as float pairs
+// (two-sum), so that a line's value does not depend on how its blocks were
+// spread over warps and lanes, i.e. on the lines it shares a chunk with.
+//
+// What bounds it: the FMA pipe.  A row of a line with N = n + 1 + D candidates
+// takes N (2n+1) Horner FMAs, about (n + 2) D for the knots, 7 (n + 1) for the
+// z_q and N to accumulate (87 at n = 3, D = 2), and N shared-memory accesses;
+// the lanes' accesses of one row fall on neighbouring columns, in distinct
+// banks.
 //
 // The adjoint accumulates its strip in 32-bit fixed point: a shared-memory
 // integer reduction costs about what a plain shared store does on this GPU,
@@ -30,12 +57,12 @@
 // that puts its largest contribution h |p| phi (phi <= sqrt(2) < 1.5 for
 // every basis here) at 2^21 or less; a pair then adds round(S h p phi) to its
 // node, at most 2^26 in magnitude after 32 lines, and the flush adds the
-// sums times 1/S (exact) to the image.  The rounding rides on the last FMA
-// of the Horner scheme: its constant term carries M = 1.5 2^23, so the
-// result lies in [2^23, 2^24) where floats are the integers, and its bits
-// minus M's bits are round(S h p phi).  Per pair that is an error of at most
-// one unit, 1/S <= 1.5 h max|p| 2^-21 = 7e-7 h max|p|.
+// sums times 1/S (exact) to the image.  Adding M = 1.5 2^23 does the rounding:
+// the result lies in [2^23, 2^24) where floats are the integers, and its bits
+// minus M's bits are round(S h p phi).  Per pair that is an error of about
+// half a unit, 1/S <= 1.5 h max|p| 2^-21 = 7e-7 h max|p|.
 #include <climits>
+#include <cfloat>
 
 #include "common.cuh"
 
@@ -44,33 +71,29 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kThreads = kWarps * 32;
-constexpr int kChunk = 32;          // lines per chunk
-constexpr int kPitch = 44;          // strip row length (floats), whole 16-byte chunks
-constexpr int kWin = kPitch - 3;    // window width that fits once its start is rounded down to 4 columns
-constexpr int kSlabRows = 360;      // strip rows held at once (one sorting batch per line and slab)
-constexpr int kDummy = 16;          // zero floats after the strip: target of padding records
-constexpr int kBatch = 384;         // rows of one line per sorting batch (12 per lane), >= kSlabRows
-constexpr int kRowsPerLane = kBatch / 32;
-constexpr int kEntCap = kBatch + 4 * kMaxSig;   // sorted row records, segments padded to multiples of 4
+constexpr int kChunk = 32;          // lines per chunk (lanes of a warp)
+constexpr int kRowBlock = 4;        // rows summed in one FP32 chain
+constexpr int kSlopeBits = 15;      // fractional bits of the window's slope
+constexpr int kMaxWidth = 192;      // widest strip row (floats)
+constexpr int kStripFloats = 25280; // strip rows held at once times their width
+constexpr int kBasePitch = kSigStride + kTabHead + 4;   // a line's base polynomials and table head, spaced so that
+                                                        // 16-byte reads of 8 lanes meet 32 banks
 
-constexpr size_t kStripBytes = sizeof(float) * (kSlabRows * kPitch + kDummy);
-constexpr size_t kCloBytes = sizeof(int) * kSlabRows;
-// Per warp: two table buffers (current line and the next one, loaded
-// asynchronously) and the sorted row records of one batch.
-constexpr size_t kTabBufBytes = sizeof(float) * kTabFloats;
-constexpr size_t kWarpBytes = 2 * kTabBufBytes + 2 * sizeof(float) * kEntCap;   // + t[] and offset[]
-constexpr size_t kAccBytes = sizeof(float) * kChunk;
-constexpr size_t kMiscBytes = 32 + 4 * 64;
+constexpr size_t kStripBytes = sizeof(float) * kStripFloats;
+constexpr size_t kBaseBytes = sizeof(float) * kBasePitch * kChunk;
 constexpr size_t kHdrBytes = sizeof(LineHdr) * kChunk;
-constexpr size_t kRecOffBytes = sizeof(int) * kChunk;
-constexpr size_t kSmemBytes =
-    kStripBytes + kCloBytes + kWarps * kWarpBytes + kAccBytes + kMiscBytes + kHdrBytes + kRecOffBytes;
-static_assert(kTabBufBytes % 16 == 0 && kWarpBytes % 16 == 0 && kStripBytes % 16 == 0 && kCloBytes % 16 == 0,
-              "16-byte alignment of the shared-memory regions");
+constexpr size_t kPartBytes = 2 * sizeof(float) * kWarps * kChunk;
+constexpr size_t kSmemBytes = kStripBytes + kBaseBytes + kHdrBytes + kPartBytes;
+static_assert(kStripBytes % 16 == 0 && kBaseBytes % 16 == 0 && kHdrBytes % 16 == 0, "16-byte alignment of the regions");
 static_assert(kSmemBytes <= 115712, "two CTAs per SM");
-static_assert(kPitch % 4 == 0, "strip rows of whole 16-byte chunks");
-static_assert(kSlabRows * kPitch + kDummy < (1 << 16), "strip offsets fit 16 bits (phase A packs sigma above them)");
-static_assert(kBatch >= kSlabRows && kEntCap < 512, "one batch per line and slab; 9-bit counters of the sort");
+static_assert(kStripFloats / kMaxWidth >= 8 * kRowBlock, "the widest strip holds a row block per warp");
+static_assert(kBasePitch % 8 == 4, "conflict-free 16-byte reads");
+
+// What the kernels are instantiated for: the B-spline degrees, and the
+// 3-direction box-spline (whose footprint is piecewise quadratic with knots
+// in its first two derivatives).
+constexpr int kKindBox = 4;
+inline int strip_kind(const GridDev &g) { return g.basis == SP_BASIS_BOX3 ? kKindBox : g.kdeg; }
 
 // ------------------------------------------------------------------ packed FP32
 typedef unsigned long long f2;
@@ -94,6 +117,29 @@ __device__ __forceinline__ f2 f2fma(f2 a, f2 b, f2 c)
     return d;
 }
 
+__device__ __forceinline__ f2 f2mul(f2 a, f2 b)
+{
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ f2 f2add(f2 a, f2 b)
+{
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// (hi, lo) += x, hi + lo kept to about 48 bits (two-sum).
+__device__ __forceinline__ void pair_add(float &hi, float &lo, float x)
+{
+    const float s = __fadd_rn(hi, x);
+    const float bb = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+    hi = s;
+}
+
 __device__ __forceinline__ void red_shared(float *p, float v)
 {
     asm volatile("red.shared.add.f32 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(p)), "f"(v)
@@ -101,8 +147,7 @@ __device__ __forceinline__ void red_shared(float *p, float v)
 }
 
 // No "memory" clobber: the strip is read only after the block's barrier
-// before its flush, so the reductions need not order the row-record and table
-// loads of the next groups, which the compiler may then issue early.
+// before its flush, so the reductions need not order any other access.
 __device__ __forceinline__ void red_shared_u32(int *p, int v)
 {
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(p)), "r"(v));
@@ -116,412 +161,568 @@ constexpr int kFixMagicBits = 0x4B400000;
 constexpr float kFixMax = 2097152.0f;   // 2^21
 constexpr float kPhiBound = 1.5f;
 
-// Row records kept by a plan (see spline_plan_prepare): kRecWrite runs the
-// traversal (line groups, strip slabs, row batches, phase A and the sort) and
-// stores each batch's sorted records instead of projecting; kRecRead loads
-// them in the same order and runs phase B only.  Per line a region of
-// strip_rec_line_bytes(); per batch a 16-byte header (padded segment lengths,
-// and a flag for batches with runs outside the staged window, which the
-// replay recomputes), then t[R] and the strip offsets[R].
-enum RecMode { kRecNone = 0, kRecWrite = 1, kRecRead = 2 };
 // Which chunks an adjoint call runs (strip_chunk's FM).
 enum FixMode { kFmAll = 0, kFmFixed = 1, kFmFloat = 2 };
-constexpr unsigned long long kRecSlowBit = 1ull << 63;
 
-template <int NS>
-__device__ __forceinline__ int4 rec_pack(const int (&segn)[NS], bool slow)
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool in = true)
 {
-    int n[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-    for (int q = 0; q < NS; ++q) n[q] = segn[q];
-    return make_int4(n[0] | (n[1] << 16), n[2] | (n[3] << 16), n[4], slow ? (1 << 16) : 0);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+// 4 bytes, or zeros where in is false (src is then not read).
+__device__ __forceinline__ void cp_async4(unsigned dst, const void *src, bool in)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// (xh + xl) / a in fixed point with F fractional bits, a = H.a_hi + H.a_lo:
+// the float quotient and one correction step.
+template <int F>
+__device__ __forceinline__ long long fix_quot(const LineHdr &H, float inv_a, float xh, float xl)
+{
+    constexpr float kOne = F == 32 ? 4294967296.f : 281474976710656.f;
+    const float q1 = xh * inv_a;
+    const float r = __fmaf_rn(-q1, H.a_lo, __fmaf_rn(-q1, H.a_hi, xh) + xl);
+    return __float2ll_rn(q1 * kOne) + __float2ll_rn(r * inv_a * kOne);
 }
 
-template <int NS>
-__device__ __forceinline__ int rec_unpack(int4 hd, int (&segb)[NS], int (&segn)[NS])
+// W of row 0 and its step per row.
+template <int F>
+__device__ __forceinline__ void row_stepping(const LineHdr &H, long long &W, long long &step)
 {
-    const int n[5] = {hd.x & 0xffff, hd.x >> 16, hd.y & 0xffff, hd.y >> 16, hd.z & 0xffff};
-    int b = 0;
+    const float inv_a = 1.0f / H.a;
+    step = fix_quot<F>(H, inv_a, H.rho_hi, H.rho_lo);
+    W = fix_quot<F>(H, inv_a, H.U0, H.U0_lo) - 1 - H.r_ref * step;
+}
+
+// The row records a plan keeps: every line's W of row 0 and its step, from
+// which all its rows follow (degree >= 1).
+__global__ void row_record_kernel(const LineHdr *__restrict__ hdr, int64_t m, longlong2 *__restrict__ rec)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const LineHdr H = hdr[i];
+    long long W = 0, step = 0;
+    if (!(H.flags & kEmpty)) row_stepping<32>(H, W, step);
+    rec[i] = make_longlong2(W, step);
+}
+
+// ------------------------------------------------------------------ one line on a strip
+// A lane's line on a strip: W of strip row 0 and the step per row; a run
+// starts in column q_ref minus W's high part.
+struct LaneLine {
+    long long W0, Wstep;
+    int q_ref;
+    float a, ua;               // a, and a / 2^F
+    float hp;                  // adjoint: h p (times the chunk's scale S for fixed-point strips)
+    // 1 at run time: multiplied by it the polynomials settle in register pairs;
+    // left as loaded, the compiler packs them anew in every row (48 moves a row
+    // at degree 3, 1.39 against 1.19 ms at the 512 x 512 cubic fan)
+    float one;
+    const float *base;         // B_i [8][8], then the table head
+    float s_base;              // the base interval's start
+    // the rows whose run reaches the line's last candidate slot (x up to the
+    // end of the support): slot N - 1 of lines with the warp's most slots N,
+    // slot N - 2 of the others
+    bool has_last;
+    unsigned x_end;
+};
+
+// The strip in shared memory: `rows` rows of `pitch` floats, row rr starting
+// at the column c0 + slope rr 2^-kSlopeBits rounded down to a multiple of 4.
+struct Strip {
+    float *p;
+    int pitch, rows, c0, slope;
+    __device__ __forceinline__ int first(int rr) const { return (c0 + ((slope * rr) >> kSlopeBits)) & ~3; }
+};
+
+// Candidate pair (2p, 2p+1)'s weights for the knots with floor(q b / a) = f:
+// (-1)^k C(m, k) at k = 2p - f and 2p + 1 - f.
+__host__ __device__ constexpr float knot_weight(int m, int k)
+{
+    if (k < 0 || k > m) return 0.f;
+    float r = 1.f;
+    for (int i = 1; i <= k; ++i) r = r * (float)(m - k + i) / (float)i;
+    return (k & 1) ? -r : r;
+}
+
+// The values of f = floor(q b / a) that knot q can have in a warp whose lines
+// have D or D - 1 of them (b / a in (max(D - 2, 0) / m, D / m)).
+__host__ __device__ constexpr int knot_f_lo(int m, int D, int q) { return D >= 2 ? q * (D - 2) / m : 0; }
+__host__ __device__ constexpr int knot_f_hi(int m, int D, int q) { return (q * D + m - 1) / m - 1; }
+
+// Rows [r0, r1) of a block for one B-spline line of degree DEG, m = DEG + 1,
+// N = m + D candidates: the polynomials and knots in registers.
+template <int DEG, int D, bool ADJ, bool FIX>
+struct SplineRows {
+    static constexpr int F = 32;
+    static constexpr int m = DEG + 1, NC = 2 * DEG + 2, N = m + D, NP = N / 2;
+    static constexpr int NQ = (m + 1) / 2;   // knots, two per packed operation
+    f2 C[NP][NC];      // candidates 2p, 2p + 1
+    float cl[NC];      // the last one of an odd N
+    f2 zs[NQ], zb[NQ]; // distance to knot q: zs u + zb, positive beyond it
+    float g[m][D];     // Z_f = sum_q g[q][f] z_q
+    float ua, ub;      // t = ua x + ub
+    float hp;          // float adjoint: the factor of phi
+    unsigned x_last, x_prev;   // rows that have candidates N - 1 and N - 2: x up to these
+    bool has_last;
+
+    __device__ __forceinline__ void load(const LaneLine &ln)
+    {
 #pragma unroll
-    for (int q = 0; q < NS; ++q) {
-        segb[q] = b;
-        segn[q] = n[q];
-        b += n[q];
+        for (int i = 0; i < N; ++i) {
+            float c[8];
+#pragma unroll
+            for (int d4 = 0; d4 < (NC + 3) / 4; ++d4) {
+                const float4 w = *reinterpret_cast<const float4 *>(ln.base + i * kNC + 4 * d4);
+                c[4 * d4] = w.x; c[4 * d4 + 1] = w.y; c[4 * d4 + 2] = w.z; c[4 * d4 + 3] = w.w;
+            }
+#pragma unroll
+            for (int d = 0; d < NC; ++d) {
+                const float v = c[d] * (FIX ? ln.hp : ln.one);
+                if (i == 2 * NP) {
+                    cl[d] = v;
+                } else if (i & 1) {
+                    float lo, hi;
+                    f2unpack(C[i / 2][d], lo, hi);
+                    C[i / 2][d] = f2pack(lo, v);
+                } else {
+                    C[i / 2][d] = f2pack(v, 0.f);
+                }
+            }
+        }
+        const float a = ln.a, b = ln.base[kSigStride + kTabB], inv_a = 1.0f / a;
+        // 1 / ((2n+1)! (a b)^(n+1)); no knots in b = 0 (the Dirac of Prop. 1)
+        float ab = a * b, kap = ab;
+#pragma unroll
+        for (int k = 1; k < m; ++k) kap *= ab;
+        constexpr float kFact = DEG == 3 ? 5040.f : DEG == 2 ? 120.f : 6.f;
+        kap = b > 0.f ? 1.0f / (kFact * kap) : 0.f;
+        if constexpr (FIX) kap *= ln.hp;
+        float zsv[2 * NQ], zbv[2 * NQ];
+#pragma unroll
+        for (int k = 0; k < 2 * NQ; ++k) { zsv[k] = 0.f; zbv[k] = 0.f; }
+#pragma unroll
+        for (int q = 1; q <= m; ++q) {
+            // s_q = q b - f a in (0, a], as the table builder takes it
+            int f = (int)floorf((float)q * b * inv_a);
+            float s = __fmaf_rn((float)(-f), a, (float)q * b);
+            if (s <= 0.f) { f -= 1; s = __fmaf_rn((float)(-f), a, (float)q * b); }
+            else if (s > a) { f += 1; s = __fmaf_rn((float)(-f), a, (float)q * b); }
+            const float sg = s <= ln.s_base ? -1.f : 1.f;   // knots below the base interval look down
+            zsv[q - 1] = sg * ln.ua;
+            zbv[q - 1] = sg * (ln.ua - s);
+            // (a value of f outside the range only arises at s_q = 0 or a to
+            // rounding, where z_q vanishes)
+#pragma unroll
+            for (int k = 0; k < D; ++k) {
+                const bool can = k >= knot_f_lo(m, D, q) && k <= knot_f_hi(m, D, q);
+                g[q - 1][k] = (can && f == k) ? kap * knot_weight(m, q) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            zs[k] = f2pack(zsv[2 * k], zsv[2 * k + 1]);
+            zb[k] = f2pack(zbv[2 * k], zbv[2 * k + 1]);
+        }
+        ua = ln.ua;
+        ub = ln.ua - ln.s_base;
+        hp = ln.hp;
+        has_last = ln.has_last;
+        x_last = ln.x_end;
+        x_prev = has_last ? 0xffffffffu : ln.x_end;
     }
-    return b;
+
+    // One row at strip address sp (the run's first column).
+    __device__ __forceinline__ void row(long long W, float *sp, f2 &acc) const
+    {
+        const float xf = (float)(unsigned)W;
+                const bool on_last = has_last && (unsigned)W <= x_last, on_prev = (unsigned)W <= x_prev;
+        const float t = __fmaf_rn(xf, ua, ub);
+        const f2 tt = f2pack(t, t), xx = f2pack(xf, xf);
+        float z[2 * NQ];
+#pragma unroll
+        for (int k = 0; k < NQ; ++k) {
+            float d0, d1;
+            f2unpack(f2fma(xx, zs[k], zb[k]), d0, d1);
+            const f2 d = f2pack(fmaxf(d0, 0.f), fmaxf(d1, 0.f));
+            const f2 d2 = f2mul(d, d);
+            f2 w = f2mul(d2, d);                     // d^3
+            if constexpr (DEG == 2) w = f2mul(w, d2);                  // d^5
+            if constexpr (DEG == 3) w = f2mul(w, f2mul(d2, d2));       // d^7
+            f2unpack(w, z[2 * k], z[2 * k + 1]);
+        }
+        float Z[D];
+#pragma unroll
+        for (int f = 0; f < D; ++f) {
+            bool any = false;
+            Z[f] = 0.f;
+#pragma unroll
+            for (int q = 1; q <= m; ++q)
+                if (f >= knot_f_lo(m, D, q) && f <= knot_f_hi(m, D, q)) {
+                    Z[f] = any ? __fmaf_rn(g[q - 1][f], z[q - 1], Z[f]) : g[q - 1][f] * z[q - 1];
+                    any = true;
+                }
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            f2 e = C[p][0], phi = C[p][NC - 1];
+#pragma unroll
+            for (int f = 0; f < D; ++f)
+                if (2 * p + 1 - f >= 0 && 2 * p - f <= m) {
+                    // (scalar FMAs with immediate weights: packed ones need
+                    // two moves per weight pair and row, 4 % slower)
+                    float e0, e1;
+                    f2unpack(e, e0, e1);
+                    if (2 * p - f >= 0 && 2 * p - f <= m) e0 = __fmaf_rn(Z[f], knot_weight(m, 2 * p - f), e0);
+                    if (2 * p + 1 - f >= 0 && 2 * p + 1 - f <= m) e1 = __fmaf_rn(Z[f], knot_weight(m, 2 * p + 1 - f), e1);
+                    e = f2pack(e0, e1);
+                }
+#pragma unroll
+            for (int d = NC - 2; d >= 1; --d) phi = f2fma(phi, tt, C[p][d]);
+            phi = f2fma(phi, tt, e);
+            const bool on0 = 2 * p == N - 2 ? on_prev : true;
+            const bool on1 = 2 * p + 1 == N - 1 ? on_last : 2 * p + 1 == N - 2 ? on_prev : true;
+            if constexpr (ADJ) {
+                float v0, v1;
+                if constexpr (FIX) {
+                    int *ip = reinterpret_cast<int *>(sp);
+                    f2unpack(f2add(phi, f2pack(kFixMagic, kFixMagic)), v0, v1);
+                    // (adding zero instead of branching)
+                    red_shared_u32(ip + 2 * p, on0 ? __float_as_int(v0) - kFixMagicBits : 0);
+                    red_shared_u32(ip + 2 * p + 1, on1 ? __float_as_int(v1) - kFixMagicBits : 0);
+                } else {
+                    f2unpack(phi, v0, v1);
+                    if (on0) red_shared(sp + 2 * p, hp * v0);
+                    if (on1) red_shared(sp + 2 * p + 1, hp * v1);
+                }
+            } else {
+                float c0 = 0.f, c1 = 0.f;
+                if (on0) c0 = sp[2 * p];
+                if (on1) c1 = sp[2 * p + 1];
+                acc = f2fma(f2pack(c0, c1), phi, acc);
+            }
+        }
+        if constexpr (N & 1) {
+            float e = cl[0], phi = cl[NC - 1];
+#pragma unroll
+            for (int f = 0; f < D; ++f)
+                if (N - 1 - f <= m) e = __fmaf_rn(Z[f], knot_weight(m, N - 1 - f), e);
+#pragma unroll
+            for (int d = NC - 2; d >= 1; --d) phi = __fmaf_rn(phi, t, cl[d]);
+            phi = __fmaf_rn(phi, t, e);
+            if constexpr (ADJ) {
+                if constexpr (FIX) {
+                    red_shared_u32(reinterpret_cast<int *>(sp) + N - 1,
+                                   on_last ? __float_as_int(phi + kFixMagic) - kFixMagicBits : 0);
+                } else {
+                    if (on_last) red_shared(sp + N - 1, hp * phi);
+                }
+            } else {
+                float c = 0.f, a0, a1;
+                if (on_last) c = sp[N - 1];
+                f2unpack(acc, a0, a1);
+                acc = f2pack(__fmaf_rn(c, phi, a0), a1);
+            }
+        }
+    }
+};
+
+// The same for the 3-direction box-spline: at most three breakpoints, across
+// which the first two derivatives jump (the first one where a box is as
+// narrow as a Dirac), per candidate as the table's polynomials differ.
+template <int N, bool ADJ, bool FIX>
+struct BoxRows {
+    static constexpr int F = 32, NB = 3;
+    float c[N][3], j1[NB][N], j2[NB][N];
+    float zs[NB], zb[NB];
+    float ua, ub, hp;
+    unsigned x_last, x_prev;
+    bool has_last;
+
+    __device__ __forceinline__ void load(const LaneLine &ln, const float *tab)
+    {
+        float s[NB + 1];
+        s[0] = 0.f;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) s[k + 1] = fminf(tab[k], ln.a);
+        const float sc = FIX ? ln.hp : 1.f;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) c[i][d] = ln.base[i * kNC + d] * sc;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            // breakpoint s[k + 1] between the intervals k and k + 1
+            const float L = s[k + 1] - s[k];
+            const float sg = s[k + 1] <= ln.s_base ? -1.f : 1.f;
+            zs[k] = sg * ln.ua;
+            zb[k] = sg * (ln.ua - s[k + 1]);
+            const bool real = s[k + 1] < ln.a;
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const float *lo = tab + tab_poly(k, i), *hi = tab + tab_poly(k + 1, i);
+                const float d1 = hi[1] - __fmaf_rn(2.f * lo[2], L, lo[1]), d2 = hi[2] - lo[2];
+                j1[k][i] = real ? d1 * sc : 0.f;
+                j2[k][i] = real ? sg * d2 * sc : 0.f;
+            }
+        }
+        ua = ln.ua;
+        ub = ln.ua - ln.s_base;
+        hp = ln.hp;
+        has_last = ln.has_last;
+        x_last = ln.x_end;
+        x_prev = has_last ? 0xffffffffu : ln.x_end;
+    }
+
+    __device__ __forceinline__ void row(long long W, float *sp, f2 &acc) const
+    {
+        const float xf = (float)(unsigned)W;
+        const bool on_last = has_last && (unsigned)W <= x_last, on_prev = (unsigned)W <= x_prev;
+        const float t = __fmaf_rn(xf, ua, ub);
+        float d[NB], dd[NB], a0, a1;
+        f2unpack(acc, a0, a1);
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            d[k] = fmaxf(__fmaf_rn(xf, zs[k], zb[k]), 0.f);
+            dd[k] = d[k] * d[k];
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            float phi = __fmaf_rn(__fmaf_rn(c[i][2], t, c[i][1]), t, c[i][0]);
+#pragma unroll
+            for (int k = 0; k < NB; ++k) phi = __fmaf_rn(j1[k][i], d[k], __fmaf_rn(j2[k][i], dd[k], phi));
+            const bool on = i == N - 1 ? on_last : i == N - 2 ? on_prev : true;
+            if constexpr (ADJ) {
+                if constexpr (FIX) {
+                    if (on) red_shared_u32(reinterpret_cast<int *>(sp) + i, __float_as_int(phi + kFixMagic) - kFixMagicBits);
+                } else {
+                    if (on) red_shared(sp + i, hp * phi);
+                }
+            } else {
+                float v = 0.f;
+                if (on) v = sp[i];
+                if (i & 1) a1 = __fmaf_rn(v, phi, a1);
+                else a0 = __fmaf_rn(v, phi, a0);
+            }
+        }
+        acc = f2pack(a0, a1);
+    }
+};
+
+// The strip's row blocks [b0, b1) of this lane's line.  Forward: adds their
+// sums to (hi, lo).
+template <typename Rows>
+__device__ __forceinline__ void walk_blocks(const Rows &R, const LaneLine &ln, const Strip &st, int b0, int b1, bool adj,
+                                            float &hi, float &lo)
+{
+    long long W = ln.W0 + (long long)(b0 * kRowBlock) * ln.Wstep;
+    for (int b = b0; b < b1; ++b) {
+        f2 acc = 0ull;
+        int rr = b * kRowBlock;
+#pragma unroll
+        for (int k = 0; k < kRowBlock; ++k, ++rr) {
+            float *sp = st.p + (rr * st.pitch + (ln.q_ref - (int)(W >> Rows::F) - st.first(rr)));
+            R.row(W, sp, acc);
+            W += ln.Wstep;
+        }
+        if (!adj) {
+            float a0, a1;
+            f2unpack(acc, a0, a1);
+            pair_add(hi, lo, a0 + a1);
+        }
+    }
 }
 
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// ------------------------------------------------------------------ degree 0
+// Degree 0 has at most two candidates per row and two intervals; its lanes
+// select the (linear) polynomials.  Its footprint can have ramps far narrower
+// than one float ulp of u, so W carries 48 fractional bits.
+constexpr int kFrac0 = 48;
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+// One row of a degree-0 line exactly along an axis (kDeg0Axis), whose
+// footprint is a rectangle with edges on nodes, each taking the midpoint value
+// on both sides (so a row has one more candidate): straight from or to global
+// memory.  Such lines occur only at views exactly along an axis.
+__device__ __noinline__ float axis_row0(const LineHdr &H, const float *tab, int r, const float *__restrict__ src,
+                                        float *dst, int Nq, float hp, bool adj)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-                 "l"(src)
-                 : "memory");
+    const float inv_a = 1.0f / H.a;
+    float s0[1] = {tab[0]};
+    float acc = 0.f;
+    const RowEval e = row_eval<0>(H, s0, inv_a, r);
+    for (int i = -1; i < H.K; ++i) {
+        const int q = e.q0 + i;
+        if ((unsigned)q >= (unsigned)Nq) continue;
+        float phi;
+        if (i < 0) {
+            if (!e.tie) continue;
+            phi = 0.5f * inv_a;   // the run also starts at u = 0
+        } else {
+            phi = horner<0>(tab + tab_poly(e.sg, i), __fmaf_rn((float)i, H.a_corr, e.t));
+            if (e.tie) phi = 0.5f * phi;
+        }
+        if (adj) atomicAdd(dst + (size_t)r * Nq + q, hp * phi);
+        else acc = __fmaf_rn(__ldg(src + (size_t)r * Nq + q), phi, acc);
+    }
+    return acc;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-constexpr int kTabLines = (kTabFloats * 4 + 127) / 128;   // 128-byte lines of one table
+template <bool ADJ, bool FIX>
+struct PixelRows {
+    static constexpr int F = kFrac0;
+    // c0 + c1 t of candidates 0 and 1 in the intervals 0 and 1 (candidate 1
+    // with its argument shift |kappa| - a folded in)
+    float c0[2][2], c1[2][2];
+    unsigned long long S1;   // the interval's boundary
+    float ua, hp;
+    bool has_last;
 
-// First and last column of the run of line H in row r, for a run of K nodes.
-__device__ __forceinline__ void run_columns(const LineHdr &H, float inv_a, int r, int &lo, int &hi)
+    __device__ __forceinline__ void load(const LaneLine &ln, const float *tab, float a_corr)
+    {
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float *T = tab + tab_poly(sg, i);
+                c1[sg][i] = T[1];
+                c0[sg][i] = i ? __fmaf_rn(T[1], a_corr, T[0]) : T[0];
+                if constexpr (FIX) {
+                    c0[sg][i] = __fmaf_rn(c0[sg][i], ln.hp, kFixMagic);
+                    c1[sg][i] *= ln.hp;
+                }
+            }
+        const float s = tab[0], a = ln.a, inv_a = 1.0f / a;
+        const float q1 = fminf(s * inv_a, 2.f);
+        const float r = fminf(__fmaf_rn(-q1, a, s) * inv_a, 1.f);
+        S1 = (unsigned long long)max(__float2ll_rn(q1 * 281474976710656.f) + __float2ll_rn(r * 281474976710656.f), 0ll);
+        ua = ln.ua;
+        hp = ln.hp;
+        has_last = ln.has_last;
+    }
+
+    __device__ __forceinline__ void row(long long W, float *sp, f2 &acc) const
+    {
+        const unsigned long long x = (unsigned long long)W & ((1ull << kFrac0) - 1ull);
+        const bool up = x >= S1, on_last = has_last && !up;   // candidate 1 ends with interval 0
+        const float t = (float)(x - (up ? S1 : 0ull) + 1ull) * ua;
+        const float p0 = __fmaf_rn(up ? c1[1][0] : c1[0][0], t, up ? c0[1][0] : c0[0][0]);
+        const float p1 = __fmaf_rn(up ? c1[1][1] : c1[0][1], t, up ? c0[1][1] : c0[0][1]);
+        if constexpr (FIX) {
+            red_shared_u32(reinterpret_cast<int *>(sp), __float_as_int(p0) - kFixMagicBits);
+            if (on_last) red_shared_u32(reinterpret_cast<int *>(sp) + 1, __float_as_int(p1) - kFixMagicBits);
+        } else if constexpr (ADJ) {
+            red_shared(sp, hp * p0);
+            if (on_last) red_shared(sp + 1, hp * p1);
+        } else {
+            float v = 0.f;
+            if (on_last) v = sp[1];
+            acc = f2fma(f2pack(sp[0], v), f2pack(p0, p1), acc);
+        }
+    }
+};
+
+// ------------------------------------------------------------------ chunks
+// The rows of this lane's line on a strip, blocks [b0, b1) (none where the
+// lane has no line): loads the line's polynomials and walks.  n: the
+// candidates of the warp's lines (the most).
+template <int KIND, bool ADJ, bool FIX>
+__device__ __forceinline__ void strip_line(int n, const LaneLine &ln, const LineHdr &H, const float *tab, const Strip &st,
+                                           int S0, int b0, int b1, const float *__restrict__ src, float *dst, int Nq,
+                                           float hp_raw, float &hi, float &lo)
 {
-    int k;
-    row_start(H, inv_a, r, k);
-    const int sgn = (H.flags & kKapNeg) ? -1 : 1;
-    const int q0 = H.q_ref - sgn * k;
-    const int q1 = q0 + sgn * (H.K - 1);
-    lo = min(q0, q1);
-    hi = max(q0, q1);
+    if constexpr (KIND == 0) {
+        if (H.flags & kDeg0Axis) {
+            for (int b = b0; b < b1; ++b) {
+                float acc = 0.f;
+                for (int r = max(S0 + b * kRowBlock, H.r_begin); r < min(S0 + (b + 1) * kRowBlock, H.r_end); ++r)
+                    acc += axis_row0(H, tab, r, src, dst, Nq, hp_raw, ADJ);
+                pair_add(hi, lo, acc);
+            }
+            return;
+        }
+        PixelRows<ADJ, FIX> R;
+        R.load(ln, tab, H.a_corr);
+        walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
+    } else if constexpr (KIND == kKindBox) {
+        switch (n) {
+        case 6: { BoxRows<6, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        case 5: { BoxRows<5, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        case 4: { BoxRows<4, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        default: { BoxRows<3, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        }
+    } else {
+        constexpr int m = KIND + 1;
+        switch (n - m) {
+        case 4: if constexpr (m >= 4) { SplineRows<KIND, m >= 4 ? 4 : 1, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); } break;
+        case 3: if constexpr (m >= 3) { SplineRows<KIND, m >= 3 ? 3 : 1, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); } break;
+        case 2: { SplineRows<KIND, 2, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        default: { SplineRows<KIND, 1, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        }
+    }
 }
 
-// Copy the first n16 16-byte chunks of a footprint table (all kTabFloats / 4
-// of them, or its head alone) to shared memory.
-__device__ __forceinline__ void table_copy_async(float *dst, const float *src, int lane, int n16 = kTabFloats / 4)
+// The fewest candidates that strip_line is instantiated for.
+template <int KIND>
+__device__ __forceinline__ int fewest_slots() { return KIND == 0 ? 2 : KIND == kKindBox ? 3 : KIND + 2; }
+
+// Adds the accumulated strip into the image: 16-byte reductions where the
+// image rows allow it.
+__device__ __forceinline__ void strip_flush(const Strip &st, int S0, int Nr, int Nq, float *dst, bool fixed, float finv,
+                                            int vec)
 {
-    for (int i = lane; i < n16; i += 32) cp_async16(dst + 4 * i, src + 4 * i);
+    if (vec) {
+        const int nch = st.pitch / 4;
+        const unsigned inv = 0xffffffffu / (unsigned)nch + 1u;   // i / nch = umulhi(i, inv) for every strip index
+        for (int i = threadIdx.x; i < st.rows * nch; i += kThreads) {
+            const int rr = (int)__umulhi((unsigned)i, inv), q = st.first(rr) + 4 * (i - rr * nch);
+            const int4 n4 = reinterpret_cast<const int4 *>(st.p)[i];
+            float4 v = make_float4(__int_as_float(n4.x), __int_as_float(n4.y), __int_as_float(n4.z), __int_as_float(n4.w));
+            if (fixed)
+                v = make_float4((float)n4.x * finv, (float)n4.y * finv, (float)n4.z * finv, (float)n4.w * finv);
+            if ((unsigned)q < (unsigned)Nq && S0 + rr < Nr && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f))
+                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)(S0 + rr) * Nq + q),
+                             "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                             : "memory");
+        }
+    } else {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int rr = warp; rr < st.rows && S0 + rr < Nr; rr += kWarps)
+            for (int c = lane; c < st.pitch; c += 32) {
+                const int w = reinterpret_cast<const int *>(st.p)[rr * st.pitch + c], q = st.first(rr) + c;
+                const float v = fixed ? (float)w * finv : __int_as_float(w);
+                if ((unsigned)q < (unsigned)Nq && v != 0.f) atomicAdd(dst + (size_t)(S0 + rr) * Nq + q, v);
+            }
+    }
+}
+
+// Stages the strip's coefficients, zeros outside the grid.
+__device__ __forceinline__ void strip_stage(const Strip &st, int S0, int Nr, int Nq, const float *__restrict__ src, int vec)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(st.p);
+    if (vec) {
+        // asynchronous 16-byte copies; chunks are wholly inside or outside the
+        // grid (Nq and chunk starts are multiples of 4)
+        const int nch = st.pitch / 4;
+        const unsigned inv = 0xffffffffu / (unsigned)nch + 1u;
+        for (int i = threadIdx.x; i < st.rows * nch; i += kThreads) {
+            const int rr = (int)__umulhi((unsigned)i, inv), q = st.first(rr) + 4 * (i - rr * nch);
+            const bool in = (unsigned)q < (unsigned)Nq && S0 + rr < Nr;
+            cp_async16(sa + 16 * i, in ? src + (size_t)(S0 + rr) * Nq + q : src, in);
+        }
+    } else {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int rr = warp; rr < st.rows; rr += kWarps)
+            for (int c = lane; c < st.pitch; c += 32) {
+                const int q = st.first(rr) + c;
+                const bool in = (unsigned)q < (unsigned)Nq && S0 + rr < Nr;
+                cp_async4(sa + 4 * (rr * st.pitch + c), in ? src + (size_t)(S0 + rr) * Nq + q : src, in);
+            }
+    }
 }
 
 // floor(a / b) for b > 0.
-__device__ __forceinline__ long long floor_div(long long a, long long b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
-
-// Prefetch `bytes` from p towards L2 (one 128-byte line per lane and pass).
-__device__ __forceinline__ void prefetch_span_l2(const unsigned char *p, int bytes, int lane)
-{
-    for (int o = lane * 128; o < bytes; o += 32 * 128) prefetch_l2(p + o);
-}
-
-// Phase B helpers of strip_line.  load_poly: the packed coefficients of
-// T[q][ci] (times hp for the adjoint; degree 0 with candidate ci's argument
-// shift ci (|kappa| - a) folded into the constant term).
-template <int DEG, bool ADJ, bool FIX = false>
-__device__ __forceinline__ void load_poly(const float *tabw, int q, int ci, float hp, float a_corr,
-                                          f2 (&C)[2 * DEG + 2])
-{
-    constexpr int NC = 2 * DEG + 2;
-    // T[sigma][ci]: 32-byte aligned (table buffers and entries are)
-    const float4 *Tq4 = reinterpret_cast<const float4 *>(tabw + tab_poly(q, ci));
-    float cq[NC];
-#pragma unroll
-    for (int d4 = 0; d4 < (NC + 3) / 4; ++d4) {
-        const float4 w = Tq4[d4];
-        const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (4 * d4 + u < NC) cq[4 * d4 + u] = wv[u];
-    }
-    if constexpr (DEG == 0) cq[0] = __fmaf_rn(cq[1], (float)ci * a_corr, cq[0]);
-#pragma unroll
-    for (int d = 0; d < NC; ++d) {
-        float c = ADJ ? cq[d] * hp : cq[d];
-        if (FIX && d == 0) c += kFixMagic;   // hp carries the chunk's scale S
-        C[d] = f2pack(c, c);
-    }
-}
-
-// run_group: the 4 sorted row records at e (one interval), two rows per packed
-// Horner chain; forward: acc2 += c phi from the strip; adjoint: reductions of
-// phi into the strip.
-template <int DEG, bool ADJ, bool FIX = false>
-__device__ __forceinline__ void run_group(const f2 (&C)[2 * DEG + 2], const float *ent_t, const int *ent_p, int e,
-                                          float *strip, int coloff, f2 &acc2)
-{
-    constexpr int NC = 2 * DEG + 2;
-    const ulonglong2 tt = *reinterpret_cast<const ulonglong2 *>(ent_t + e);
-    const int4 P = *reinterpret_cast<const int4 *>(ent_p + e);
-    f2 pa = C[NC - 1], pb = C[NC - 1];
-#pragma unroll
-    for (int d = NC - 2; d >= 0; --d) {
-        pa = f2fma(pa, tt.x, C[d]);
-        pb = f2fma(pb, tt.y, C[d]);
-    }
-    if constexpr (ADJ && FIX) {
-        float f0, f1, f2_, f3;
-        f2unpack(pa, f0, f1);
-        f2unpack(pb, f2_, f3);
-        int *istrip = reinterpret_cast<int *>(strip);
-        red_shared_u32(istrip + P.x + coloff, __float_as_int(f0) - kFixMagicBits);
-        red_shared_u32(istrip + P.y + coloff, __float_as_int(f1) - kFixMagicBits);
-        red_shared_u32(istrip + P.z + coloff, __float_as_int(f2_) - kFixMagicBits);
-        red_shared_u32(istrip + P.w + coloff, __float_as_int(f3) - kFixMagicBits);
-    } else if constexpr (ADJ) {
-        float f0, f1, f2_, f3;
-        f2unpack(pa, f0, f1);
-        f2unpack(pb, f2_, f3);
-        red_shared(strip + P.x + coloff, f0);
-        red_shared(strip + P.y + coloff, f1);
-        red_shared(strip + P.z + coloff, f2_);
-        red_shared(strip + P.w + coloff, f3);
-    } else {
-        acc2 = f2fma(f2pack(strip[P.x + coloff], strip[P.y + coloff]), pa, acc2);
-        acc2 = f2fma(f2pack(strip[P.z + coloff], strip[P.w + coloff]), pb, acc2);
-    }
-}
-
-// Degree 0 exactly along an axis (kDeg0Axis): the footprint is a rectangle
-// whose edges fall on nodes, each taking the midpoint value on both sides, so
-// a row has one more candidate.  Such lines run lane per row straight from or
-// to global memory (as the general kernels do); they occur only at views
-// exactly along an axis.
-__device__ float strip_tie_line(const LineHdr &H, const float *tabw, int S0, int S1, int lane,
-                                const float *__restrict__ src, float *dst, int Nq, float hp, bool adj)
-{
-    const int sgn = (H.flags & kKapNeg) ? -1 : 1;
-    const float inv_a = 1.0f / H.a;
-    float s0[1] = {tabw[0]};
-    float acc = 0.f;
-    const int rb = max(H.r_begin, S0), re = min(H.r_end, S1);
-    for (int r = rb + lane; r < re; r += 32) {
-        const RowEval e = row_eval<0>(H, s0, inv_a, sgn, r);
-        for (int i = -1; i < H.K; ++i) {
-            const int q = e.q0 + sgn * i;
-            if ((unsigned)q >= (unsigned)Nq) continue;
-            float phi;
-            if (i < 0) {
-                if (!e.tie) continue;
-                phi = 0.5f * inv_a;   // the run also starts at u = 0
-            } else {
-                phi = horner<0>(tabw + tab_poly(e.sg, i), __fmaf_rn((float)i, H.a_corr, e.t));
-                if (e.tie) phi = 0.5f * phi;
-            }
-            if (adj) atomicAdd(dst + (size_t)r * Nq + q, hp * phi);
-            else acc = __fmaf_rn(__ldg(src + (size_t)r * Nq + q), phi, acc);
-        }
-    }
-    return acc;
-}
-
-// One line over the strip rows [S0, S1).  Forward (ADJ false): returns this
-// lane's part of sum_k c_k phi (no factor h).  Adjoint: adds hp * phi into the
-// strip.  tabw is the line's table in shared memory; ent_t / ent_p hold the
-// warp's sorted row records (t, strip offset of candidate 0).  FIX: the
-// adjoint's fixed-point strip (hpS = hp S); RM: the row-record mode.
-// A row whose run fell outside the staged window: its candidates straight
-// from (forward; returns the partial sum) or to (adjoint) global memory, and
-// counted.  Kept out of line: it runs only on geometries the windows do not
-// anticipate, and inlined into every unrolled row of phase A it only
-// lengthened the kernel.
-template <int DEG, bool ADJ>
-__device__ __noinline__ float strip_slow_row(const float *tabw, int sg, float t, int q0, int sgn, int K, float a_corr,
-                                             int r, int Nq, const float *__restrict__ src, float *dst, float hp,
-                                             int *err)
-{
-    atomicAdd(err, 1);
-    const float *T0 = tabw + tab_poly(sg, 0);
-    float acc = 0.f;
-    for (int i = 0; i < K; ++i) {
-        const int q = q0 + sgn * i;
-        if ((unsigned)q < (unsigned)Nq) {
-            const float ti = (DEG == 0) ? __fmaf_rn((float)i, a_corr, t) : t;
-            const float phi = horner<DEG>(T0 + i * kNC, ti);
-            if constexpr (ADJ) atomicAdd(dst + (size_t)r * Nq + q, hp * phi);
-            else acc = __fmaf_rn(__ldg(src + (size_t)r * Nq + q), phi, acc);
-        }
-    }
-    return acc;
-}
-
-template <int DEG, bool ADJ, bool FIX = false, int RM = kRecNone>
-__device__ float strip_line(const LineHdr &H, const float *tabw, float *ent_t, int *ent_p, float *strip, const int *clo,
-                            int S0, int S1, int lane, const float *__restrict__ src, float *dst, int Nq,
-                            int *err, float hp, float hpS, unsigned char *&rp, const unsigned char *rend)
-{
-    constexpr int rmode = RM;
-    constexpr int NC = 2 * DEG + 2;
-    constexpr int NS = DEG + 2;       // intervals sigma
-    if constexpr (DEG == 0)
-        if (H.flags & kDeg0Axis) return strip_tie_line(H, tabw, S0, S1, lane, src, dst, Nq, hp, ADJ);
-    const int sgn = (H.flags & kKapNeg) ? -1 : 1;
-    const float inv_a = 1.0f / H.a;
-    float s[DEG + 1];
-#pragma unroll
-    for (int q = 0; q <= DEG; ++q) s[q] = tabw[q];
-    const int K = H.K;
-    // phase B lane roles: candidate ci of row slot sl (nsl slots of K lanes)
-    const int rk = (int)ceilf(256.0f * __frcp_rn((float)K));   // ceil(256 / K): (l * rk) >> 8 == l / K for l < 32, K <= 8
-    const int nsl = (32 * rk) >> 8;
-    const int sl = (lane * rk) >> 8;
-    const int ci = lane - sl * K;
-    const bool lane_on = sl < nsl;
-    const int coloff = sgn * ci;
-    f2 acc2 = 0ull;
-    float acc_slow = 0.f;
-    // a run fits the strip row iff its first column oq satisfies
-    // oq_lo <= oq <= oq_lo + kPitch - K (the run spans oq .. oq + sgn (K - 1))
-    const int oq_lo = sgn > 0 ? 0 : K - 1;
-    const unsigned oq_span = (unsigned)(kPitch - K);
-    // Row stepping in fixed point (degree >= 1): W(r) = 2^32 u(r)/a - 1 as a
-    // 64-bit integer, u(r) = U0 + (r - r_ref) rho the offset of row r at
-    // column q_ref.  Its high word is the row's step count k (u_0 = u - k a
-    // in (0, a]) and u_0 = (low word + 1) a 2^-32.  rho/a and U0/a enter as
-    // float pairs (one correction step of the float quotient), rounded to 32
-    // fractional bits: over 2^11 rows that is within 2^-21 a of the exact u_0.
-    long long Wstep = 0, Wbase = 0;
-    float ua = 0.f;
-    if constexpr (DEG >= 1) {
-        auto fix_quot = [&](float xh, float xl) {
-            const float q1 = xh * inv_a;
-            const float r = __fmaf_rn(-q1, H.a_lo, __fmaf_rn(-q1, H.a_hi, xh) + xl);
-            const float q2 = r * inv_a;
-            return __float2ll_rn(q1 * 4294967296.f) + __float2ll_rn(q2 * 4294967296.f);
-        };
-        Wstep = fix_quot(H.rho_hi, H.rho_lo);
-        Wbase = fix_quot(H.U0, H.U0_lo) - 1 - (long long)H.r_ref * Wstep;
-        ua = H.a * 2.3283064365386963e-10f;   // a 2^-32
-    }
-
-    const int dummy_pos = kSlabRows * kPitch + kDummy / 2;
-    const int rb = max(H.r_begin, S0), re = min(H.r_end, S1);
-    for (int r0 = rb; r0 < re; r0 += kBatch) {
-        int segb[NS], segn[NS];   // segment start and padded length (a multiple of 4)
-        bool ready = false;
-        if (rmode == kRecRead && rp + 16 <= rend) {
-            // the batch as the record pass left it: header, then its t and offsets
-            const int4 hd = __ldg(reinterpret_cast<const int4 *>(rp));
-            const int R = rec_unpack(hd, segb, segn);
-            const bool slow = (hd.w >> 16) != 0;
-            if (!slow) {
-                const float4 *gt = reinterpret_cast<const float4 *>(rp + 16);
-                const int4 *gp = reinterpret_cast<const int4 *>(rp + 16 + 4 * R);
-                for (int i = lane; i < R / 4; i += 32) {
-                    reinterpret_cast<float4 *>(ent_t)[i] = __ldg(gt + i);
-                    reinterpret_cast<int4 *>(ent_p)[i] = __ldg(gp + i);
-                }
-                __syncwarp();
-                ready = true;
-            }
-            rp += 16 + 8 * (slow ? 0 : R);   // a flagged batch was stored without records
-        }
-        if (!ready) {
-        // ---- A: lane per row
-        float tv[kRowsPerLane];
-        int pv[kRowsPerLane];
-        unsigned long long own = 0ull;
-        long long W = Wbase + (long long)(r0 + lane) * Wstep;   // W of this lane's first row
-#pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j) {
-            const int r = r0 + j * 32 + lane;
-            const long long Wr = W;
-            W += 32 * Wstep;
-            tv[j] = 0.f;
-            pv[j] = -1;
-            if (r < re) {
-                RowEval e;
-                if constexpr (DEG == 0) {
-                    e = row_eval<0>(H, s, inv_a, sgn, r);
-                } else {
-                    const int k = (int)(Wr >> 32);
-                    const float u0 = __fmaf_rn((float)(unsigned)Wr, ua, ua);
-                    float s_lo;
-                    e.sg = sigma_of<DEG>(s, u0, s_lo);
-                    e.t = u0 - s_lo;
-                    e.q0 = H.q_ref - sgn * k;
-                }
-                const int rr = r - S0;
-                const int oq = e.q0 - clo[rr];
-                if ((unsigned)(oq - oq_lo) <= oq_span) {
-                    tv[j] = e.t;
-                    pv[j] = (rr * kPitch + oq) | (e.sg << 16);
-                    own += 1ull << (9 * e.sg);
-                } else if (rmode == kRecWrite) {
-                    // the replay recomputes this batch (and reaches global memory then)
-                    own |= kRecSlowBit;
-                } else {
-                    // run outside the staged window: straight from or to global memory
-                    acc_slow += strip_slow_row<DEG, ADJ>(tabw, e.sg, e.t, e.q0, sgn, K, H.a_corr, r, Nq, src, dst,
-                                                         hp, err);
-                }
-            }
-        }
-        // counting sort by sigma: 9-bit counters per interval, packed
-        const bool slow_batch = rmode == kRecWrite && __any_sync(0xffffffffu, (own & kRecSlowBit) != 0ull);
-        own &= ~kRecSlowBit;
-        unsigned long long inc = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        const unsigned long long tot = __shfl_sync(0xffffffffu, inc, 31);
-        unsigned long long basep = 0ull;
-        {
-            int b = 0;
-#pragma unroll
-            for (int q = 0; q < NS; ++q) {
-                const int c = (int)((tot >> (9 * q)) & 511ull);
-                const int cp = (c + 3) & ~3;
-                segb[q] = b;
-                segn[q] = cp;
-                basep |= (unsigned long long)b << (9 * q);
-                // padding records (t = 0, zero target) complete the segment
-                if (lane < cp - c) { ent_t[b + c + lane] = 0.f; ent_p[b + c + lane] = dummy_pos; }
-                b += cp;
-            }
-        }
-        unsigned long long cur = basep + (inc - own);
-#pragma unroll
-        for (int j = 0; j < kRowsPerLane; ++j) {
-            if (pv[j] >= 0) {
-                const int sh = 9 * (pv[j] >> 16);
-                const int idx = (int)((cur >> sh) & 511ull);
-                cur += 1ull << sh;
-                ent_t[idx] = tv[j];
-                ent_p[idx] = pv[j] & 0xffff;
-            }
-        }
-        __syncwarp();
-        if (rmode == kRecWrite) {
-            // store the batch for the replays: header, t[R], offsets[R] (a
-            // batch that would not fit the line's region is stored flagged,
-            // without records; past its end nothing is stored, and the
-            // replay, reading the same positions, recomputes those batches)
-            if (rp + 16 > rend) continue;
-            int R = 0;
-#pragma unroll
-            for (int q = 0; q < NS; ++q) R += segn[q];
-            const bool flag = slow_batch || rp + 16 + 8 * R > rend;
-            if (flag) R = 0;
-            if (lane == 0) *reinterpret_cast<int4 *>(rp) = rec_pack(segn, flag);
-            float4 *gt = reinterpret_cast<float4 *>(rp + 16);
-            int4 *gp = reinterpret_cast<int4 *>(rp + 16 + 4 * R);
-            for (int i = lane; i < R / 4; i += 32) {
-                gt[i] = reinterpret_cast<const float4 *>(ent_t)[i];
-                gp[i] = reinterpret_cast<const int4 *>(ent_p)[i];
-            }
-            rp += 16 + 8 * R;
-            __syncwarp();
-            continue;
-        }
-        }   // !ready
-        // ---- B: lane per (candidate, row slot), four rows per step
-        if (lane_on) {
-            f2 C[NC];
-            // one interval at a time (an interval's last step may leave some
-            // row slots idle; walking the concatenated intervals instead costs
-            // a segment test per step and was slower in both directions once
-            // the adjoint's reductions became integer ones)
-#pragma unroll
-            for (int q = 0; q < NS; ++q) {
-                const int n = segn[q];
-                if (n == 0) continue;
-                load_poly<DEG, ADJ, FIX>(tabw, q, ci, FIX ? hpS : hp, H.a_corr, C);
-                const int end = segb[q] + n;
-                for (int e = segb[q] + 4 * sl; e < end; e += 4 * nsl)
-                    run_group<DEG, ADJ, FIX>(C, ent_t, ent_p, e, strip, coloff, acc2);
-            }
-        }
-        __syncwarp();
-    }
-    if constexpr (ADJ) {
-        return 0.f;
-    } else {
-        float a0, a1;
-        f2unpack(acc2, a0, a1);
-        return (a0 + a1) + acc_slow;
-    }
-}
+__device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 // Forward (ADJ false): sino[line] = h sum c phi.  Adjoint (ADJ true): adds
 // h sino[line] phi to out (vertical lines) or outT (horizontal lines, the
@@ -531,364 +732,241 @@ __device__ float strip_line(const LineHdr &H, const float *tabw, float *ent_t, i
 // FM (adjoint only) picks the chunks a call runs: kFmFixed only those that
 // accumulate in fixed point, kFmFloat only the others (non-finite values, or
 // a scale outside the safe range; see the top of the file), with float
-// strips.  A launch of each covers every chunk, and the fixed-point kernel
-// carries no second copy of the line code (a second inlined copy, or a call
-// anywhere in the kernel, made the fixed-point adjoint about a tenth
-// slower).  The forward takes kFmAll.
-template <int DEG, bool ADJ, int RM = kRecNone, int FM = kFmAll>
+// strips; returns whether the chunk was one of them.  The forward takes
+// kFmAll.
+template <int KIND, bool ADJ, int FM = kFmAll>
 __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g, const LinesDev L,
                                             const LineHdr *__restrict__ hdr, const float *__restrict__ tabs,
                                             const float *__restrict__ coef, const float *__restrict__ coefT,
                                             float *__restrict__ sino, float *__restrict__ out,
-                                            float *__restrict__ outT, int chunks_per_view, int vec, int *err,
-                                            int chunk, unsigned char *rec = nullptr, long long rec_cap = 0)
+                                            float *__restrict__ outT, int chunks_per_view, int vec, int chunk,
+                                            const longlong2 *__restrict__ rec)
 {
-    constexpr int rmode = RM;
+    static_assert(!ADJ || FM != kFmAll, "the adjoint runs as fixed-point and float launches");
+    constexpr bool FIX = ADJ && FM == kFmFixed;
+    constexpr int F = KIND == 0 ? kFrac0 : 32;
     float *strip = reinterpret_cast<float *>(smem);
-    size_t o = kStripBytes;
-    int *clo = reinterpret_cast<int *>(smem + o);
-    o += kCloBytes;
-    unsigned char *warp_area = smem + o;
-    o += kWarps * kWarpBytes;
-    float *line_acc = reinterpret_cast<float *>(smem + o);
-    o += kAccBytes;
-    int *misc = reinterpret_cast<int *>(smem + o);
-    o += kMiscBytes;
-    int *gstack = misc + 8;   // pending line groups, (first | last << 8)
-    LineHdr *hdr_s = reinterpret_cast<LineHdr *>(smem + o);
-    o += kHdrBytes;
-    int *rec_off = reinterpret_cast<int *>(smem + o);   // per line: bytes of its records used so far
+    float *base_s = reinterpret_cast<float *>(smem + kStripBytes);
+    LineHdr *hdr_s = reinterpret_cast<LineHdr *>(smem + kStripBytes + kBaseBytes);
+    float2 *part_s = reinterpret_cast<float2 *>(smem + kStripBytes + kBaseBytes + kHdrBytes);   // [warp][line]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *tabbuf = reinterpret_cast<float *>(warp_area + warp * kWarpBytes);   // [2][kTabFloats]
-    float *ent_t = reinterpret_cast<float *>(warp_area + warp * kWarpBytes + 2 * kTabBufBytes);
-    int *ent_p = reinterpret_cast<int *>(ent_t + kEntCap);
     const int v = chunk / chunks_per_view, cb = chunk - v * chunks_per_view;
     const int j0 = cb * kChunk;
     const int64_t nd = chunk_bins(L);
     const int nl = (int)min((int64_t)kChunk, nd - j0);
-    // position of the chunk's first line (in the sorted order for free lists;
-    // records are kept by position), and lane l's line index in every warp
+    // position of the chunk's first line (in the sorted order for free lists),
+    // and lane l's line and table index in every warp (one table per view for
+    // parallel beams, else table = line)
     const int64_t line0 = (int64_t)v * nd + j0;
     const int my_line = lane < nl ? (L.order ? __ldg(L.order + line0 + lane) : (int)(line0 + lane)) : 0;
+    const bool shared_tab = L.kind == SP_LINES_PARALLEL;
+    const float *my_tab = tabs + (shared_tab ? (int64_t)v : (int64_t)my_line) * kTabFloats;
 
+    // The adjoint's values, and the chunk's fixed-point scale (a power of two;
+    // see the top of the file).  Non-finite values, or values so large or
+    // small that it leaves a safe exponent range, keep the float reductions.
+    float pv = 0.f, fscale = 1.f, finv = 1.f;
     if constexpr (ADJ) {
-        // The chunk's fixed-point scale S (a power of two; see the top of the
-        // file): misc[5] = 1 if the strip accumulates in fixed point, misc[6]
-        // and misc[7] the bits of S and 1/S.  Non-finite values, or values so
-        // large or small that S leaves a safe exponent range, keep the float
-        // reductions.
-        if (warp == 0) {
-            const float pv = lane < nl ? sino[my_line] : 0.f;
-            const bool bad = !isfinite(pv);
-            float pm = fabsf(pv);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-            const float top = kPhiBound * g.h * pm;   // largest |h p phi| of the chunk
-            // (an all-zero chunk counts as fixed point: its lines are skipped)
-            const bool fix = !__any_sync(0xffffffffu, bad) && (top == 0.f || (top >= 1e-20f && top <= 1e20f));
-            if (lane == 0) {
-                int e = 0;
-                if (fix && top > 0.f) {
-                    frexpf(kFixMax / top, &e);   // kFixMax / top in [2^(e-1), 2^e)
-                    e -= 1;                      // S = 2^e <= kFixMax / top
-                }
-                misc[5] = fix ? 1 : 0;
-                misc[6] = __float_as_int(ldexpf(1.f, e));
-                misc[7] = __float_as_int(ldexpf(1.f, -e));
-            }
-        }
-        __syncthreads();
-        const bool fx = misc[5] != 0;
-        static_assert(!ADJ || FM != kFmAll, "the adjoint runs as fixed-point and float launches");
-        if constexpr (FM == kFmFixed) {
-            if (!fx) return false;   // left to the float launch
-        } else if constexpr (FM == kFmFloat) {
-            if (fx) return false;    // done by the fixed-point launch
+        if (lane < nl) pv = sino[my_line];
+        // (bits of non-negative floats order like the floats; non-finite ones on top)
+        const unsigned pm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(pv)));
+        const float top = kPhiBound * g.h * __uint_as_float(pm);   // largest |h p phi| of the chunk
+        // (an all-zero chunk counts as fixed point: its lines are skipped)
+        const bool fix = pm < 0x7f800000u && (top == 0.f || (top >= 1e-20f && top <= 1e20f));
+        if (fix != FIX) return false;   // left to the other launch
+        if (FIX && top > 0.f) {
+            int e;
+            frexpf(kFixMax / top, &e);   // kFixMax / top in [2^(e-1), 2^e)
+            e -= 1;                      // S = 2^e <= kFixMax / top
+            fscale = ldexpf(1.f, e);
+            finv = ldexpf(1.f, -e);
         }
     }
 
-    if (!ADJ && threadIdx.x < kChunk) line_acc[threadIdx.x] = 0.f;
-    if (threadIdx.x < kChunk) rec_off[threadIdx.x] = 0;
-    if (!ADJ && threadIdx.x < kDummy) strip[kSlabRows * kPitch + threadIdx.x] = 0.f;
-    // the chunk's line records into shared memory, its tables towards L2
-    // (lines other than parallel beams have one table each, indexed by line)
-    static_assert(kChunk * 4 <= kThreads, "one pass over the chunk's line records");
+    // the chunk's line records into shared memory, and every line's base
+    // interval: the one that leaves u_0 the shortest way to the ends of (0, a]
+    static_assert(kChunk * 4 <= kThreads && sizeof(LineHdr) == 64, "one pass over the chunk's line records");
     {
         const int src = __shfl_sync(0xffffffffu, my_line, (threadIdx.x >> 2) & 31);
         if ((int)threadIdx.x < nl * 4)
             reinterpret_cast<int4 *>(hdr_s)[threadIdx.x] =
                 __ldg(reinterpret_cast<const int4 *>(hdr + src) + (threadIdx.x & 3));
     }
-    if (L.kind != SP_LINES_PARALLEL)
-        for (int i0 = 0; i0 < kChunk * kTabLines; i0 += kThreads) {
-            const int i = i0 + threadIdx.x;
-            const int src = __shfl_sync(0xffffffffu, my_line, min(i / kTabLines, kChunk - 1));
-            if (i < nl * kTabLines) prefetch_l2(tabs + (int64_t)src * kTabFloats + (i % kTabLines) * 32);
+    int sg_base = 0;
+    float s_base = 0.f;
+    if constexpr (KIND != 0) {
+        const float4 h0 = __ldg(reinterpret_cast<const float4 *>(my_tab));
+        const float a = __ldg(my_tab + kTabA);
+        const float s[5] = {h0.x, h0.y, h0.z, h0.w, a};
+        constexpr int NI = KIND == kKindBox ? 4 : KIND + 2;   // intervals
+        float lo = 0.f, best = FLT_MAX;
+#pragma unroll
+        for (int k = 0; k < NI; ++k) {
+            const float end = k < NI - 1 ? fminf(s[k], a) : a;
+            const float far = fmaxf(lo, a - end);
+            if (far < best && end > lo) { best = far; sg_base = k; s_base = lo; }
+            lo = end;
         }
-    bool fixed = false;
-    float fscale = 1.f, finv = 1.f;
+        // the base polynomials and the table head
+        const int nt = shared_tab ? 1 : nl;
+        constexpr int kCh = (kSigStride + kTabHead) / 4;
+        const unsigned ba = (unsigned)__cvta_generic_to_shared(base_s);
+        for (int i0 = warp * 32; i0 < nt * kCh; i0 += kThreads) {
+            const int i = i0 + lane, li = min(i / kCh, kChunk - 1), c = i - li * kCh;
+            const int sg = __shfl_sync(0xffffffffu, sg_base, li);
+            const int ti = shared_tab ? v : __shfl_sync(0xffffffffu, my_line, li);
+            const float *t = tabs + (int64_t)ti * kTabFloats;
+            if (i < nt * kCh)
+                cp_async16(ba + 4 * (li * kBasePitch + 4 * c),
+                           c < kSigStride / 4 ? t + tab_poly(sg, 0) + 4 * c : t + 4 * (c - kSigStride / 4));
+        }
+    }
+    if (!ADJ) part_s[warp * kChunk + lane] = make_float2(0.f, 0.f);
+    __syncthreads();
+
+    // this lane's line: W at its reference row, and the step per row
+    bool mine = false, mine_vert = false;
+    long long my_W = 0, my_step = 0;
+    int my_K = 0;
+    if (lane < nl) {
+        const LineHdr &H = hdr_s[lane];
+        mine = !(H.flags & kEmpty) && H.r_end > H.r_begin && (!ADJ || pv != 0.f);
+        mine_vert = (H.flags & kVert) != 0;
+        if (mine) {
+            if (rec) {
+                const longlong2 t = __ldg(rec + my_line);
+                my_W = t.x;
+                my_step = t.y;
+            } else {
+                row_stepping<F>(H, my_W, my_step);
+            }
+            my_K = max(H.K, fewest_slots<KIND>() - 1);
+        }
+    }
     for (int axis = 0; axis < 2; ++axis) {
-        __syncthreads();
-        if (ADJ && axis == 0) {
-            fixed = FM != kFmFloat && misc[5] != 0;
-            fscale = __int_as_float(misc[6]);
-            finv = __int_as_float(misc[7]);
-        }
-        if (warp == 0) {
-            bool mine = false;
-            if (lane < nl) {
-                const LineHdr &H = hdr_s[lane];
-                mine = !(H.flags & kEmpty) && (((H.flags & kVert) != 0) == (axis == 0)) && H.r_end > H.r_begin;
-                // (with kept records the groups must be those of the record pass,
-                // so lines with p = 0 stay in them and are skipped below)
-                if (ADJ && mine && rmode == kRecNone) mine = sino[my_line] != 0.f;
-            }
-            const unsigned mask = __ballot_sync(0xffffffffu, mine);
-            if (lane == 0) {
-                misc[0] = (int)mask;
-                if (mask) { gstack[0] = (__ffs(mask) - 1) | ((31 - __clz(mask)) << 8); misc[3] = 1; }
-                else misc[3] = 0;
-            }
-        }
-        __syncthreads();
-        const unsigned mask = (unsigned)misc[0];
-        if (mask == 0u) continue;
-        const bool vert = (axis == 0);
-        const int Nq = vert ? g.nx : g.ny;
+        const bool vert = axis == 0;
+        const unsigned mask = __ballot_sync(0xffffffffu, mine && mine_vert == vert);
+        const int Nq = vert ? g.nx : g.ny, Nr = vert ? g.ny : g.nx;
         const float *src = vert ? coef : coefT;
         float *dst = vert ? out : outT;
-        // Groups of lines whose runs fit the pitch; a group that is too wide
-        // (lines fanning out) is split in halves.
-        for (;;) {
-            __syncthreads();
-            const int sp = misc[3];
-            if (sp == 0) break;
-            const int top = gstack[sp - 1];
-            const int ga = top & 255, gb = top >> 8;
-            const unsigned span = (gb >= 31 ? 0xffffffffu : ((1u << (gb + 1)) - 1u)) & ~((1u << ga) - 1u);
-            const unsigned gmask = mask & span;
-            __syncthreads();
-            if (threadIdx.x == 0) { misc[3] = sp - 1; misc[4] = 0; }
-            if (gmask == 0u) continue;
-            const int first = __ffs(gmask) - 1, last = 31 - __clz(gmask);
-            const LineHdr Hf = hdr_s[first], Hl = hdr_s[last];
-            const float inv_af = 1.0f / Hf.a, inv_al = 1.0f / Hl.a;
-            // row range of the group (lane = line), and the widest window:
-            // the outermost runs move linearly with the row, so it is at an end
-            int R0 = INT_MAX, R1 = INT_MIN;
-            if ((gmask >> lane) & 1u) { R0 = hdr_s[lane].r_begin; R1 = hdr_s[lane].r_end; }
-#pragma unroll
-            for (int o2 = 16; o2 > 0; o2 >>= 1) {
-                R0 = min(R0, __shfl_xor_sync(0xffffffffu, R0, o2));
-                R1 = max(R1, __shfl_xor_sync(0xffffffffu, R1, o2));
+        // Groups: aligned spans of lines [ga, ga + len), len a power of two,
+        // whose runs fit a strip row and whose candidate slots differ by at
+        // most one; others are halved.  Every warp finds the same ones.
+        for (int ga = 0, len = kChunk; ga < kChunk; ga += len, len = ga & -ga) {
+            auto in_span = [&](int a, int n) { return mask & ((n >= 32 ? 0xffffffffu : (1u << n) - 1u) << a); };
+            if (in_span(ga, len) == 0u) continue;
+            int R0, R1, la, lb, n, width;
+            for (;;) {
+                // a half without lines is left out
+                while (len > 1 && in_span(ga + (len >> 1), len >> 1) == 0u) len >>= 1;
+                const bool in = (in_span(ga, len) >> lane) & 1u;
+                // row range of the group in whole blocks, and the lowest and
+                // highest run start of its lines in the first and the last
+                // row.  A run starts within one column above its line, and
+                // lines are straight, so between the two rows the starts stay
+                // within a column of the chords through the extremes.
+                R0 = __reduce_min_sync(0xffffffffu, in ? hdr_s[lane].r_begin : INT_MAX) & -kRowBlock;
+                R1 = (__reduce_max_sync(0xffffffffu, in ? hdr_s[lane].r_end : INT_MIN) + kRowBlock - 1) & -kRowBlock;
+                const int qa = in ? hdr_s[lane].q_ref - (int)((my_W + R0 * my_step) >> F) : 0;
+                const int qb = in ? hdr_s[lane].q_ref - (int)((my_W + (R1 - 1) * my_step) >> F) : 0;
+                la = __reduce_min_sync(0xffffffffu, in ? qa : INT_MAX);
+                lb = __reduce_min_sync(0xffffffffu, in ? qb : INT_MAX);
+                const int ha = __reduce_max_sync(0xffffffffu, in ? qa : INT_MIN);
+                const int hb = __reduce_max_sync(0xffffffffu, in ? qb : INT_MIN);
+                n = max(__reduce_max_sync(0xffffffffu, in ? my_K : 0), fewest_slots<KIND>());
+                const int nmin = __reduce_min_sync(0xffffffffu, in ? my_K : INT_MAX);
+                // 3 columns below the lowest start, 3 beyond the highest run,
+                // 3 for the start rounded down to a multiple of 4
+                width = (max(ha - la, hb - lb) + n + 9 + 3) & ~3;
+                if (len == 1 || (width <= kMaxWidth && n - nmin <= 1)) break;
+                len >>= 1;
+                if (in_span(ga, len) == 0u) ga += len;
             }
-            int wmax = 0;
-            // free lists: the extreme run columns over all lines of the group
-            // at the first and the last row (la..ha, lb..hb); between them the
-            // window follows the chords, which bound the runs: each run moves
-            // linearly with the row, so the lowest start is concave in the row
-            // and the highest end convex
-            int la = 0, ha = 0, lb = 0, hb = 0;
-            if (L.order) {
-                la = lb = INT_MAX;
-                ha = hb = INT_MIN;
-                if ((gmask >> lane) & 1u) {
-                    const LineHdr &Hx = hdr_s[lane];
-                    const float ia = 1.0f / Hx.a;
-                    run_columns(Hx, ia, R0, la, ha);
-                    run_columns(Hx, ia, R1 - 1, lb, hb);
-                }
-#pragma unroll
-                for (int o2 = 16; o2 > 0; o2 >>= 1) {
-                    la = min(la, __shfl_xor_sync(0xffffffffu, la, o2));
-                    ha = max(ha, __shfl_xor_sync(0xffffffffu, ha, o2));
-                    lb = min(lb, __shfl_xor_sync(0xffffffffu, lb, o2));
-                    hb = max(hb, __shfl_xor_sync(0xffffffffu, hb, o2));
-                }
-                wmax = max(ha - la, hb - lb) + 7;
-            } else {
-                int lo1, hi1, lo2, hi2;
-                run_columns(Hf, inv_af, R0, lo1, hi1);
-                run_columns(Hl, inv_al, R0, lo2, hi2);
-                wmax = max(hi1, hi2) - min(lo1, lo2) + 5;
-                run_columns(Hf, inv_af, R1 - 1, lo1, hi1);
-                run_columns(Hl, inv_al, R1 - 1, lo2, hi2);
-                wmax = max(wmax, max(hi1, hi2) - min(lo1, lo2) + 5);
+
+            // this lane's line of the group (groups of fewer than 32 lines:
+            // several lanes per line, on consecutive rows)
+            const int li = ga + (lane & (len - 1)), parts = kChunk / len;
+            const bool on = in_span(li, 1) != 0u;
+            const int lj = on ? li : __ffs(in_span(ga, len)) - 1;   // (a lane without one looks at another's)
+            const LineHdr &H = hdr_s[lj];
+            LaneLine ln;
+            ln.Wstep = __shfl_sync(0xffffffffu, my_step, lj);
+            const long long W_row0 = __shfl_sync(0xffffffffu, my_W, lj);
+            ln.q_ref = H.q_ref;
+            ln.one = __uint_as_float(0x3f800000u + (unsigned)(nd >> 62));
+            ln.a = H.a;
+            ln.ua = H.a * (F == 32 ? 2.3283064365386963e-10f : 3.5527136788005009e-15f);
+            const float hp_raw = ADJ ? g.h * __shfl_sync(0xffffffffu, pv, lj) : 0.f;
+            ln.hp = hp_raw * fscale;
+            ln.base = base_s + (shared_tab ? 0 : lj) * kBasePitch;
+            ln.s_base = __shfl_sync(0xffffffffu, s_base, lj);
+            ln.has_last = __shfl_sync(0xffffffffu, my_K, lj) >= n;
+            {
+                // 2w - (K - 1) a in units of a 2^-32
+                const float end = H.two_w / H.a - (float)(H.K - 1);
+                ln.x_end = end >= 1.f ? 0xffffffffu : (unsigned)(fmaxf(end, 0.f) * 4294967296.f);
             }
-            __syncthreads();
-            if (wmax > kWin && first < last) {
-                if (threadIdx.x == 0) {
-                    const int mid = (first + last) >> 1;
-                    const int s2 = misc[3];
-                    gstack[s2] = first | (mid << 8);
-                    gstack[s2 + 1] = (mid + 1) | (last << 8);
-                    misc[3] = s2 + 2;
-                }
-                continue;
-            }
-            for (int S0 = R0; S0 < R1; S0 += kSlabRows) {
-                const int S1 = min(S0 + kSlabRows, R1);
-                const int nrows = S1 - S0;
-                __syncthreads();
-                // window of each strip row from the two outermost lines of the
-                // group (lines of a view do not cross inside the grid), margin 2
-                for (int rr = threadIdx.x; rr < nrows; rr += kThreads) {
-                    int lo, hi;
-                    if (L.order) {
-                        // the chords, rounded outwards, margin 3 (a run lies
-                        // within one column of its line)
-                        const long long span = max(R1 - 1 - R0, 1), dr = S0 + rr - R0;
-                        lo = la + (int)floor_div((long long)(lb - la) * dr, span) - 3;
-                        hi = ha - (int)floor_div(-(long long)(hb - ha) * dr, span) + 3;
-                    } else {
-                        int lo1, hi1, lo2, hi2;
-                        run_columns(Hf, inv_af, S0 + rr, lo1, hi1);
-                        run_columns(Hl, inv_al, S0 + rr, lo2, hi2);
-                        lo = min(lo1, lo2) - 2;
-                        hi = max(hi1, hi2) + 2;
-                    }
-                    // centred in the usable width, start rounded down to a 16-byte chunk
-                    clo[rr] = (lo - max(0, (kWin - (hi - lo + 1)) / 2)) & ~3;
-                }
-                __syncthreads();
-                constexpr int kCh = kPitch / 4;   // 16-byte chunks per strip row
-                if (rmode == kRecWrite) {
-                    // the record pass projects nothing: no strip
-                } else if constexpr (ADJ) {
+            const float *tab = tabs + (shared_tab ? (int64_t)v : (int64_t)__shfl_sync(0xffffffffu, my_line, lj)) * kTabFloats;
+
+            Strip st;
+            st.p = strip;
+            st.pitch = width;
+            const int span = max(R1 - 1 - R0, 1);
+            st.slope = floor_div((lb - la) * (1 << kSlopeBits), span);
+            // slabs of equal height that the strip can hold
+            const int most = (kStripFloats / width) & -kRowBlock;
+            const int slabs = (R1 - R0 + most - 1) / most;
+            const int per = ((R1 - R0 + slabs - 1) / slabs + kRowBlock - 1) & -kRowBlock;
+            float hi = 0.f, lo = 0.f;
+            for (int S0 = R0; S0 < R1; S0 += per) {
+                st.rows = min(per, R1 - S0);
+                st.c0 = la + floor_div((lb - la) * (S0 - R0), span) - 3;
+                __syncthreads();   // the strip's last readers are done
+                if constexpr (ADJ) {
                     float4 *s4 = reinterpret_cast<float4 *>(strip);
-                    for (int i = threadIdx.x; i < nrows * kCh; i += kThreads) s4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                } else if (vec) {
-                    // asynchronous 16-byte copies; chunks are wholly inside or
-                    // outside the grid (Nq and chunk starts are multiples of 4)
-                    for (int i = threadIdx.x; i < nrows * kCh; i += kThreads) {
-                        const int rr = i / kCh, cc = i - rr * kCh;
-                        const int q = clo[rr] + 4 * cc;
-                        const bool in = (unsigned)q < (unsigned)Nq;
-                        const float *gp = in ? src + (size_t)(S0 + rr) * Nq + q : src;
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                                         (unsigned)__cvta_generic_to_shared(strip + 4 * i)),
-                                     "l"(gp), "r"(in ? 16 : 0)
-                                     : "memory");
-                    }
-                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    for (int i = threadIdx.x; i < st.rows * width / 4; i += kThreads) s4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 } else {
-                    // 4-byte copies, zero-filled outside the grid
-                    for (int i = threadIdx.x; i < nrows * kPitch; i += kThreads) {
-                        const int rr = i / kPitch, cc = i - rr * kPitch;
-                        const int q = clo[rr] + cc;
-                        const bool in = (unsigned)q < (unsigned)Nq;
-                        const float *gp = in ? src + (size_t)(S0 + rr) * Nq + q : src;
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                                         (unsigned)__cvta_generic_to_shared(strip + i)),
-                                     "l"(gp), "r"(in ? 4 : 0)
-                                     : "memory");
-                    }
-                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    strip_stage(st, S0, Nr, Nq, src, vec);
                 }
+                cp_async_wait_all();   // the strip's copies, and the base polynomials'
                 __syncthreads();
-                // this warp's lines of the group: li = first + warp + k kWarps in
-                // wmask (gmask less, in the adjoint with kept records, lines with
-                // p = 0); the table of the next one is loaded while the current
-                // one runs.  The record pass needs only each table's head (the
-                // interval ends s_q); replays prefetch a line's records one line
-                // ahead.
-                unsigned wmask = gmask;
-                if (ADJ && rmode == kRecRead) {
-                    const bool nz = lane < nl && sino[my_line] != 0.f;
-                    wmask &= __ballot_sync(0xffffffffu, nz);
-                }
-                int li = first + warp;
-                while (li <= last && !((wmask >> li) & 1u)) li += kWarps;
-                int buf = 0;
-                const int tab16 = rmode == kRecWrite ? kTabHead / 4 : kTabFloats / 4;
-                constexpr int kRecAhead = 4096;
-                if (li <= last) {
-                    table_copy_async(tabbuf, tabs + (int64_t)hdr_s[li].tab * kTabFloats, lane, tab16);
-                    cp_async_commit();
-                    if (rmode == kRecRead)
-                        prefetch_span_l2(rec + (line0 + li) * rec_cap + rec_off[li],
-                                         (int)min((long long)kRecAhead, rec_cap - rec_off[li]), lane);
-                }
-                while (li <= last) {
-                    int ln = li + kWarps;
-                    while (ln <= last && !((wmask >> ln) & 1u)) ln += kWarps;
-                    if (ln <= last) {
-                        table_copy_async(tabbuf + (buf ^ 1) * kTabFloats,
-                                         tabs + (int64_t)hdr_s[ln].tab * kTabFloats, lane, tab16);
-                        if (rmode == kRecRead)
-                            prefetch_span_l2(rec + (line0 + ln) * rec_cap + rec_off[ln],
-                                             (int)min((long long)kRecAhead, rec_cap - rec_off[ln]), lane);
-                    }
-                    cp_async_commit();
-                    cp_async_wait<1>();
-                    __syncwarp();
-                    const LineHdr H = hdr_s[li];
-                    const float hp = ADJ ? g.h * sino[__shfl_sync(0xffffffffu, my_line, li)] : 0.f;
-                    unsigned char *lrec = rec ? rec + (line0 + li) * rec_cap : nullptr;
-                    unsigned char *rp = lrec ? lrec + rec_off[li] : nullptr;
-                    const unsigned char *rend = lrec ? lrec + rec_cap : nullptr;
-                    float part;
-                    if constexpr (ADJ) {
-                        part = strip_line<DEG, true, FM != kFmFloat, RM>(H, tabbuf + buf * kTabFloats, ent_t, ent_p,
-                                                                         strip, clo, S0, S1, lane, src, dst, Nq, err,
-                                                                         hp, FM != kFmFloat ? hp * fscale : 0.f, rp,
-                                                                         rend);
-                    } else {
-                        part = strip_line<DEG, false, false, RM>(H, tabbuf + buf * kTabFloats, ent_t, ent_p, strip,
-                                                                 clo, S0, S1, lane, src, dst, Nq, err, hp, 0.f, rp,
-                                                                 rend);
-                    }
-                    if (!ADJ && rmode != kRecWrite) {
-                        const float sum = warp_sum(part);
-                        if (lane == 0) line_acc[li] += sum;
-                    }
-                    if (lrec && lane == 0) rec_off[li] = (int)(rp - lrec);
-                    __syncwarp();
-                    li = ln;
-                    buf ^= 1;
-                }
-                cp_async_wait<0>();
-                if (ADJ && rmode != kRecWrite) {
+                const int nb = st.rows / kRowBlock, unit = warp * parts + lane / len, units = kWarps * parts;
+                const int b0 = nb * unit / units, b1 = on ? nb * (unit + 1) / units : b0;
+                ln.W0 = W_row0 + S0 * ln.Wstep;
+                strip_line<KIND, ADJ, FIX>(n, ln, H, tab, st, S0, b0, b1, src, dst, Nq, hp_raw, hi, lo);
+                if constexpr (ADJ) {
                     __syncthreads();
-                    // add the accumulated strip into the image
-                    if (vec) {
-                        const float4 *s4 = reinterpret_cast<const float4 *>(strip);
-                        const int4 *i4 = reinterpret_cast<const int4 *>(strip);
-                        for (int i = threadIdx.x; i < nrows * kCh; i += kThreads) {
-                            const int rr = i / kCh, cc = i - rr * kCh;
-                            const int q = clo[rr] + 4 * cc;
-                            float4 v4;
-                            if (fixed) {
-                                const int4 n4 = i4[i];
-                                v4 = make_float4((float)n4.x * finv, (float)n4.y * finv, (float)n4.z * finv,
-                                                 (float)n4.w * finv);
-                            } else {
-                                v4 = s4[i];
-                            }
-                            if ((unsigned)q < (unsigned)Nq &&
-                                (v4.x != 0.f || v4.y != 0.f || v4.z != 0.f || v4.w != 0.f))
-                                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(
-                                                 dst + (size_t)(S0 + rr) * Nq + q),
-                                             "f"(v4.x), "f"(v4.y), "f"(v4.z), "f"(v4.w)
-                                             : "memory");
-                        }
-                    } else {
-                        for (int i = threadIdx.x; i < nrows * kPitch; i += kThreads) {
-                            const int rr = i / kPitch, cc = i - rr * kPitch;
-                            const int q = clo[rr] + cc;
-                            const float val = fixed ? (float)reinterpret_cast<const int *>(strip)[i] * finv : strip[i];
-                            if ((unsigned)q < (unsigned)Nq && val != 0.f)
-                                atomicAdd(dst + (size_t)(S0 + rr) * Nq + q, val);
-                        }
-                    }
+                    strip_flush(st, S0, Nr, Nq, dst, FIX, finv, vec);
+                }
+            }
+            if constexpr (!ADJ) {
+                for (int o = len; o < 32; o <<= 1) {
+                    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+                    pair_add(hi, lo, h2);
+                    lo += l2;
+                }
+                if (on && lane < len) {
+                    float2 t = part_s[warp * kChunk + li];
+                    pair_add(t.x, t.y, hi);
+                    part_s[warp * kChunk + li] = make_float2(t.x, t.y + lo);
                 }
             }
         }
     }
-    if (!ADJ && rmode != kRecWrite) {
+    cp_async_wait_all();   // (a chunk without lines still has its copies in flight)
+    if constexpr (!ADJ) {
         __syncthreads();
-        if ((int)threadIdx.x < nl) sino[my_line] = g.h * line_acc[threadIdx.x];   // warp 0: lane = line
+        if ((int)threadIdx.x < nl) {   // warp 0: lane = line
+            float hi = 0.f, lo = 0.f;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const float2 t = part_s[w * kChunk + lane];
+                pair_add(hi, lo, t.x);
+                lo += t.y;
+            }
+            sino[my_line] = g.h * (hi + lo);
+        }
     }
     return true;
 }
@@ -896,26 +974,26 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g
 // One CTA per chunk.  The adjoint runs the fixed-point chunks (FM kFmFixed:
 // nearly all) and appends the others to defer[2..] (count defer[0]) for
 // strip_float_kernel.
-template <int DEG, bool ADJ, int RM, int FM = kFmAll>
+template <int KIND, bool ADJ, int FM = kFmAll>
 __global__ void __launch_bounds__(kThreads, 2)
 strip_kernel(GridDev g, LinesDev L, const LineHdr *__restrict__ hdr, const float *__restrict__ tabs,
              const float *__restrict__ coef, const float *__restrict__ coefT, float *__restrict__ sino,
-             float *__restrict__ out, float *__restrict__ outT, int chunks_per_view, int vec, int *err,
-             unsigned char *rec, long long rec_cap, unsigned *defer)
+             float *__restrict__ out, float *__restrict__ outT, int chunks_per_view, int vec, unsigned *defer,
+             const longlong2 *__restrict__ rec)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const bool ran = strip_chunk<DEG, ADJ, RM, FM>(smem, g, L, hdr, tabs, coef, coefT, sino, out, outT,
-                                                   chunks_per_view, vec, err, (int)blockIdx.x, rec, rec_cap);
+    const bool ran = strip_chunk<KIND, ADJ, FM>(smem, g, L, hdr, tabs, coef, coefT, sino, out, outT, chunks_per_view,
+                                                vec, (int)blockIdx.x, rec);
     if (FM == kFmFixed && !ran && threadIdx.x == 0) defer[2 + atomicAdd(defer, 1u)] = blockIdx.x;
 }
 
 // The deferred adjoint chunks (float strip accumulators): a small persistent
 // grid over defer[2 .. 2 + defer[0]), defer[1] its counter.
-template <int DEG, int RM>
+template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2)
 strip_float_kernel(GridDev g, LinesDev L, const LineHdr *__restrict__ hdr, const float *__restrict__ tabs,
                    float *__restrict__ sino, float *__restrict__ out, float *__restrict__ outT, int chunks_per_view,
-                   int vec, int *err, unsigned char *rec, long long rec_cap, unsigned *defer)
+                   int vec, unsigned *defer, const longlong2 *__restrict__ rec)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned cur;
@@ -925,12 +1003,13 @@ strip_float_kernel(GridDev g, LinesDev L, const LineHdr *__restrict__ hdr, const
         if (threadIdx.x == 0) cur = atomicAdd(defer + 1, 1u);
         __syncthreads();
         if (cur >= n) break;
-        strip_chunk<DEG, true, RM, kFmFloat>(smem, g, L, hdr, tabs, nullptr, nullptr, sino, out, outT,
-                                             chunks_per_view, vec, err, (int)defer[2 + cur], rec, rec_cap);
+        strip_chunk<KIND, true, kFmFloat>(smem, g, L, hdr, tabs, nullptr, nullptr, sino, out, outT, chunks_per_view,
+                                          vec, (int)defer[2 + cur], rec);
     }
 }
 
-// Persistent kernel over the chunks of several instances of one degree: each
+// Persistent kernel over the chunks of several instances of one kind (B-spline
+// degree, or box-spline): each
 // CTA takes the next chunk from one counter (atomicAdd; no CTA waits on
 // another) and runs it with its instance's parameters, until every chunk is
 // taken.  Instance k owns chunks [jobs[k].chunk0, jobs[k + 1].chunk0).  The
@@ -949,7 +1028,7 @@ __device__ __forceinline__ const StripJob *queue_job(const StripJob *__restrict_
     return jobs + lo;
 }
 
-template <int DEG, bool ADJ>
+template <int KIND, bool ADJ>
 __global__ void __launch_bounds__(kThreads, 2)
 strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total, unsigned long long *counter,
                    long long *defer, unsigned long long *defer_n)
@@ -963,15 +1042,15 @@ strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total
         const long long c = cur;
         if (c >= total) break;
         const StripJob *J = queue_job(jobs, njobs, c);
-        const bool ran = strip_chunk<DEG, ADJ, kRecNone, ADJ ? kFmFixed : kFmAll>(
-            smem, J->g, J->L, J->hdr, J->tabs, J->coef, J->coefT, J->sino, J->out, J->outT, J->cpv, J->vec, J->err,
-            (int)(c - J->chunk0));
+        const bool ran = strip_chunk<KIND, ADJ, ADJ ? kFmFixed : kFmAll>(
+            smem, J->g, J->L, J->hdr, J->tabs, J->coef, J->coefT, J->sino, J->out, J->outT, J->cpv, J->vec,
+            (int)(c - J->chunk0), nullptr);
         if (ADJ && !ran && threadIdx.x == 0) defer[atomicAdd(defer_n, 1ull)] = c;
     }
 }
 
 // The deferred adjoint chunks (float strip accumulators), persistent likewise.
-template <int DEG>
+template <int KIND>
 __global__ void __launch_bounds__(kThreads, 2)
 strip_queue_float_kernel(const StripJob *__restrict__ jobs, int njobs, const long long *__restrict__ defer,
                          const unsigned long long *__restrict__ defer_n, unsigned long long *counter)
@@ -987,36 +1066,44 @@ strip_queue_float_kernel(const StripJob *__restrict__ jobs, int njobs, const lon
         if (k >= (long long)n) break;
         const long long c = defer[k];
         const StripJob *J = queue_job(jobs, njobs, c);
-        strip_chunk<DEG, true, kRecNone, kFmFloat>(smem, J->g, J->L, J->hdr, J->tabs, J->coef, J->coefT, J->sino,
-                                                   J->out, J->outT, J->cpv, J->vec, J->err, (int)(c - J->chunk0));
+        strip_chunk<KIND, true, kFmFloat>(smem, J->g, J->L, J->hdr, J->tabs, J->coef, J->coefT, J->sino,
+                                                   J->out, J->outT, J->cpv, J->vec, (int)(c - J->chunk0),
+                                         nullptr);
     }
 }
 
-template <int DEG>
+// 16-byte staging and flushing: image rows (nx and ny floats) and bases aligned.
+inline int strip_vec(const GridDev &g, const void *img, const void *imgT)
+{
+    return (g.nx % 4 == 0) && (g.ny % 4 == 0) && ((reinterpret_cast<uintptr_t>(img) & 15) == 0) &&
+           ((reinterpret_cast<uintptr_t>(imgT) & 15) == 0);
+}
+
+template <int KIND>
 cudaError_t launch_queue_t(bool adj, const StripJob *jobs, int njobs, int64_t total, unsigned long long *counter,
                            long long *defer, int64_t grid, int sms, cudaStream_t s)
 {
     cudaError_t e;
     if (adj) {
-        e = cudaFuncSetAttribute(strip_queue_kernel<DEG, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(strip_queue_kernel<KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kSmemBytes);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(strip_queue_float_kernel<DEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            e = cudaFuncSetAttribute(strip_queue_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemBytes);
         if (e != cudaSuccess) return e;
-        strip_queue_kernel<DEG, true><<<(unsigned)grid, kThreads, kSmemBytes, s>>>(jobs, njobs, (long long)total,
+        strip_queue_kernel<KIND, true><<<(unsigned)grid, kThreads, kSmemBytes, s>>>(jobs, njobs, (long long)total,
                                                                                   counter, defer, counter + 1);
         e = cudaGetLastError();
         // the deferred chunks are few (non-finite or extreme sinogram values): a small grid
         if (e == cudaSuccess)
-            strip_queue_float_kernel<DEG><<<(unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s>>>(
+            strip_queue_float_kernel<KIND><<<(unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s>>>(
                 jobs, njobs, defer, counter + 1, counter + 2);
         return e == cudaSuccess ? cudaGetLastError() : e;
     }
-    e = cudaFuncSetAttribute(strip_queue_kernel<DEG, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(strip_queue_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    strip_queue_kernel<DEG, false><<<(unsigned)grid, kThreads, kSmemBytes, s>>>(jobs, njobs, (long long)total, counter,
+    strip_queue_kernel<KIND, false><<<(unsigned)grid, kThreads, kSmemBytes, s>>>(jobs, njobs, (long long)total, counter,
                                                                                nullptr, nullptr);
     return cudaGetLastError();
 }
@@ -1052,20 +1139,15 @@ __global__ void add_transposed_kernel(const float *__restrict__ inT, float *__re
     }
 }
 
-template <int DEG, bool ADJ>
+template <int KIND, bool ADJ>
 cudaError_t launch_strip_t(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                           const float *coef, float *imgT, float *sino, float *out, int *err, cudaStream_t s,
-                           const StripRec *rec = nullptr, int rmode = kRecNone, unsigned *defer = nullptr)
+                           const float *coef, float *imgT, float *sino, float *out, cudaStream_t s, const longlong2 *rec,
+                           unsigned *defer = nullptr)
 {
     const dim3 tb(32, 8), tg((g.nx + 31) / 32, (g.ny + 31) / 32);
     cudaError_t e;
-    unsigned char *rb = (rec && rmode != kRecNone) ? rec->base : nullptr;
-    const long long rcap = rb ? rec->line_bytes : 0;
-    if (!rb) rmode = kRecNone;
     if (ADJ && !defer) return cudaErrorInvalidValue;
-    if (rmode == kRecWrite) {
-        // records only: no image in or out
-    } else if (!ADJ) {
+    if (!ADJ) {
         transpose_kernel<<<tg, tb, 0, s>>>(coef, imgT, g.nx, g.ny);
     } else {
         e = cudaMemsetAsync(out, 0, sizeof(float) * (size_t)g.nx * g.ny, s);
@@ -1076,23 +1158,17 @@ cudaError_t launch_strip_t(const GridDev &g, const LinesDev &L, const LineHdr *h
     // the adjoint: fixed-point chunks, then (a small second launch) the
     // chunks they deferred to float strips
     constexpr int FM1 = ADJ ? kFmFixed : kFmAll;
-    auto kern = rmode == kRecRead ? strip_kernel<DEG, ADJ, kRecRead, FM1>
-                : rmode == kRecWrite ? strip_kernel<DEG, ADJ, (ADJ ? kRecNone : kRecWrite), FM1>
-                                     : strip_kernel<DEG, ADJ, kRecNone, FM1>;
-    auto kern2 = rmode == kRecRead ? strip_float_kernel<DEG, kRecRead> : strip_float_kernel<DEG, kRecNone>;
+    auto kern = strip_kernel<KIND, ADJ, FM1>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e == cudaSuccess && ADJ)
-        e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        e = cudaFuncSetAttribute(strip_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
     if (strip_needs_order(L) && !L.order) return cudaErrorInvalidValue;   // free lists need their order
     const int cpv = (int)((chunk_bins(L) + kChunk - 1) / kChunk);
     const unsigned grid = (unsigned)(chunk_views(L) * cpv);
-    // 16-byte staging and flushing: image rows (nx and ny floats) and bases aligned
-    const float *img = ADJ ? out : coef;
-    const int vec = (g.nx % 4 == 0) && (g.ny % 4 == 0) && ((reinterpret_cast<uintptr_t>(img) & 15) == 0) &&
-                    ((reinterpret_cast<uintptr_t>(imgT) & 15) == 0);
+    const int vec = strip_vec(g, ADJ ? out : coef, imgT);
     kern<<<grid, kThreads, kSmemBytes, s>>>(g, L, hdr, tabs, coef, imgT, const_cast<float *>(sino), out, imgT, cpv,
-                                            vec, err, rb, rcap, defer);
+                                            vec, defer, rec);
     e = cudaGetLastError();
     if (e == cudaSuccess && ADJ) {
         int dev = 0, sms = 0;
@@ -1100,11 +1176,11 @@ cudaError_t launch_strip_t(const GridDev &g, const LinesDev &L, const LineHdr *h
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const unsigned g2 = grid < (unsigned)sms ? grid : (unsigned)sms;
         if (e == cudaSuccess)
-            kern2<<<g2, kThreads, kSmemBytes, s>>>(g, L, hdr, tabs, const_cast<float *>(sino), out, imgT, cpv, vec,
-                                                   err, rb, rcap, defer);
+            strip_float_kernel<KIND><<<g2, kThreads, kSmemBytes, s>>>(g, L, hdr, tabs, const_cast<float *>(sino), out,
+                                                                     imgT, cpv, vec, defer, rec);
         if (e == cudaSuccess) e = cudaGetLastError();
     }
-    if (e == cudaSuccess && ADJ && rmode != kRecWrite) {
+    if (e == cudaSuccess && ADJ) {
         add_transposed_kernel<<<tg, tb, 0, s>>>(imgT, out, g.nx, g.ny);
         e = cudaGetLastError();
     }
@@ -1113,8 +1189,10 @@ cudaError_t launch_strip_t(const GridDev &g, const LinesDev &L, const LineHdr *h
 
 }  // namespace
 
+int strip_queue_kind(const GridDev &g) { return strip_kind(g); }
+
 StripJob make_strip_job(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs, bool adj,
-                        const float *img_in, float *sino, float *img_out, void *scratch, int *err)
+                        const float *img_in, float *sino, float *img_out, void *scratch)
 {
     StripJob J;
     J.g = g;
@@ -1126,11 +1204,8 @@ StripJob make_strip_job(const GridDev &g, const LinesDev &L, const LineHdr *hdr,
     J.sino = sino;
     J.out = adj ? img_out : nullptr;
     J.outT = static_cast<float *>(scratch);
-    J.err = err;
     J.cpv = (int)((chunk_bins(L) + kChunk - 1) / kChunk);
-    const void *img = adj ? static_cast<const void *>(img_out) : static_cast<const void *>(img_in);
-    J.vec = (g.nx % 4 == 0) && (g.ny % 4 == 0) && ((reinterpret_cast<uintptr_t>(img) & 15) == 0) &&
-            ((reinterpret_cast<uintptr_t>(scratch) & 15) == 0);
+    J.vec = strip_vec(g, adj ? img_out : img_in, scratch);
     J.chunk0 = 0;
     return J;
 }
@@ -1157,11 +1232,11 @@ cudaError_t launch_strip_post(const StripJob &J, bool adj, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_strip_queue(int deg, bool adj, const StripJob *jobs, int njobs, int64_t total,
+cudaError_t launch_strip_queue(int kind, bool adj, const StripJob *jobs, int njobs, int64_t total,
                                unsigned long long *counter, long long *defer, cudaStream_t s)
 {
     if (njobs <= 0 || total <= 0) return cudaSuccess;
-    if (deg < 0 || deg > 3 || (adj && !defer)) return cudaErrorInvalidValue;
+    if (kind < 0 || kind > kKindBox || (adj && !defer)) return cudaErrorInvalidValue;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1169,11 +1244,12 @@ cudaError_t launch_strip_queue(int deg, bool adj, const StripJob *jobs, int njob
     if (e != cudaSuccess) return e;
     int64_t grid = 2 * (int64_t)sms;   // two CTAs per SM, resident at once
     if (grid > total) grid = total;
-    switch (deg) {
+    switch (kind) {
     case 0: return launch_queue_t<0>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
     case 1: return launch_queue_t<1>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
     case 2: return launch_queue_t<2>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
-    default: return launch_queue_t<3>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
+    case 3: return launch_queue_t<3>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
+    default: return launch_queue_t<kKindBox>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
     }
 }
 
@@ -1184,58 +1260,40 @@ bool strip_supported(const GridDev &g, const LinesDev &L)
 
 size_t strip_scratch_bytes(const GridDev &g) { return sizeof(float) * (size_t)g.nx * g.ny + 256; }
 
-long long strip_rec_line_bytes(const GridDev &g)
-{
-    // A line's rows lie in [0, Nr) (Nr the grid's extent along its major
-    // axis) and are split into strip slabs of kSlabRows, each into batches of
-    // kBatch: at most nb = 2 ceil(Nr / kSlabRows) batches, hence at most
-    // Nr + nb 3 (n + 2) records (each interval segment padded by at most 3),
-    // 8 bytes each, and a 16-byte header per batch.
-    const long long nr = g.nx > g.ny ? g.nx : g.ny;
-    const long long nb = 2 * ((nr + kSlabRows - 1) / kSlabRows) + 2;
-    const long long bytes = nb * 16 + 8 * (nr + nb * 3 * (g.kdeg + 2));
-    return (bytes + 15) & ~15LL;
-}
-
 cudaError_t launch_fwd_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *coef, void *scratch, float *sino, int *err, cudaStream_t s,
-                             const StripRec *rec)
+                             const float *coef, void *scratch, float *sino, cudaStream_t s, const longlong2 *rec)
 {
     float *coefT = static_cast<float *>(scratch);
-    const int rm = rec ? kRecRead : kRecNone;
-    switch (g.kdeg) {
-    case 0: return launch_strip_t<0, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, err, s, rec, rm);
-    case 1: return launch_strip_t<1, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, err, s, rec, rm);
-    case 2: return launch_strip_t<2, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, err, s, rec, rm);
-    default: return launch_strip_t<3, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, err, s, rec, rm);
+    switch (strip_kind(g)) {
+    case 0: return launch_strip_t<0, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
+    case 1: return launch_strip_t<1, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
+    case 2: return launch_strip_t<2, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
+    case 3: return launch_strip_t<3, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
+    default: return launch_strip_t<kKindBox, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
     }
+}
+
+cudaError_t launch_row_records(const LineHdr *hdr, int64_t m, longlong2 *rec, cudaStream_t s)
+{
+    if (m <= 0) return cudaSuccess;
+    row_record_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(hdr, m, rec);
+    return cudaGetLastError();
 }
 
 int64_t strip_chunk_count(const LinesDev &L) { return chunk_views(L) * ((chunk_bins(L) + kChunk - 1) / kChunk); }
 
 cudaError_t launch_adj_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *sino, void *scratch, float *coef_out, int *err, cudaStream_t s,
-                             const StripRec *rec, unsigned *defer)
+                             const float *sino, void *scratch, float *coef_out, cudaStream_t s, const longlong2 *rec,
+                             unsigned *defer)
 {
     float *outT = static_cast<float *>(scratch);
     float *p = const_cast<float *>(sino);
-    const int rm = rec ? kRecRead : kRecNone;
-    switch (g.kdeg) {
-    case 0: return launch_strip_t<0, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, err, s, rec, rm, defer);
-    case 1: return launch_strip_t<1, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, err, s, rec, rm, defer);
-    case 2: return launch_strip_t<2, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, err, s, rec, rm, defer);
-    default: return launch_strip_t<3, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, err, s, rec, rm, defer);
-    }
-}
-
-cudaError_t launch_strip_record(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                                const StripRec &rec, cudaStream_t s)
-{
-    switch (g.kdeg) {
-    case 0: return launch_strip_t<0, false>(g, L, hdr, tabs, nullptr, nullptr, nullptr, nullptr, nullptr, s, &rec, kRecWrite);
-    case 1: return launch_strip_t<1, false>(g, L, hdr, tabs, nullptr, nullptr, nullptr, nullptr, nullptr, s, &rec, kRecWrite);
-    case 2: return launch_strip_t<2, false>(g, L, hdr, tabs, nullptr, nullptr, nullptr, nullptr, nullptr, s, &rec, kRecWrite);
-    default: return launch_strip_t<3, false>(g, L, hdr, tabs, nullptr, nullptr, nullptr, nullptr, nullptr, s, &rec, kRecWrite);
+    switch (strip_kind(g)) {
+    case 0: return launch_strip_t<0, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
+    case 1: return launch_strip_t<1, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
+    case 2: return launch_strip_t<2, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
+    case 3: return launch_strip_t<3, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
+    default: return launch_strip_t<kKindBox, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
     }
 }
 
