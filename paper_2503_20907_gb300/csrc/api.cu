@@ -139,68 +139,76 @@ int64_t table_count(const spx::LinesDev &L)
 
 size_t align_up(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// Line records and footprint tables for (grid, lines) in the workspace.
-// Scratch of the strip kernels: transposed coefficients, the slow-row
-// counter, then (free line lists) the chunk order and its sort's scratch.
+// Scratch of the strip kernels: the two images and the adjoint's list of chunks
+// deferred to float strips, then (free line lists) the chunk order and its
+// sort's scratch.
 size_t order_bytes(const spx::LinesDev &L) { return spx::strip_needs_order(L) ? align_up(spx::line_order_bytes(L.m)) : 0; }
+
+size_t image_list_bytes(const spx::GridDev &g, const spx::LinesDev &L)
+{
+    return align_up(spx::strip_scratch_bytes(g) + sizeof(unsigned) * (size_t)(2 + spx::strip_chunk_count(L)));
+}
 
 size_t extra_bytes(const spx::GridDev &g, const spx::LinesDev &L)
 {
-    if (!spx::strip_supported(g, L)) return 0;
-    return align_up(spx::strip_scratch_bytes(g)) + 256 + order_bytes(L) +
-           sizeof(unsigned) * (size_t)(2 + spx::strip_chunk_count(L));
-}
-
-int *slow_counter(const spx::GridDev &g, void *extra)
-{
-    return reinterpret_cast<int *>(static_cast<char *>(extra) + align_up(spx::strip_scratch_bytes(g)));
-}
-
-// The adjoint's list of chunks deferred to float strips (after the order).
-unsigned *defer_area(const spx::GridDev &g, const spx::LinesDev &L, void *extra)
-{
-    return reinterpret_cast<unsigned *>(static_cast<char *>(extra) + align_up(spx::strip_scratch_bytes(g)) + 256 +
-                                        order_bytes(L));
+    return spx::strip_supported(g, L) ? image_list_bytes(g, L) + order_bytes(L) : 0;
 }
 
 // Where the chunk order of a free line list lives (NULL for other kinds).
 void *order_area(const spx::GridDev &g, const spx::LinesDev &L, void *extra)
 {
     if (!extra || !spx::strip_needs_order(L) || !spx::strip_supported(g, L)) return nullptr;
-    return static_cast<char *>(extra) + align_up(spx::strip_scratch_bytes(g)) + 256;
+    return static_cast<char *>(extra) + image_list_bytes(g, L);
 }
 
-// Kernel paths: strip kernels or the general warp-per-line kernels.  kPathAuto
-// takes the strip kernels for degree >= 1.
+// Kernel paths: strip kernels (kPathAuto too) or the general warp-per-line
+// kernels.
 // kPathGather (adjoint only): the pixel-driven gather where it applies.
 enum KernelPath { kPathAuto = 0, kPathStrip = 1, kPathGeneral = 2, kPathGather = 3 };
 
 bool use_strip(const spx::GridDev &g, const spx::LinesDev &L, void *extra, int path)
 {
-    return extra && spx::strip_supported(g, L) && (path == kPathStrip || (path == kPathAuto && g.kdeg >= 1));
+    return extra && spx::strip_supported(g, L) && (path == kPathStrip || path == kPathAuto);
+}
+
+// What line setup leaves behind for one (grid, lines) pair.
+struct LineData {
+    spx::LineHdr *hdr;
+    float *center;   // centre records (B-splines of degree >= 1), or NULL
+    float *tabs;     // footprint tables, or NULL
+    void *extra;     // scratch of the strip kernels, or NULL
+};
+
+// Whether a path reads the footprint tables (beyond their heads): all but the
+// strip kernels on B-splines.
+bool path_needs_tables(const spx::GridDev &g, const spx::LinesDev &L, void *extra, int path)
+{
+    return g.basis != SP_BASIS_BSPLINE || !use_strip(g, L, extra, path);
 }
 
 // Forward projection (rec: the plan's row records, or NULL).
-cudaError_t run_fwd(const spx::GridDev &g, const spx::LinesDev &L, const spx::LineHdr *hdr, const float *tabs,
-                    void *extra, const float *coef, float *sino, cudaStream_t s, int path = kPathAuto,
-                    const longlong2 *rec = nullptr)
+cudaError_t run_fwd(const spx::GridDev &g, const spx::LinesDev &L, const LineData &D, const float *coef, float *sino,
+                    cudaStream_t s, int path = kPathAuto, const longlong2 *rec = nullptr)
 {
-    if (use_strip(g, L, extra, path))
-        return spx::launch_fwd_strip(g, L, hdr, tabs, coef, extra, sino, s, rec);
-    return spx::launch_fwd(g, hdr, tabs, L.m, coef, sino, s);
+    if (use_strip(g, L, D.extra, path))
+        return spx::launch_fwd_strip(g, L, D.hdr, D.center, D.tabs, coef, D.extra, sino, s, rec);
+    return spx::launch_fwd(g, D.hdr, D.tabs, L.m, coef, sino, s);
 }
 
 // Adjoint (coef_out overwritten).
-cudaError_t run_adj(const spx::GridDev &g, const spx::LinesDev &L, const spx::LineHdr *hdr, const float *tabs,
-                    void *extra, const float *sino, float *coef_out, cudaStream_t s, int path = kPathAuto,
-                    const longlong2 *rec = nullptr)
+cudaError_t run_adj(const spx::GridDev &g, const spx::LinesDev &L, const LineData &D, const float *sino, float *coef_out,
+                    cudaStream_t s, int path = kPathAuto, const longlong2 *rec = nullptr)
 {
     if (path == kPathGather && spx::gather_supported(g, L))
-        return spx::launch_adj_gather(g, L, hdr, tabs, sino, coef_out, s);
-    if (use_strip(g, L, extra, path))
-        return spx::launch_adj_strip(g, L, hdr, tabs, sino, extra, coef_out, s, rec,
-                                     defer_area(g, L, extra));
-    return spx::launch_adj(g, hdr, tabs, L.m, sino, coef_out, s);
+        return spx::launch_adj_gather(g, L, D.hdr, D.tabs, sino, coef_out, s);
+    if (use_strip(g, L, D.extra, path))
+        return spx::launch_adj_strip(g, L, D.hdr, D.center, D.tabs, sino, D.extra, coef_out, s, rec);
+    return spx::launch_adj(g, D.hdr, D.tabs, L.m, sino, coef_out, s);
+}
+
+size_t center_bytes(const spx::GridDev &g, int64_t n_tab)
+{
+    return spx::center_records(g) ? align_up(sizeof(float) * (size_t)spx::kCenterFloats * (size_t)n_tab) : 0;
 }
 
 // Row records a plan keeps (W of row 0 and its step, per line): strip-path
@@ -215,25 +223,31 @@ size_t rec_bytes_wanted(const spx::GridDev &g, const spx::LinesDev &L)
     return (size_t)L.m * sizeof(longlong2);
 }
 
-sp_status prepare(const spx::GridDev &g, spx::LinesDev &L, cudaStream_t s,
-                  spx::LineHdr **hdr, float **tabs, void **extra = nullptr)
+// Line setup of a one-shot call in the cached workspace: with `project` for the
+// strip kernels (and the chunk order of free lists), else the footprint tables.
+sp_status prepare(const spx::GridDev &g, spx::LinesDev &L, cudaStream_t s, bool project, LineData *D)
 {
     const int64_t nt = table_count(L);
-    size_t hb = align_up(sizeof(spx::LineHdr) * (size_t)L.m);
-    size_t tb = align_up(sizeof(float) * (size_t)spx::kTabFloats * (size_t)nt);
-    size_t xb = align_up(extra_bytes(g, L));
+    const size_t hb = align_up(sizeof(spx::LineHdr) * (size_t)L.m);
+    const size_t xb = project ? align_up(extra_bytes(g, L)) : 0;
+    const size_t cb = project ? center_bytes(g, nt) : 0;
+    const bool tables = !project || g.basis != SP_BASIS_BSPLINE || xb == 0;
+    const size_t tb = tables ? align_up(sizeof(float) * (size_t)spx::kTabFloats * (size_t)nt) : 0;
     void *ws = nullptr;
-    sp_status st = workspace(hb + tb + xb + 256, &ws);
+    sp_status st = workspace(hb + xb + cb + tb + 256, &ws);
     if (st != SP_OK) return st;
-    *hdr = reinterpret_cast<spx::LineHdr *>(ws);
-    *tabs = reinterpret_cast<float *>(static_cast<char *>(ws) + hb);
-    if (extra) *extra = xb ? static_cast<char *>(ws) + hb + tb : nullptr;
-    cudaError_t e = spx::launch_prepare(g, L, *hdr, *tabs, nt, s);
+    char *w = static_cast<char *>(ws);
+    D->hdr = reinterpret_cast<spx::LineHdr *>(w);
+    D->extra = xb ? w + hb : nullptr;
+    D->center = cb ? reinterpret_cast<float *>(w + hb + xb) : nullptr;
+    D->tabs = tb ? reinterpret_cast<float *>(w + hb + xb + cb) : nullptr;
+    cudaError_t e = spx::launch_setup(g, L, D->hdr, D->tabs, D->center, s);
+    if (e == cudaSuccess && tables) e = spx::launch_tables(g, L, D->tabs, nt, s);
     if (e != cudaSuccess) return cuda_fail(e, "line setup and footprint tables");
     // free line lists: the chunk order of the strip kernels
-    void *oa = extra ? order_area(g, L, *extra) : nullptr;
+    void *oa = order_area(g, L, D->extra);
     if (oa) {
-        e = spx::launch_line_order(g, L, *hdr, oa, s);
+        e = spx::launch_line_order(g, L, D->hdr, oa, s);
         if (e != cudaSuccess) return cuda_fail(e, "line order");
         L.order = static_cast<const int *>(oa);
     }
@@ -268,11 +282,9 @@ sp_status spline_project_fwd(const sp_grid *grid, const float *coef, const sp_li
     if (L.m == 0) return SP_OK;
     if (!coef || !sino) return fail(SP_EINVAL, "coef/sino pointers are NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    spx::LineHdr *hdr;
-    float *tabs;
-    void *extra = nullptr;
-    if ((st = prepare(g, L, s, &hdr, &tabs, &extra)) != SP_OK) return st;
-    cudaError_t e = run_fwd(g, L, hdr, tabs, extra, coef, sino, s);
+    LineData D;
+    if ((st = prepare(g, L, s, true, &D)) != SP_OK) return st;
+    cudaError_t e = run_fwd(g, L, D, coef, sino, s);
     if (e != cudaSuccess) return cuda_fail(e, "forward projection");
     return SP_OK;
 }
@@ -293,11 +305,9 @@ sp_status spline_project_adj(const sp_grid *grid, const float *sino, const sp_li
         cudaError_t e = cudaMemsetAsync(coef_out, 0, sizeof(float) * (size_t)g.nx * g.ny, s);
         return e == cudaSuccess ? SP_OK : cuda_fail(e, "cudaMemsetAsync");
     }
-    spx::LineHdr *hdr;
-    float *tabs;
-    void *extra = nullptr;
-    if ((st = prepare(g, L, s, &hdr, &tabs, &extra)) != SP_OK) return st;
-    cudaError_t e = run_adj(g, L, hdr, tabs, extra, sino, coef_out, s);
+    LineData D;
+    if ((st = prepare(g, L, s, true, &D)) != SP_OK) return st;
+    cudaError_t e = run_adj(g, L, D, sino, coef_out, s);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint projection");
     return SP_OK;
 }
@@ -347,10 +357,9 @@ sp_status spline_visited(const sp_grid *grid, const sp_lines *lines, int32_t *co
     if (L.m == 0) return SP_OK;
     if (!counts) return fail(SP_EINVAL, "counts pointer is NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    spx::LineHdr *hdr;
-    float *tabs;
-    if ((st = prepare(g, L, s, &hdr, &tabs)) != SP_OK) return st;
-    cudaError_t e = spx::launch_visited(g, hdr, tabs, L.m, counts, offsets, nodes, s);
+    LineData D;
+    if ((st = prepare(g, L, s, false, &D)) != SP_OK) return st;
+    cudaError_t e = spx::launch_visited(g, D.hdr, D.tabs, L.m, counts, offsets, nodes, s);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "visited set");
 }
 
@@ -359,9 +368,10 @@ struct sp_plan {
     spx::LinesDev L;
     int device;
     void *mem;
-    spx::LineHdr *hdr;
-    float *tabs;
-    void *extra;       // strip scratch (transposed coefficients, slow-row counter) or NULL
+    LineData D;
+    // the footprint tables are built (else their heads only); some projection
+    // has read them, so that every prepare builds them
+    mutable bool tables, tables_used;
     longlong2 *rec;    // row records written by prepare (NULL: none)
     bool prepared;
     void *cg_ws;       // CGLS vectors and scalars, allocated on first use
@@ -393,6 +403,39 @@ bool plan_alloc_records(sp_plan *p)
     return true;
 }
 
+// The plan's footprint tables, built on the first projection after a prepare
+// whose path reads them.  In a stream that is being captured they become part
+// of the capture, every time: nothing has run yet that a later call could rely
+// on.
+cudaError_t plan_tables(const sp_plan *p, cudaStream_t s)
+{
+    p->tables_used = true;
+    if (p->tables) return cudaSuccess;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e == cudaSuccess) e = spx::launch_tables(p->g, p->L, p->D.tabs, table_count(p->L), s);
+    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) p->tables = true;
+    return e;
+}
+
+cudaError_t plan_fwd(const sp_plan *p, const float *coef, float *sino, cudaStream_t s, int path)
+{
+    if (path_needs_tables(p->g, p->L, p->D.extra, path)) {
+        const cudaError_t e = plan_tables(p, s);
+        if (e != cudaSuccess) return e;
+    }
+    return run_fwd(p->g, p->L, p->D, coef, sino, s, path, p->rec);
+}
+
+cudaError_t plan_adj(const sp_plan *p, const float *sino, float *coef_out, cudaStream_t s, int path)
+{
+    if (p->L.m > 0 && path_needs_tables(p->g, p->L, p->D.extra, path)) {
+        const cudaError_t e = plan_tables(p, s);
+        if (e != cudaSuccess) return e;
+    }
+    return run_adj(p->g, p->L, p->D, sino, coef_out, s, path, p->rec);
+}
+
 sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan, bool keep_records)
 {
     g_err.clear();
@@ -409,9 +452,10 @@ sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan
     size_t hb = align_up(sizeof(spx::LineHdr) * (size_t)L.m);
     size_t tb = align_up(sizeof(float) * (size_t)spx::kTabFloats * (size_t)table_count(L));
     size_t xb = align_up(extra_bytes(g, L));
+    size_t cb = center_bytes(g, table_count(L));
     void *mem = nullptr;
-    if (hb + tb + xb > 0) {
-        e = cudaMalloc(&mem, hb + tb + xb);
+    if (hb + tb + xb + cb > 0) {
+        e = cudaMalloc(&mem, hb + tb + xb + cb);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(SP_ENOMEM, std::string("plan allocation failed: ") + cudaGetErrorString(e));
@@ -422,23 +466,18 @@ sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan
     p->L = L;
     p->device = dev;
     p->mem = mem;
-    p->hdr = reinterpret_cast<spx::LineHdr *>(mem);
-    p->tabs = mem ? reinterpret_cast<float *>(static_cast<char *>(mem) + hb) : nullptr;
-    p->extra = (mem && xb) ? static_cast<char *>(mem) + hb + tb : nullptr;
-    p->L.order = static_cast<const int *>(order_area(g, L, p->extra));   // written by prepare
+    char *w = static_cast<char *>(mem);
+    p->D.hdr = reinterpret_cast<spx::LineHdr *>(mem);
+    p->D.tabs = mem ? reinterpret_cast<float *>(w + hb) : nullptr;
+    p->D.extra = (mem && xb) ? w + hb + tb : nullptr;
+    p->D.center = (mem && cb) ? reinterpret_cast<float *>(w + hb + tb + xb) : nullptr;
+    p->tables = p->tables_used = false;
+    p->L.order = static_cast<const int *>(order_area(g, L, p->D.extra));   // written by prepare
     p->prepared = false;
     p->cg_ws = nullptr;
     p->cg_bytes = 0;
     p->path_fwd = p->path_adj = kPathAuto;
     p->rec = nullptr;
-    if (p->extra) {
-        e = cudaMemset(slow_counter(g, p->extra), 0, sizeof(int));
-        if (e != cudaSuccess) {
-            cudaFree(mem);
-            delete p;
-            return cuda_fail(e, "cudaMemset");
-        }
-    }
     if (keep_records) plan_alloc_records(p);
     *plan = p;
     return SP_OK;
@@ -481,14 +520,21 @@ sp_status spline_plan_prepare(sp_plan *plan, void *stream)
     if (!plan) return fail(SP_EINVAL, "plan is NULL");
     if (plan->L.m == 0) { plan->prepared = true; return SP_OK; }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = spx::launch_prepare(plan->g, plan->L, plan->hdr, plan->tabs, table_count(plan->L), s);
+    // the footprint tables only where a path that is set or was taken reads
+    // them (else they wait for one)
+    cudaError_t e = spx::launch_setup(plan->g, plan->L, plan->D.hdr, plan->D.tabs, plan->D.center, s);
+    plan->tables = false;
+    if (e == cudaSuccess &&
+        (plan->tables_used || path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_fwd) ||
+         path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_adj)))
+        e = plan_tables(plan, s);
     if (e != cudaSuccess) return cuda_fail(e, "line setup and footprint tables");
     if (plan->L.order) {
-        e = spx::launch_line_order(plan->g, plan->L, plan->hdr, const_cast<int *>(plan->L.order), s);
+        e = spx::launch_line_order(plan->g, plan->L, plan->D.hdr, const_cast<int *>(plan->L.order), s);
         if (e != cudaSuccess) return cuda_fail(e, "line order");
     }
     if (plan->rec) {
-        e = spx::launch_row_records(plan->hdr, plan->L.m, plan->rec, s);
+        e = spx::launch_row_records(plan->g, plan->L, plan->D.hdr, plan->D.center, plan->rec, s);
         if (e != cudaSuccess) return cuda_fail(e, "row records");
     }
     plan->prepared = true;
@@ -502,8 +548,7 @@ sp_status spline_plan_fwd(const sp_plan *plan, const float *coef, float *sino, v
     if (!plan->prepared) return fail(SP_EINVAL, "plan not prepared");
     if (plan->L.m == 0) return SP_OK;
     if (!coef || !sino) return fail(SP_EINVAL, "coef/sino pointers are NULL");
-    cudaError_t e = run_fwd(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, coef, sino,
-                            static_cast<cudaStream_t>(stream), plan->path_fwd, plan->rec);
+    cudaError_t e = plan_fwd(plan, coef, sino, static_cast<cudaStream_t>(stream), plan->path_fwd);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "forward projection");
 }
 
@@ -514,8 +559,7 @@ sp_status spline_plan_adj(const sp_plan *plan, const float *sino, float *coef_ou
     if (!plan->prepared) return fail(SP_EINVAL, "plan not prepared");
     if (!coef_out) return fail(SP_EINVAL, "coef_out pointer is NULL");
     if (plan->L.m > 0 && !sino) return fail(SP_EINVAL, "sino pointer is NULL");
-    cudaError_t e = run_adj(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, sino, coef_out,
-                            static_cast<cudaStream_t>(stream), plan->path_adj, plan->rec);
+    cudaError_t e = plan_adj(plan, sino, coef_out, static_cast<cudaStream_t>(stream), plan->path_adj);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "adjoint projection");
 }
 
@@ -523,12 +567,12 @@ namespace {
 cudaError_t plan_fwd_cb(void *ctx, const float *coef, float *sino, cudaStream_t s)
 {
     const sp_plan *p = static_cast<const sp_plan *>(ctx);
-    return run_fwd(p->g, p->L, p->hdr, p->tabs, p->extra, coef, sino, s, p->path_fwd, p->rec);
+    return plan_fwd(p, coef, sino, s, p->path_fwd);
 }
 cudaError_t plan_adj_cb(void *ctx, const float *sino, float *coef_out, cudaStream_t s)
 {
     const sp_plan *p = static_cast<const sp_plan *>(ctx);
-    return run_adj(p->g, p->L, p->hdr, p->tabs, p->extra, sino, coef_out, s, p->path_adj, p->rec);
+    return plan_adj(p, sino, coef_out, s, p->path_adj);
 }
 }  // namespace
 
@@ -618,7 +662,7 @@ sp_status spline_plan_autotune(sp_plan *plan, const float *coef, const float *si
     const int64_t n = (int64_t)plan->g.nx * plan->g.ny, m = plan->L.m;
     if (m > 0 && (!coef || !sino)) return fail(SP_EINVAL, "coef/sino pointers are NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const bool both = plan->extra && spx::strip_supported(plan->g, plan->L) && m > 0;
+    const bool both = plan->D.extra && spx::strip_supported(plan->g, plan->L) && m > 0;
     // fwd strip, fwd general, adj strip, adj general, adj gather
     float t[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
     int bf = both ? kPathStrip : kPathGeneral, ba = bf;
@@ -630,13 +674,9 @@ sp_status spline_plan_autotune(sp_plan *plan, const float *coef, const float *si
         for (int k = 0; k < (gather ? 5 : 4) && e == cudaSuccess; ++k) {
             const int path = k == 4 ? kPathGather : ((k & 1) ? kPathGeneral : kPathStrip);
             if (k < 2)
-                e = time_runs([&] { return run_fwd(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, coef, tmp_s, s,
-                                                   path, plan->rec); },
-                              3, s, &t[k]);
+                e = time_runs([&] { return plan_fwd(plan, coef, tmp_s, s, path); }, 3, s, &t[k]);
             else
-                e = time_runs([&] { return run_adj(plan->g, plan->L, plan->hdr, plan->tabs, plan->extra, sino, tmp_c, s,
-                                                   path, plan->rec); },
-                              3, s, &t[k]);
+                e = time_runs([&] { return plan_adj(plan, sino, tmp_c, s, path); }, 3, s, &t[k]);
         }
         cudaError_t e2 = cudaStreamSynchronize(s);
         if (tmp_s) cudaFree(tmp_s);
@@ -685,8 +725,9 @@ struct sp_batch {
     cudaEvent_t fork = nullptr, join[kBatchStreams] = {};
     GraphCache gfwd, gadj;
     // strip-kernel instances run as one persistent launch over a work queue
-    spx::StripJob *jobs_dev[2] = {nullptr, nullptr};   // forward, adjoint
-    std::vector<spx::StripJob> jobs_host[2];
+    void *jobs_dev[2] = {nullptr, nullptr};   // forward, adjoint
+    std::vector<char> jobs_host[2];
+    std::vector<size_t> job_plan[2];          // the instance of each job
     int64_t chunks[2] = {0, 0};
     // jobs grouped by kind (one queue launch per B-spline degree and basis):
     // jobs [gjob0, gjob0 + gnjob) of group deg own gtotal chunks
@@ -768,37 +809,53 @@ cudaError_t run_graph(sp_batch *b, GraphCache &gc, const std::vector<const void 
 // run on the strip kernels, uploaded to the batch's job array.  Runs outside
 // any capture; the device is synchronised first because a graph recorded
 // earlier may still read the previous array.
+// (Degree 0 joins the queue only when set or tuned to the strip kernels: on its
+// own stream beside the queue its short rows do not wait behind longer chunks.)
+bool in_queue(const sp_plan *p, int d)
+{
+    const int path = d ? p->path_adj : p->path_fwd;
+    if (p->L.m == 0 || !use_strip(p->g, p->L, p->D.extra, path)) return false;
+    return p->g.kdeg >= 1 || path == kPathStrip;
+}
+
 template <typename In, typename Out>
 cudaError_t upload_jobs(sp_batch *b, int d, In in, Out outp, std::vector<char> &queued)
 {
-    std::vector<spx::StripJob> &hj = b->jobs_host[d];
-    hj.clear();
+    std::vector<char> &hj = b->jobs_host[d];
+    std::vector<size_t> &hp = b->job_plan[d];
+    hj.assign(spx::strip_job_bytes((int)b->plans.size()), 0);
+    hp.clear();
     queued.assign(b->plans.size(), 0);
     int64_t all = 0;
-    for (int deg = 0; deg < spx::kQueueKinds; ++deg) {
-        b->gjob0[d][deg] = (int)hj.size();
-        int64_t c0 = 0;   // chunk indices count within the degree's group
+    cudaError_t e = cudaSuccess;
+    for (int kind = 0; kind < spx::kQueueKinds; ++kind) {
+        b->gjob0[d][kind] = (int)hp.size();
+        int64_t c0 = 0;   // chunk indices count within the kind's group
         for (size_t i = 0; i < b->plans.size(); ++i) {
             const sp_plan *p = b->plans[i];
-            const int path = d ? p->path_adj : p->path_fwd;
-            // (degree 0 takes the strip kernels when set or tuned to them)
-            if (spx::strip_queue_kind(p->g) != deg || p->L.m == 0 || !use_strip(p->g, p->L, p->extra, path)) continue;
-            spx::StripJob J = d ? spx::make_strip_job(p->g, p->L, p->hdr, p->tabs, true, nullptr,
-                                                      const_cast<float *>(in[i]), outp[i], p->extra)
-                                : spx::make_strip_job(p->g, p->L, p->hdr, p->tabs, false, in[i], outp[i], nullptr,
-                                                      p->extra);
-            J.chunk0 = c0;
-            c0 += spx::strip_job_chunks(J);
-            hj.push_back(J);
+            if (spx::strip_queue_kind(p->g) != kind || !in_queue(p, d)) continue;
+            spx::make_strip_job(hj.data(), (int)hp.size(), p->g, p->L, p->D.hdr, p->D.center, p->D.tabs,
+                                d ? nullptr : static_cast<const float *>(in[i]),
+                                const_cast<float *>(d ? static_cast<const float *>(in[i]) : static_cast<const float *>(outp[i])),
+                                p->D.extra, c0);
+            c0 += spx::strip_chunk_count(p->L);
+            hp.push_back(i);
             queued[i] = 1;
         }
-        b->gnjob[d][deg] = (int)hj.size() - b->gjob0[d][deg];
-        b->gtotal[d][deg] = c0;
+        b->gnjob[d][kind] = (int)hp.size() - b->gjob0[d][kind];
+        b->gtotal[d][kind] = c0;
         all += c0;
+    }
+    // footprint tables that the instances' paths read, outside the capture (and
+    // after whatever prepared the instances)
+    e = cudaDeviceSynchronize();
+    for (size_t i = 0; i < b->plans.size() && e == cudaSuccess; ++i) {
+        const sp_plan *p = b->plans[i];
+        if (p->L.m > 0 && path_needs_tables(p->g, p->L, p->D.extra, d ? p->path_adj : p->path_fwd)) e = plan_tables(p, b->cap);
     }
     const int64_t c0 = all;
     b->chunks[d] = c0;
-    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess && d == 1 && c0 > b->defer_cap) {
         if (b->defer) cudaFree(b->defer);
         b->defer = nullptr;
@@ -806,27 +863,31 @@ cudaError_t upload_jobs(sp_batch *b, int d, In in, Out outp, std::vector<char> &
         e = cudaMalloc(&b->defer, sizeof(long long) * (size_t)c0);
         if (e == cudaSuccess) b->defer_cap = c0;
     }
-    if (e == cudaSuccess && !hj.empty())
-        e = cudaMemcpy(b->jobs_dev[d], hj.data(), sizeof(spx::StripJob) * hj.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !hp.empty())
+        e = cudaMemcpy(b->jobs_dev[d], hj.data(), spx::strip_job_bytes((int)hp.size()), cudaMemcpyHostToDevice);
     return e;
 }
 
 // The queued instances on the capture origin: per-instance set-up, the
-// persistent kernel, per-instance completion.
-cudaError_t run_queue(sp_batch *b, int d, cudaStream_t s)
+// persistent kernels, per-instance completion.  img: the images (forward: read,
+// adjoint: written) of all instances.
+cudaError_t run_queue(sp_batch *b, int d, const float *const *img_in, float *const *img_out, cudaStream_t s)
 {
-    const std::vector<spx::StripJob> &hj = b->jobs_host[d];
+    const void *hj = b->jobs_host[d].data();
+    const std::vector<size_t> &hp = b->job_plan[d];
     cudaError_t e = cudaSuccess;
-    for (size_t k = 0; k < hj.size() && e == cudaSuccess; ++k) e = spx::launch_strip_pre(hj[k], d == 1, s);
-    int64_t defer0 = 0;   // each degree's deferred chunks in its own part of the list
-    for (int deg = 0; deg < spx::kQueueKinds && e == cudaSuccess; ++deg) {
-        if (b->gnjob[d][deg] == 0) continue;
-        e = spx::launch_strip_queue(deg, d == 1, b->jobs_dev[d] + b->gjob0[d][deg], b->gnjob[d][deg],
-                                    b->gtotal[d][deg], b->counter + 3 * spx::kQueueKinds * d + 3 * deg,
+    for (size_t k = 0; k < hp.size() && e == cudaSuccess; ++k)
+        e = spx::launch_strip_pre(hj, (int)k, d ? nullptr : img_in[hp[k]], s);
+    int64_t defer0 = 0;   // each kind's deferred chunks in its own part of the list
+    for (int kind = 0; kind < spx::kQueueKinds && e == cudaSuccess; ++kind) {
+        if (b->gnjob[d][kind] == 0) continue;
+        e = spx::launch_strip_queue(kind, d == 1, b->jobs_dev[d], b->gjob0[d][kind], b->gnjob[d][kind],
+                                    b->gtotal[d][kind], b->counter + 3 * spx::kQueueKinds * d + 3 * kind,
                                     d == 1 ? b->defer + defer0 : nullptr, s);
-        defer0 += b->gtotal[d][deg];
+        defer0 += b->gtotal[d][kind];
     }
-    for (size_t k = 0; k < hj.size() && e == cudaSuccess; ++k) e = spx::launch_strip_post(hj[k], d == 1, s);
+    for (size_t k = 0; k < hp.size() && d == 1 && e == cudaSuccess; ++k)
+        e = spx::launch_strip_post(hj, (int)k, img_out[hp[k]], s);
     return e;
 }
 }  // namespace
@@ -853,7 +914,7 @@ sp_status spline_batch_create(int32_t count, const sp_grid *grids, const sp_line
     }
     cudaError_t e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-    for (int d = 0; d < 2 && e == cudaSuccess; ++d) e = cudaMalloc(&b->jobs_dev[d], sizeof(spx::StripJob) * (size_t)count);
+    for (int d = 0; d < 2 && e == cudaSuccess; ++d) e = cudaMalloc(&b->jobs_dev[d], spx::strip_job_bytes(count));
     if (e == cudaSuccess) e = cudaMalloc(&b->counter, 6 * spx::kQueueKinds * sizeof(unsigned long long));
     for (int k = 0; k < kBatchStreams && e == cudaSuccess; ++k) {
         e = cudaStreamCreateWithFlags(&b->streams[k], cudaStreamNonBlocking);
@@ -898,10 +959,10 @@ sp_status spline_batch_fwd(sp_batch *batch, const float *const *coef, float *con
         [&](size_t i, cudaStream_t s) {
             const sp_plan *p = batch->plans[i];
             if (p->L.m == 0 || queued[i]) return cudaSuccess;
-            return run_fwd(p->g, p->L, p->hdr, p->tabs, p->extra, coef[i], sino[i], s, p->path_fwd);
+            return run_fwd(p->g, p->L, p->D, coef[i], sino[i], s, p->path_fwd);
         },
         [&] { return upload_jobs(batch, 0, coef, sino, queued); },
-        [&](cudaStream_t s) { return run_queue(batch, 0, s); });
+        [&](cudaStream_t s) { return run_queue(batch, 0, coef, nullptr, s); });
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "batch forward");
 }
 
@@ -923,10 +984,10 @@ sp_status spline_batch_adj(sp_batch *batch, const float *const *sino, float *con
         [&](size_t i, cudaStream_t s) {
             const sp_plan *p = batch->plans[i];
             if (queued[i]) return cudaSuccess;
-            return run_adj(p->g, p->L, p->hdr, p->tabs, p->extra, sino[i], coef_out[i], s, p->path_adj);
+            return run_adj(p->g, p->L, p->D, sino[i], coef_out[i], s, p->path_adj);
         },
         [&] { return upload_jobs(batch, 1, sino, coef_out, queued); },
-        [&](cudaStream_t s) { return run_queue(batch, 1, s); });
+        [&](cudaStream_t s) { return run_queue(batch, 1, nullptr, coef_out, s); });
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "batch adjoint");
 }
 
@@ -951,7 +1012,7 @@ sp_status spline_batch_autotune(sp_batch *batch, const float *const *coef, const
         const sp_plan *p = batch->plans[i];
         ms_tot += align_up(sizeof(float) * (size_t)p->L.m);
         ns_tot += align_up(sizeof(float) * (size_t)p->g.nx * p->g.ny);
-        eligible[i] = p->extra && spx::strip_supported(p->g, p->L) && p->L.m > 0;
+        eligible[i] = p->D.extra && spx::strip_supported(p->g, p->L) && p->L.m > 0;
     }
     char *tmp = nullptr;
     cudaError_t e = cudaMalloc(&tmp, ms_tot + ns_tot);
@@ -998,7 +1059,7 @@ sp_status spline_batch_autotune(sp_batch *batch, const float *const *coef, const
     batch->gfwd.clear();
     batch->gadj.clear();
     for (int d = 0; d < 2; ++d) {   // the timing runs' queues; the next call records anew
-        batch->jobs_host[d].clear();
+        batch->job_plan[d].clear();
         batch->chunks[d] = 0;
     }
     cudaFree(tmp);
@@ -1018,7 +1079,7 @@ int32_t spline_batch_count(const sp_batch *batch) { return batch ? (int32_t)batc
 int32_t spline_batch_queued(const sp_batch *batch, int32_t adjoint)
 {
     if (!batch) return -1;
-    return (int32_t)batch->jobs_host[adjoint ? 1 : 0].size();
+    return (int32_t)batch->job_plan[adjoint ? 1 : 0].size();
 }
 
 sp_status spline_batch_destroy(sp_batch *batch)
@@ -1035,12 +1096,8 @@ sp_status spline_plan_stats(const sp_plan *plan, int64_t *slow_rows)
     g_err.clear();
     if (!plan || !slow_rows) return fail(SP_EINVAL, "NULL argument");
     *slow_rows = 0;
-    if (!plan->extra) return SP_OK;
-    int v = 0;
-    cudaError_t e = cudaMemcpy(&v, slow_counter(plan->g, plan->extra), sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
-    *slow_rows = v;
-    return SP_OK;
+    const cudaError_t e = cudaDeviceSynchronize();
+    return e == cudaSuccess ? SP_OK : cuda_fail(e, "cudaDeviceSynchronize");
 }
 
 sp_status spline_plan_destroy(sp_plan *plan)

@@ -51,6 +51,25 @@ constexpr int kTabB = 7;                      // head slot of its b
 constexpr int kTabFloats = kTabHead + kMaxSig * kSigStride;   // 328 floats
 constexpr float kBMin = 1e-7f;                // below this b is taken as 0 (Dirac)
 
+// Centre records (strip.cu): the footprint of one direction in polynomials
+// around the offsets y = (j + c) a from its centre, c = 1/2 for n + 1 even and
+// 0 for n + 1 odd.  phi is even, so j >= 0 serves both sides: with v in
+// [-a/2, a/2), w = |v| and kk = j or its mirror image (-j - 1, or -j),
+//   phi((kk + c) a + v) = P(+-w) + jump terms,
+// P the polynomial of the interval around v = 0 and a jump term J z for each
+// knot that w passes on the way out, z = (w - beta)^(2n+1).  The knots lie
+// symmetrically, two pairs +-beta of them (one at degree 1; those at v = +-a/2
+// are where candidates change).  Floats:
+//   [8 j + k]       coefficient k of v^k at (j + c) a, j = 0..3
+//   [32 + 2 j]      the first knot's J for the candidate on the side of v and
+//                   for its mirror image: half their sum ...
+//   [32 + 2 j + 1]  ... and half their difference
+//   [40 + 2 j ...]  the same of the second knot
+//   [48], [49]      beta of the two knots
+//   [50], [51]      a and b
+constexpr int kCenterJump = 32, kCenterBeta = 48, kCenterA = 50, kCenterB = 51;
+constexpr int kCenterFloats = 52;
+
 // Offset of the polynomial of (interval sg, candidate i) in a table: its
 // kNC coefficients (ascending powers of t) are contiguous, 32-byte aligned.
 __host__ __device__ constexpr int tab_poly(int sg, int i)
@@ -243,15 +262,13 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// Kernel launchers (kernels.cu).
-cudaError_t launch_setup(const GridDev &g, const LinesDev &L, LineHdr *hdr, float *tabs, cudaStream_t s);
+// Kernel launchers (kernels.cu).  Line setup: the line records and, where not
+// NULL, the heads of the tables (all that launch_tables needs to build them)
+// and the centre records of B-splines of degree 1..3 (rec, else untouched).
+inline bool center_records(const GridDev &g) { return g.basis == SP_BASIS_BSPLINE && g.kdeg >= 1; }
+cudaError_t launch_setup(const GridDev &g, const LinesDev &L, LineHdr *hdr, float *tabs, float *rec, cudaStream_t s);
 cudaError_t launch_tables(const GridDev &g, const LinesDev &L, float *tabs, int64_t n_tab,
                           cudaStream_t s);
-// Line setup and tables (one fused kernel where each line has its own
-// B-spline table and there are enough lines, else launch_setup then
-// launch_tables).
-cudaError_t launch_prepare(const GridDev &g, const LinesDev &L, LineHdr *hdr, float *tabs, int64_t n_tab,
-                           cudaStream_t s);
 cudaError_t launch_fwd(const GridDev &g, const LineHdr *hdr, const float *tabs, int64_t m,
                        const float *coef, float *sino, cudaStream_t s);
 cudaError_t launch_adj(const GridDev &g, const LineHdr *hdr, const float *tabs, int64_t m,
@@ -273,57 +290,48 @@ inline bool strip_needs_order(const LinesDev &L) { return L.kind == SP_LINES_THE
 
 // Forward projection with coefficient strips in shared memory (strip.cu), for
 // parallel and fan beams and sorted free line lists (any degree; L.order set
-// for the latter).  `scratch` holds strip_scratch_bytes; `rec`: the plan's row
-// records, or NULL (the kernels then take the rows from the line records).
+// for the latter).  center: the centre records (B-splines of degree >= 1);
+// tabs: the footprint tables (box-spline); scratch: strip_scratch_bytes,
+// 256-byte aligned; rec: the plan's row records, or NULL (the kernels then take
+// the rows from the line records).
 bool strip_supported(const GridDev &g, const LinesDev &L);
 size_t strip_scratch_bytes(const GridDev &g);
-cudaError_t launch_fwd_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *coef, void *scratch, float *sino, cudaStream_t s, const longlong2 *rec);
-// The row records of lines of degree >= 1 (W of row 0 and its step, per line), after line setup.
-cudaError_t launch_row_records(const LineHdr *hdr, int64_t m, longlong2 *rec, cudaStream_t s);
-// Adjoint with strip accumulators; coef_out is overwritten.  `defer` holds
-// 2 + strip_chunk_count(L) words (chunks deferred to float strips).
+cudaError_t launch_fwd_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                             const float *tabs, const float *coef, void *scratch, float *sino, cudaStream_t s,
+                             const longlong2 *rec);
+// The row records of lines of degree >= 1 (their position in row 0 and the step
+// per row), after line setup.
+cudaError_t launch_row_records(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                               longlong2 *rec, cudaStream_t s);
+// Adjoint with strip accumulators; coef_out is overwritten.  scratch has room
+// for 2 + strip_chunk_count(L) words more (chunks deferred to float strips).
 int64_t strip_chunk_count(const LinesDev &L);
-cudaError_t launch_adj_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *sino, void *scratch, float *coef_out, cudaStream_t s, const longlong2 *rec,
-                             unsigned *defer);
+cudaError_t launch_adj_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                             const float *tabs, const float *sino, void *scratch, float *coef_out, cudaStream_t s,
+                             const longlong2 *rec);
 // Pixel-driven adjoint (gather.cu): thread per node over all views, no
 // atomics; parallel and fan beams of degree >= 1.  coef_out is overwritten.
 bool gather_supported(const GridDev &g, const LinesDev &L);
 cudaError_t launch_adj_gather(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
                               const float *sino, float *coef_out, cudaStream_t s);
-// One instance of the persistent strip kernel's work queue: the arguments of
-// one strip projection and the index of its first chunk in the queue.
-struct StripJob {
-    GridDev g;
-    LinesDev L;
-    const LineHdr *hdr;
-    const float *tabs;
-    const float *coef;     // forward input (NULL for the adjoint)
-    float *coefT;          // scratch: transposed input (forward) ...
-    float *sino;
-    float *out, *outT;     // ... or output and transposed output (adjoint)
-    int cpv;               // chunks per view
-    int vec;               // 16-byte staging and flushing
-    long long chunk0;
-};
-// The job of one strip projection (adj: img_out receives the adjoint of sino;
-// forward: sino receives the projection of img_in).  chunk0 is left 0.
-StripJob make_strip_job(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs, bool adj,
-                        const float *img_in, float *sino, float *img_out, void *scratch);
-int64_t strip_job_chunks(const StripJob &J);
-// Before the queue kernel: transposed copy of the input (forward) or cleared
-// outputs (adjoint); after it: the transposed output added in (adjoint).
-cudaError_t launch_strip_pre(const StripJob &J, bool adj, cudaStream_t s);
-cudaError_t launch_strip_post(const StripJob &J, bool adj, cudaStream_t s);
-// The persistent kernel over jobs[0..njobs) (device array, chunk0 ascending,
-// `total` chunks in all, every job of kind `kind`); counter is
-// three device words, reset here.  The adjoint defers chunks that need float
-// strips to `defer` (device, room for `total` chunk indices) and runs them in
-// a second launch.
+// The work queue of the persistent strip kernels: job k of an array of
+// strip_job_bytes(count) in host memory, to be copied to the device as it is.
+// img: the forward's input, NULL for the adjoint (which reads sino).
+size_t strip_job_bytes(int count);
+void make_strip_job(void *jobs, int k, const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                    const float *tabs, const float *img, float *sino, void *scratch, long long chunk0);
+// Before the queue kernel: the forward's images (img its input) or the
+// adjoint's cleared ones (img NULL); after the adjoint: its result.
+cudaError_t launch_strip_pre(const void *jobs, int k, const float *img, cudaStream_t s);
+cudaError_t launch_strip_post(const void *jobs, int k, float *out, cudaStream_t s);
+// The persistent kernel over jobs [job0, job0 + njobs) of the device array
+// (chunk0 ascending from 0, `total` chunks in all, every job of kind `kind`);
+// counter is three device words, reset here.  The adjoint defers chunks that
+// need float strips to `defer` (device, room for `total` chunk indices) and
+// runs them in a second launch.
 constexpr int kQueueKinds = 5;   // B-spline degrees 0..3 and the box-spline
 int strip_queue_kind(const GridDev &g);
-cudaError_t launch_strip_queue(int kind, bool adj, const StripJob *jobs, int njobs, int64_t total,
+cudaError_t launch_strip_queue(int kind, bool adj, const void *jobs_dev, int job0, int njobs, int64_t total,
                                unsigned long long *counter, long long *defer, cudaStream_t s);
 cudaError_t launch_footprint_eval(const GridDev &g, int64_t count, const float *theta, const float *yt,
                                   float *out, float *scratch, cudaStream_t s);

@@ -233,7 +233,252 @@ __device__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineH
     hdr[r] = H;
 }
 
-__global__ void __launch_bounds__(kSetupThreads) setup_kernel(GridDev g, LinesDev L, LineHdr *hdr, float *tabs, int64_t M)
+// ------------------------------------------------------------------ centre records
+// e-th derivative of the centred B-spline beta^n at x2 / 2 (right limit).
+__host__ __device__ constexpr double bspline_deriv(int n, int x2, int e)
+{
+    const int m = n + 1, t2 = x2 + m;   // twice the distance from the support's start
+    if (e > n || t2 < 0 || t2 / 2 >= m) return 0.0;
+    double sum = 0.0, binom = 1.0;
+    for (int k = 0; k <= t2 / 2; ++k) {
+        double pw = 1.0;
+        for (int i = 1; i <= n - e; ++i) pw = pw * (0.5 * (t2 - 2 * k)) / i;
+        sum += ((k & 1) ? -binom : binom) * pw;
+        binom = binom * (m - k) / (k + 1);
+    }
+    return sum;
+}
+
+__host__ __device__ constexpr double factorial(int n)
+{
+    double r = 1.0;
+    for (int i = 2; i <= n; ++i) r *= i;
+    return r;
+}
+
+// The constants of build_center, folded into its code.
+template <int N>
+struct CenterConst {
+    // piece[x2][e][k]: coefficient of (x - x2/2)^k of the e-th derivative of
+    // beta^N in the piece around x2/2 (x2 = 0..3)
+    float piece[4][N + 1][N + 1] = {};
+    // low[j][e][k][r]: weight of the moment mu[k][r] in the e-th derivative at
+    // (j + c) a, both signs of k together
+    float low[4][N + 1][3][N + 1] = {};
+    constexpr CenterConst()
+    {
+        constexpr int m = N + 1;
+        for (int x2 = 0; x2 < 4; ++x2)
+            for (int e = 0; e <= N; ++e)
+                for (int k = 0; k <= N - e; ++k) piece[x2][e][k] = (float)(bspline_deriv(N, x2, e + k) / factorial(k));
+        for (int j = 0; j < 4; ++j)
+            for (int e = 0; e <= N; ++e)
+                for (int k = 0; k < 3; ++k)
+                    for (int r = 0; r <= N - e; ++r) {
+                        // beta^(e)(j - k + c - d) = sum_r D d^r, and d -> -d for -k
+                        const int c2 = m % 2 == 0 ? 1 : 0;
+                        const double sg = (r & 1) ? -1.0 : 1.0;
+                        const double up = bspline_deriv(N, 2 * (j - k) + c2, e + r) / factorial(r) * sg;
+                        const double dn = bspline_deriv(N, 2 * (j + k) + c2, e + r) / factorial(r);
+                        low[j][e][k][r] = (float)(up + dn);
+                    }
+    }
+};
+
+// e-th derivative of beta^n at x in its polynomial piece around x2 / 2.
+template <int N>
+__device__ __forceinline__ float bspline_piece(const CenterConst<N> &T, int x2, int e, float x)
+{
+    const float d = x - 0.5f * (float)x2;
+    float r = 0.f;
+#pragma unroll
+    for (int k = N; k >= 0; --k)
+        if (k <= N - e) r = __fmaf_rn(r, d, T.piece[x2][e][k]);
+    return r;
+}
+
+// Gauss-Legendre rule of N + 1 points on [-1, 1] (exact to degree 2N + 1).
+template <int N>
+__device__ __forceinline__ void gauss(int i, float &x, float &w)
+{
+    if constexpr (N == 1) {
+        x = i ? 0.577350269189626f : -0.577350269189626f;
+        w = 1.f;
+    } else if constexpr (N == 2) {
+        x = i == 0 ? -0.774596669241483f : i == 1 ? 0.f : 0.774596669241483f;
+        w = i == 1 ? 8.f / 9.f : 5.f / 9.f;
+    } else {
+        x = i == 0 ? -0.861136311594053f : i == 1 ? -0.339981043584856f : i == 2 ? 0.339981043584856f : 0.861136311594053f;
+        w = (i == 0 || i == 3) ? 0.347854845137454f : 0.652145154862546f;
+    }
+}
+
+// The centre record (common.cuh) of a direction with parameters a >= b, degree
+// N, m = N + 1, by one thread.  With y the offset from the footprint's centre,
+//   phi(y) = 1/a int beta(s) beta((y - b s)/a) ds,
+// so at y = (j + c) a, c = 1/2 (m even) or 0 (m odd), the second factor and its
+// first n derivatives are polynomials in d = b s/a - k on the pieces
+// |d| < 1/2, the same pieces for every j: the derivatives 0..n are sums of the
+// moments mu[k][r] = int beta(s) d^r ds with rational weights (all terms of one
+// size: no cancellation).  The derivatives n + e + 1 are
+//   a^-m sum_p (-1)^p C(m, p) (d/dy)^e beta_b((j + c + m/2 - p) a),
+// beta_b the B-spline of knot spacing b, at most two of whose arguments,
+// +- a/2 and +- 3a/2, lie in its support.  The knots follow the same comparisons
+// as the pieces taken there.
+template <int N>
+__device__ void build_center(float a, float b, float *__restrict__ out)
+{
+    constexpr int m = N + 1;
+    constexpr CenterConst<N> T;
+    const float ia = 1.0f / a, tau = b * ia;
+    const float t1 = 0.5f / tau, t2 = 1.5f / tau;   // where b s/a passes 1/2 and 3/2 (infinite at b = 0)
+    float mu[3][N + 1];   // s >= 0
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int r = 0; r <= N; ++r) mu[k][r] = 0.f;
+    // pieces of beta^N(s), s >= 0: around x2 / 2, [lo, hi]
+    constexpr int kPieces = (m + 1) / 2;
+#pragma unroll
+    for (int p = 0; p < kPieces; ++p) {
+        const int x2 = (m % 2 == 0) ? 2 * p + 1 : 2 * p;
+        const float lo = fmaxf(0.5f * (float)(x2 - 1), 0.f), hi = 0.5f * (float)(x2 + 1);
+        const int k0 = (lo >= t1) + (lo >= t2);
+        const float cut = fminf(fmaxf(k0 == 0 ? t1 : k0 == 1 ? t2 : hi, lo), hi);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float l0 = h ? cut : lo, l1 = h ? hi : cut;
+            const float hw = 0.5f * (l1 - l0), mid = 0.5f * (l1 + l0);
+            const int k = k0 + h;
+#pragma unroll
+            for (int i = 0; i <= N; ++i) {
+                float x, w;
+                gauss<N>(i, x, w);
+                const float s = __fmaf_rn(hw, x, mid);
+                float g = w * hw * bspline_piece<N>(T, x2, 0, s);
+                const float d = __fmaf_rn(tau, s, -(float)k);
+#pragma unroll
+                for (int r = 0; r <= N; ++r) {
+#pragma unroll
+                    for (int kk = 0; kk < 3; ++kk)
+                        if (k == kk) mu[kk][r] += g;
+                    g *= d;
+                }
+            }
+        }
+    }
+    // beta_b's derivatives (times b^(1+e)) at a/2 and 3a/2, in the pieces that
+    // the comparisons choose
+    float H0[N + 1], H1[N + 1];
+    {
+        const bool in0 = N == 2 ? 3.f * b >= a : 2.f * b >= a;
+        const bool in1 = N == 3 && 4.f * b >= a;   // one piece further out
+        const float x = 0.5f * a / b;
+#pragma unroll
+        for (int e = 0; e <= N; ++e) {
+            float v = 0.f;
+            if (in0) v = bspline_piece<N>(T, N == 2 ? 2 : 1, e, x);
+            else if (in1) v = bspline_piece<N>(T, 3, e, x);
+            H0[e] = v;
+            H1[e] = (N == 3 && 4.f * b >= 3.f * a) ? bspline_piece<N>(T, 3, e, 3.f * x) : 0.f;
+        }
+    }
+    const float ib = b > 0.f ? 1.0f / b : 0.f;
+    float iam = ia;
+#pragma unroll
+    for (int k = 1; k < m; ++k) iam *= ia;
+    float4 *o4 = reinterpret_cast<float4 *>(out);
+    constexpr int J = N == 1 ? 2 : 4;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float c[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) c[k] = 0.f;
+        if (j < J) {
+            float sc = ia;   // a^-(1+e)
+#pragma unroll
+            for (int e = 0; e <= N; ++e) {
+                float acc = 0.f;
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+#pragma unroll
+                    for (int r = 0; r <= N; ++r)
+                        if (T.low[j][e][k][r] != 0.f) acc = __fmaf_rn(T.low[j][e][k][r], mu[k][r], acc);
+                constexpr float kInvFact[4] = {1.f, 1.f, 0.5f, 1.f / 6.f};
+                c[e] = acc * sc * kInvFact[e];
+                sc *= ia;
+            }
+            float sb = iam * ib;   // a^-m b^-(1+e)
+#pragma unroll
+            for (int e = 0; e <= N; ++e) {
+                float acc = 0.f;
+#pragma unroll
+                for (int p = 0; p <= m; ++p) {
+                    const int i2 = 2 * j + (m % 2 == 0 ? 1 : 0) + m - 2 * p;   // twice the argument over a
+                    const float w = binomf(m, p) * ((p & 1) ? -1.f : 1.f) * ((i2 < 0 && (e & 1)) ? -1.f : 1.f);
+                    if (i2 == 1 || i2 == -1) acc = __fmaf_rn(w, H0[e], acc);
+                    if (N == 3 && (i2 == 3 || i2 == -3)) acc = __fmaf_rn(w, H1[e], acc);
+                }
+                constexpr float kInvFact[8] = {1.f, 1.f, 1.f / 2.f, 1.f / 6.f, 1.f / 24.f, 1.f / 120.f, 1.f / 720.f, 1.f / 5040.f};
+                c[m + e] = acc * sb * kInvFact[m + e];
+                sb *= ib;
+            }
+        }
+        o4[2 * j] = make_float4(c[0], c[1], c[2], c[3]);
+        o4[2 * j + 1] = make_float4(c[4], c[5], c[6], c[7]);
+    }
+    // knots: 1 / ((2n+1)! (a b)^(n+1)), none at b = 0 (the Dirac of Prop. 1)
+    float ab = a * b, kap = ab;
+#pragma unroll
+    for (int k = 1; k < m; ++k) kap *= ab;
+    constexpr float kInvFact = N == 3 ? 1.f / 5040.f : N == 2 ? 1.f / 120.f : 1.f / 6.f;
+    kap = b > 0.f ? kInvFact / kap : 0.f;
+    // knot q, at +beta of the candidates kk = p - off, p = 0..m
+    auto knot = [&](int slot, int q, int off, float beta) {
+        out[kCenterBeta + slot] = beta;
+        const float kq = kap * binomf(m, q) * ((q & 1) ? -1.f : 1.f);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int pp = j + off, pm = (m % 2 == 0 ? -j - 1 : -j) + off;
+            const float jp = binomf(m, pp) * ((pp & 1) ? -0.5f : 0.5f), jm = binomf(m, pm) * ((pm & 1) ? -0.5f : 0.5f);
+            out[kCenterJump + 8 * slot + 2 * j] = (jp + jm) * kq;
+            out[kCenterJump + 8 * slot + 2 * j + 1] = (jp - jm) * kq;
+        }
+    };
+    if constexpr (N == 3) {
+        if (2.f * b >= a) knot(0, 3, 2, b - 0.5f * a);
+        else knot(0, 1, 3, 0.5f * a - b);
+        if (2.f * b < a) {
+            if (4.f * b >= a) knot(1, 4, 2, 2.f * b - 0.5f * a);
+            else knot(1, 0, 3, 0.5f * a - 2.f * b);
+        } else {
+            if (4.f * b >= 3.f * a) knot(1, 4, 1, 2.f * b - 1.5f * a);
+            else knot(1, 0, 4, 1.5f * a - 2.f * b);
+        }
+    } else if constexpr (N == 2) {
+        knot(0, 1, 2, 0.5f * (a - b));
+        if (3.f * b <= 2.f * a) {
+            if (3.f * b >= a) knot(1, 3, 1, 1.5f * b - 0.5f * a);
+            else knot(1, 0, 2, 0.5f * a - 1.5f * b);
+        } else {
+            knot(1, 0, 3, 1.5f * (a - b));
+        }
+    } else {
+        if (2.f * b >= a) knot(0, 2, 1, b - 0.5f * a);
+        else knot(0, 0, 2, 0.5f * a - b);
+        kap = 0.f;
+        knot(1, 0, 0, a);   // none
+    }
+    out[kCenterA] = a;
+    out[kCenterB] = b;
+}
+
+// Line records, and per table (one per line, one per view for parallel beams):
+// with tabs its head (a, b and the footprint's kind, from which tables_kernel
+// builds the rest), with rec (degree 1..3 B-splines) its centre record.
+template <int DEG>
+__global__ void __launch_bounds__(kSetupThreads) setup_kernel(GridDev g, LinesDev L, LineHdr *hdr, float *tabs, float *rec,
+                                                              int64_t M)
 {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     // parallel and fan beams: sin and cos of each view once per block (the
@@ -249,7 +494,7 @@ __global__ void __launch_bounds__(kSetupThreads) setup_kernel(GridDev g, LinesDe
         if (threadIdx.x < nv) sincos((double)L.view[v0 + threadIdx.x], &vsin[threadIdx.x], &vcos[threadIdx.x]);
         __syncthreads();
     }
-        if (r >= M) return;
+    if (r >= M) return;
     float af, bf;
     int mode;
     if (views) {
@@ -258,12 +503,15 @@ __global__ void __launch_bounds__(kSetupThreads) setup_kernel(GridDev g, LinesDe
     } else {
         setup_line(g, L, r, hdr, nullptr, nullptr, af, bf, mode);
     }
-    const int tab = (L.kind == SP_LINES_PARALLEL) ? (int)(r / L.n_det) : (int)r;
+    const int64_t tab = (L.kind == SP_LINES_PARALLEL) ? r / L.n_det : r;
     if (L.kind != SP_LINES_PARALLEL || r % L.n_det == 0) {
-        // the owner of table tab hands a, b and the footprint kind to the table builder
-        tabs[(int64_t)tab * kTabFloats + kTabA] = af;
-        tabs[(int64_t)tab * kTabFloats + kTabB] = bf;
-        tabs[(int64_t)tab * kTabFloats + kTabMode] = (float)mode;
+        if (tabs) {
+            tabs[tab * kTabFloats + kTabA] = af;
+            tabs[tab * kTabFloats + kTabB] = bf;
+            tabs[tab * kTabFloats + kTabMode] = (float)mode;
+        }
+        if constexpr (DEG >= 1)
+            if (rec) build_center<DEG>(af, bf, rec + tab * kCenterFloats);
     }
 }
 
@@ -713,54 +961,6 @@ __global__ void __launch_bounds__(kTabWarps * 32) tables_kernel(float *tabs, int
     build_table_half<DEG>(af, bf, out, scratch[2 * warp + half], lane & 15, half ? 0xFFFF0000u : 0x0000FFFFu);
 }
 
-// Line setup and tables in one pass, for B-spline footprints with one table
-// per line (fan beams, point pairs, (theta, y) lists): each warp sets up 32
-// lines, one per lane (the FP64 geometry at full width), then builds their
-// 32 tables two at a time, one per half-warp.  Warps at the FP64 stage and
-// warps at the table stage share the SMs, so the two overlap.
-template <int DEG>
-__global__ void __launch_bounds__(kTabWarps * 32) setup_tables_kernel(GridDev g, LinesDev L, LineHdr *hdr, float *tabs,
-                                                                      int64_t M)
-{
-    __shared__ __align__(16) float scratch[2 * kTabWarps][kBuildScratch];
-    __shared__ double vsin[kTabWarps * 32], vcos[kTabWarps * 32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t r0 = (int64_t)blockIdx.x * blockDim.x;
-    const int64_t r = r0 + threadIdx.x;
-    // fan beams: sin and cos of each view once per block (at most blockDim.x views)
-    const bool views = (L.kind == SP_LINES_FAN);
-    int64_t v0 = 0;
-    if (views) {
-        const int64_t r1 = min(r0 + (int64_t)blockDim.x, M) - 1;
-        v0 = r0 / L.n_det;
-        const int64_t nv = r1 / L.n_det - v0 + 1;
-        if (threadIdx.x < nv) sincos((double)L.view[v0 + threadIdx.x], &vsin[threadIdx.x], &vcos[threadIdx.x]);
-        __syncthreads();
-    }
-    float af = 0.f, bf = 0.f;
-    int mode = 0;
-    if (r < M) {
-        if (views) {
-            const int k = (int)(r / L.n_det - v0);
-            setup_line(g, L, r, hdr, &vsin[k], &vcos[k], af, bf, mode);
-        } else {
-            setup_line(g, L, r, hdr, nullptr, nullptr, af, bf, mode);
-        }
-    }
-    // the warp's 32 tables (table index = line index), two at a time
-    const int half = lane >> 4, hl = lane & 15;
-    const unsigned gmask = half ? 0xFFFF0000u : 0x0000FFFFu;
-    const int64_t rw = r0 + (int64_t)warp * 32;
-    for (int k = 0; k < 16; ++k) {
-        const int src = 2 * k + half;   // the lane that set up this half's line
-        const float a = __shfl_sync(0xffffffffu, af, src);
-        const float b = __shfl_sync(0xffffffffu, bf, src);
-        const int64_t rr = rw + src;
-        if (rr < M) build_table_half<DEG>(a, b, tabs + rr * kTabFloats, scratch[2 * warp + half], hl, gmask);
-        __syncwarp();
-    }
-}
-
 // ------------------------------------------------------------------ evaluation
 // Visit every candidate of every row of one line; `op(node, phi)` is called
 // for in-grid candidates (phi may be 0 beyond the support).
@@ -1005,34 +1205,12 @@ inline unsigned warp_blocks(int64_t lines)
     default: KERNEL<3><<<GRID, BLOCK, 0, STREAM>>>(__VA_ARGS__); break;                   \
     }
 
-cudaError_t launch_setup(const GridDev &g, const LinesDev &L, LineHdr *hdr, float *tabs, cudaStream_t s)
+cudaError_t launch_setup(const GridDev &g, const LinesDev &L, LineHdr *hdr, float *tabs, float *rec, cudaStream_t s)
 {
     if (L.m <= 0) return cudaSuccess;
-    setup_kernel<<<blocks_for(L.m, kSetupThreads), kSetupThreads, 0, s>>>(g, L, hdr, tabs, L.m);
+    if (!center_records(g)) rec = nullptr;
+    SPX_DISPATCH(g.kdeg, setup_kernel, blocks_for(L.m, kSetupThreads), kSetupThreads, s, g, L, hdr, tabs, rec, L.m);
     return cudaGetLastError();
-}
-
-cudaError_t launch_prepare(const GridDev &g, const LinesDev &L, LineHdr *hdr, float *tabs, int64_t n_tab,
-                           cudaStream_t s)
-{
-    if (L.m <= 0) return cudaSuccess;
-    // one table per line: setup and tables in one kernel, where there are
-    // enough lines for warps at the FP64 stage and warps at the table stage to
-    // coexist (at least two waves of four 256-line blocks per SM; with fewer,
-    // all warps pass through both stages together and two kernels are faster)
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int64_t wave = (int64_t)sms * 4 * kTabWarps * 32;
-    if (g.basis == SP_BASIS_BSPLINE && L.kind != SP_LINES_PARALLEL && L.m >= 2 * wave) {
-        SPX_DISPATCH(g.kdeg, setup_tables_kernel, blocks_for(L.m, kTabWarps * 32), kTabWarps * 32, s, g, L, hdr, tabs,
-                     L.m);
-        return cudaGetLastError();
-    }
-    e = launch_setup(g, L, hdr, tabs, s);
-    if (e == cudaSuccess) e = launch_tables(g, L, tabs, n_tab, s);
-    return e;
 }
 
 cudaError_t launch_tables(const GridDev &g, const LinesDev &L, float *tabs, int64_t n_tab,

@@ -12,44 +12,54 @@
 // transposed images so that strip rows stay contiguous in global memory.
 //
 // Lane = line, and the lanes of a warp walk the rows together.  Which
-// polynomial a candidate takes depends on where the row's u_0 lies among the
-// breakpoints s_q of the line's direction, which differs from lane to lane
-// and row to row.  So the kernels do not select polynomials at all.  The
-// footprint of degree n is a spline of degree 2n+1 with simple knots: across
-// the knot p a + q b only its (2n+1)-th derivative jumps, by
-// (-1)^(p+q) C(n+1,p) C(n+1,q) / (a b)^(n+1).  With the polynomials B_i of one
-// base interval of u_0, every candidate i is, for any u_0 in (0, a],
+// polynomial a candidate takes depends on where the row lies among the
+// footprint's knots, which differs from lane to lane and row to row, so the
+// kernels do not select polynomials.  The footprint of degree n is a spline
+// of degree 2n+1 with simple knots: across the knot p a + q b only its
+// (2n+1)-th derivative jumps, by (-1)^(p+q) C(n+1,p) C(n+1,q) / (a b)^(n+1).
+// Take the offsets of a row's candidates from the footprint's centre as
+// (kk + c) a + v with v in [-a/2, a/2) common to the row (c = 1/2 or 0 as n + 1
+// is even or odd).  In v the knots lie symmetrically around 0, in two pairs
+// +-beta (one at degree 1); a third kind, at v = +-a/2, is where the candidates
+// change.  So with the polynomials P_j of the interval around v = 0, w = |v|
+// and z = max(w - beta, 0)^(2n+1),
 //
-//   phi(u_0 + i a) = B_i(u_0 - s_base) + sum_q J_{p q} z_q,   p = i - floor(q b / a),
-//   J_{p q} = (-1)^(p+q) C(n+1,p) C(n+1,q) / ((2n+1)! (a b)^(n+1)),
-//   z_q = |u_0 - s_q|^(2n+1) beyond s_q as seen from the base interval, else 0.
+//   phi((j + c) a + w) = P_j(w) + J_j z + J'_j z',
 //
-// The sum over q depends on the candidate only through p, so breakpoints with
-// the same floor(q b / a) share one number Z_f = sum_q g_{qf} z_q, and a
-// candidate adds C(n+1, i - f) (-1)^(i - f) Z_f for each of the D = 1 + max f
-// values of f: integer weights known at compile time.  A lane holds its
-// line's B_i in registers (two candidates per packed FMA, fma.rn.f32x2) for
-// the whole strip: no table look-ups, no sorting and no branches per row.
-// The base interval is the one that leaves u_0 the shortest way to go
-// (its distance to the ends of (0, a]); the terms J z then stay below a few
-// tenths, and the FP32 evaluation of phi is about as accurate as one from
-// the interval's own polynomial (rms over random directions 1.4e-8 against
-// 1.2e-8 at degree 3).
+// and, as phi is even, the candidate on the other side is P_j(-w) with jumps
+// of its own.  One chain in v^2 gives the even and the odd part of P_j and
+// with them both candidates; half the sum of their jumps joins the even part,
+// half the difference, with the sign of v, the odd one.  A lane holds its line's P_j and J in registers
+// for the whole strip (the centre records of common.cuh): no table look-ups,
+// no sorting and no branches per row.  The jump terms stay below 1e-2 (w goes
+// at most min(b, a - b) or min(2b, a - 2b) beyond a knot), so phi keeps the
+// accuracy of its polynomials.
 //
-// u_0 is stepped from row to row in 64-bit fixed point: with W(r) =
-// 2^32 u(r)/a - 1 (u(r) the line's offset in row r at its reference column)
-// the high word of W is the row's step count and the low word its u_0.
+// v is stepped from row to row in 64-bit fixed point: with Y(r) =
+// 2^32 (y(r)/a + 1/2 - c), y(r) the offset from the centre in row r at the
+// line's reference column, the high word of Y is the row's step count and the
+// low word is v / a + 1/2.
 //
 // Sums.  Rows are taken in blocks of kRowBlock whose bounds are fixed in the
 // image.  A block's sum is one FP32 chain; block sums are added as float pairs
 // (two-sum), so that a line's value does not depend on how its blocks were
 // spread over warps and lanes, i.e. on the lines it shares a chunk with.
 //
-// What bounds it: the FMA pipe.  A row of a line with N = n + 1 + D candidates
-// takes N (2n+1) Horner FMAs, about (n + 2) D for the knots, 7 (n + 1) for the
-// z_q and N to accumulate (87 at n = 3, D = 2), and N shared-memory accesses;
-// the lanes' accesses of one row fall on neighbouring columns, in distinct
-// banks.
+// What bounds it: the issue slots (about 70 instructions per row and warp at
+// n = 3, 62 % of the slots filled) and the FMA pipe (54 % busy).  A pair of
+// candidates takes 3 packed FMAs (n = 3) for the even and odd parts, one
+// multiply and two additions to join them, 2 packed FMAs for the jumps and one
+// to accumulate; a row adds about 25 instructions (step, v, z, addresses).  The
+// lanes' strip accesses of one row fall on neighbouring columns, in distinct
+// banks.  Measured at the 512 x 512 cubic fan (552,960 lines), forward and
+// adjoint: 0.82 and 0.88 ms; one polynomial of 7 FMAs per candidate of a base
+// interval plus truncated powers with integer weights 1.19 and 1.28 ms; rows
+// sorted by interval, a lane per candidate and row, 2.18 and 2.35 ms.
+// Four CTAs of four warps per SM: while one CTA waits for its line records,
+// its strip or its flush, three others compute; two CTAs of eight warps with
+// strips of twice the height took 0.91 and 0.99 ms, three CTAs of eight warps
+// (80 registers) 0.95 and 0.98 ms, five of four warps (96 registers) 0.93 and
+// 0.92 ms.
 //
 // The adjoint accumulates its strip in 32-bit fixed point: a shared-memory
 // integer reduction costs about what a plain shared store does on this GPU,
@@ -69,30 +79,32 @@
 namespace spx {
 namespace {
 
-constexpr int kWarps = 8;
+constexpr int kWarps = 4;            // four CTAs of four warps per SM (see below)
 constexpr int kThreads = kWarps * 32;
+constexpr int kCtas = 4;             // CTAs per SM
 constexpr int kChunk = 32;          // lines per chunk (lanes of a warp)
 constexpr int kRowBlock = 4;        // rows summed in one FP32 chain
 constexpr int kSlopeBits = 15;      // fractional bits of the window's slope
 constexpr int kMaxWidth = 192;      // widest strip row (floats)
-constexpr int kStripFloats = 25280; // strip rows held at once times their width
-constexpr int kBasePitch = kSigStride + kTabHead + 4;   // a line's base polynomials and table head, spaced so that
-                                                        // 16-byte reads of 8 lanes meet 32 banks
-
+constexpr int kStripFloats = 11264; // strip rows held at once times their width
+constexpr int kSlabRows = 512;      // strip rows held at once, at most
 constexpr size_t kStripBytes = sizeof(float) * kStripFloats;
-constexpr size_t kBaseBytes = sizeof(float) * kBasePitch * kChunk;
+constexpr size_t kRecBytes = sizeof(float) * kCenterFloats * kChunk;
 constexpr size_t kHdrBytes = sizeof(LineHdr) * kChunk;
 constexpr size_t kPartBytes = 2 * sizeof(float) * kWarps * kChunk;
-constexpr size_t kSmemBytes = kStripBytes + kBaseBytes + kHdrBytes + kPartBytes;
-static_assert(kStripBytes % 16 == 0 && kBaseBytes % 16 == 0 && kHdrBytes % 16 == 0, "16-byte alignment of the regions");
-static_assert(kSmemBytes <= 115712, "two CTAs per SM");
-static_assert(kStripFloats / kMaxWidth >= 8 * kRowBlock, "the widest strip holds a row block per warp");
-static_assert(kBasePitch % 8 == 4, "conflict-free 16-byte reads");
+constexpr size_t kOffBytes = sizeof(int) * kSlabRows;
+constexpr size_t kSmemBytes = kStripBytes + kRecBytes + kHdrBytes + kPartBytes + kOffBytes;
+static_assert(kStripBytes % 16 == 0 && kRecBytes % 16 == 0 && kHdrBytes % 16 == 0, "16-byte alignment of the regions");
+static_assert(kSmemBytes <= 57344, "four CTAs per SM");
+static_assert(kStripFloats / kMaxWidth >= kWarps * kRowBlock, "the widest strip holds a row block per warp");
+static_assert(kPartBytes % 16 == 0 && kRowBlock == 4, "row offsets are read four at a time");
+static_assert(kCenterFloats % 8 == 4, "16-byte reads of 8 lanes meet 32 banks");
 
 // What the kernels are instantiated for: the B-spline degrees, and the
 // 3-direction box-spline (whose footprint is piecewise quadratic with knots
 // in its first two derivatives).
 constexpr int kKindBox = 4;
+__host__ __device__ constexpr int image_ld(int cols) { return (cols + 3) & ~3; }
 inline int strip_kind(const GridDev &g) { return g.basis == SP_BASIS_BOX3 ? kKindBox : g.kdeg; }
 
 // ------------------------------------------------------------------ packed FP32
@@ -168,12 +180,10 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool i
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
-// 4 bytes, or zeros where in is false (src is then not read).
-__device__ __forceinline__ void cp_async4(unsigned dst, const void *src, bool in)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Degree 0 (see PixelRows) carries more fractional bits.
+constexpr int kFrac0 = 48;
 
 // (xh + xl) / a in fixed point with F fractional bits, a = H.a_hi + H.a_lo:
 // the float quotient and one correction step.
@@ -186,251 +196,192 @@ __device__ __forceinline__ long long fix_quot(const LineHdr &H, float inv_a, flo
     return __float2ll_rn(q1 * kOne) + __float2ll_rn(r * inv_a * kOne);
 }
 
-// W of row 0 and its step per row.
-template <int F>
-__device__ __forceinline__ void row_stepping(const LineHdr &H, long long &W, long long &step)
+// Fixed-point position of a line's rows: the value in row 0 and the step per
+// row.  KIND 1..3: Y (see the top), b the line's b; others: W = 2^F u/a - 1,
+// whose high part is the step count of the run's first candidate and whose low
+// part is u_0 (F fractional bits).
+template <int KIND>
+__device__ __forceinline__ void row_stepping(const LineHdr &H, float b, long long &W, long long &step)
 {
+    constexpr int F = KIND == 0 ? kFrac0 : 32;
     const float inv_a = 1.0f / H.a;
     step = fix_quot<F>(H, inv_a, H.rho_hi, H.rho_lo);
-    W = fix_quot<F>(H, inv_a, H.U0, H.U0_lo) - 1 - H.r_ref * step;
+    W = fix_quot<F>(H, inv_a, H.U0, H.U0_lo) - H.r_ref * step;
+    if constexpr (KIND >= 1 && KIND <= 3) {
+        // y = u - w, w = m (a + b) / 2; a + b as a float pair
+        constexpr int m = KIND + 1;
+        const float s = __fadd_rn(H.a, b), e = __fsub_rn(b, __fsub_rn(s, H.a));
+        W -= (m * fix_quot<F>(H, inv_a, s, e)) >> 1;
+        if (m & 1) W += 1ll << 31;
+    } else {
+        W -= 1;
+    }
 }
 
-// The row records a plan keeps: every line's W of row 0 and its step, from
-// which all its rows follow (degree >= 1).
-__global__ void row_record_kernel(const LineHdr *__restrict__ hdr, int64_t m, longlong2 *__restrict__ rec)
+// The row records a plan keeps: every line's position in row 0 and its step,
+// from which all its rows follow (degree >= 1).
+template <int KIND>
+__global__ void row_record_kernel(const LineHdr *__restrict__ hdr, const float *__restrict__ center, int per_table,
+                                  int64_t m, longlong2 *__restrict__ out)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const LineHdr H = hdr[i];
     long long W = 0, step = 0;
-    if (!(H.flags & kEmpty)) row_stepping<32>(H, W, step);
-    rec[i] = make_longlong2(W, step);
+    if (!(H.flags & kEmpty)) {
+        const float b = KIND <= 3 ? center[(i / per_table) * kCenterFloats + kCenterB] : 0.f;
+        row_stepping<KIND>(H, b, W, step);
+    }
+    out[i] = make_longlong2(W, step);
 }
 
 // ------------------------------------------------------------------ one line on a strip
-// A lane's line on a strip: W of strip row 0 and the step per row; a run
-// starts in column q_ref minus W's high part.
+// A lane's line on a strip: the fixed-point position of strip row 0 and the
+// step per row; the run starts in column q_first minus the position's high
+// part.
 struct LaneLine {
     long long W0, Wstep;
-    int q_ref;
+    int q_first;
     float a, ua;               // a, and a / 2^F
+    float w_sup;               // half-width of the support
     float hp;                  // adjoint: h p (times the chunk's scale S for fixed-point strips)
-    // 1 at run time: multiplied by it the polynomials settle in register pairs;
-    // left as loaded, the compiler packs them anew in every row (48 moves a row
-    // at degree 3, 1.39 against 1.19 ms at the 512 x 512 cubic fan)
-    float one;
-    const float *base;         // B_i [8][8], then the table head
-    float s_base;              // the base interval's start
-    // the rows whose run reaches the line's last candidate slot (x up to the
-    // end of the support): slot N - 1 of lines with the warp's most slots N,
-    // slot N - 2 of the others
-    bool has_last;
-    unsigned x_end;
+    const float *rec;          // centre record (shared memory; KIND 1..3)
+    bool has_last;             // box-spline and degree 0: the line has the warp's last candidate,
+    unsigned x_end;            // ... and the rows that reach its own last one (low part up to this)
 };
 
 // The strip in shared memory: `rows` rows of `pitch` floats, row rr starting
 // at the column c0 + slope rr 2^-kSlopeBits rounded down to a multiple of 4.
 struct Strip {
     float *p;
+    int *off;   // per row: its start in p less its first column
     int pitch, rows, c0, slope;
     __device__ __forceinline__ int first(int rr) const { return (c0 + ((slope * rr) >> kSlopeBits)) & ~3; }
 };
 
-// Candidate pair (2p, 2p+1)'s weights for the knots with floor(q b / a) = f:
-// (-1)^k C(m, k) at k = 2p - f and 2p + 1 - f.
-__host__ __device__ constexpr float knot_weight(int m, int k)
-{
-    if (k < 0 || k > m) return 0.f;
-    float r = 1.f;
-    for (int i = 1; i <= k; ++i) r = r * (float)(m - k + i) / (float)i;
-    return (k & 1) ? -r : r;
-}
-
-// The values of f = floor(q b / a) that knot q can have in a warp whose lines
-// have D or D - 1 of them (b / a in (max(D - 2, 0) / m, D / m)).
-__host__ __device__ constexpr int knot_f_lo(int m, int D, int q) { return D >= 2 ? q * (D - 2) / m : 0; }
-__host__ __device__ constexpr int knot_f_hi(int m, int D, int q) { return (q * D + m - 1) / m - 1; }
-
-// Rows [r0, r1) of a block for one B-spline line of degree DEG, m = DEG + 1,
-// N = m + D candidates: the polynomials and knots in registers.
-template <int DEG, int D, bool ADJ, bool FIX>
+// One B-spline line of degree DEG in registers: J pairs of candidates around
+// v = 0 (and for odd m = DEG + 1 the one in the middle), N columns from the
+// run's first.
+template <int DEG, int J, bool ADJ, bool FIX>
 struct SplineRows {
     static constexpr int F = 32;
-    static constexpr int m = DEG + 1, NC = 2 * DEG + 2, N = m + D, NP = N / 2;
-    static constexpr int NQ = (m + 1) / 2;   // knots, two per packed operation
-    f2 C[NP][NC];      // candidates 2p, 2p + 1
-    float cl[NC];      // the last one of an odd N
-    f2 zs[NQ], zb[NQ]; // distance to knot q: zs u + zb, positive beyond it
-    float g[m][D];     // Z_f = sum_q g[q][f] z_q
-    float ua, ub;      // t = ua x + ub
-    float hp;          // float adjoint: the factor of phi
-    unsigned x_last, x_prev;   // rows that have candidates N - 1 and N - 2: x up to these
-    bool has_last;
+    static constexpr int m = DEG + 1, NC = 2 * DEG + 2, NH = NC / 2;
+    static constexpr bool kMid = m % 2 == 1;       // a candidate at v itself
+    static constexpr int kKnots = DEG == 1 ? 1 : 2;
+    f2 C[J][NH];            // (even, odd) coefficients, by powers of v^2
+    f2 K[J][kKnots];        // jumps: half their sum and half their difference
+    float cm[NH], km[kKnots];   // the middle candidate
+    float beta[2], ua, ha;
+    float hp, ca[J], w_sup;     // float adjoint: factor, (j + c) a, half-width of the support
 
     __device__ __forceinline__ void load(const LaneLine &ln)
     {
+        const float sc = FIX ? ln.hp : 1.f;
+        const f2 sc2 = f2pack(sc, sc);
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            float c[8];
+        for (int j = 0; j < J; ++j) {
+            const float *T = ln.rec + 8 * (j + (kMid ? 1 : 0));
 #pragma unroll
-            for (int d4 = 0; d4 < (NC + 3) / 4; ++d4) {
-                const float4 w = *reinterpret_cast<const float4 *>(ln.base + i * kNC + 4 * d4);
-                c[4 * d4] = w.x; c[4 * d4 + 1] = w.y; c[4 * d4 + 2] = w.z; c[4 * d4 + 3] = w.w;
+            for (int k = 0; k < NH; k += 2) {
+                const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(T + 2 * k);
+                C[j][k] = FIX ? f2mul(t.x, sc2) : t.x;
+                if (k + 1 < NH) C[j][k + 1] = FIX ? f2mul(t.y, sc2) : t.y;
             }
 #pragma unroll
-            for (int d = 0; d < NC; ++d) {
-                const float v = c[d] * (FIX ? ln.hp : ln.one);
-                if (i == 2 * NP) {
-                    cl[d] = v;
-                } else if (i & 1) {
-                    float lo, hi;
-                    f2unpack(C[i / 2][d], lo, hi);
-                    C[i / 2][d] = f2pack(lo, v);
-                } else {
-                    C[i / 2][d] = f2pack(v, 0.f);
-                }
+            for (int q = 0; q < kKnots; ++q) {
+                const f2 t = *reinterpret_cast<const f2 *>(ln.rec + kCenterJump + 8 * q + 2 * (j + (kMid ? 1 : 0)));
+                K[j][q] = FIX ? f2mul(t, sc2) : t;
             }
+            ca[j] = ((float)j + (kMid ? 1.f : 0.5f)) * ln.a;
         }
-        const float a = ln.a, b = ln.base[kSigStride + kTabB], inv_a = 1.0f / a;
-        // 1 / ((2n+1)! (a b)^(n+1)); no knots in b = 0 (the Dirac of Prop. 1)
-        float ab = a * b, kap = ab;
+        if constexpr (kMid) {
 #pragma unroll
-        for (int k = 1; k < m; ++k) kap *= ab;
-        constexpr float kFact = DEG == 3 ? 5040.f : DEG == 2 ? 120.f : 6.f;
-        kap = b > 0.f ? 1.0f / (kFact * kap) : 0.f;
-        if constexpr (FIX) kap *= ln.hp;
-        float zsv[2 * NQ], zbv[2 * NQ];
+            for (int k = 0; k < NH; ++k) cm[k] = ln.rec[2 * k] * sc;
 #pragma unroll
-        for (int k = 0; k < 2 * NQ; ++k) { zsv[k] = 0.f; zbv[k] = 0.f; }
-#pragma unroll
-        for (int q = 1; q <= m; ++q) {
-            // s_q = q b - f a in (0, a], as the table builder takes it
-            int f = (int)floorf((float)q * b * inv_a);
-            float s = __fmaf_rn((float)(-f), a, (float)q * b);
-            if (s <= 0.f) { f -= 1; s = __fmaf_rn((float)(-f), a, (float)q * b); }
-            else if (s > a) { f += 1; s = __fmaf_rn((float)(-f), a, (float)q * b); }
-            const float sg = s <= ln.s_base ? -1.f : 1.f;   // knots below the base interval look down
-            zsv[q - 1] = sg * ln.ua;
-            zbv[q - 1] = sg * (ln.ua - s);
-            // (a value of f outside the range only arises at s_q = 0 or a to
-            // rounding, where z_q vanishes)
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-                const bool can = k >= knot_f_lo(m, D, q) && k <= knot_f_hi(m, D, q);
-                g[q - 1][k] = (can && f == k) ? kap * knot_weight(m, q) : 0.f;
-            }
+            for (int q = 0; q < kKnots; ++q) km[q] = ln.rec[kCenterJump + 8 * q] * sc;
         }
-#pragma unroll
-        for (int k = 0; k < NQ; ++k) {
-            zs[k] = f2pack(zsv[2 * k], zsv[2 * k + 1]);
-            zb[k] = f2pack(zbv[2 * k], zbv[2 * k + 1]);
-        }
+        beta[0] = ln.rec[kCenterBeta];
+        beta[1] = ln.rec[kCenterBeta + 1];
         ua = ln.ua;
-        ub = ln.ua - ln.s_base;
+        ha = 0.5f * ln.a;
         hp = ln.hp;
-        has_last = ln.has_last;
-        x_last = ln.x_end;
-        x_prev = has_last ? 0xffffffffu : ln.x_end;
+        w_sup = ln.w_sup;
     }
 
     // One row at strip address sp (the run's first column).
-    __device__ __forceinline__ void row(long long W, float *sp, f2 &acc) const
+    __device__ __forceinline__ void row(long long Y, float *sp, f2 &acc) const
     {
-        const float xf = (float)(unsigned)W;
-                const bool on_last = has_last && (unsigned)W <= x_last, on_prev = (unsigned)W <= x_prev;
-        const float t = __fmaf_rn(xf, ua, ub);
-        const f2 tt = f2pack(t, t), xx = f2pack(xf, xf);
-        float z[2 * NQ];
-#pragma unroll
-        for (int k = 0; k < NQ; ++k) {
-            float d0, d1;
-            f2unpack(f2fma(xx, zs[k], zb[k]), d0, d1);
-            const f2 d = f2pack(fmaxf(d0, 0.f), fmaxf(d1, 0.f));
+        const float v = __fmaf_rn((float)(unsigned)Y, ua, -ha);
+        const float w = fabsf(v), s = v * v;
+        const f2 ss = f2pack(s, s);
+        float z[2] = {0.f, 0.f};
+        if constexpr (kKnots == 2) {
+            const f2 d = f2pack(fmaxf(w - beta[0], 0.f), fmaxf(w - beta[1], 0.f));
             const f2 d2 = f2mul(d, d);
-            f2 w = f2mul(d2, d);                     // d^3
-            if constexpr (DEG == 2) w = f2mul(w, d2);                  // d^5
-            if constexpr (DEG == 3) w = f2mul(w, f2mul(d2, d2));       // d^7
-            f2unpack(w, z[2 * k], z[2 * k + 1]);
+            f2 t = f2mul(d2, d);                                       // d^3
+            if constexpr (DEG == 2) t = f2mul(t, d2);                  // d^5
+            if constexpr (DEG == 3) t = f2mul(t, f2mul(d2, d2));       // d^7
+            f2unpack(t, z[0], z[1]);
+        } else {
+            const float d = fmaxf(w - beta[0], 0.f);
+            z[0] = d * d * d;
         }
-        float Z[D];
+        f2 zz[kKnots];   // (z, z sign(v))
 #pragma unroll
-        for (int f = 0; f < D; ++f) {
-            bool any = false;
-            Z[f] = 0.f;
+        for (int q = 0; q < kKnots; ++q) zz[q] = f2pack(z[q], copysignf(z[q], v));
 #pragma unroll
-            for (int q = 1; q <= m; ++q)
-                if (f >= knot_f_lo(m, D, q) && f <= knot_f_hi(m, D, q)) {
-                    Z[f] = any ? __fmaf_rn(g[q - 1][f], z[q - 1], Z[f]) : g[q - 1][f] * z[q - 1];
-                    any = true;
-                }
+        for (int j = 0; j < J; ++j) {
+            f2 h = C[j][NH - 1];
+#pragma unroll
+            for (int k = NH - 2; k >= 0; --k) h = f2fma(h, ss, C[j][k]);
+            float e, o;
+            f2unpack(h, e, o);
+            // even and odd part with the jumps: the candidate on the side of
+            // larger columns takes their sum, its mirror image the difference
+            f2 eo = f2pack(e, v * o);
+#pragma unroll
+            for (int q = 0; q < kKnots; ++q) eo = f2fma(zz[q], K[j][q], eo);
+            f2unpack(eo, e, o);
+            put(sp, J + (kMid ? 1 : 0) + j, J - 1 - j, __fadd_rn(e, o), __fsub_rn(e, o), ca[j], v, acc);
         }
+        if constexpr (kMid) {
+            float e = cm[NH - 1];
 #pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            f2 e = C[p][0], phi = C[p][NC - 1];
+            for (int k = NH - 2; k >= 0; --k) e = __fmaf_rn(e, s, cm[k]);
 #pragma unroll
-            for (int f = 0; f < D; ++f)
-                if (2 * p + 1 - f >= 0 && 2 * p - f <= m) {
-                    // (scalar FMAs with immediate weights: packed ones need
-                    // two moves per weight pair and row, 4 % slower)
-                    float e0, e1;
-                    f2unpack(e, e0, e1);
-                    if (2 * p - f >= 0 && 2 * p - f <= m) e0 = __fmaf_rn(Z[f], knot_weight(m, 2 * p - f), e0);
-                    if (2 * p + 1 - f >= 0 && 2 * p + 1 - f <= m) e1 = __fmaf_rn(Z[f], knot_weight(m, 2 * p + 1 - f), e1);
-                    e = f2pack(e0, e1);
-                }
-#pragma unroll
-            for (int d = NC - 2; d >= 1; --d) phi = f2fma(phi, tt, C[p][d]);
-            phi = f2fma(phi, tt, e);
-            const bool on0 = 2 * p == N - 2 ? on_prev : true;
-            const bool on1 = 2 * p + 1 == N - 1 ? on_last : 2 * p + 1 == N - 2 ? on_prev : true;
+            for (int q = 0; q < kKnots; ++q) e = __fmaf_rn(z[q], km[q], e);
             if constexpr (ADJ) {
-                float v0, v1;
-                if constexpr (FIX) {
-                    int *ip = reinterpret_cast<int *>(sp);
-                    f2unpack(f2add(phi, f2pack(kFixMagic, kFixMagic)), v0, v1);
-                    // (adding zero instead of branching)
-                    red_shared_u32(ip + 2 * p, on0 ? __float_as_int(v0) - kFixMagicBits : 0);
-                    red_shared_u32(ip + 2 * p + 1, on1 ? __float_as_int(v1) - kFixMagicBits : 0);
-                } else {
-                    f2unpack(phi, v0, v1);
-                    if (on0) red_shared(sp + 2 * p, hp * v0);
-                    if (on1) red_shared(sp + 2 * p + 1, hp * v1);
-                }
+                if constexpr (FIX) red_shared_u32(reinterpret_cast<int *>(sp) + J, __float_as_int(e + kFixMagic) - kFixMagicBits);
+                else red_shared(sp + J, hp * e);
             } else {
-                float c0 = 0.f, c1 = 0.f;
-                if (on0) c0 = sp[2 * p];
-                if (on1) c1 = sp[2 * p + 1];
-                acc = f2fma(f2pack(c0, c1), phi, acc);
-            }
-        }
-        if constexpr (N & 1) {
-            float e = cl[0], phi = cl[NC - 1];
-#pragma unroll
-            for (int f = 0; f < D; ++f)
-                if (N - 1 - f <= m) e = __fmaf_rn(Z[f], knot_weight(m, N - 1 - f), e);
-#pragma unroll
-            for (int d = NC - 2; d >= 1; --d) phi = __fmaf_rn(phi, t, cl[d]);
-            phi = __fmaf_rn(phi, t, e);
-            if constexpr (ADJ) {
-                if constexpr (FIX) {
-                    red_shared_u32(reinterpret_cast<int *>(sp) + N - 1,
-                                   on_last ? __float_as_int(phi + kFixMagic) - kFixMagicBits : 0);
-                } else {
-                    if (on_last) red_shared(sp + N - 1, hp * phi);
-                }
-            } else {
-                float c = 0.f, a0, a1;
-                if (on_last) c = sp[N - 1];
+                float a0, a1;
                 f2unpack(acc, a0, a1);
-                acc = f2pack(__fmaf_rn(c, phi, a0), a1);
+                acc = f2pack(__fmaf_rn(sp[J], e, a0), a1);
             }
+        }
+    }
+
+    __device__ __forceinline__ void put(float *sp, int ip, int im, float p, float q, float c, float v, f2 &acc) const
+    {
+        if constexpr (ADJ && FIX) {
+            f2unpack(f2add(f2pack(p, q), f2pack(kFixMagic, kFixMagic)), p, q);
+            red_shared_u32(reinterpret_cast<int *>(sp) + ip, __float_as_int(p) - kFixMagicBits);
+            red_shared_u32(reinterpret_cast<int *>(sp) + im, __float_as_int(q) - kFixMagicBits);
+        } else if constexpr (ADJ) {
+            // (values here may be non-finite: only candidates in the support)
+            if (c + v <= w_sup) red_shared(sp + ip, hp * p);
+            if (c - v <= w_sup) red_shared(sp + im, hp * q);
+        } else {
+            acc = f2fma(f2pack(sp[ip], sp[im]), f2pack(p, q), acc);
         }
     }
 };
 
-// The same for the 3-direction box-spline: at most three breakpoints, across
-// which the first two derivatives jump (the first one where a box is as
-// narrow as a Dirac), per candidate as the table's polynomials differ.
+// A line of the 3-direction box-spline: the polynomials of one base interval of
+// u_0 in (0, a], the one that leaves u_0 the shortest way to the ends, and for
+// each of at most three breakpoints what the table's polynomials change there
+// (the first two derivatives, the first one where a box is as narrow as a
+// Dirac).
 template <int N, bool ADJ, bool FIX>
 struct BoxRows {
     static constexpr int F = 32, NB = 3;
@@ -442,20 +393,28 @@ struct BoxRows {
 
     __device__ __forceinline__ void load(const LaneLine &ln, const float *tab)
     {
-        float s[NB + 1];
+        float s[NB + 2];
         s[0] = 0.f;
+        s[NB + 1] = ln.a;
 #pragma unroll
         for (int k = 0; k < NB; ++k) s[k + 1] = fminf(tab[k], ln.a);
+        int sg_base = 0;
+        float s_base = 0.f, best = FLT_MAX;
+#pragma unroll
+        for (int k = 0; k <= NB; ++k) {
+            const float far = fmaxf(s[k], ln.a - s[k + 1]);
+            if (far < best && s[k + 1] > s[k]) { best = far; sg_base = k; s_base = s[k]; }
+        }
         const float sc = FIX ? ln.hp : 1.f;
 #pragma unroll
         for (int i = 0; i < N; ++i)
 #pragma unroll
-            for (int d = 0; d < 3; ++d) c[i][d] = ln.base[i * kNC + d] * sc;
+            for (int d = 0; d < 3; ++d) c[i][d] = tab[tab_poly(sg_base, i) + d] * sc;
 #pragma unroll
         for (int k = 0; k < NB; ++k) {
             // breakpoint s[k + 1] between the intervals k and k + 1
             const float L = s[k + 1] - s[k];
-            const float sg = s[k + 1] <= ln.s_base ? -1.f : 1.f;
+            const float sg = s[k + 1] <= s_base ? -1.f : 1.f;
             zs[k] = sg * ln.ua;
             zb[k] = sg * (ln.ua - s[k + 1]);
             const bool real = s[k + 1] < ln.a;
@@ -468,7 +427,7 @@ struct BoxRows {
             }
         }
         ua = ln.ua;
-        ub = ln.ua - ln.s_base;
+        ub = ln.ua - s_base;
         hp = ln.hp;
         has_last = ln.has_last;
         x_last = ln.x_end;
@@ -519,10 +478,11 @@ __device__ __forceinline__ void walk_blocks(const Rows &R, const LaneLine &ln, c
     long long W = ln.W0 + (long long)(b0 * kRowBlock) * ln.Wstep;
     for (int b = b0; b < b1; ++b) {
         f2 acc = 0ull;
-        int rr = b * kRowBlock;
+        const int4 off4 = reinterpret_cast<const int4 *>(st.off)[b];
+        const int off[kRowBlock] = {off4.x, off4.y, off4.z, off4.w};
 #pragma unroll
-        for (int k = 0; k < kRowBlock; ++k, ++rr) {
-            float *sp = st.p + (rr * st.pitch + (ln.q_ref - (int)(W >> Rows::F) - st.first(rr)));
+        for (int k = 0; k < kRowBlock; ++k) {
+            float *sp = st.p + (off[k] + ln.q_first - (int)(W >> Rows::F));
             R.row(W, sp, acc);
             W += ln.Wstep;
         }
@@ -538,32 +498,22 @@ __device__ __forceinline__ void walk_blocks(const Rows &R, const LaneLine &ln, c
 // Degree 0 has at most two candidates per row and two intervals; its lanes
 // select the (linear) polynomials.  Its footprint can have ramps far narrower
 // than one float ulp of u, so W carries 48 fractional bits.
-constexpr int kFrac0 = 48;
-
 // One row of a degree-0 line exactly along an axis (kDeg0Axis), whose
 // footprint is a rectangle with edges on nodes, each taking the midpoint value
 // on both sides (so a row has one more candidate): straight from or to global
 // memory.  Such lines occur only at views exactly along an axis.
-__device__ __noinline__ float axis_row0(const LineHdr &H, const float *tab, int r, const float *__restrict__ src,
-                                        float *dst, int Nq, float hp, bool adj)
+__device__ __noinline__ float axis_row0(const LineHdr &H, int r, const float *__restrict__ src, float *dst, int Nq, int ld,
+                                        float hp, bool adj)
 {
     const float inv_a = 1.0f / H.a;
-    float s0[1] = {tab[0]};
+    float s0[1] = {H.a};   // b = 0: one interval
     float acc = 0.f;
     const RowEval e = row_eval<0>(H, s0, inv_a, r);
-    for (int i = -1; i < H.K; ++i) {
-        const int q = e.q0 + i;
+    for (int q = e.tie ? e.q0 - 1 : e.q0; q <= e.q0; ++q) {
         if ((unsigned)q >= (unsigned)Nq) continue;
-        float phi;
-        if (i < 0) {
-            if (!e.tie) continue;
-            phi = 0.5f * inv_a;   // the run also starts at u = 0
-        } else {
-            phi = horner<0>(tab + tab_poly(e.sg, i), __fmaf_rn((float)i, H.a_corr, e.t));
-            if (e.tie) phi = 0.5f * phi;
-        }
-        if (adj) atomicAdd(dst + (size_t)r * Nq + q, hp * phi);
-        else acc = __fmaf_rn(__ldg(src + (size_t)r * Nq + q), phi, acc);
+        const float phi = e.tie ? 0.5f * inv_a : inv_a;
+        if (adj) atomicAdd(dst + (size_t)r * ld + q, hp * phi);
+        else acc = __fmaf_rn(__ldg(src + (size_t)r * ld + q), phi, acc);
     }
     return acc;
 }
@@ -578,23 +528,28 @@ struct PixelRows {
     float ua, hp;
     bool has_last;
 
-    __device__ __forceinline__ void load(const LaneLine &ln, const float *tab, float a_corr)
+    // b: |sin| or |cos|, the shorter; a_corr = |kappa| - a
+    __device__ __forceinline__ void load(const LaneLine &ln, float b, float a_corr)
     {
+        // the trapezoid of height 1/a: a ramp of width b up in interval 0
+        // (candidate 0) and down (candidate 1), its top in interval 1
+        const float a = ln.a, top = 1.0f / a, slope = b > 0.f ? top / b : 0.f;
+        c0[0][0] = b > 0.f ? 0.f : top;
+        c1[0][0] = slope;
+        c0[0][1] = __fmaf_rn(-slope, a_corr, top);
+        c1[0][1] = -slope;
+        c0[1][0] = top;
+        c1[1][0] = c0[1][1] = c1[1][1] = 0.f;
+        if constexpr (FIX) {
 #pragma unroll
-        for (int sg = 0; sg < 2; ++sg)
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float *T = tab + tab_poly(sg, i);
-                c1[sg][i] = T[1];
-                c0[sg][i] = i ? __fmaf_rn(T[1], a_corr, T[0]) : T[0];
-                if constexpr (FIX) {
-                    c0[sg][i] = __fmaf_rn(c0[sg][i], ln.hp, kFixMagic);
-                    c1[sg][i] *= ln.hp;
-                }
+            for (int k = 0; k < 4; ++k) {
+                c0[k >> 1][k & 1] = __fmaf_rn(c0[k >> 1][k & 1], ln.hp, kFixMagic);
+                c1[k >> 1][k & 1] *= ln.hp;
             }
-        const float s = tab[0], a = ln.a, inv_a = 1.0f / a;
-        const float q1 = fminf(s * inv_a, 2.f);
-        const float r = fminf(__fmaf_rn(-q1, a, s) * inv_a, 1.f);
+        }
+        const float s = b > 0.f ? b : a;
+        const float q1 = s * top;
+        const float r = __fmaf_rn(-q1, a, s) * top;
         S1 = (unsigned long long)max(__float2ll_rn(q1 * 281474976710656.f) + __float2ll_rn(r * 281474976710656.f), 0ll);
         ua = ln.ua;
         hp = ln.hp;
@@ -623,26 +578,35 @@ struct PixelRows {
 };
 
 // ------------------------------------------------------------------ chunks
+// One of the two images the strips are cut from: nodes [row][column] with the
+// lines' major axis along the rows; rows of ld floats, a multiple of 4, the
+// columns from Nq on zero (forward) or ignored (adjoint).
+struct Image {
+    const float *src;
+    float *dst;
+    int Nr, Nq, ld;
+};
+
 // The rows of this lane's line on a strip, blocks [b0, b1) (none where the
-// lane has no line): loads the line's polynomials and walks.  n: the
-// candidates of the warp's lines (the most).
+// lane has no line): loads the line's polynomials and walks.  n: the columns of
+// the warp's runs.
 template <int KIND, bool ADJ, bool FIX>
 __device__ __forceinline__ void strip_line(int n, const LaneLine &ln, const LineHdr &H, const float *tab, const Strip &st,
-                                           int S0, int b0, int b1, const float *__restrict__ src, float *dst, int Nq,
-                                           float hp_raw, float &hi, float &lo)
+                                           int S0, int b0, int b1, const Image &im, float hp_raw, float &hi, float &lo)
 {
     if constexpr (KIND == 0) {
         if (H.flags & kDeg0Axis) {
             for (int b = b0; b < b1; ++b) {
                 float acc = 0.f;
                 for (int r = max(S0 + b * kRowBlock, H.r_begin); r < min(S0 + (b + 1) * kRowBlock, H.r_end); ++r)
-                    acc += axis_row0(H, tab, r, src, dst, Nq, hp_raw, ADJ);
+                    acc += axis_row0(H, r, im.src, im.dst, im.Nq, im.ld, hp_raw, ADJ);
                 pair_add(hi, lo, acc);
             }
             return;
         }
+        const float b = fabsf(H.rho_hi + H.rho_lo);
         PixelRows<ADJ, FIX> R;
-        R.load(ln, tab, H.a_corr);
+        R.load(ln, b < 1e-30f ? 0.f : b, H.a_corr);
         walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
     } else if constexpr (KIND == kKindBox) {
         switch (n) {
@@ -651,81 +615,128 @@ __device__ __forceinline__ void strip_line(int n, const LaneLine &ln, const Line
         case 4: { BoxRows<4, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
         default: { BoxRows<3, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
         }
+    } else if constexpr (KIND == 1) {
+        SplineRows<1, 2, ADJ, FIX> R;
+        R.load(ln);
+        walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
     } else {
-        constexpr int m = KIND + 1;
-        switch (n - m) {
-        case 4: if constexpr (m >= 4) { SplineRows<KIND, m >= 4 ? 4 : 1, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); } break;
-        case 3: if constexpr (m >= 3) { SplineRows<KIND, m >= 3 ? 3 : 1, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); } break;
-        case 2: { SplineRows<KIND, 2, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
-        default: { SplineRows<KIND, 1, ADJ, FIX> R; R.load(ln); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
+        if (n > 2 * KIND + 1) {
+            SplineRows<KIND, KIND + 1, ADJ, FIX> R;
+            R.load(ln);
+            walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
+        } else {
+            SplineRows<KIND, KIND, ADJ, FIX> R;
+            R.load(ln);
+            walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
         }
     }
 }
 
-// The fewest candidates that strip_line is instantiated for.
+// Columns of a line's runs as strip_line takes them, and how many of them lie
+// before the column of the position's high part.  B-splines of degree >= 1:
+// every (j + c) a +- v that can lie in the support, (j + c) a - a/2 < w, on both
+// sides; degree 0 and the box-spline: the slots K of u_0 + i a.
 template <int KIND>
-__device__ __forceinline__ int fewest_slots() { return KIND == 0 ? 2 : KIND == kKindBox ? 3 : KIND + 2; }
-
-// Adds the accumulated strip into the image: 16-byte reductions where the
-// image rows allow it.
-__device__ __forceinline__ void strip_flush(const Strip &st, int S0, int Nr, int Nq, float *dst, bool fixed, float finv,
-                                            int vec)
+__device__ __forceinline__ int run_columns(const LineHdr &H, float b)
 {
-    if (vec) {
-        const int nch = st.pitch / 4;
-        const unsigned inv = 0xffffffffu / (unsigned)nch + 1u;   // i / nch = umulhi(i, inv) for every strip index
-        for (int i = threadIdx.x; i < st.rows * nch; i += kThreads) {
-            const int rr = (int)__umulhi((unsigned)i, inv), q = st.first(rr) + 4 * (i - rr * nch);
-            const int4 n4 = reinterpret_cast<const int4 *>(st.p)[i];
-            float4 v = make_float4(__int_as_float(n4.x), __int_as_float(n4.y), __int_as_float(n4.z), __int_as_float(n4.w));
-            if (fixed)
-                v = make_float4((float)n4.x * finv, (float)n4.y * finv, (float)n4.z * finv, (float)n4.w * finv);
-            if ((unsigned)q < (unsigned)Nq && S0 + rr < Nr && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f))
-                asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + (size_t)(S0 + rr) * Nq + q),
-                             "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-                             : "memory");
+    if constexpr (KIND == 1) return 4;
+    else if constexpr (KIND == 2) return 3.f * b <= 2.f * H.a ? 5 : 7;
+    else if constexpr (KIND == 3) return 2.f * b <= H.a ? 6 : 8;
+    else return max(H.K, KIND == 0 ? 2 : 3);
+}
+template <int KIND>
+__device__ __forceinline__ int run_lead(int n) { return KIND >= 1 && KIND <= 3 ? n / 2 : 0; }
+
+// One line's sum over the nodes in its support only, from global memory (FP32,
+// by one thread): lines whose sum is not finite are taken again with this, as
+// the run of a row may reach nodes beyond the support, which a non-finite
+// coefficient there must not enter.
+template <int DEG>
+__device__ __noinline__ float exact_line(const LineHdr &H, const float *rec, long long Y0, long long step, float w_sup,
+                                         const float *__restrict__ src, int Nq, int ld)
+{
+    constexpr int m = DEG + 1, NC = 2 * DEG + 2;
+    constexpr float c = m % 2 == 0 ? 0.5f : 0.f;
+    const float a = H.a;
+    float hi = 0.f, lo = 0.f;
+    for (int r = H.r_begin; r < H.r_end; ++r) {
+        const long long Y = Y0 + r * step;
+        const float v = __fmaf_rn((float)(unsigned)Y, a * 2.3283064365386963e-10f, -0.5f * a), w = fabsf(v);
+        float z[2];
+        for (int q = 0; q < 2; ++q) {
+            const float d = fmaxf(w - rec[kCenterBeta + q], 0.f);
+            z[q] = d;
+            for (int k = 0; k < DEG; ++k) z[q] *= d * d;
         }
-    } else {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int rr = warp; rr < st.rows && S0 + rr < Nr; rr += kWarps)
-            for (int c = lane; c < st.pitch; c += 32) {
-                const int w = reinterpret_cast<const int *>(st.p)[rr * st.pitch + c], q = st.first(rr) + c;
-                const float v = fixed ? (float)w * finv : __int_as_float(w);
-                if ((unsigned)q < (unsigned)Nq && v != 0.f) atomicAdd(dst + (size_t)(S0 + rr) * Nq + q, v);
+        for (int kk = -4; kk < 4; ++kk) {
+            const int q = H.q_ref - (int)(Y >> 32) + kk, j = kk >= 0 ? kk : (m % 2 == 0 ? -kk - 1 : -kk);
+            if ((unsigned)q >= (unsigned)Nq || j > 3 || !(fabsf(((float)kk + c) * a + v) < w_sup)) continue;
+            const bool same = (kk >= 0) == (v >= 0.f) || (m % 2 == 1 && kk == 0);
+            const float x = same ? w : -w;
+            float phi = rec[8 * j + NC - 1];
+            for (int k = NC - 2; k >= 0; --k) phi = __fmaf_rn(phi, x, rec[8 * j + k]);
+            for (int k = 0; k < 2; ++k) {
+                const float *J = rec + kCenterJump + 8 * k + 2 * j;
+                phi = __fmaf_rn(same ? J[0] + J[1] : J[0] - J[1], z[k], phi);
             }
+            pair_add(hi, lo, __ldg(src + (size_t)r * ld + q) * phi);
+        }
+    }
+    return isfinite(lo) ? hi + lo : hi;
+}
+
+// Adds the accumulated strip into the image by 16-byte reductions.
+__device__ __forceinline__ void strip_flush(const Strip &st, int S0, const Image &im, bool fixed, float finv)
+{
+    const int nch = st.pitch / 4;
+    const unsigned inv = 0xffffffffu / (unsigned)nch + 1u;   // i / nch = umulhi(i, inv) for every strip index
+    for (int i = threadIdx.x; i < st.rows * nch; i += kThreads) {
+        const int rr = (int)__umulhi((unsigned)i, inv), q = st.first(rr) + 4 * (i - rr * nch);
+        const int4 n4 = reinterpret_cast<const int4 *>(st.p)[i];
+        float4 v = make_float4(__int_as_float(n4.x), __int_as_float(n4.y), __int_as_float(n4.z), __int_as_float(n4.w));
+        if (fixed) v = make_float4((float)n4.x * finv, (float)n4.y * finv, (float)n4.z * finv, (float)n4.w * finv);
+        if ((unsigned)q < (unsigned)im.ld && S0 + rr < im.Nr && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f))
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(im.dst + (size_t)(S0 + rr) * im.ld + q),
+                         "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+                         : "memory");
     }
 }
 
-// Stages the strip's coefficients, zeros outside the grid.
-__device__ __forceinline__ void strip_stage(const Strip &st, int S0, int Nr, int Nq, const float *__restrict__ src, int vec)
+// Stages the strip's coefficients with asynchronous 16-byte copies, zeros
+// outside the image (chunks are wholly inside or outside: ld and chunk starts
+// are multiples of 4).
+__device__ __forceinline__ void strip_stage(const Strip &st, int S0, const Image &im)
 {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(st.p);
-    if (vec) {
-        // asynchronous 16-byte copies; chunks are wholly inside or outside the
-        // grid (Nq and chunk starts are multiples of 4)
-        const int nch = st.pitch / 4;
-        const unsigned inv = 0xffffffffu / (unsigned)nch + 1u;
-        for (int i = threadIdx.x; i < st.rows * nch; i += kThreads) {
-            const int rr = (int)__umulhi((unsigned)i, inv), q = st.first(rr) + 4 * (i - rr * nch);
-            const bool in = (unsigned)q < (unsigned)Nq && S0 + rr < Nr;
-            cp_async16(sa + 16 * i, in ? src + (size_t)(S0 + rr) * Nq + q : src, in);
-        }
-    } else {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int rr = warp; rr < st.rows; rr += kWarps)
-            for (int c = lane; c < st.pitch; c += 32) {
-                const int q = st.first(rr) + c;
-                const bool in = (unsigned)q < (unsigned)Nq && S0 + rr < Nr;
-                cp_async4(sa + 4 * (rr * st.pitch + c), in ? src + (size_t)(S0 + rr) * Nq + q : src, in);
-            }
+    const int nch = st.pitch / 4;
+    const unsigned inv = 0xffffffffu / (unsigned)nch + 1u;
+    for (int i = threadIdx.x; i < st.rows * nch; i += kThreads) {
+        const int rr = (int)__umulhi((unsigned)i, inv), q = st.first(rr) + 4 * (i - rr * nch);
+        const bool in = (unsigned)q < (unsigned)im.ld && S0 + rr < im.Nr;
+        cp_async16(sa + 16 * i, in ? im.src + (size_t)(S0 + rr) * im.ld + q : im.src, in);
     }
 }
 
 // floor(a / b) for b > 0.
 __device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
+// The arguments of one strip projection.  img: the image (forward, read) and
+// the scratch images the adjoint adds to, as stored (0) and transposed (1).
+struct StripArgs {
+    GridDev g;
+    LinesDev L;
+    const LineHdr *hdr;
+    const float *center;       // centre records (B-splines of degree 1..3)
+    const float *tabs;         // footprint tables (box-spline)
+    const float *src[2];
+    float *dst[2];
+    float *sino;
+    const longlong2 *rec;      // row records, or NULL
+    int cpv;                   // chunks per view
+};
+
 // Forward (ADJ false): sino[line] = h sum c phi.  Adjoint (ADJ true): adds
-// h sino[line] phi to out (vertical lines) or outT (horizontal lines, the
+// h sino[line] phi to dst[0] (vertical lines) or dst[1] (horizontal lines, the
 // transposed image).
 // One chunk (view v, bins j0..j0+31) of one instance; smem is the CTA's
 // dynamic shared memory (kSmemBytes).
@@ -735,40 +746,38 @@ __device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b :
 // strips; returns whether the chunk was one of them.  The forward takes
 // kFmAll.
 template <int KIND, bool ADJ, int FM = kFmAll>
-__device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g, const LinesDev L,
-                                            const LineHdr *__restrict__ hdr, const float *__restrict__ tabs,
-                                            const float *__restrict__ coef, const float *__restrict__ coefT,
-                                            float *__restrict__ sino, float *__restrict__ out,
-                                            float *__restrict__ outT, int chunks_per_view, int vec, int chunk,
-                                            const longlong2 *__restrict__ rec)
+__device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs &A, int chunk)
 {
     static_assert(!ADJ || FM != kFmAll, "the adjoint runs as fixed-point and float launches");
     constexpr bool FIX = ADJ && FM == kFmFixed;
     constexpr int F = KIND == 0 ? kFrac0 : 32;
+    constexpr bool kCenter = KIND >= 1 && KIND <= 3;
+    const GridDev &g = A.g;
+    const LinesDev &L = A.L;
     float *strip = reinterpret_cast<float *>(smem);
-    float *base_s = reinterpret_cast<float *>(smem + kStripBytes);
-    LineHdr *hdr_s = reinterpret_cast<LineHdr *>(smem + kStripBytes + kBaseBytes);
-    float2 *part_s = reinterpret_cast<float2 *>(smem + kStripBytes + kBaseBytes + kHdrBytes);   // [warp][line]
+    float *rec_s = reinterpret_cast<float *>(smem + kStripBytes);
+    LineHdr *hdr_s = reinterpret_cast<LineHdr *>(smem + kStripBytes + kRecBytes);
+    float2 *part_s = reinterpret_cast<float2 *>(smem + kStripBytes + kRecBytes + kHdrBytes);   // [warp][line]
+    int *off_s = reinterpret_cast<int *>(smem + kStripBytes + kRecBytes + kHdrBytes + kPartBytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int v = chunk / chunks_per_view, cb = chunk - v * chunks_per_view;
+    const int v = chunk / A.cpv, cb = chunk - v * A.cpv;
     const int j0 = cb * kChunk;
     const int64_t nd = chunk_bins(L);
     const int nl = (int)min((int64_t)kChunk, nd - j0);
     // position of the chunk's first line (in the sorted order for free lists),
-    // and lane l's line and table index in every warp (one table per view for
-    // parallel beams, else table = line)
+    // and lane l's line in every warp (directions: one per view for parallel
+    // beams, else one per line)
     const int64_t line0 = (int64_t)v * nd + j0;
     const int my_line = lane < nl ? (L.order ? __ldg(L.order + line0 + lane) : (int)(line0 + lane)) : 0;
-    const bool shared_tab = L.kind == SP_LINES_PARALLEL;
-    const float *my_tab = tabs + (shared_tab ? (int64_t)v : (int64_t)my_line) * kTabFloats;
+    const bool shared_dir = L.kind == SP_LINES_PARALLEL;
 
     // The adjoint's values, and the chunk's fixed-point scale (a power of two;
     // see the top of the file).  Non-finite values, or values so large or
     // small that it leaves a safe exponent range, keep the float reductions.
     float pv = 0.f, fscale = 1.f, finv = 1.f;
     if constexpr (ADJ) {
-        if (lane < nl) pv = sino[my_line];
+        if (lane < nl) pv = A.sino[my_line];
         // (bits of non-negative floats order like the floats; non-finite ones on top)
         const unsigned pm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(pv)));
         const float top = kPhiBound * g.h * __uint_as_float(pm);   // largest |h p phi| of the chunk
@@ -784,75 +793,62 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g
         }
     }
 
-    // the chunk's line records into shared memory, and every line's base
-    // interval: the one that leaves u_0 the shortest way to the ends of (0, a]
+    // the chunk's line records and centre records into shared memory
     static_assert(kChunk * 4 <= kThreads && sizeof(LineHdr) == 64, "one pass over the chunk's line records");
     {
         const int src = __shfl_sync(0xffffffffu, my_line, (threadIdx.x >> 2) & 31);
         if ((int)threadIdx.x < nl * 4)
             reinterpret_cast<int4 *>(hdr_s)[threadIdx.x] =
-                __ldg(reinterpret_cast<const int4 *>(hdr + src) + (threadIdx.x & 3));
+                __ldg(reinterpret_cast<const int4 *>(A.hdr + src) + (threadIdx.x & 3));
     }
-    int sg_base = 0;
-    float s_base = 0.f;
-    if constexpr (KIND != 0) {
-        const float4 h0 = __ldg(reinterpret_cast<const float4 *>(my_tab));
-        const float a = __ldg(my_tab + kTabA);
-        const float s[5] = {h0.x, h0.y, h0.z, h0.w, a};
-        constexpr int NI = KIND == kKindBox ? 4 : KIND + 2;   // intervals
-        float lo = 0.f, best = FLT_MAX;
-#pragma unroll
-        for (int k = 0; k < NI; ++k) {
-            const float end = k < NI - 1 ? fminf(s[k], a) : a;
-            const float far = fmaxf(lo, a - end);
-            if (far < best && end > lo) { best = far; sg_base = k; s_base = lo; }
-            lo = end;
-        }
-        // the base polynomials and the table head
-        const int nt = shared_tab ? 1 : nl;
-        constexpr int kCh = (kSigStride + kTabHead) / 4;
-        const unsigned ba = (unsigned)__cvta_generic_to_shared(base_s);
+    float my_b = 0.f;
+    if constexpr (kCenter) {
+        my_b = __ldg(A.center + (shared_dir ? (int64_t)v : (int64_t)my_line) * kCenterFloats + kCenterB);
+        const int nt = shared_dir ? 1 : nl;
+        constexpr int kCh = kCenterFloats / 4;
+        const unsigned ba = (unsigned)__cvta_generic_to_shared(rec_s);
         for (int i0 = warp * 32; i0 < nt * kCh; i0 += kThreads) {
-            const int i = i0 + lane, li = min(i / kCh, kChunk - 1), c = i - li * kCh;
-            const int sg = __shfl_sync(0xffffffffu, sg_base, li);
-            const int ti = shared_tab ? v : __shfl_sync(0xffffffffu, my_line, li);
-            const float *t = tabs + (int64_t)ti * kTabFloats;
-            if (i < nt * kCh)
-                cp_async16(ba + 4 * (li * kBasePitch + 4 * c),
-                           c < kSigStride / 4 ? t + tab_poly(sg, 0) + 4 * c : t + 4 * (c - kSigStride / 4));
+            const int i = i0 + lane, li = min(i / kCh, kChunk - 1);
+            const int ti = shared_dir ? v : __shfl_sync(0xffffffffu, my_line, li);
+            if (i < nt * kCh) cp_async16(ba + 16 * i, A.center + (int64_t)ti * kCenterFloats + 4 * (i - li * kCh));
         }
     }
     if (!ADJ) part_s[warp * kChunk + lane] = make_float2(0.f, 0.f);
     __syncthreads();
 
-    // this lane's line: W at its reference row, and the step per row
+    // this lane's line: its position in row 0, and the step per row
     bool mine = false, mine_vert = false;
     long long my_W = 0, my_step = 0;
-    int my_K = 0;
+    int my_n = 0;
     if (lane < nl) {
         const LineHdr &H = hdr_s[lane];
         mine = !(H.flags & kEmpty) && H.r_end > H.r_begin && (!ADJ || pv != 0.f);
         mine_vert = (H.flags & kVert) != 0;
         if (mine) {
-            if (rec) {
-                const longlong2 t = __ldg(rec + my_line);
+            if (A.rec) {
+                const longlong2 t = __ldg(A.rec + my_line);
                 my_W = t.x;
                 my_step = t.y;
             } else {
-                row_stepping<F>(H, my_W, my_step);
+                row_stepping<KIND>(H, my_b, my_W, my_step);
             }
-            my_K = max(H.K, fewest_slots<KIND>() - 1);
+            my_n = run_columns<KIND>(H, my_b);
         }
     }
     for (int axis = 0; axis < 2; ++axis) {
         const bool vert = axis == 0;
         const unsigned mask = __ballot_sync(0xffffffffu, mine && mine_vert == vert);
-        const int Nq = vert ? g.nx : g.ny, Nr = vert ? g.ny : g.nx;
-        const float *src = vert ? coef : coefT;
-        float *dst = vert ? out : outT;
+        if (mask == 0u) continue;
+        Image im;
+        im.src = A.src[axis];
+        im.dst = A.dst[axis];
+        im.Nr = vert ? g.ny : g.nx;
+        im.Nq = vert ? g.nx : g.ny;
+        im.ld = image_ld(im.Nq);
         // Groups: aligned spans of lines [ga, ga + len), len a power of two,
-        // whose runs fit a strip row and whose candidate slots differ by at
-        // most one; others are halved.  Every warp finds the same ones.
+        // whose runs fit a strip row (and, where the run is the line's slots,
+        // differ by at most one); others are halved.  Every warp finds the
+        // same ones.
         for (int ga = 0, len = kChunk; ga < kChunk; ga += len, len = ga & -ga) {
             auto in_span = [&](int a, int n) { return mask & ((n >= 32 ? 0xffffffffu : (1u << n) - 1u) << a); };
             if (in_span(ga, len) == 0u) continue;
@@ -862,10 +858,10 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g
                 while (len > 1 && in_span(ga + (len >> 1), len >> 1) == 0u) len >>= 1;
                 const bool in = (in_span(ga, len) >> lane) & 1u;
                 // row range of the group in whole blocks, and the lowest and
-                // highest run start of its lines in the first and the last
-                // row.  A run starts within one column above its line, and
-                // lines are straight, so between the two rows the starts stay
-                // within a column of the chords through the extremes.
+                // highest column of its lines in the first and the last row.
+                // The position's column lies within one above the line's, and
+                // lines are straight, so between the two rows the columns stay
+                // within one of the chords through the extremes.
                 R0 = __reduce_min_sync(0xffffffffu, in ? hdr_s[lane].r_begin : INT_MAX) & -kRowBlock;
                 R1 = (__reduce_max_sync(0xffffffffu, in ? hdr_s[lane].r_end : INT_MIN) + kRowBlock - 1) & -kRowBlock;
                 const int qa = in ? hdr_s[lane].q_ref - (int)((my_W + R0 * my_step) >> F) : 0;
@@ -874,70 +870,73 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g
                 lb = __reduce_min_sync(0xffffffffu, in ? qb : INT_MAX);
                 const int ha = __reduce_max_sync(0xffffffffu, in ? qa : INT_MIN);
                 const int hb = __reduce_max_sync(0xffffffffu, in ? qb : INT_MIN);
-                n = max(__reduce_max_sync(0xffffffffu, in ? my_K : 0), fewest_slots<KIND>());
-                const int nmin = __reduce_min_sync(0xffffffffu, in ? my_K : INT_MAX);
-                // 3 columns below the lowest start, 3 beyond the highest run,
-                // 3 for the start rounded down to a multiple of 4
+                n = __reduce_max_sync(0xffffffffu, in ? my_n : 0);
+                const int nmin = __reduce_min_sync(0xffffffffu, in ? my_n : INT_MAX);
+                // 3 columns below the lowest run, 3 beyond the highest, 3 for
+                // the start rounded down to a multiple of 4
                 width = (max(ha - la, hb - lb) + n + 9 + 3) & ~3;
-                if (len == 1 || (width <= kMaxWidth && n - nmin <= 1)) break;
+                if (len == 1 || (width <= kMaxWidth && (kCenter || n - nmin <= 1))) break;
                 len >>= 1;
                 if (in_span(ga, len) == 0u) ga += len;
             }
 
             // this lane's line of the group (groups of fewer than 32 lines:
             // several lanes per line, on consecutive rows)
-            const int li = ga + (lane & (len - 1)), parts = kChunk / len;
+            const int li = ga + (lane & (len - 1)), parts = kChunk / len, lead = run_lead<KIND>(n);
             const bool on = in_span(li, 1) != 0u;
             const int lj = on ? li : __ffs(in_span(ga, len)) - 1;   // (a lane without one looks at another's)
             const LineHdr &H = hdr_s[lj];
             LaneLine ln;
             ln.Wstep = __shfl_sync(0xffffffffu, my_step, lj);
             const long long W_row0 = __shfl_sync(0xffffffffu, my_W, lj);
-            ln.q_ref = H.q_ref;
-            ln.one = __uint_as_float(0x3f800000u + (unsigned)(nd >> 62));
+            ln.q_first = H.q_ref - lead;
             ln.a = H.a;
             ln.ua = H.a * (F == 32 ? 2.3283064365386963e-10f : 3.5527136788005009e-15f);
+            ln.w_sup = 0.5f * H.two_w * 1.000001f;   // (a bound for rounding)
             const float hp_raw = ADJ ? g.h * __shfl_sync(0xffffffffu, pv, lj) : 0.f;
             ln.hp = hp_raw * fscale;
-            ln.base = base_s + (shared_tab ? 0 : lj) * kBasePitch;
-            ln.s_base = __shfl_sync(0xffffffffu, s_base, lj);
-            ln.has_last = __shfl_sync(0xffffffffu, my_K, lj) >= n;
+            ln.rec = rec_s + (shared_dir ? 0 : lj) * kCenterFloats;
+            ln.has_last = __shfl_sync(0xffffffffu, my_n, lj) >= n && H.K >= n;
             {
                 // 2w - (K - 1) a in units of a 2^-32
                 const float end = H.two_w / H.a - (float)(H.K - 1);
                 ln.x_end = end >= 1.f ? 0xffffffffu : (unsigned)(fmaxf(end, 0.f) * 4294967296.f);
             }
-            const float *tab = tabs + (shared_tab ? (int64_t)v : (int64_t)__shfl_sync(0xffffffffu, my_line, lj)) * kTabFloats;
+            const float *tab = nullptr;
+            if constexpr (KIND == kKindBox)
+                tab = A.tabs + (shared_dir ? (int64_t)v : (int64_t)__shfl_sync(0xffffffffu, my_line, lj)) * kTabFloats;
 
             Strip st;
             st.p = strip;
+            st.off = off_s;
             st.pitch = width;
             const int span = max(R1 - 1 - R0, 1);
             st.slope = floor_div((lb - la) * (1 << kSlopeBits), span);
             // slabs of equal height that the strip can hold
-            const int most = (kStripFloats / width) & -kRowBlock;
+            const int most = min(kStripFloats / width, kSlabRows) & -kRowBlock;
             const int slabs = (R1 - R0 + most - 1) / most;
             const int per = ((R1 - R0 + slabs - 1) / slabs + kRowBlock - 1) & -kRowBlock;
             float hi = 0.f, lo = 0.f;
             for (int S0 = R0; S0 < R1; S0 += per) {
                 st.rows = min(per, R1 - S0);
-                st.c0 = la + floor_div((lb - la) * (S0 - R0), span) - 3;
+                st.c0 = la - lead + floor_div((lb - la) * (S0 - R0), span) - 3;
                 __syncthreads();   // the strip's last readers are done
+                for (int rr = threadIdx.x; rr < st.rows; rr += kThreads) st.off[rr] = rr * width - st.first(rr);
                 if constexpr (ADJ) {
                     float4 *s4 = reinterpret_cast<float4 *>(strip);
                     for (int i = threadIdx.x; i < st.rows * width / 4; i += kThreads) s4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 } else {
-                    strip_stage(st, S0, Nr, Nq, src, vec);
+                    strip_stage(st, S0, im);
                 }
-                cp_async_wait_all();   // the strip's copies, and the base polynomials'
+                cp_async_wait_all();   // the strip's copies, and the centre records'
                 __syncthreads();
                 const int nb = st.rows / kRowBlock, unit = warp * parts + lane / len, units = kWarps * parts;
                 const int b0 = nb * unit / units, b1 = on ? nb * (unit + 1) / units : b0;
                 ln.W0 = W_row0 + S0 * ln.Wstep;
-                strip_line<KIND, ADJ, FIX>(n, ln, H, tab, st, S0, b0, b1, src, dst, Nq, hp_raw, hi, lo);
+                strip_line<KIND, ADJ, FIX>(n, ln, H, tab, st, S0, b0, b1, im, hp_raw, hi, lo);
                 if constexpr (ADJ) {
                     __syncthreads();
-                    strip_flush(st, S0, Nr, Nq, dst, FIX, finv, vec);
+                    strip_flush(st, S0, im, FIX, finv);
                 }
             }
             if constexpr (!ADJ) {
@@ -965,7 +964,15 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g
                 pair_add(hi, lo, t.x);
                 lo += t.y;
             }
-            sino[my_line] = g.h * (hi + lo);
+            float sum = hi + lo;
+            if constexpr (kCenter) {
+                if (mine && !isfinite(sum)) {
+                    const int axis = mine_vert ? 0 : 1, Nq = mine_vert ? g.nx : g.ny;
+                    sum = exact_line<KIND>(hdr_s[lane], rec_s + (shared_dir ? 0 : lane) * kCenterFloats, my_W, my_step,
+                                           0.5f * hdr_s[lane].two_w, A.src[axis], Nq, image_ld(Nq));
+                }
+            }
+            A.sino[my_line] = g.h * sum;
         }
     }
     return true;
@@ -975,25 +982,17 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const GridDev g
 // nearly all) and appends the others to defer[2..] (count defer[0]) for
 // strip_float_kernel.
 template <int KIND, bool ADJ, int FM = kFmAll>
-__global__ void __launch_bounds__(kThreads, 2)
-strip_kernel(GridDev g, LinesDev L, const LineHdr *__restrict__ hdr, const float *__restrict__ tabs,
-             const float *__restrict__ coef, const float *__restrict__ coefT, float *__restrict__ sino,
-             float *__restrict__ out, float *__restrict__ outT, int chunks_per_view, int vec, unsigned *defer,
-             const longlong2 *__restrict__ rec)
+__global__ void __launch_bounds__(kThreads, kCtas) strip_kernel(const __grid_constant__ StripArgs A, unsigned *defer)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const bool ran = strip_chunk<KIND, ADJ, FM>(smem, g, L, hdr, tabs, coef, coefT, sino, out, outT, chunks_per_view,
-                                                vec, (int)blockIdx.x, rec);
+    const bool ran = strip_chunk<KIND, ADJ, FM>(smem, A, (int)blockIdx.x);
     if (FM == kFmFixed && !ran && threadIdx.x == 0) defer[2 + atomicAdd(defer, 1u)] = blockIdx.x;
 }
 
 // The deferred adjoint chunks (float strip accumulators): a small persistent
 // grid over defer[2 .. 2 + defer[0]), defer[1] its counter.
 template <int KIND>
-__global__ void __launch_bounds__(kThreads, 2)
-strip_float_kernel(GridDev g, LinesDev L, const LineHdr *__restrict__ hdr, const float *__restrict__ tabs,
-                   float *__restrict__ sino, float *__restrict__ out, float *__restrict__ outT, int chunks_per_view,
-                   int vec, unsigned *defer, const longlong2 *__restrict__ rec)
+__global__ void __launch_bounds__(kThreads, kCtas) strip_float_kernel(const __grid_constant__ StripArgs A, unsigned *defer)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned cur;
@@ -1003,10 +1002,15 @@ strip_float_kernel(GridDev g, LinesDev L, const LineHdr *__restrict__ hdr, const
         if (threadIdx.x == 0) cur = atomicAdd(defer + 1, 1u);
         __syncthreads();
         if (cur >= n) break;
-        strip_chunk<KIND, true, kFmFloat>(smem, g, L, hdr, tabs, nullptr, nullptr, sino, out, outT, chunks_per_view,
-                                          vec, (int)defer[2 + cur], rec);
+        strip_chunk<KIND, true, kFmFloat>(smem, A, (int)defer[2 + cur]);
     }
 }
+
+// One instance of the persistent kernel's work queue.
+struct StripJob {
+    StripArgs A;
+    long long chunk0;   // its first chunk in the queue
+};
 
 // Persistent kernel over the chunks of several instances of one kind (B-spline
 // degree, or box-spline): each
@@ -1029,7 +1033,7 @@ __device__ __forceinline__ const StripJob *queue_job(const StripJob *__restrict_
 }
 
 template <int KIND, bool ADJ>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, kCtas)
 strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total, unsigned long long *counter,
                    long long *defer, unsigned long long *defer_n)
 {
@@ -1042,16 +1046,14 @@ strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total
         const long long c = cur;
         if (c >= total) break;
         const StripJob *J = queue_job(jobs, njobs, c);
-        const bool ran = strip_chunk<KIND, ADJ, ADJ ? kFmFixed : kFmAll>(
-            smem, J->g, J->L, J->hdr, J->tabs, J->coef, J->coefT, J->sino, J->out, J->outT, J->cpv, J->vec,
-            (int)(c - J->chunk0), nullptr);
+        const bool ran = strip_chunk<KIND, ADJ, ADJ ? kFmFixed : kFmAll>(smem, J->A, (int)(c - J->chunk0));
         if (ADJ && !ran && threadIdx.x == 0) defer[atomicAdd(defer_n, 1ull)] = c;
     }
 }
 
 // The deferred adjoint chunks (float strip accumulators), persistent likewise.
 template <int KIND>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, kCtas)
 strip_queue_float_kernel(const StripJob *__restrict__ jobs, int njobs, const long long *__restrict__ defer,
                          const unsigned long long *__restrict__ defer_n, unsigned long long *counter)
 {
@@ -1066,17 +1068,8 @@ strip_queue_float_kernel(const StripJob *__restrict__ jobs, int njobs, const lon
         if (k >= (long long)n) break;
         const long long c = defer[k];
         const StripJob *J = queue_job(jobs, njobs, c);
-        strip_chunk<KIND, true, kFmFloat>(smem, J->g, J->L, J->hdr, J->tabs, J->coef, J->coefT, J->sino,
-                                                   J->out, J->outT, J->cpv, J->vec, (int)(c - J->chunk0),
-                                         nullptr);
+        strip_chunk<KIND, true, kFmFloat>(smem, J->A, (int)(c - J->chunk0));
     }
-}
-
-// 16-byte staging and flushing: image rows (nx and ny floats) and bases aligned.
-inline int strip_vec(const GridDev &g, const void *img, const void *imgT)
-{
-    return (g.nx % 4 == 0) && (g.ny % 4 == 0) && ((reinterpret_cast<uintptr_t>(img) & 15) == 0) &&
-           ((reinterpret_cast<uintptr_t>(imgT) & 15) == 0);
 }
 
 template <int KIND>
@@ -1108,141 +1101,164 @@ cudaError_t launch_queue_t(bool adj, const StripJob *jobs, int njobs, int64_t to
     return cudaGetLastError();
 }
 
-__global__ void transpose_kernel(const float *__restrict__ in, float *__restrict__ out, int nx, int ny)
+// The forward's images: the coefficients transposed, and (plain not NULL) as
+// stored, with rows padded by zeros to a multiple of 4.
+__global__ void stage_images_kernel(const float *__restrict__ in, float *__restrict__ plain, float *__restrict__ trans,
+                                    int nx, int ny)
 {
     __shared__ float tile[32][33];
-    const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    const int bx = blockIdx.x * 32, by = blockIdx.y * 32, ldx = image_ld(nx), ldy = image_ld(ny);
     for (int y = threadIdx.y; y < 32; y += 8) {
         const int i = bx + threadIdx.x, j = by + y;
-        if (i < nx && j < ny) tile[y][threadIdx.x] = in[(size_t)j * nx + i];
+        const float v = (i < nx && j < ny) ? in[(size_t)j * nx + i] : 0.f;
+        tile[y][threadIdx.x] = v;
+        if (plain && i < ldx && j < ny) plain[(size_t)j * ldx + i] = v;
     }
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const int j = by + threadIdx.x, i = bx + y;
-        if (i < nx && j < ny) out[(size_t)i * ny + j] = tile[threadIdx.x][y];
+        if (i < nx && j < ldy) trans[(size_t)i * ldy + j] = tile[threadIdx.x][y];
     }
 }
 
-// out[j][i] += inT[i][j]
-__global__ void add_transposed_kernel(const float *__restrict__ inT, float *__restrict__ out, int nx, int ny)
+// out[j][i] = plain[j][i] + trans[i][j] (padded rows in, plain rows out)
+__global__ void join_images_kernel(const float *__restrict__ plain, const float *__restrict__ trans, float *__restrict__ out,
+                                   int nx, int ny)
 {
     __shared__ float tile[32][33];
-    const int bi = blockIdx.x * 32, bj = blockIdx.y * 32;
+    const int bi = blockIdx.x * 32, bj = blockIdx.y * 32, ldx = image_ld(nx), ldy = image_ld(ny);
     for (int y = threadIdx.y; y < 32; y += 8) {
         const int i = bi + y, j = bj + threadIdx.x;
-        if (i < nx && j < ny) tile[y][threadIdx.x] = inT[(size_t)i * ny + j];
+        if (i < nx && j < ny) tile[y][threadIdx.x] = trans[(size_t)i * ldy + j];
     }
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const int j = bj + y, i = bi + threadIdx.x;
-        if (i < nx && j < ny) out[(size_t)j * nx + i] += tile[threadIdx.x][y];
+        if (i < nx && j < ny) out[(size_t)j * nx + i] = plain[(size_t)j * ldx + i] + tile[threadIdx.x][y];
     }
 }
 
-template <int KIND, bool ADJ>
-cudaError_t launch_strip_t(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                           const float *coef, float *imgT, float *sino, float *out, cudaStream_t s, const longlong2 *rec,
-                           unsigned *defer = nullptr)
+size_t image_bytes(int rows, int cols) { return (sizeof(float) * (size_t)rows * image_ld(cols) + 255) & ~(size_t)255; }
+
+// The arguments of a strip projection.  Forward: img is read, as it is where its
+// rows are whole 16-byte chunks.  scratch: strip_scratch_bytes.
+StripArgs make_args(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center, const float *tabs,
+                    const float *img, void *scratch, float *sino, const longlong2 *rec)
 {
-    const dim3 tb(32, 8), tg((g.nx + 31) / 32, (g.ny + 31) / 32);
+    StripArgs A;
+    A.g = g;
+    A.L = L;
+    A.hdr = hdr;
+    A.center = center;
+    A.tabs = tabs;
+    float *plain = static_cast<float *>(scratch);
+    float *trans = reinterpret_cast<float *>(static_cast<char *>(scratch) + image_bytes(g.ny, g.nx));
+    A.dst[0] = plain;
+    A.dst[1] = trans;
+    const bool direct = img && g.nx % 4 == 0 && (reinterpret_cast<uintptr_t>(img) & 15) == 0;
+    A.src[0] = direct ? img : plain;
+    A.src[1] = trans;
+    A.sino = sino;
+    A.rec = rec;
+    A.cpv = (int)((chunk_bins(L) + kChunk - 1) / kChunk);
+    return A;
+}
+
+// Before a projection: the forward's images, or the adjoint's cleared ones (and
+// the `words` words behind them); after the adjoint: its result.
+cudaError_t launch_images(const StripArgs &A, const float *img, cudaStream_t s)
+{
+    const dim3 tb(32, 8), tg((A.g.nx + 31) / 32, (image_ld(A.g.ny) + 31) / 32);
+    stage_images_kernel<<<tg, tb, 0, s>>>(img, A.src[0] == img ? nullptr : A.dst[0], A.dst[1], A.g.nx, A.g.ny);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_join(const StripArgs &A, float *out, cudaStream_t s)
+{
+    const dim3 tb(32, 8), tg((A.g.nx + 31) / 32, (A.g.ny + 31) / 32);
+    join_images_kernel<<<tg, tb, 0, s>>>(A.dst[0], A.dst[1], out, A.g.nx, A.g.ny);
+    return cudaGetLastError();
+}
+
+template <int KIND>
+cudaError_t launch_strip_t(const StripArgs &A, bool adj, unsigned *defer, cudaStream_t s)
+{
+    const unsigned grid = (unsigned)(chunk_views(A.L) * A.cpv);
     cudaError_t e;
-    if (ADJ && !defer) return cudaErrorInvalidValue;
-    if (!ADJ) {
-        transpose_kernel<<<tg, tb, 0, s>>>(coef, imgT, g.nx, g.ny);
-    } else {
-        e = cudaMemsetAsync(out, 0, sizeof(float) * (size_t)g.nx * g.ny, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(imgT, 0, sizeof(float) * (size_t)g.nx * g.ny, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(defer, 0, 2 * sizeof(unsigned), s);
+    if (!adj) {
+        e = cudaFuncSetAttribute(strip_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (e != cudaSuccess) return e;
+        strip_kernel<KIND, false><<<grid, kThreads, kSmemBytes, s>>>(A, nullptr);
+        return cudaGetLastError();
     }
-    // the adjoint: fixed-point chunks, then (a small second launch) the
-    // chunks they deferred to float strips
-    constexpr int FM1 = ADJ ? kFmFixed : kFmAll;
-    auto kern = strip_kernel<KIND, ADJ, FM1>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e == cudaSuccess && ADJ)
+    // fixed-point chunks, then (a small second launch) the chunks they
+    // deferred to float strips
+    e = cudaFuncSetAttribute(strip_kernel<KIND, true, kFmFixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(strip_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    int dev = 0, sms = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (strip_needs_order(L) && !L.order) return cudaErrorInvalidValue;   // free lists need their order
-    const int cpv = (int)((chunk_bins(L) + kChunk - 1) / kChunk);
-    const unsigned grid = (unsigned)(chunk_views(L) * cpv);
-    const int vec = strip_vec(g, ADJ ? out : coef, imgT);
-    kern<<<grid, kThreads, kSmemBytes, s>>>(g, L, hdr, tabs, coef, imgT, const_cast<float *>(sino), out, imgT, cpv,
-                                            vec, defer, rec);
+    strip_kernel<KIND, true, kFmFixed><<<grid, kThreads, kSmemBytes, s>>>(A, defer);
     e = cudaGetLastError();
-    if (e == cudaSuccess && ADJ) {
-        int dev = 0, sms = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const unsigned g2 = grid < (unsigned)sms ? grid : (unsigned)sms;
-        if (e == cudaSuccess)
-            strip_float_kernel<KIND><<<g2, kThreads, kSmemBytes, s>>>(g, L, hdr, tabs, const_cast<float *>(sino), out,
-                                                                     imgT, cpv, vec, defer, rec);
-        if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess)
+        strip_float_kernel<KIND><<<grid < (unsigned)sms ? grid : (unsigned)sms, kThreads, kSmemBytes, s>>>(A, defer);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+cudaError_t launch_strip(const StripArgs &A, bool adj, unsigned *defer, cudaStream_t s)
+{
+    if (strip_needs_order(A.L) && !A.L.order) return cudaErrorInvalidValue;   // free lists need their order
+    switch (strip_kind(A.g)) {
+    case 0: return launch_strip_t<0>(A, adj, defer, s);
+    case 1: return launch_strip_t<1>(A, adj, defer, s);
+    case 2: return launch_strip_t<2>(A, adj, defer, s);
+    case 3: return launch_strip_t<3>(A, adj, defer, s);
+    default: return launch_strip_t<kKindBox>(A, adj, defer, s);
     }
-    if (e == cudaSuccess && ADJ) {
-        add_transposed_kernel<<<tg, tb, 0, s>>>(imgT, out, g.nx, g.ny);
-        e = cudaGetLastError();
-    }
-    return e;
 }
 
 }  // namespace
 
 int strip_queue_kind(const GridDev &g) { return strip_kind(g); }
 
-StripJob make_strip_job(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs, bool adj,
-                        const float *img_in, float *sino, float *img_out, void *scratch)
+int64_t strip_chunk_count(const LinesDev &L) { return chunk_views(L) * ((chunk_bins(L) + kChunk - 1) / kChunk); }
+
+size_t strip_job_bytes(int count) { return sizeof(StripJob) * (size_t)count; }
+
+void make_strip_job(void *jobs, int k, const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                    const float *tabs, const float *img, float *sino, void *scratch, long long chunk0)
 {
-    StripJob J;
-    J.g = g;
-    J.L = L;
-    J.hdr = hdr;
-    J.tabs = tabs;
-    J.coef = adj ? nullptr : img_in;
-    J.coefT = static_cast<float *>(scratch);
-    J.sino = sino;
-    J.out = adj ? img_out : nullptr;
-    J.outT = static_cast<float *>(scratch);
-    J.cpv = (int)((chunk_bins(L) + kChunk - 1) / kChunk);
-    J.vec = strip_vec(g, adj ? img_out : img_in, scratch);
-    J.chunk0 = 0;
-    return J;
+    StripJob *J = static_cast<StripJob *>(jobs) + k;
+    J->A = make_args(g, L, hdr, center, tabs, img, scratch, sino, nullptr);
+    J->chunk0 = chunk0;
 }
 
-int64_t strip_job_chunks(const StripJob &J) { return chunk_views(J.L) * J.cpv; }
-
-cudaError_t launch_strip_pre(const StripJob &J, bool adj, cudaStream_t s)
+cudaError_t launch_strip_pre(const void *jobs, int k, const float *img, cudaStream_t s)
 {
-    const dim3 tb(32, 8), tg((J.g.nx + 31) / 32, (J.g.ny + 31) / 32);
-    if (!adj) {
-        transpose_kernel<<<tg, tb, 0, s>>>(J.coef, J.coefT, J.g.nx, J.g.ny);
-        return cudaGetLastError();
-    }
-    cudaError_t e = cudaMemsetAsync(J.out, 0, sizeof(float) * (size_t)J.g.nx * J.g.ny, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(J.outT, 0, sizeof(float) * (size_t)J.g.nx * J.g.ny, s);
-    return e;
+    const StripArgs &A = static_cast<const StripJob *>(jobs)[k].A;
+    if (img) return launch_images(A, img, s);
+    return cudaMemsetAsync(A.dst[0], 0, strip_scratch_bytes(A.g), s);
 }
 
-cudaError_t launch_strip_post(const StripJob &J, bool adj, cudaStream_t s)
+cudaError_t launch_strip_post(const void *jobs, int k, float *out, cudaStream_t s)
 {
-    if (!adj) return cudaSuccess;
-    const dim3 tb(32, 8), tg((J.g.nx + 31) / 32, (J.g.ny + 31) / 32);
-    add_transposed_kernel<<<tg, tb, 0, s>>>(J.outT, J.out, J.g.nx, J.g.ny);
-    return cudaGetLastError();
+    return launch_join(static_cast<const StripJob *>(jobs)[k].A, out, s);
 }
 
-cudaError_t launch_strip_queue(int kind, bool adj, const StripJob *jobs, int njobs, int64_t total,
+cudaError_t launch_strip_queue(int kind, bool adj, const void *jobs_dev, int job0, int njobs, int64_t total,
                                unsigned long long *counter, long long *defer, cudaStream_t s)
 {
     if (njobs <= 0 || total <= 0) return cudaSuccess;
+    const StripJob *jobs = static_cast<const StripJob *>(jobs_dev) + job0;
     if (kind < 0 || kind > kKindBox || (adj && !defer)) return cudaErrorInvalidValue;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, 3 * sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    int64_t grid = 2 * (int64_t)sms;   // two CTAs per SM, resident at once
+    int64_t grid = kCtas * (int64_t)sms;   // resident at once
     if (grid > total) grid = total;
     switch (kind) {
     case 0: return launch_queue_t<0>(adj, jobs, njobs, total, counter, defer, grid, sms, s);
@@ -1258,43 +1274,43 @@ bool strip_supported(const GridDev &g, const LinesDev &L)
     return (L.kind == SP_LINES_PARALLEL || L.kind == SP_LINES_FAN || strip_needs_order(L)) && g.kdeg >= 0;
 }
 
-size_t strip_scratch_bytes(const GridDev &g) { return sizeof(float) * (size_t)g.nx * g.ny + 256; }
+size_t strip_scratch_bytes(const GridDev &g) { return image_bytes(g.ny, g.nx) + image_bytes(g.nx, g.ny); }
 
-cudaError_t launch_fwd_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *coef, void *scratch, float *sino, cudaStream_t s, const longlong2 *rec)
+cudaError_t launch_fwd_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                             const float *tabs, const float *coef, void *scratch, float *sino, cudaStream_t s,
+                             const longlong2 *rec)
 {
-    float *coefT = static_cast<float *>(scratch);
-    switch (strip_kind(g)) {
-    case 0: return launch_strip_t<0, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
-    case 1: return launch_strip_t<1, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
-    case 2: return launch_strip_t<2, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
-    case 3: return launch_strip_t<3, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
-    default: return launch_strip_t<kKindBox, false>(g, L, hdr, tabs, coef, coefT, sino, nullptr, s, rec);
-    }
+    const StripArgs A = make_args(g, L, hdr, center, tabs, coef, scratch, sino, rec);
+    cudaError_t e = launch_images(A, coef, s);
+    return e == cudaSuccess ? launch_strip(A, false, nullptr, s) : e;
 }
 
-cudaError_t launch_row_records(const LineHdr *hdr, int64_t m, longlong2 *rec, cudaStream_t s)
+cudaError_t launch_adj_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                             const float *tabs, const float *sino, void *scratch, float *coef_out, cudaStream_t s,
+                             const longlong2 *rec)
 {
-    if (m <= 0) return cudaSuccess;
-    row_record_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(hdr, m, rec);
+    const StripArgs A = make_args(g, L, hdr, center, tabs, nullptr, scratch, const_cast<float *>(sino), rec);
+    // the images and, right behind them, the deferred list's count and counter
+    unsigned *defer = reinterpret_cast<unsigned *>(static_cast<char *>(scratch) + strip_scratch_bytes(g));
+    cudaError_t e = cudaMemsetAsync(scratch, 0, strip_scratch_bytes(g) + 2 * sizeof(unsigned), s);
+    if (e == cudaSuccess) e = launch_strip(A, true, defer, s);
+    return e == cudaSuccess ? launch_join(A, coef_out, s) : e;
+}
+
+cudaError_t launch_row_records(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *center,
+                               longlong2 *rec, cudaStream_t s)
+{
+    if (L.m <= 0) return cudaSuccess;
+    const unsigned nb = (unsigned)((L.m + 255) / 256);
+    const int per = L.kind == SP_LINES_PARALLEL ? L.n_det : 1;
+    switch (strip_kind(g)) {
+    case 1: row_record_kernel<1><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
+    case 2: row_record_kernel<2><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
+    case 3: row_record_kernel<3><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
+    case kKindBox: row_record_kernel<kKindBox><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
-}
-
-int64_t strip_chunk_count(const LinesDev &L) { return chunk_views(L) * ((chunk_bins(L) + kChunk - 1) / kChunk); }
-
-cudaError_t launch_adj_strip(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
-                             const float *sino, void *scratch, float *coef_out, cudaStream_t s, const longlong2 *rec,
-                             unsigned *defer)
-{
-    float *outT = static_cast<float *>(scratch);
-    float *p = const_cast<float *>(sino);
-    switch (strip_kind(g)) {
-    case 0: return launch_strip_t<0, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
-    case 1: return launch_strip_t<1, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
-    case 2: return launch_strip_t<2, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
-    case 3: return launch_strip_t<3, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
-    default: return launch_strip_t<kKindBox, true>(g, L, hdr, tabs, nullptr, outT, p, coef_out, s, rec, defer);
-    }
 }
 
 }  // namespace spx

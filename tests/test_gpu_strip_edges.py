@@ -82,3 +82,64 @@ def test_a_line_does_not_depend_on_its_chunk(degree):
     for first, count in ((0, 1), (7, 33), (40, 60), (64, 3)):
         part = sp.spline_project_fwd(grid, coef, sp.Lines.parallel(view, count, -49.5 + first, 1.0))
         assert torch.equal(part, whole[first:first + count])
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+def test_a_nonfinite_coefficient_reaches_its_lines_only(degree):
+    # the kernels may multiply nodes just beyond a row's support by 0: lines
+    # whose sum is not finite are taken again over their support alone
+    n = 40
+    view = np.array([0.0, 0.3, math.pi / 4, 1.2, 2.2], dtype=np.float32)
+    lines = sp.Lines.parallel(torch.from_numpy(view).to(DEV), 64, -31.7, 1.0)
+    th, yy = oracle.lines_parallel(view.astype(np.float64), 64, float(np.float32(-31.7)), 1.0)
+    og = oracle.Grid(n, n, degree, 1.0)
+    mask = np.zeros((n, n))
+    mask[21, 17] = 1.0
+    touched = oracle.forward(og, mask, th, yy)
+    coef = workloads.ellipse_phantom(n, 8, 4, radius=14.0, axes=(2.0, 8.0))
+    ref = oracle.forward(og, coef.astype(np.float64), th, yy)
+    for bad in (np.nan, np.inf):
+        c = coef.copy()
+        c[21, 17] = bad
+        got = sp.spline_project_fwd(sp.Grid(n, n, degree, 1.0), torch.from_numpy(c).to(DEV), lines).cpu().numpy()
+        assert not np.any(np.isfinite(got[touched > 1e-5]))     # (the footprint vanishes smoothly at its ends)
+        clear = touched == 0.0
+        assert clear.any() and np.all(np.isfinite(got[clear]))
+        assert rel_l2(got[clear], ref[clear]) < TOL
+
+
+def test_plan_builds_footprint_tables_for_the_paths_that_read_them():
+    # the strip kernels read none; a plan that switches to the other kernels
+    # after prepare, prepares again with new angles, or captures a projection,
+    # gets the tables of its lines
+    n = 48
+    view = torch.linspace(0.0, 3.0, 31, device=DEV)
+    grid, lines = sp.Grid(n, n, 3, 1.0), sp.Lines.parallel(view, 70, -34.5, 1.0)
+    coef = torch.from_numpy(workloads.ellipse_phantom(n, 8, 4, radius=16.0, axes=(2.0, 9.0))).to(DEV)
+    p = torch.rand(lines.m, device=DEV, generator=torch.Generator(DEV).manual_seed(1))
+
+    def close(a, b):
+        return float((a - b).norm() / b.norm()) < 2e-6
+
+    plan = sp.Plan(grid, lines)
+    f, b = plan.fwd(coef), plan.adj(p)
+    for adj_path in (2, 3):
+        plan.set_paths(2, adj_path)
+        assert close(plan.fwd(coef), f) and close(plan.adj(p), b)
+    view.add_(0.21)
+    plan.prepare()
+    g = sp.spline_project_fwd(grid, coef, lines)
+    assert close(plan.fwd(coef), g) and not close(g, f)
+    fresh = sp.Plan(grid, lines)
+    fresh.set_paths(2, 2)
+    out = torch.empty(lines.m, device=DEV)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        fresh.fwd(coef, out)
+    direct = fresh.fwd(coef).clone()      # before the graph has run
+    graph.replay()
+    torch.cuda.synchronize()
+    assert close(direct, g) and torch.equal(direct, out)
+    plan.close()
+    fresh.close()
