@@ -59,6 +59,34 @@ sp_status sp_conv3x3_bwd_weight(int32_t B, int32_t H, int32_t W, int32_t cin, in
 sp_status sp_conv3x3_flip_weights(int32_t cin, int32_t cout, const void *w, void *wf,
                                   void *stream);
 
+/*
+ * The whole network x0 = z + f(z): `layers` (2..16) convolutions 1 -> 32,
+ * 32 -> 32, ..., 32 -> 1 with dilations dilation[k] (host array) and ReLU
+ * between them, on z FP32 [B][H][W] (rounded to BF16 as f's input).  w and bias
+ * are host arrays of device pointers to the FP32 master weights
+ * [cout][3][3][cin] (used in BF16) and biases (NULL = 0).
+ *
+ * Forward: out FP32 [B][H][W].  acts BF16: the activations of the layers but the
+ * last, [layers - 1][B][H][W][32] with keep != 0 (for the backward), else two
+ * such slabs of scratch; then z as rounded, [B][H][W].  pack BF16
+ * [sp_convnet_pack_elems]: the weights as the kernels take them, for the backward
+ * too.
+ *
+ * Backward: g FP32 [B][H][W], the gradient of out; acts and pack as the forward
+ * left them (keep != 0).  dparam FP32, overwritten: per layer dW
+ * [cout][3][3][cin], then dbias [cout].  dx (may be NULL) FP32 [B][H][W]: the
+ * gradient through f (rounded to BF16, as z was; the one through z is g).  work
+ * BF16: two slabs of scratch.  Gradients between layers are BF16, those of the
+ * last layer's output FP32; sums are FP32, over blocks by atomic adds (their
+ * order may vary between runs).
+ */
+int64_t sp_convnet_pack_elems(int32_t layers);
+sp_status sp_convnet_fwd(int32_t B, int32_t H, int32_t W, int32_t layers, const int32_t *dilation,
+                         const float *const *w, const float *const *bias, const float *z, int32_t keep, void *acts,
+                         void *pack, float *out, void *stream);
+sp_status sp_convnet_bwd(int32_t B, int32_t H, int32_t W, int32_t layers, const int32_t *dilation, const void *acts,
+                         const void *pack, const float *g, void *work, float *dparam, float *dx, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

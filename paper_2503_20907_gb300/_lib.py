@@ -51,7 +51,8 @@ EXPORTED = ("sp_lines_count", "spline_project_fwd", "spline_project_adj", "splin
             "spline_plan_autotune", "spline_batch_create", "spline_batch_prepare", "spline_batch_fwd",
             "spline_batch_adj", "spline_batch_autotune", "spline_batch_count", "spline_batch_queued",
             "spline_batch_destroy",
-            "sp_conv3x3_fwd", "sp_conv3x3_bwd_data", "sp_conv3x3_bwd_weight", "sp_conv3x3_flip_weights")
+            "sp_conv3x3_fwd", "sp_conv3x3_bwd_data", "sp_conv3x3_bwd_weight", "sp_conv3x3_flip_weights",
+            "sp_convnet_pack_elems", "sp_convnet_fwd", "sp_convnet_bwd")
 
 
 def load(build_if_stale: bool = True) -> ctypes.CDLL:
@@ -124,6 +125,12 @@ def load(build_if_stale: bool = True) -> ctypes.CDLL:
     lib.sp_conv3x3_bwd_weight.argtypes = [i32, i32, i32, i32, i32, i32, P, P, P, P, P]
     lib.sp_conv3x3_flip_weights.restype = st
     lib.sp_conv3x3_flip_weights.argtypes = [i32, i32, P, P, P]
+    lib.sp_convnet_pack_elems.restype = ctypes.c_int64
+    lib.sp_convnet_pack_elems.argtypes = [i32]
+    lib.sp_convnet_fwd.restype = st
+    lib.sp_convnet_fwd.argtypes = [i32, i32, i32, i32, P, P, P, P, i32, P, P, P, P]
+    lib.sp_convnet_bwd.restype = st
+    lib.sp_convnet_bwd.argtypes = [i32, i32, i32, i32, P, P, P, P, P, P, P, P]
     lib.spline_plan_destroy.restype = st
     lib.spline_plan_destroy.argtypes = [P]
     lib.sp_release_workspace.restype = st

@@ -16,6 +16,7 @@ library's projector.
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import math
 import time
@@ -80,6 +81,47 @@ def conv3x3(x, w, b, relu: bool, dil: int = 1):
     return _Conv3x3.apply(x, w, b, int(w.shape[3]), int(w.shape[0]), bool(relu), int(dil))
 
 
+class _Net(torch.autograd.Function):
+    """x_0 = z + f(z) in one call per direction (sp_convnet_fwd, sp_convnet_bwd)."""
+
+    @staticmethod
+    def forward(ctx, z, dils, keep, *params):
+        n = len(dils)
+        z = z.detach().contiguous()
+        B, H, W = z.shape
+        # activations, then z in BF16
+        acts = torch.empty((((n - 1) if keep else 2) * CH + 1) * B * H * W, dtype=torch.bfloat16, device=z.device)
+        pack = torch.empty(load().sp_convnet_pack_elems(n), dtype=torch.bfloat16, device=z.device)
+        out = torch.empty_like(z)
+        pointers = [p.data_ptr() for p in params]
+        _check(load().sp_convnet_fwd(B, H, W, n, (ctypes.c_int32 * n)(*dils), (ctypes.c_void_p * n)(*pointers[:n]),
+                                     (ctypes.c_void_p * n)(*pointers[n:]), z.data_ptr(), int(keep), acts.data_ptr(),
+                                     pack.data_ptr(), out.data_ptr(), _stream(None)))
+        if keep:
+            ctx.save_for_backward(acts, pack)
+            ctx.meta = z.shape, dils, [p.shape for p in params]
+        return out
+
+    @staticmethod
+    def backward(ctx, gy):
+        acts, pack = ctx.saved_tensors
+        (B, H, W), dils, shapes = ctx.meta
+        n = len(dils)
+        g = gy.contiguous()
+        work = torch.empty(2 * CH * B * H * W, dtype=torch.bfloat16, device=g.device)
+        sizes = [math.prod(s) for s in shapes]
+        dparam = torch.empty(sum(sizes), dtype=torch.float32, device=g.device)
+        dx = torch.empty((B, H, W), dtype=torch.float32, device=g.device) if ctx.needs_input_grad[0] else None
+        _check(load().sp_convnet_bwd(B, H, W, n, (ctypes.c_int32 * n)(*dils), acts.data_ptr(), pack.data_ptr(),
+                                     g.data_ptr(), work.data_ptr(), dparam.data_ptr(),
+                                     None if dx is None else dx.data_ptr(), _stream(None)))
+        order = [j for k in range(n) for j in (k, n + k)]   # dparam: dW, then dbias, layer by layer
+        grads = [None] * (2 * n)
+        for j, d in zip(order, dparam.split([sizes[j] for j in order])):
+            grads[j] = d.view(shapes[j])
+        return (None if dx is None else gy + dx, None, None, *grads)
+
+
 class WarmStartNet(torch.nn.Module):
     """x_0 = z + f(z), z [B,H,W] FP32."""
 
@@ -97,6 +139,14 @@ class WarmStartNet(torch.nn.Module):
             self.b.append(torch.nn.Parameter(torch.zeros(cout)))
 
     def forward(self, z):
+        params = [*self.w, *self.b]
+        if (z.is_cuda and z.dtype == torch.float32 and z.dim() == 3
+                and all(p.dtype == torch.float32 and p.device == z.device and p.is_contiguous() for p in params)
+                and all(w.shape == (cout, 3, 3, cin) and b.shape == (cout,)
+                        for w, b, (cin, cout, _, _) in zip(params, params[len(LAYERS):], LAYERS))):
+            keep = torch.is_grad_enabled() and (z.requires_grad or any(p.requires_grad for p in params))
+            return _Net.apply(z, tuple(layer[3] for layer in LAYERS), keep, *params)
+        # other dtypes and devices: layer by layer
         x = z.to(torch.bfloat16).unsqueeze(-1).contiguous()
         for k, (_, _, relu, dil) in enumerate(LAYERS):
             x = conv3x3(x, self.w[k], self.b[k], relu, dil)
