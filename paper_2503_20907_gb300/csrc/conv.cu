@@ -18,6 +18,7 @@
 
 #include <cstdint>
 #include <string>
+#include <type_traits>
 
 #include "common.cuh"
 #include "../../include/warmstart_conv.h"
@@ -34,11 +35,12 @@ constexpr int kMaxDil = 16;         // largest dilation of the taps
 // Four lanes hold a pixel's 32 channels, eight each (an octet: 16 bytes of
 // BF16); a warp takes eight consecutive pixels of an image row at a time.  What
 // an octet needs of the nine taps (weights, or partial weight gradients) stays
-// in 72 registers.  All three kernels are bound by memory: 64 bytes per pixel
-// once, against 288 FMAs per pixel (8 x 256 x 256 pixels: 5 us of HBM, 4 us of
-// FMA issue).  One thread per pixel or per output instead (2-byte loads, 64
-// bytes apart, or a block per 16 rows) took 54 to 267 us forward and 0.72 and
-// 1.81 ms for the two weight gradients at that size.
+// in 72 registers (16 warps per SM).  The floor is 5 us of HBM (64 bytes per
+// pixel) and 4 us of FMAs (288 per pixel) at 8 x 256 x 256 pixels; measured are
+// 28 us out, 52 us in and 28 and 32 us for the weight gradients, with the issue
+// slots 33 to 50 % busy and the rest load latency.  One thread per pixel or per
+// output instead (2-byte loads, 64 bytes apart, or a block per 16 rows) took 54
+// to 267 us forward and 0.72 and 1.81 ms for the two weight gradients.
 constexpr int kEdgeThreads = 256;
 
 struct EdgeArgs {
@@ -104,7 +106,9 @@ __device__ __forceinline__ float masked(float v, bool on)
 }
 
 // This warp's pixel groups: group k is row k / gw (over B H), columns
-// 8 (k % gw) .. + 7.  Calls f(row, h, w, in) with the lane's pixel.
+// 8 (k % gw) .. + 7.  Calls f(inner, row, h, w, in) with the lane's pixel; inner
+// (a type) says that all of the group's pixels and their taps are in the image:
+// without a test at each tap their loads are in flight together.
 template <typename F>
 __device__ __forceinline__ void for_pixels(const EdgeArgs &a, F f)
 {
@@ -116,8 +120,11 @@ __device__ __forceinline__ void for_pixels(const EdgeArgs &a, F f)
     int64_t row = first / gw;
     unsigned gi = first - (unsigned)row * gw, h = (unsigned)row % (unsigned)a.H;
     while (row < rows) {
-        const int w = (int)gi * 8 + (int)((threadIdx.x & 31) >> 2);
-        f(row, (int)h, w, w < a.W);
+        const int w0 = (int)gi * 8, w = w0 + (int)((threadIdx.x & 31) >> 2);
+        if ((int)h >= a.dil && (int)h + a.dil < a.H && w0 >= a.dil && w0 + 7 + a.dil < a.W)
+            f(std::true_type{}, row, (int)h, w, true);
+        else
+            f(std::false_type{}, row, (int)h, w, w < a.W);
         row += srow; gi += sg; h += sh;
         if (gi >= gw) { gi -= gw; ++row; ++h; }
         if (h >= (unsigned)a.H) h -= (unsigned)a.H;
@@ -126,11 +133,12 @@ __device__ __forceinline__ void for_pixels(const EdgeArgs &a, F f)
 
 // The offset of a tap's pixel from (row, w) in pixels, and whether it is in the
 // image.
-__device__ __forceinline__ bool tap_at(const EdgeArgs &a, int tap, int h, int w, int64_t &off)
+template <typename INNER>
+__device__ __forceinline__ bool tap_at(const EdgeArgs &a, INNER, int tap, int h, int w, int64_t &off)
 {
     const int dy = a.sign * (tap / 3 - 1) * a.dil, dx = a.sign * (tap % 3 - 1) * a.dil;
     off = (int64_t)dy * a.W + dx;
-    return (unsigned)(h + dy) < (unsigned)a.H && (unsigned)(w + dx) < (unsigned)a.W;
+    return INNER::value || ((unsigned)(h + dy) < (unsigned)a.H && (unsigned)(w + dx) < (unsigned)a.W);
 }
 
 // One channel in, 32 out: y[p, c] = bias[c] + sum_tap s[p + off(tap)] w[c][tap]
@@ -152,7 +160,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 #pragma unroll
         for (int t = 0; t < 9; ++t) wr[t][k] = __bfloat162float(GRAD ? wt[t * kC + c0 + k] : wt[(c0 + k) * 9 + t]);
     }
-    for_pixels(a, [&](int64_t row, int h, int w, bool in) {
+    for_pixels(a, [&](auto inner, int64_t row, int h, int w, bool in) {
         if (!in) return;
         const int64_t p = row * a.W + w;
         float acc[8];
@@ -161,7 +169,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             int64_t off;
-            if (!tap_at(a, t, h, w, off)) continue;
+            if (!tap_at(a, inner, t, h, w, off)) continue;
             float v = as_float(s[p + off]);
             if (ROUND) v = round_bf16(v);
             if (ROUND && t == 4 && c0 == 0) sb[p] = __float2bfloat16(v);
@@ -210,13 +218,13 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, con
 #pragma unroll
         for (int t = 0; t < 9; ++t) wr[t][k] = __bfloat162float(GRAD ? wt[(c0 + k) * 9 + t] : wt[t * kC + c0 + k]);
     const float b0 = bias ? bias[0] : 0.f;
-    for_pixels(a, [&](int64_t row, int h, int w, bool in) {
+    for_pixels(a, [&](auto inner, int64_t row, int h, int w, bool in) {
         const int64_t p = row * a.W + w;
         float acc = 0.f;
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             int64_t off;
-            if (!in || !tap_at(a, t, h, w, off)) continue;
+            if (!in || !tap_at(a, inner, t, h, w, off)) continue;
             float f[8];
             load8(v + (p + off) * kC + c0, vec, f);
 #pragma unroll
@@ -254,7 +262,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, co
 #pragma unroll
         for (int t = 0; t < 9; ++t) acc[t][k] = 0.f;
     }
-    for_pixels(a, [&](int64_t row, int h, int w, bool in) {
+    for_pixels(a, [&](auto inner, int64_t row, int h, int w, bool in) {
         if (!in) return;
         const int64_t p = row * a.W + w;
         float f[8];
@@ -262,7 +270,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, co
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             int64_t off;
-            if (!tap_at(a, t, h, w, off)) continue;
+            if (!tap_at(a, inner, t, h, w, off)) continue;
             const float x = as_float(s[p + off]);
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc[t][k] = __fmaf_rn(x, f[k], acc[t][k]);
@@ -358,6 +366,10 @@ __host__ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t saddr, uint
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
 
+// The same operand `bytes` further on (a multiple of 16; shared-memory addresses
+// stay below 2^18, so the sum does not leave the address field).
+__device__ __forceinline__ uint64_t umma_step(uint64_t desc, uint32_t bytes) { return desc + (bytes >> 4); }
+
 // Instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
 // (bits 7-9 and 10-12 = 1), K-major (bits 15, 16 = 0) or MN-major (1), N >> 3 at
 // bit 17, M >> 4 at bit 24.
@@ -412,8 +424,8 @@ __device__ __forceinline__ void tmem_load32(uint32_t taddr, uint32_t (&acc)[kC])
 }
 
 // Warp 0 allocates `cols` columns of tensor memory (a power of two >= 32) and
-// thread 0 the completion barrier; call before a __syncthreads.
-__device__ __forceinline__ void tc05_begin(uint32_t *tslot, void *mbar, uint32_t cols)
+// thread 0 the two completion barriers; call before a __syncthreads.
+__device__ __forceinline__ void tc05_begin(uint32_t *tslot, unsigned long long *mbar, uint32_t cols)
 {
     if (threadIdx.x < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_u32(tslot)), "r"(cols)
@@ -422,6 +434,7 @@ __device__ __forceinline__ void tc05_begin(uint32_t *tslot, void *mbar, uint32_t
     }
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(mbar)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_u32(mbar + 1)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
 }
@@ -441,14 +454,92 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void *src, bool in)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
 }
 
-// Staged operands visible to the tensor cores, then all threads together.
-__device__ __forceinline__ void staged_sync()
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+// Waits until at most PENDING of this thread's copy groups are under way, makes
+// what was staged visible to the tensor cores, and joins the block; true if
+// `good` holds for all threads.
+template <int PENDING>
+__device__ __forceinline__ bool staged_sync(bool good)
 {
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    good = __syncthreads_and(good) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return good;
+}
+
+// How the image rows of a 32 -> 32 layer are shared out.  Rows of one residue
+// modulo the dilation form a chain: each row of the chain meets its neighbours
+// in it, so a CTA that walks along a chain stages every input row once, in a
+// ring, instead of three times.  A unit is 128 columns of `rows` successive
+// rows of a chain; one CTA per unit.
+struct ChainArgs {
+    int B, H, W, dil;
+    int strips, chains, segs, rows;   // per image: 128-column strips, chains; per chain: segments of `rows`
+};
+
+struct Unit {
+    int64_t b;
+    int h0, n, w0;   // image, first row, rows, first column
+};
+
+__device__ __forceinline__ Unit unit_of(const ChainArgs &a, unsigned u)
+{
+    Unit t;
+    const unsigned seg = u % (unsigned)a.segs;
+    u /= (unsigned)a.segs;
+    const unsigned c = u % (unsigned)a.chains;
+    u /= (unsigned)a.chains;
+    t.w0 = (int)(u % (unsigned)a.strips) * 128;
+    t.b = u / (unsigned)a.strips;
+    const int64_t h0 = c + (int64_t)seg * a.rows * a.dil;
+    t.n = h0 < a.H ? min(a.rows, (int)((a.H - h0 + a.dil - 1) / a.dil)) : 0;
+    t.h0 = (int)h0;
+    return t;
+}
+
+// Four warps stage, and store the results; a fifth issues the MMAs meanwhile
+// (issued by one of the four, they held up the block's next copies: 32 to 35 us
+// and 57 us instead of 26 to 28 us and 49 us forward and weight gradient, 8 x 256 x
+// 256 pixels).
+constexpr int kThreads5 = 160;
+constexpr int kTile5 = 128;                   // pixels of a row per tile: M forward, K of the weight gradient
+constexpr int kHalo5 = kTile5 + 2 * kMaxDil;  // with the taps on both sides
+// Staged rows are [channel group of 8][pixel][8]; a group is 32 bytes longer
+// than its pixels, so that the four groups of two pixels, which eight lanes
+// write together, lie in different banks.
+constexpr int kHaloGroup5 = kHalo5 * 16 + 32;   // 2,592
+constexpr int kHaloRow5 = 4 * kHaloGroup5;
+constexpr int kTileGroup5 = kTile5 * 16 + 32;   // 2,080
+constexpr int kTileRow5 = 4 * kTileGroup5;
+
+// Stages `pixels` pixels of image row (b, h) from column w on (zeros outside the
+// image) at dst and, unless NULL, again at copy: 16 bytes per copy, FP32 input
+// rounded to BF16 on the way.
+template <typename IN>
+__device__ __forceinline__ void stage_row(const ChainArgs &a, const IN *__restrict__ x, int64_t b, int h, int w,
+                                          int pixels, int group, unsigned char *dst, unsigned char *copy)
+{
+    const bool rin = (unsigned)h < (unsigned)a.H;
+    const IN *src = x + ((b * a.H + (rin ? h : 0)) * a.W) * kC;
+    const int cg = threadIdx.x & 3;
+    for (int p = threadIdx.x >> 2; p < pixels; p += 32) {
+        const bool in = rin && (unsigned)(w + p) < (unsigned)a.W;
+        const IN *s = src + (in ? (int64_t)(w + p) * kC + cg * 8 : 0);
+        const int at = cg * group + p * 16;
+        if constexpr (sizeof(IN) == 2) {
+            cp16(s_u32(dst + at), s, in);
+            if (copy) cp16(s_u32(copy + at), s, in);
+        } else {
+            float f[8] = {};
+            if (in) load8(s, true, f);
+            const uint4 v = pack8(f);
+            *reinterpret_cast<uint4 *>(dst + at) = v;
+            if (copy) *reinterpret_cast<uint4 *>(copy + at) = v;
+        }
+    }
 }
 
 // The 32 -> 32 convolution: a tile is 128 output pixels of one image row as
@@ -459,85 +550,54 @@ __device__ __forceinline__ void staged_sync()
 // Shared-memory operands use the canonical no-swizzle K-major layout: core
 // matrices of 8 rows x 16 bytes stored contiguously (128 bytes), LBO the
 // byte distance between core matrices along K, SBO along M (or N).
-//   input  xs[cg][row][pixel][8]: channel group cg (8 channels) of the three
-//          rows h - d, h, h + d and pixels w0 - d .. w0 + 127 + d.  A tap's
-//          A operand is the same array read from another start address:
-//          LBO = one channel group (kXRows5 * kXPix5 * 16 B), SBO = 128 B
-//          (8 pixels of 16 B).
+//   input  a ring of staged rows, pixels w0 - d .. w0 + 127 + d.  A tap's A
+//          operand is its row read from another pixel on: LBO = one channel
+//          group, SBO = 128 B (8 pixels of 16 B).
 //   weights wb[kc][n][8]: K = tap 32 + input channel in groups kc of 8,
 //          n the output channel; LBO = 32 * 16 B, SBO = 128 B.
 //
-// A CTA of 128 threads keeps the weights and walks over tiles with two input
-// buffers: the copies of the next tile run while the tensor cores work on the
-// present one and its epilogue stores it.  Bound by the memory system (64
-// bytes in and out per pixel from HBM, three rows per tile from L2); a CTA per
-// tile that staged the weights anew, and had nothing to do while its copies
-// were under way, took 62 us forward and 97 us for the gradient at 8 x 256 x
-// 256 pixels.
-constexpr int kTile5 = 128;                  // output pixels of one tile (M)
-constexpr int kXPix5 = kTile5 + 2 * kMaxDil;  // staged pixels per row
-constexpr int kXRows5 = 3;
-constexpr int kXBytes5 = 4 * kXRows5 * kXPix5 * 16;   // 30,720
-constexpr int kWBytes5 = 36 * kC * 16;                // 18,432
-constexpr int kSmem5 = 2 * kXBytes5 + kWBytes5 + kC * 4 + 16;   // + bias, mbarrier and TMEM address
-constexpr uint32_t kTmemCols5 = 32;                   // FP32 accumulators: N = 32 columns
+// Three CTAs of 128 threads per SM, each with its weights, a ring of five rows
+// and two accumulators: while the tensor cores work on a tile, the block stores
+// the one before and copies the row two tiles ahead.  Bound by the latency of a
+// tile's chain (copies, MMAs, read-back, stores; 64 bytes in and out per pixel
+// at 2.6 TB/s): 26 us forward and 28 us for the gradient at 8 x 256 x 256
+// pixels.  A CTA per tile, staging the weights and all three rows anew, took 62
+// and 97 us; several tiles per CTA but three rows per tile 50 and 60 us.
+constexpr int kRing5 = 5;
+constexpr int kWBytes5 = 36 * kC * 16;   // 18,432
+constexpr int kSmem5 = kRing5 * kHaloRow5 + kWBytes5 + kC * 4 + 24;   // + bias, barriers and TMEM address
+constexpr int kCtas5 = 3;                // per SM
+constexpr uint32_t kTmemCols5 = 64;      // two accumulators of 32 columns
 
 enum WeightForm { kWPacked = 0, kWPlain = 1, kWFlip = 2 };
 
 struct ConvArgs {
-    int B, H, W, dil, relu;
-    int form;              // WeightForm of w
+    int relu, form;        // form: WeightForm of w
     const bf16 *w;
     const float *bias;     // may be NULL
-    const bf16 *gate;      // may be NULL: results are zeroed where gate <= 0
+    const bf16 *gate;      // may be NULL: results are masked where gate <= 0
 };
 
-template <typename IN>
-__device__ __forceinline__ void stage_tile(const ConvArgs &a, const IN *__restrict__ x, unsigned char *xs, int64_t tile)
-{
-    const int tiles_w = (a.W + kTile5 - 1) / kTile5;
-    const int64_t row = tile / tiles_w;
-    const int w0 = (int)(tile - row * tiles_w) * kTile5, h = (int)(row % a.H);
-    const int n4 = (kTile5 + 2 * a.dil) * 4;
-#pragma unroll
-    for (int r = 0; r < kXRows5; ++r) {
-        const int hh = h + (r - 1) * a.dil;
-        const bool rin = (unsigned)hh < (unsigned)a.H;
-        const IN *src = x + ((row + (rin ? (int64_t)(r - 1) * a.dil : 0)) * a.W) * kC;
-        for (int i = threadIdx.x; i < n4; i += 128) {
-            const int p = i >> 2, cg = i & 3, ww = w0 + p - a.dil;
-            const bool in = rin && (unsigned)ww < (unsigned)a.W;
-            const IN *s = src + (in ? (int64_t)ww * kC + cg * 8 : 0);
-            unsigned char *dst = xs + ((cg * kXRows5 + r) * kXPix5 + p) * 16;
-            if constexpr (sizeof(IN) == 2) {
-                cp16(s_u32(dst), s, in);
-            } else {
-                float f[8] = {};
-                if (in) load8(s, true, f);
-                *reinterpret_cast<uint4 *>(dst) = pack8(f);
-            }
-        }
-    }
-}
-
 // IN, OUT: bf16 or float (float input is rounded to BF16 while staged).  Every
-// wait is bounded; a CTA whose MMAs did not complete writes NaN, stops, and
-// still frees its tensor memory.
+// wait is bounded; when MMAs do not complete, the rest of the unit is NaN and
+// the block still frees its tensor memory.
 template <typename IN, typename OUT>
-__global__ void __launch_bounds__(128) conv32_tc05_kernel(ConvArgs a, const IN *__restrict__ x, OUT *__restrict__ y,
-                                                          int64_t tiles)
+__global__ void __launch_bounds__(kThreads5) conv32_tc05_kernel(ChainArgs ch, ConvArgs a, const IN *__restrict__ x,
+                                                          OUT *__restrict__ y)
 {
     extern __shared__ __align__(128) unsigned char sm5[];
-    unsigned char *wsb = sm5 + 2 * kXBytes5;
+    unsigned char *wsb = sm5 + kRing5 * kHaloRow5;
     float *bias_s = reinterpret_cast<float *>(wsb + kWBytes5);
     unsigned long long *mbar = reinterpret_cast<unsigned long long *>(bias_s + kC);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 1);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 2);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const Unit u = unit_of(ch, blockIdx.x);
+    if (u.n < 1) return;
 
     tc05_begin(tslot, mbar, kTmemCols5);
     // weights: wb[kc][n][8] = W[n][kc 8 .. kc 8 + 7] (W is [n][tap][i], K = tap 32 + i);
     // flipped for the input gradient: n = i, K = tap' 32 + o, W[o][8 - tap'][i]
-    for (int i = threadIdx.x; i < 36 * kC; i += 128) {
+    for (int i = threadIdx.x; i < 36 * kC; i += kThreads5) {
         if (a.form == kWPacked) {
             cp16(s_u32(wsb + i * 16), a.w + (size_t)i * 8, true);
             continue;
@@ -551,51 +611,67 @@ __global__ void __launch_bounds__(128) conv32_tc05_kernel(ConvArgs a, const IN *
         *reinterpret_cast<uint4 *>(wsb + i * 16) = *reinterpret_cast<const uint4 *>(e);
     }
     if (threadIdx.x < kC) bias_s[threadIdx.x] = a.bias ? a.bias[threadIdx.x] : 0.f;
-    int64_t tile = blockIdx.x;
-    if (tile < tiles) stage_tile(a, x, sm5, tile);
-    const int tiles_w = (a.W + kTile5 - 1) / kTile5;
-    uint32_t k = 0;
+    // staged row j is image row h0 + (j - 1) d; tile k takes rows k, k + 1, k + 2.  One copy
+    // group per row, empty past the last.
+    auto stage = [&](int j) {
+        if (warp < 4 && j < u.n + 2)
+            stage_row(ch, x, u.b, u.h0 + (j - 1) * ch.dil, u.w0 - ch.dil, kTile5 + 2 * ch.dil, kHaloGroup5,
+                      sm5 + (j % kRing5) * kHaloRow5, nullptr);
+        cp_commit();
+    };
+    for (int j = 0; j < kRing5; ++j) stage(j);
+    bool good = true;
     uint32_t taddr = 0;
-    bool done = true;
-    for (; tile < tiles && done; tile += gridDim.x, ++k) {
-        unsigned char *xs = sm5 + (k & 1) * kXBytes5;
-        staged_sync();
-        taddr = *tslot;
-        if (threadIdx.x == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(kTile5, kC);
-            const uint32_t xbase = s_u32(xs), wbase = s_u32(wsb);
-            constexpr uint32_t kGroup = kXRows5 * kXPix5 * 16;   // A: LBO (next 8 channels)
-#pragma unroll 1
-            for (int s = 0; s < 18; ++s) {
-                const int tap = s >> 1, half = s & 1;
-                const int ky = tap / 3, kx = tap - 3 * ky;
-                const uint32_t a_addr = xbase + (uint32_t)(2 * half) * kGroup + (uint32_t)(ky * kXPix5 * 16) +
-                                        (uint32_t)(kx * a.dil) * 16u;
-                umma_bf16(taddr, umma_smem_desc(a_addr, kGroup, 128),
-                          umma_smem_desc(wbase + (uint32_t)s * 2u * kC * 16u, kC * 16, 128), idesc, (uint32_t)s);
+    for (int k = 0; k <= u.n; ++k) {
+        if (k < u.n) {
+            good = staged_sync<kRing5 - 4>(good);   // rows up to k + 2 are there
+            taddr = *tslot;
+            if (good && threadIdx.x == 128) {
+                constexpr uint32_t idesc = umma_idesc_bf16(kTile5, kC);
+                const uint32_t d = taddr + (uint32_t)(k & 1) * kC;
+                const uint64_t wdesc = umma_smem_desc(s_u32(wsb), kC * 16, 128);
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+                    const uint64_t row = umma_smem_desc(s_u32(sm5) + (uint32_t)((k + ky) % kRing5) * kHaloRow5, kHaloGroup5, 128);
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+                        for (int half = 0; half < 2; ++half) {
+                            const uint32_t s = (uint32_t)((ky * 3 + kx) * 2 + half);
+                            umma_bf16(d, umma_step(row, 2u * half * kHaloGroup5 + (uint32_t)(kx * ch.dil) * 16u),
+                                      umma_step(wdesc, s * 2u * kC * 16u), idesc, s);
+                        }
+                }
+                umma_commit(mbar + (k & 1));
             }
-            umma_commit(mbar);
         }
-        // the next tile into the other buffer (its MMAs were waited for)
-        if (tile + gridDim.x < tiles) stage_tile(a, x, sm5 + ((k + 1) & 1) * kXBytes5, tile + gridDim.x);
-        done = mbar_wait(mbar, k & 1);
+        if (k == 0) continue;
+        const int t = k - 1;   // the tile whose MMAs end next; its first row then makes room
+        const int w = u.w0 + warp * 32 + lane;   // this thread's pixel (the fifth warp has none)
+        const bool mine = warp < 4 && w < ch.W;
+        const int64_t off = ((u.b * ch.H + u.h0 + t * ch.dil) * ch.W + w) * kC;
+        uint4 gate[4] = {};
+        if (a.gate && mine)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) gate[j] = reinterpret_cast<const uint4 *>(a.gate + off)[j];
+        if (good) good = mbar_wait(mbar + (t & 1), (uint32_t)(t >> 1) & 1u);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        stage(t + kRing5);
+        if (warp == 4) continue;
         // accumulators of this warp's 32 pixels: 32 columns (output channels)
         uint32_t acc[kC];
-        tmem_load32(taddr + ((uint32_t)(warp * 32) << 16), acc);
-        // epilogue: pixel w0 + 32 warp + lane, 32 channels
-        const int64_t row = tile / tiles_w;
-        const int ww = (int)(tile - row * tiles_w) * kTile5 + warp * 32 + lane;
-        if (ww < a.W) {
-            const int64_t off = (row * a.W + ww) * kC;
+        __syncwarp();
+        tmem_load32(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t & 1) * kC, acc);
+        if (mine) {
             const float bad = __int_as_float(0x7fc00000);
 #pragma unroll
             for (int o = 0; o < kC; o += 8) {
-                float f[8], gt[8];
-                if (a.gate) load8(a.gate + off + o, true, gt);
+                float f[8], gt[8], bv[8];
+                if (a.gate) unpack8(gate[o / 8], gt);
+                load8(bias_s + o, true, bv);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    float v = done ? __uint_as_float(acc[o + j]) + bias_s[o + j] : bad;
+                    float v = good ? __uint_as_float(acc[o + j]) + bv[j] : bad;
                     if (a.relu) v = fmaxf(v, 0.f);
                     if (a.gate) v = masked<OUT>(v, gt[j] > 0.f);
                     f[j] = v;
@@ -608,146 +684,130 @@ __global__ void __launch_bounds__(128) conv32_tc05_kernel(ConvArgs a, const IN *
                 }
             }
         }
-        done = __syncthreads_and(done) != 0;   // block-uniform: stop at the first failure
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    tc05_end(*tslot, kTmemCols5);
+    tc05_end(taddr, kTmemCols5);
 }
 
 // The 32 -> 32 weight gradient on tcgen05:
 //   dW[o, (ky, kx), i] = sum_p g[p, o] x[p + off, i],  dbias[o] = sum_p g[p, o]
-// as, per ky, D[(kx, o)][i] = sum over pixels of A[(kx, o)][pixel] B[i][pixel]:
-// M = 3 shifts kx x 32 output channels (rows 96..127 zero), N = the 32 input
-// channels, K = the 128 pixels of a segment of one image row, 16 per MMA.  The
-// shifts are on g: for the x at column w of row h + (ky - 1) d, g at column
-// w - (kx - 1) d of row h.  Both operands are MN-major: a pixel's channels are
-// contiguous, so the staged data are plain 16-byte copies of what is in memory,
-// [channel group][pixel][8], and nothing is transposed (core matrices of 8
-// pixels x 8 channels, 128 bytes; LBO the distance of 8 pixels, SBO the one of
-// 8 channels).  At the end warp kx reads the accumulators of its shift for each
-// ky, the block lays them out as dW in shared memory and adds them to dw, and
-// its FP32 sums of g to dbias; a block whose MMAs did not complete adds NaN.
+// as, per kx, D[(ky, i)][o] = sum over pixels of A[(ky, i)][pixel] B[o][pixel]:
+// M = 3 rows of x x 32 input channels (a fourth row of the ring rides along
+// unused), N = the 32 output channels, K = the 128 pixels of a tile of one image
+// row, 16 per MMA.  For the x at column w of row h + (ky - 1) d, g at column
+// w - (kx - 1) d of row h: the staged row of g read from another pixel on.  Both
+// operands are MN-major: a pixel's channels are contiguous, so what is staged is
+// a plain copy of memory and nothing is transposed (core matrices of 8 pixels x
+// 8 channels, 128 bytes; LBO the distance of 8 pixels, SBO the one of 8
+// channels).  A's rows must lie in a row: the ring of six rows of x has its first
+// three again behind the sixth.  At the end warp ky adds the accumulators of its
+// row to dw, 32 input channels at a time, and the block its FP32 sums of g to
+// dbias; a block whose MMAs did not complete adds NaN.
 //
-// Bound by L2 reads (six rows of 64 bytes per pixel and segment).  The operands
-// transposed while staged (K-major, 2-byte stores, nine shifted copies of x)
-// took 145 us at 8 x 256 x 256 pixels.
-constexpr int kWgGroup5 = kTile5 * 16;                 // one channel group: 128 pixels x 16 bytes
-constexpr int kWgABytes5 = 16 * kWgGroup5;             // 3 shifts x 4 groups, 4 zero groups
-constexpr int kWgBBytes5 = 3 * 4 * kWgGroup5;          // three rows of x
-constexpr int kWgSmem5 = kWgABytes5 + kWgBBytes5 + 16; // + mbarrier and TMEM address
+// Bound by the chain of a tile (copies, MMAs, sums of g, about 1 us each for 16
+// tiles per CTA): 38 us at 8 x 256 x 256 pixels.  The operands transposed while
+// staged (K-major, 2-byte stores, nine shifted copies of x) took 145 us, three
+// rows of x and three shifted copies of g per tile 99 us.
+constexpr int kWgRing5 = 6, kWgG5 = 3;                 // staged rows of x (and 3 again) and of g
+constexpr int kWgABytes5 = (kWgRing5 + 3) * kTileRow5;
+constexpr int kWgSmem5 = kWgABytes5 + kWgG5 * kHaloRow5 + 24;   // + barriers and TMEM address
 constexpr uint32_t kWgCols5 = 128;                     // 3 x 32 columns, as a power of two
-constexpr int kWgCtas5 = 3;                            // CTAs per SM
-static_assert(9 * kC * kC * 4 <= kWgABytes5 + kWgBBytes5, "dW fits the staging area");
+constexpr int kWgCtas5 = 2;                            // CTAs per SM
 
 template <typename G>
-__global__ void __launch_bounds__(128) conv32_wgrad_tc05_kernel(const bf16 *__restrict__ x, const G *__restrict__ g,
-                                                                float *__restrict__ dw, float *__restrict__ db, int B,
-                                                                int H, int W, int rows, int dil)
+__global__ void __launch_bounds__(kThreads5) conv32_wgrad_tc05_kernel(ChainArgs ch, const bf16 *__restrict__ x,
+                                                                const G *__restrict__ g, float *__restrict__ dw,
+                                                                float *__restrict__ db)
 {
     extern __shared__ __align__(128) unsigned char smw[];
-    unsigned char *as = smw;
-    unsigned char *bs = smw + kWgABytes5;
-    unsigned long long *mbar = reinterpret_cast<unsigned long long *>(smw + kWgABytes5 + kWgBBytes5);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ float bias_s[4][kC];
+    unsigned char *gs = smw + kWgABytes5;
+    unsigned long long *mbar = reinterpret_cast<unsigned long long *>(gs + kWgG5 * kHaloRow5);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(mbar + 2);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cg = threadIdx.x & 3;
+    const Unit u = unit_of(ch, blockIdx.x);
+    if (u.n < 1) return;
 
     tc05_begin(tslot, mbar, kWgCols5);
-    for (int k = threadIdx.x; k < 4 * kTile5; k += 128)
-        *reinterpret_cast<uint4 *>(as + 12 * kWgGroup5 + k * 16) = make_uint4(0u, 0u, 0u, 0u);
-
-    float gsum[kC];   // FP32 sums of g over this thread's pixels (bias gradient)
-#pragma unroll
-    for (int o = 0; o < kC; ++o) gsum[o] = 0.f;
-    const int r0 = blockIdx.x * rows, r1 = min(r0 + rows, B * H);
-    const int segs = (W + kTile5 - 1) / kTile5;
-    bool done = true;
-    uint32_t nseg = 0;
-    for (int r = r0; r < r1 && done; ++r) {
-        const int h = r % H;
-        const G *grow = g + (int64_t)r * W * kC;
-        for (int sg = 0; sg < segs && done; ++sg, ++nseg) {
-            const int w0 = sg * kTile5;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                // A: g shifted by (q - 1) d; B: row h + (q - 1) d of x
-                const int hh = h + (q - 1) * dil;
-                const bool rin = (unsigned)hh < (unsigned)H;
-                const bf16 *xrow = x + ((int64_t)r + (rin ? (q - 1) * dil : 0)) * W * kC;
-                for (int i = threadIdx.x; i < 4 * kTile5; i += 128) {
-                    const int p = i >> 2, cg = i & 3, w = w0 + p, wg = w - (q - 1) * dil;
-                    const bool xin = rin && w < W, gin = w < W && (unsigned)wg < (unsigned)W;
-                    cp16(s_u32(bs + (q * 4 + cg) * kWgGroup5 + p * 16), xin ? xrow + (int64_t)w * kC + cg * 8 : x, xin);
-                    unsigned char *ad = as + (q * 4 + cg) * kWgGroup5 + p * 16;
-                    if constexpr (sizeof(G) == 2) {
-                        cp16(s_u32(ad), gin ? grow + (int64_t)wg * kC + cg * 8 : g, gin);
-                    } else {
-                        float f[8] = {};
-                        if (gin) load8(grow + (int64_t)wg * kC + cg * 8, true, f);
-                        *reinterpret_cast<uint4 *>(ad) = pack8(f);
-                    }
-                }
-            }
-            staged_sync();
-            if (threadIdx.x == 0) {
-                constexpr uint32_t idesc = umma_idesc_bf16(kTile5, kC, true);
-                const uint32_t abase = s_u32(as), bbase = s_u32(bs), taddr = *tslot;
-#pragma unroll 1
-                for (int k = 0; k < kTile5 / 16; ++k) {
-                    const uint64_t adesc = umma_smem_desc(abase + (uint32_t)(k * 256), 128, kWgGroup5);
-#pragma unroll 1
-                    for (int q = 0; q < 3; ++q)
-                        umma_bf16(taddr + (uint32_t)(q * kC), adesc,
-                                  umma_smem_desc(bbase + (uint32_t)(q * 4 * kWgGroup5 + k * 256), 128, kWgGroup5), idesc,
-                                  (nseg > 0 || k > 0) ? 1u : 0u);
-                }
-                umma_commit(mbar);
-            }
-            // meanwhile the sums of g (the unshifted copy; FP32 g from memory)
-            if (w0 + (int)threadIdx.x < W) {
-#pragma unroll
-                for (int cg = 0; cg < 4; ++cg) {
-                    float f[8];
-                    if constexpr (sizeof(G) == 2)
-                        unpack8(*reinterpret_cast<const uint4 *>(as + (4 + cg) * kWgGroup5 + threadIdx.x * 16), f);
-                    else
-                        load8(grow + (int64_t)(w0 + (int)threadIdx.x) * kC + cg * 8, true, f);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) gsum[cg * 8 + j] += f[j];
-                }
-            }
-            // bounded wait for the segment's MMAs before its operands are overwritten
-            done = __syncthreads_and(mbar_wait(mbar, nseg & 1u)) != 0;   // block-uniform: stop at the first failure
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // copy group j: row j of x (image row h0 + (j - 1) d) and row j - 3 of g (h0 + (j - 3) d).
+    // Tile k takes rows k .. k + 2 of x and row k of g, and its MMAs read row k + 3 of x.
+    auto stage = [&](int j) {
+        if (warp < 4 && j < u.n + 2) {
+            const int slot = j % kWgRing5;
+            stage_row(ch, x, u.b, u.h0 + (j - 1) * ch.dil, u.w0, kTile5, kTileGroup5, smw + slot * kTileRow5,
+                      slot < 3 ? smw + (kWgRing5 + slot) * kTileRow5 : nullptr);
         }
-    }
-    __syncthreads();
-    const uint32_t taddr = *tslot;
-    const float bad = __int_as_float(0x7fc00000);
-    // bias gradient: the warp's sums, one atomic per channel and warp
+        if (warp < 4 && j >= 3 && j < u.n + 3)
+            stage_row(ch, g, u.b, u.h0 + (j - 3) * ch.dil, u.w0 - ch.dil, kTile5 + 2 * ch.dil, kHaloGroup5,
+                      gs + (j % kWgG5) * kHaloRow5, nullptr);
+        cp_commit();
+    };
+    for (int j = 0; j < kWgRing5; ++j) stage(j);
+
+    float gsum[8];   // FP32 sums of g over this thread's pixels, channels 8 cg .. (bias gradient)
 #pragma unroll
-    for (int o = 0; o < kC; ++o) {
+    for (int o = 0; o < 8; ++o) gsum[o] = 0.f;
+    bool good = true;
+    uint32_t taddr = 0;
+    for (int k = 0; k <= u.n; ++k) {
+        if (k < u.n) {
+            good = staged_sync<1>(good);   // groups up to k + 3 are there
+            taddr = *tslot;
+            const unsigned char *grow = gs + (k % kWgG5) * kHaloRow5;
+            if (good && threadIdx.x == 128) {
+                constexpr uint32_t idesc = umma_idesc_bf16(kTile5, kC, true);
+                const uint64_t adesc = umma_smem_desc(s_u32(smw) + (uint32_t)(k % kWgRing5) * kTileRow5, 128, kTileGroup5);
+                const uint64_t gdesc = umma_smem_desc(s_u32(grow), 128, kHaloGroup5);
+#pragma unroll
+                for (int s = 0; s < kTile5 / 16; ++s)
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx)
+                        umma_bf16(taddr + (uint32_t)(kx * kC), umma_step(adesc, (uint32_t)s * 256u),
+                                  umma_step(gdesc, (uint32_t)s * 256u + (uint32_t)((2 - kx) * ch.dil) * 16u), idesc,
+                                  (k > 0 || s > 0) ? 1u : 0u);
+                umma_commit(mbar + (k & 1));
+            }
+            // meanwhile the sums of g (FP32 g from memory)
+            for (int p = threadIdx.x >> 2; warp < 4 && p < kTile5 && u.w0 + p < ch.W; p += 32) {
+                float f[8];
+                if constexpr (sizeof(G) == 2)
+                    unpack8(*reinterpret_cast<const uint4 *>(grow + cg * kHaloGroup5 + (p + ch.dil) * 16), f);
+                else
+                    load8(g + ((u.b * ch.H + u.h0 + k * ch.dil) * ch.W + u.w0 + p) * kC + cg * 8, true, f);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) gsum[j] += f[j];
+            }
+        }
+        if (k == 0) continue;
+        if (good) good = mbar_wait(mbar + ((k - 1) & 1), (uint32_t)((k - 1) >> 1) & 1u);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        stage(k - 1 + kWgRing5);
+    }
+    good = __syncthreads_and(good) != 0;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const float bad = __int_as_float(0x7fc00000);
+    // bias gradient: the warps' sums, then one 128-byte addition per block (every block adds to
+    // the same line: one atomic per channel and warp took 15 us at 8 x 256 x 256 pixels)
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
         float v = gsum[o];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) atomicAdd(db + o, done ? v : bad);
-    }
-    // weight gradient: warp kx holds rows o = lane of shift kx
-    float *out = reinterpret_cast<float *>(smw);   // dW of this block
-#pragma unroll 1
-    for (int q = 0; q < 3; ++q) {
-        uint32_t acc[kC];
-        tmem_load32(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)(q * kC), acc);
-        if (warp < 3)
-#pragma unroll
-            for (int i = 0; i < kC; i += 4)
-                *reinterpret_cast<float4 *>(out + ((size_t)lane * 9 + q * 3 + warp) * kC + i) =
-                    make_float4(__uint_as_float(acc[i]), __uint_as_float(acc[i + 1]), __uint_as_float(acc[i + 2]),
-                                __uint_as_float(acc[i + 3]));
+        for (int off = 4; off < 32; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (warp < 4 && lane < 4) bias_s[warp][cg * 8 + o] = v;
     }
     __syncthreads();
-    if (nseg > 0)
-        for (int k = threadIdx.x; k < 9 * kC * kC; k += 128) atomicAdd(dw + k, done ? out[k] : bad);
+    if (warp == 4) {
+        const float v = (bias_s[0][lane] + bias_s[1][lane]) + (bias_s[2][lane] + bias_s[3][lane]);
+        atomicAdd(db + lane, good ? v : bad);
+    }
+    // weight gradient: warp ky holds rows i = lane of the row ky of x
+#pragma unroll 1
+    for (int kx = 0; kx < 3 && warp < 3; ++kx) {
+        uint32_t acc[kC];
+        tmem_load32(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)(kx * kC), acc);
+#pragma unroll
+            for (int o = 0; o < kC; ++o)
+                atomicAdd(dw + ((size_t)o * 9 + warp * 3 + kx) * kC + lane, good ? __uint_as_float(acc[o]) : bad);
+    }
     tc05_end(taddr, kWgCols5);
 }
 
@@ -764,16 +824,34 @@ int sm_count()
     return sms;
 }
 
+// Segments per chain: as many units as keep all slots (resident CTAs) busy, with
+// as few starts as possible; a start costs about `start` rows (copies until the
+// first tile can begin, and the end of the block).
+ChainArgs share_out(int B, int H, int W, int dil, int64_t slots, int start, unsigned &units)
+{
+    ChainArgs c{B, H, W, dil, (W + kTile5 - 1) / kTile5, dil < H ? dil : H, 1, 1};
+    const int64_t len = (H + c.chains - 1) / c.chains, base = (int64_t)B * c.strips * c.chains;
+    int64_t best = -1;
+    for (int waves = 1; waves <= 3; ++waves) {   // the most segments that so many waves hold
+        int64_t segs = waves * slots / base;
+        segs = segs < 1 ? 1 : segs > len ? len : segs;
+        const int64_t rows = (len + segs - 1) / segs, cost = (base * segs + slots - 1) / slots * (rows + start);
+        if (best < 0 || cost < best) { best = cost; c.segs = (int)((len + rows - 1) / rows); c.rows = (int)rows; }
+    }
+    units = (unsigned)(base * c.segs);
+    return c;
+}
+
 template <typename IN, typename OUT>
-cudaError_t launch_conv32(const ConvArgs &a, const IN *x, OUT *y, cudaStream_t s)
+cudaError_t launch_conv32(int B, int H, int W, int dil, const ConvArgs &a, const IN *x, OUT *y, cudaStream_t s)
 {
     cudaError_t e = cudaFuncSetAttribute(conv32_tc05_kernel<IN, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem5);
     if (e != cudaSuccess) return e;
     const int sms = sm_count();
     if (sms < 1) return cudaErrorUnknown;
-    const int64_t tiles = (int64_t)a.B * a.H * ((a.W + kTile5 - 1) / kTile5);
-    const int64_t most = 2 * (int64_t)sms;   // resident at once (80 KB of shared memory each)
-    conv32_tc05_kernel<IN, OUT><<<(unsigned)(tiles < most ? tiles : most), 128, kSmem5, s>>>(a, x, y, tiles);
+    unsigned units;
+    const ChainArgs c = share_out(B, H, W, dil, kCtas5 * (int64_t)sms, 4, units);
+    conv32_tc05_kernel<IN, OUT><<<units, kThreads5, kSmem5, s>>>(c, a, x, y);
     return cudaGetLastError();
 }
 
@@ -784,10 +862,9 @@ cudaError_t launch_wgrad32(int B, int H, int W, int dil, const bf16 *x, const G 
     if (e != cudaSuccess) return e;
     const int sms = sm_count();
     if (sms < 1) return cudaErrorUnknown;
-    const int64_t nrows = (int64_t)B * H, target = kWgCtas5 * (int64_t)sms;
-    const int rows = (int)((nrows + target - 1) / target);
-    const int blocks = (int)((nrows + rows - 1) / rows);
-    conv32_wgrad_tc05_kernel<G><<<blocks, 128, kWgSmem5, s>>>(x, g, dw, db, B, H, W, rows, dil);
+    unsigned units;
+    const ChainArgs c = share_out(B, H, W, dil, kWgCtas5 * (int64_t)sms, 6, units);
+    conv32_wgrad_tc05_kernel<G><<<units, kThreads5, kWgSmem5, s>>>(c, x, g, dw, db);
     return cudaGetLastError();
 }
 
@@ -831,7 +908,7 @@ sp_status sp_conv3x3_fwd(int32_t B, int32_t H, int32_t W, int32_t cin, int32_t c
     const EdgeArgs ea{B, H, W, dilation, 1};
     cudaError_t e;
     if (cin == 32 && cout == 32) {
-        e = launch_conv32(ConvArgs{B, H, W, dilation, relu, kWPlain, wb, bias, nullptr}, xb, static_cast<bf16 *>(y), s);
+        e = launch_conv32(B, H, W, dilation, ConvArgs{relu, kWPlain, wb, bias, nullptr}, xb, static_cast<bf16 *>(y), s);
     } else if (cin == 1) {
         edge_out32_kernel<bf16, false, false, bf16><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
             ea, xb, wb, bias, nullptr, relu, static_cast<bf16 *>(y), nullptr, 1);
@@ -860,7 +937,7 @@ sp_status sp_conv3x3_bwd_data(int32_t B, int32_t H, int32_t W, int32_t cin, int3
         if (!aligned16(g) || !aligned16(w) || !aligned16(dx))
             return record_error(SP_EINVAL, "g, w, dx must be 16-byte aligned");
         if (gate && !aligned16(gate)) return record_error(SP_EINVAL, "gate must be 16-byte aligned");
-        e = launch_conv32(ConvArgs{B, H, W, dilation, 0, kWFlip, wb, nullptr, gb}, g, dx, s);
+        e = launch_conv32(B, H, W, dilation, ConvArgs{0, kWFlip, wb, nullptr, gb}, g, dx, s);
     } else if (cin == 32) {
         edge_out32_kernel<float, false, true, float><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
             ea, g, wb, nullptr, gb, 0, dx, nullptr, aligned16(dx) && aligned16(gate) ? 1 : 0);
@@ -967,7 +1044,7 @@ sp_status sp_convnet_fwd(int32_t B, int32_t H, int32_t W, int32_t layers, const 
     cudaError_t e = cudaGetLastError();
     auto at = [&](int k) { return act + slab * (size_t)(keep ? k : (k & 1)); };   // layer k's activations
     for (int k = 1; k < layers - 1 && e == cudaSuccess; ++k)
-        e = launch_conv32(ConvArgs{B, H, W, dilation[k], 1, kWPacked, pk + pack_at(layers, k), bias[k], nullptr}, at(k - 1),
+        e = launch_conv32(B, H, W, dilation[k], ConvArgs{1, kWPacked, pk + pack_at(layers, k), bias[k], nullptr}, at(k - 1),
                           at(k), s);
     if (e == cudaSuccess) {
         edge_in32_kernel<bf16, false><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
@@ -1011,7 +1088,7 @@ sp_status sp_convnet_bwd(int32_t B, int32_t H, int32_t W, int32_t layers, const 
         const bf16 *below = act + slab * (size_t)(k - 1);
         e = launch_wgrad32(B, H, W, dilation[k], below, gk[cur], dw(k), db(k), s);
         if (e == cudaSuccess)
-            e = launch_conv32(ConvArgs{B, H, W, dilation[k], 0, kWPacked, pk + pack_at(layers, k) + 9 * kC * kC, nullptr, below},
+            e = launch_conv32(B, H, W, dilation[k], ConvArgs{0, kWPacked, pk + pack_at(layers, k) + 9 * kC * kC, nullptr, below},
                               gk[cur], gk[cur ^ 1], s);
         cur ^= 1;
     }

@@ -23,6 +23,7 @@ import time
 
 import numpy as np
 import torch
+from torch.autograd import forward_ad
 
 from . import _lib
 from ._lib import Grid, Lines, Plan, _check, _stream, load
@@ -81,22 +82,28 @@ def conv3x3(x, w, b, relu: bool, dil: int = 1):
     return _Conv3x3.apply(x, w, b, int(w.shape[3]), int(w.shape[0]), bool(relu), int(dil))
 
 
+def _net_forward(z, dils, keep, params):
+    """x_0, and with keep what the backward needs: the activations followed by z
+    in BF16, and the weights as the kernels take them."""
+    n = len(dils)
+    z = z.detach().contiguous()
+    B, H, W = z.shape
+    acts = torch.empty((((n - 1) if keep else 2) * CH + 1) * B * H * W, dtype=torch.bfloat16, device=z.device)
+    pack = torch.empty(load().sp_convnet_pack_elems(n), dtype=torch.bfloat16, device=z.device)
+    out = torch.empty_like(z)
+    pointers = [p.data_ptr() for p in params]
+    _check(load().sp_convnet_fwd(B, H, W, n, (ctypes.c_int32 * n)(*dils), (ctypes.c_void_p * n)(*pointers[:n]),
+                                 (ctypes.c_void_p * n)(*pointers[n:]), z.data_ptr(), int(keep), acts.data_ptr(),
+                                 pack.data_ptr(), out.data_ptr(), _stream(None)))
+    return out, acts, pack
+
+
 class _Net(torch.autograd.Function):
     """x_0 = z + f(z) in one call per direction (sp_convnet_fwd, sp_convnet_bwd)."""
 
     @staticmethod
     def forward(ctx, z, dils, keep, *params):
-        n = len(dils)
-        z = z.detach().contiguous()
-        B, H, W = z.shape
-        # activations, then z in BF16
-        acts = torch.empty((((n - 1) if keep else 2) * CH + 1) * B * H * W, dtype=torch.bfloat16, device=z.device)
-        pack = torch.empty(load().sp_convnet_pack_elems(n), dtype=torch.bfloat16, device=z.device)
-        out = torch.empty_like(z)
-        pointers = [p.data_ptr() for p in params]
-        _check(load().sp_convnet_fwd(B, H, W, n, (ctypes.c_int32 * n)(*dils), (ctypes.c_void_p * n)(*pointers[:n]),
-                                     (ctypes.c_void_p * n)(*pointers[n:]), z.data_ptr(), int(keep), acts.data_ptr(),
-                                     pack.data_ptr(), out.data_ptr(), _stream(None)))
+        out, acts, pack = _net_forward(z, dils, keep, params)
         if keep:
             ctx.save_for_backward(acts, pack)
             ctx.meta = z.shape, dils, [p.shape for p in params]
@@ -145,7 +152,12 @@ class WarmStartNet(torch.nn.Module):
                 and all(w.shape == (cout, 3, 3, cin) and b.shape == (cout,)
                         for w, b, (cin, cout, _, _) in zip(params, params[len(LAYERS):], LAYERS))):
             keep = torch.is_grad_enabled() and (z.requires_grad or any(p.requires_grad for p in params))
-            return _Net.apply(z, tuple(layer[3] for layer in LAYERS), keep, *params)
+            dils = tuple(layer[3] for layer in LAYERS)
+            # nothing to differentiate or record: without the autograd function (21 us of 97 for
+            # one 256 x 256 image), which tracing and forward mode do have to see
+            if not (keep or torch.jit.is_tracing() or forward_ad._current_level >= 0):
+                return _net_forward(z, dils, False, params)[0]
+            return _Net.apply(z, dils, keep, *params)
         # other dtypes and devices: layer by layer
         x = z.to(torch.bfloat16).unsqueeze(-1).contiguous()
         for k, (_, _, relu, dil) in enumerate(LAYERS):
