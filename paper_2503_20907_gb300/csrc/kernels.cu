@@ -41,11 +41,9 @@ __device__ __forceinline__ float factf(int n)
     return r;
 }
 
-// Unit direction (dx, dy) and a point (px, py) of line r, in double.  For
-// parallel and fan beams, vs / vc (if not NULL) hold sin and cos of the view
-// angle of line r, computed as below.
+// Unit direction (dx, dy) and a point (px, py) of line r, in double.
 __device__ void line_geometry(const LinesDev &L, int64_t r, double &dx, double &dy, double &px,
-                              double &py, const double *vs = nullptr, const double *vc = nullptr)
+                              double &py)
 {
     switch (L.kind) {
     case SP_LINES_THETA_Y: {
@@ -64,8 +62,7 @@ __device__ void line_geometry(const LinesDev &L, int64_t r, double &dx, double &
     case SP_LINES_PARALLEL: {
         int64_t v = r / L.n_det, j = r - v * L.n_det;
         double s, c;
-        if (vs) { s = *vs; c = *vc; }
-        else sincos((double)L.view[v], &s, &c);
+        sincos((double)L.view[v], &s, &c);
         double yy = (double)L.det0 + (double)j * (double)L.ddet;
         dx = c; dy = s; px = yy * s; py = -yy * c;
         break;
@@ -73,8 +70,7 @@ __device__ void line_geometry(const LinesDev &L, int64_t r, double &dx, double &
     default: {  // SP_LINES_FAN
         int64_t v = r / L.n_det, j = r - v * L.n_det;
         double sb, cb;
-        if (vs) { sb = *vs; cb = *vc; }
-        else sincos((double)L.view[v], &sb, &cb);
+        sincos((double)L.view[v], &sb, &cb);
         double sx = (double)L.dso * cb, sy = (double)L.dso * sb;
         double off = (double)L.det0 + (double)j * (double)L.ddet;
         double ex = -(double)L.dod * cb - off * sb, ey = -(double)L.dod * sb + off * cb;
@@ -136,67 +132,104 @@ __device__ __forceinline__ int footprint_mode(int basis, double dx, double dy)
     return (dx * dy >= 0.0) ? kModeBoxSame : kModeBoxOpp;
 }
 
-// Split x into hi + lo with hi carrying `bits` significant bits.
-__device__ void split_hi_lo(double x, int bits, float &hi, float &lo)
+// Split x into hi + lo with hi carrying `bits` significant bits (1..23).
+__device__ __forceinline__ void split_hi_lo(double x, int bits, float &hi, float &lo)
 {
-    if (x == 0.0) { hi = 0.f; lo = 0.f; return; }
-    int e;
-    frexp(x, &e);
-    const double sc = ldexp(1.0, bits - e), isc = ldexp(1.0, e - bits);   // powers of two: exact
-    double xh = rint(x * sc) * isc;
-    hi = (float)xh;
-    lo = (float)(x - xh);
+    const unsigned unit = 1u << (24 - bits);
+    hi = __uint_as_float((__float_as_uint((float)x) + unit / 2) & ~(unit - 1));
+    lo = (float)(x - (double)hi);
 }
 
 // ------------------------------------------------------------------ setup
+// Bound by the FP64 units (2 FMAs per clock and SM): what the records do not
+// need in FP64 (the row range, the quotients, integer parts) is not, the row
+// range with margins far above FP32's error, and what the lines of a view share
+// is computed once per view.  2.2 M parallel lines take 258 us (718 us with the
+// range and its five divisions in FP64).
 constexpr int kSetupThreads = 128;
 
-// Line setup of line r: its record hdr[r] (see LineHdr) and the footprint's
-// a, b and kind.  vs, vc: sin and cos of the line's view for parallel and fan
-// beams (NULL: computed here).
-__device__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineHdr *hdr, const double *vs,
-                           const double *vc, float &af, float &bf, int &mode)
+// What the lines of one view share, relative to the grid's centre (fan beams:
+// the source and the detector's foot point as seen from it).
+struct ViewGeo {
+    double s, c, px, py, vx, vy;
+};
+
+__device__ void view_geometry(const GridDev &g, const LinesDev &L, int64_t v, ViewGeo &V)
 {
-    double dx, dy, px, py;
-    line_geometry(L, r, dx, dy, px, py, vs, vc);
+    sincos((double)L.view[v], &V.s, &V.c);
+    if (L.kind == SP_LINES_FAN) {
+        const double dist = (double)L.dso + (double)L.dod;
+        V.px = (double)L.dso * V.c - (double)g.cx;
+        V.py = (double)L.dso * V.s - (double)g.cy;
+        V.vx = -dist * V.c;
+        V.vy = -dist * V.s;
+    } else {
+        V.px = (double)g.cy * V.c - (double)g.cx * V.s;   // the offset of the centre's line
+    }
+}
+
+// Line setup of line r: its record hdr[r] (see LineHdr) and the footprint's
+// a, b and kind.  V (parallel and fan beams, else NULL): its view; j: its bin;
+// tab: the index of its table.
+__device__ __forceinline__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineHdr *hdr, const ViewGeo *V,
+                                           int j, int tab, float &af, float &bf, int &mode)
+{
+    double dx, dy, Yhat;   // direction; ((p - centre) x direction), then over h
+    if (L.kind == SP_LINES_PARALLEL) {
+        dx = V->c;
+        dy = V->s;
+        Yhat = (double)L.det0 + (double)j * (double)L.ddet + V->px;
+    } else if (L.kind == SP_LINES_FAN) {
+        const double off = (double)L.det0 + (double)j * (double)L.ddet;
+        const double vx = V->vx - off * V->s, vy = V->vy + off * V->c;
+        const double inv = rsqrt(vx * vx + vy * vy);
+        dx = vx * inv;
+        dy = vy * inv;
+        Yhat = V->px * dy - V->py * dx;
+    } else {
+        double px, py;
+        line_geometry(L, r, dx, dy, px, py);
+        Yhat = (px - (double)g.cx) * dy - (py - (double)g.cy) * dx;
+    }
+    if (g.h != 1.f) Yhat /= (double)g.h;
     LineHdr H;
     H.U0_lo = 0.f;
     H.a_corr = 0.f;
-    H.tab = (L.kind == SP_LINES_PARALLEL) ? (int)(r / L.n_det) : (int)r;
+    H.tab = tab;
     footprint_ab(g.kdeg, dx, dy, af, bf);
     mode = footprint_mode(g.basis, dx, dy);
     double w;
     support_params(g.kdeg, af, bf, mode, H.two_w, w, H.K);
     const bool vert = fabs(dy) >= fabs(dx);
-    const double A = fmax(fabs(dx), fabs(dy));
-    const double B = fmin(fabs(dx), fabs(dy));
-    const double h = (double)g.h;
-    double Yhat = ((px - (double)g.cx) * dy - (py - (double)g.cy) * dx) / h;
-    const double ic = 0.5 * (g.nx - 1), jc = 0.5 * (g.ny - 1);
-    double kap, rho, rc, qc;
+    const float ic = 0.5f * (float)(g.nx - 1), jc = 0.5f * (float)(g.ny - 1);
+    double kap, rho;
+    float rc, qc;
     int Nr, Nq;
     if (vert) { kap = -dy; rho = dx; rc = jc; qc = ic; Nr = g.ny; Nq = g.nx; }
     else { kap = dx; rho = -dy; rc = ic; qc = jc; Nr = g.nx; Nq = g.ny; }
     // a line and its reverse are one line, and phi is even: take the direction
     // in which u grows with the column
     if (kap < 0.0) { kap = -kap; rho = -rho; Yhat = -Yhat; }
+    const double A = kap;
     // w as the table sees it (support_params, with the table's a and b)
     int flags = vert ? kVert : 0;
-    if (g.degree == 0 && B == 0.0) flags |= kDeg0Axis;
+    if (g.degree == 0 && (vert ? dx : dy) == 0.0) flags |= kDeg0Axis;
 
     // Rows whose support run meets the columns [0, Nq): the column of the
-    // support centre (u = w) moves linearly with the row.
-    const double lo = -w / A - 2.0, hi = (double)(Nq - 1) + w / A + 2.0;
-    const double c0 = qc - (Yhat - rc * rho) / kap;   // centre column at row 0
-    const double gam = -rho / kap;
+    // support centre (u = w) moves linearly with the row.  In FP32: at 16384
+    // columns it is off by less than 0.01 column, against a margin of two.
+    const float kapf = (float)kap, rhof = (float)rho, wa = (float)w / kapf + 2.f;
+    const float lo = -wa, hi = (float)(Nq - 1) + wa;
+    const float c0 = qc - ((float)Yhat - rc * rhof) / kapf;   // centre column at row 0
+    const float gam = -rhof / kapf;
     int rb = 0, re = 0;
-    if (fabs(gam) < 1e-300) {
+    if (fabsf(gam) < 1e-30f) {
         if (c0 >= lo && c0 <= hi) { rb = 0; re = Nr; }
     } else {
-        double t0 = (lo - c0) / gam, t1 = (hi - c0) / gam;
-        if (t0 > t1) { double t = t0; t0 = t1; t1 = t; }
-        t0 = fmax(floor(t0) - 1.0, 0.0);
-        t1 = fmin(ceil(t1) + 2.0, (double)Nr);
+        float t0 = (lo - c0) / gam, t1 = (hi - c0) / gam;
+        if (t0 > t1) { const float t = t0; t0 = t1; t1 = t; }
+        t0 = fmaxf(floorf(t0) - 1.f, 0.f);
+        t1 = fminf(ceilf(t1) + 2.f, (float)Nr);
         if (t1 > t0) { rb = (int)t0; re = (int)t1; }
     }
     if (rb >= re || !(Yhat == Yhat)) {
@@ -209,16 +242,14 @@ __device__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineH
     }
     const int r_ref = (rb + re) / 2;
     // u at (r_ref, q = 0), then the reference column with U0 in (0, a].
-    const double Ur = Yhat + w + ((double)r_ref - rc) * rho - qc * kap;
-    double qr = floor(-Ur / A) + 1.0;
-    double U0 = Ur + qr * kap;
-    if (U0 <= 0.0) { qr += 1.0; U0 = Ur + qr * kap; }
-    else if (U0 > A) { qr -= 1.0; U0 = Ur + qr * kap; }
+    const double Ur = Yhat + w + (double)((float)r_ref - rc) * rho - (double)qc * kap;
+    int qr = (int)floorf(-(float)Ur / kapf) + 1;   // off by one at most
+    double U0 = Ur + (double)qr * kap;
+    if (U0 <= 0.0) { ++qr; U0 = Ur + (double)qr * kap; }
+    else if (U0 > A) { --qr; U0 = Ur + (double)qr * kap; }
     // hi parts exact against |row offset| and |step count|, both < maxc
-    int maxc = (re - rb) + 8;
-    int nb = 0;
-    while ((1 << nb) <= maxc) ++nb;
-    const int bits = 23 - nb;
+    const int maxc = (re - rb) + 8;
+    const int bits = 23 - (32 - __clz(maxc));
     H.U0 = (float)U0;
     H.U0_lo = (float)(U0 - (double)H.U0);
     split_hi_lo(rho, bits, H.rho_hi, H.rho_lo);
@@ -226,7 +257,7 @@ __device__ void setup_line(const GridDev &g, const LinesDev &L, int64_t r, LineH
     H.a = af;
     H.a_corr = (float)(A - (double)af);
     H.r_ref = r_ref;
-    H.q_ref = (int)qr;
+    H.q_ref = qr;
     H.r_begin = rb;
     H.r_end = re;
     H.flags = flags;
@@ -480,31 +511,27 @@ template <int DEG>
 __global__ void __launch_bounds__(kSetupThreads) setup_kernel(GridDev g, LinesDev L, LineHdr *hdr, float *tabs, float *rec,
                                                               int64_t M)
 {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    // parallel and fan beams: sin and cos of each view once per block (the
-    // block's lines span at most blockDim.x views)
-    __shared__ double vsin[kSetupThreads], vcos[kSetupThreads];
+    const int64_t r0 = (int64_t)blockIdx.x * kSetupThreads, r = r0 + threadIdx.x;
+    // parallel and fan beams: the views of the block's lines (at most one per thread)
+    __shared__ ViewGeo geo[kSetupThreads];
     const bool views = (L.kind == SP_LINES_PARALLEL || L.kind == SP_LINES_FAN);
     int64_t v0 = 0;
+    int k = 0, j = 0;   // this line's view, from v0 on, and bin
     if (views) {
-        const int64_t r0 = (int64_t)blockIdx.x * blockDim.x;
-        const int64_t r1 = min(r0 + (int64_t)blockDim.x, M) - 1;
         v0 = r0 / L.n_det;
-        const int64_t nv = r1 / L.n_det - v0 + 1;
-        if (threadIdx.x < nv) sincos((double)L.view[v0 + threadIdx.x], &vsin[threadIdx.x], &vcos[threadIdx.x]);
+        const unsigned b0 = (unsigned)(r0 - v0 * L.n_det), n = (unsigned)L.n_det;   // the first line's bin
+        const unsigned last = b0 + (unsigned)(min((int64_t)kSetupThreads, M - r0) - 1);
+        if (threadIdx.x <= last / n) view_geometry(g, L, v0 + threadIdx.x, geo[threadIdx.x]);
+        k = (int)((b0 + threadIdx.x) / n);
+        j = (int)((b0 + threadIdx.x) - (unsigned)k * n);
         __syncthreads();
     }
     if (r >= M) return;
     float af, bf;
     int mode;
-    if (views) {
-        const int k = (int)(r / L.n_det - v0);
-        setup_line(g, L, r, hdr, &vsin[k], &vcos[k], af, bf, mode);
-    } else {
-        setup_line(g, L, r, hdr, nullptr, nullptr, af, bf, mode);
-    }
-    const int64_t tab = (L.kind == SP_LINES_PARALLEL) ? r / L.n_det : r;
-    if (L.kind != SP_LINES_PARALLEL || r % L.n_det == 0) {
+    const int64_t tab = (L.kind == SP_LINES_PARALLEL) ? v0 + k : r;
+    setup_line(g, L, r, hdr, views ? geo + k : nullptr, j, (int)tab, af, bf, mode);
+    if (L.kind != SP_LINES_PARALLEL || j == 0) {
         if (tabs) {
             tabs[tab * kTabFloats + kTabA] = af;
             tabs[tab * kTabFloats + kTabB] = bf;
