@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const float *__restric
                                                           double *__restrict__ partial, CgScalars *sc,
                                                           int role, double *hist, int k)
 {
+    chain_begin();
     __shared__ double sh[kDotThreads / 32];
     __shared__ bool last;
     double v = 0.0;
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const float *__restric
 __global__ void residual_kernel(const float *__restrict__ b, const float *__restrict__ q, float *__restrict__ r,
                                 int64_t m)
 {
+    chain_begin();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
         r[i] = b[i] - q[i];
 }
@@ -97,6 +99,7 @@ __global__ void update_xr_kernel(float *__restrict__ x, const float *__restrict_
                                  float *__restrict__ r, const float *__restrict__ q, int64_t m,
                                  const CgScalars *__restrict__ sc)
 {
+    chain_begin();
     const float alpha = (float)sc->alpha;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n || i < m; i += stride) {
@@ -109,6 +112,7 @@ __global__ void update_xr_kernel(float *__restrict__ x, const float *__restrict_
 __global__ void update_p_kernel(float *__restrict__ p, const float *__restrict__ s, int64_t n,
                                 const CgScalars *__restrict__ sc)
 {
+    chain_begin();
     const float beta = (float)sc->beta;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         p[i] = __fmaf_rn(beta, p[i], s[i]);
@@ -152,18 +156,18 @@ cudaError_t run_cgls(const CgOps &ops, int64_t n, int64_t m, const float *b, flo
     if (e != cudaSuccess) return e;
     // r = b - A x0; s = A^T r; p = s; gamma = <s, s>
     if ((e = ops.fwd(ops.ctx, x, q, s)) != cudaSuccess) return e;
-    residual_kernel<<<vec_blocks(m), 256, 0, s>>>(b, q, r, m);
+    launch_chained(residual_kernel, vec_blocks(m), 256, 0, s, b, q, r, m);
     if ((e = ops.adj(ops.ctx, r, sv, s)) != cudaSuccess) return e;
     if ((e = cudaMemcpyAsync(p, sv, sizeof(float) * (size_t)n, cudaMemcpyDeviceToDevice, s)) != cudaSuccess) return e;
-    dot_kernel<<<kDotBlocks, kDotThreads, 0, s>>>(sv, n, partial, sc, kDotGamma0, hist, 0);
+    launch_chained(dot_kernel, kDotBlocks, kDotThreads, 0, s, sv, n, partial, sc, kDotGamma0, hist, 0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int k = 1; k <= iters; ++k) {
         if ((e = ops.fwd(ops.ctx, p, q, s)) != cudaSuccess) return e;
-        dot_kernel<<<kDotBlocks, kDotThreads, 0, s>>>(q, m, partial, sc, kDotAlpha, nullptr, k);
-        update_xr_kernel<<<vec_blocks(n > m ? n : m), 256, 0, s>>>(x, p, n, r, q, m, sc);
+        launch_chained(dot_kernel, kDotBlocks, kDotThreads, 0, s, q, m, partial, sc, kDotAlpha, nullptr, k);
+        launch_chained(update_xr_kernel, vec_blocks(n > m ? n : m), 256, 0, s, x, p, n, r, q, m, sc);
         if ((e = ops.adj(ops.ctx, r, sv, s)) != cudaSuccess) return e;
-        dot_kernel<<<kDotBlocks, kDotThreads, 0, s>>>(sv, n, partial, sc, kDotGammaNext, hist, k);
-        update_p_kernel<<<vec_blocks(n), 256, 0, s>>>(p, sv, n, sc);
+        launch_chained(dot_kernel, kDotBlocks, kDotThreads, 0, s, sv, n, partial, sc, kDotGammaNext, hist, k);
+        launch_chained(update_p_kernel, vec_blocks(n), 256, 0, s, p, sv, n, sc);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
                                                                   const bf16 *__restrict__ gate, int relu,
                                                                   OUT *__restrict__ y, bf16 *__restrict__ sb, int vec)
 {
+    chain_begin();
     const int c0 = (threadIdx.x & 3) * 8;
     float wr[9][8], br[8];
 #pragma unroll
@@ -211,6 +212,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, con
                                                                  const float *__restrict__ add, float *__restrict__ y,
                                                                  int vec)
 {
+    chain_begin();
     const int c0 = (threadIdx.x & 3) * 8;
     float wr[9][8];
 #pragma unroll
@@ -251,6 +253,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, co
                                                                   const S *__restrict__ s, float *__restrict__ dw,
                                                                   float *__restrict__ db, int vec)
 {
+    chain_begin();
     __shared__ float part[9 * kC + kC];
     const int lane = threadIdx.x & 31, c0 = (threadIdx.x & 3) * 8;
     for (int k = threadIdx.x; k < 9 * kC + kC; k += kEdgeThreads) part[k] = 0.f;
@@ -312,6 +315,7 @@ unsigned edge_blocks(int B, int H, int W, int per_sm)
 // W'[i, 2-ky, 2-kx, o] = W[o, ky, kx, i] (the input gradient as a forward convolution)
 __global__ void flip_weights_kernel(const bf16 *__restrict__ w, bf16 *__restrict__ wf, int cin, int cout)
 {
+    chain_begin();
     const int n = cout * 9 * cin;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const int o = j / (9 * cin), rem = j - o * 9 * cin, tap = rem / cin, i = rem - tap * cin;
@@ -338,6 +342,7 @@ __host__ __device__ constexpr size_t pack_at(int n, int k)   // first element of
 
 __global__ void pack_weights_kernel(NetWeights N, bf16 *__restrict__ pack)
 {
+    chain_begin();
     const int k = blockIdx.y;
     const float *w = N.w[k];
     bf16 *out = pack + pack_at(N.n, k);
@@ -585,6 +590,7 @@ template <typename IN, typename OUT>
 __global__ void __launch_bounds__(kThreads5) conv32_tc05_kernel(ChainArgs ch, ConvArgs a, const IN *__restrict__ x,
                                                           OUT *__restrict__ y)
 {
+    chain_begin();
     extern __shared__ __align__(128) unsigned char sm5[];
     unsigned char *wsb = sm5 + kRing5 * kHaloRow5;
     float *bias_s = reinterpret_cast<float *>(wsb + kWBytes5);
@@ -718,6 +724,7 @@ __global__ void __launch_bounds__(kThreads5) conv32_wgrad_tc05_kernel(ChainArgs 
                                                                 const G *__restrict__ g, float *__restrict__ dw,
                                                                 float *__restrict__ db)
 {
+    chain_begin();
     extern __shared__ __align__(128) unsigned char smw[];
     __shared__ float bias_s[4][kC];
     unsigned char *gs = smw + kWgABytes5;
@@ -851,7 +858,7 @@ cudaError_t launch_conv32(int B, int H, int W, int dil, const ConvArgs &a, const
     if (sms < 1) return cudaErrorUnknown;
     unsigned units;
     const ChainArgs c = share_out(B, H, W, dil, kCtas5 * (int64_t)sms, 4, units);
-    conv32_tc05_kernel<IN, OUT><<<units, kThreads5, kSmem5, s>>>(c, a, x, y);
+    launch_chained(conv32_tc05_kernel<IN, OUT>, units, kThreads5, kSmem5, s, c, a, x, y);
     return cudaGetLastError();
 }
 
@@ -864,7 +871,7 @@ cudaError_t launch_wgrad32(int B, int H, int W, int dil, const bf16 *x, const G 
     if (sms < 1) return cudaErrorUnknown;
     unsigned units;
     const ChainArgs c = share_out(B, H, W, dil, kWgCtas5 * (int64_t)sms, 6, units);
-    conv32_wgrad_tc05_kernel<G><<<units, kThreads5, kWgSmem5, s>>>(c, x, g, dw, db);
+    launch_chained(conv32_wgrad_tc05_kernel<G>, units, kThreads5, kWgSmem5, s, c, x, g, dw, db);
     return cudaGetLastError();
 }
 
@@ -910,12 +917,10 @@ sp_status sp_conv3x3_fwd(int32_t B, int32_t H, int32_t W, int32_t cin, int32_t c
     if (cin == 32 && cout == 32) {
         e = launch_conv32(B, H, W, dilation, ConvArgs{relu, kWPlain, wb, bias, nullptr}, xb, static_cast<bf16 *>(y), s);
     } else if (cin == 1) {
-        edge_out32_kernel<bf16, false, false, bf16><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-            ea, xb, wb, bias, nullptr, relu, static_cast<bf16 *>(y), nullptr, 1);
+        launch_chained(edge_out32_kernel<bf16, false, false, bf16>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, ea, xb, wb, bias, nullptr, relu, static_cast<bf16 *>(y), nullptr, 1);
         e = cudaGetLastError();
     } else {
-        edge_in32_kernel<bf16, false><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-            ea, xb, wb, bias, relu, 0, nullptr, nullptr, static_cast<float *>(y), 1);
+        launch_chained(edge_in32_kernel<bf16, false>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, ea, xb, wb, bias, relu, 0, nullptr, nullptr, static_cast<float *>(y), 1);
         e = cudaGetLastError();
     }
     return e == cudaSuccess ? SP_OK : record_error(SP_ECUDA, cudaGetErrorString(e));
@@ -939,12 +944,10 @@ sp_status sp_conv3x3_bwd_data(int32_t B, int32_t H, int32_t W, int32_t cin, int3
         if (gate && !aligned16(gate)) return record_error(SP_EINVAL, "gate must be 16-byte aligned");
         e = launch_conv32(B, H, W, dilation, ConvArgs{0, kWFlip, wb, nullptr, gb}, g, dx, s);
     } else if (cin == 32) {
-        edge_out32_kernel<float, false, true, float><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-            ea, g, wb, nullptr, gb, 0, dx, nullptr, aligned16(dx) && aligned16(gate) ? 1 : 0);
+        launch_chained(edge_out32_kernel<float, false, true, float>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, ea, g, wb, nullptr, gb, 0, dx, nullptr, aligned16(dx) && aligned16(gate) ? 1 : 0);
         e = cudaGetLastError();
     } else {
-        edge_in32_kernel<float, true><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-            ea, g, wb, nullptr, 0, 0, gb, nullptr, dx, aligned16(g) ? 1 : 0);
+        launch_chained(edge_in32_kernel<float, true>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, ea, g, wb, nullptr, 0, 0, gb, nullptr, dx, aligned16(g) ? 1 : 0);
         e = cudaGetLastError();
     }
     return e == cudaSuccess ? SP_OK : record_error(SP_ECUDA, cudaGetErrorString(e));
@@ -972,11 +975,9 @@ sp_status sp_conv3x3_bwd_weight(int32_t B, int32_t H, int32_t W, int32_t cin, in
             return record_error(SP_EINVAL, "image too wide for the weight-gradient kernel");
         const unsigned blocks = edge_blocks(B, H, W, 2);
         if (cin == 1)
-            edge_wgrad_kernel<float, bf16, false><<<blocks, kEdgeThreads, 0, s>>>(
-                EdgeArgs{B, H, W, dilation, 1}, g, xb, dw, dbias, aligned16(g) ? 1 : 0);
+            launch_chained(edge_wgrad_kernel<float, bf16, false>, blocks, kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation, 1}, g, xb, dw, dbias, aligned16(g) ? 1 : 0);
         else
-            edge_wgrad_kernel<bf16, float, true><<<blocks, kEdgeThreads, 0, s>>>(
-                EdgeArgs{B, H, W, dilation, -1}, xb, g, dw, dbias, aligned16(xb) ? 1 : 0);
+            launch_chained(edge_wgrad_kernel<bf16, float, true>, blocks, kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation, -1}, xb, g, dw, dbias, aligned16(xb) ? 1 : 0);
         e = cudaGetLastError();
     }
     return e == cudaSuccess ? SP_OK : record_error(SP_ECUDA, cudaGetErrorString(e));
@@ -987,8 +988,7 @@ sp_status sp_conv3x3_flip_weights(int32_t cin, int32_t cout, const void *w, void
     spx::clear_error();
     if (cin < 1 || cout < 1 || !w || !wf) return spx::record_error(SP_EINVAL, "bad arguments");
     const int n = cout * 9 * cin;
-    spx::flip_weights_kernel<<<(n + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const spx::bf16 *>(w), static_cast<spx::bf16 *>(wf), cin, cout);
+    spx::launch_chained(spx::flip_weights_kernel, (n + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream), static_cast<const spx::bf16 *>(w), static_cast<spx::bf16 *>(wf), cin, cout);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? SP_OK : spx::record_error(SP_ECUDA, cudaGetErrorString(e));
 }
@@ -1038,17 +1038,15 @@ sp_status sp_convnet_fwd(int32_t B, int32_t H, int32_t W, int32_t layers, const 
     bf16 *pk = static_cast<bf16 *>(pack), *act = static_cast<bf16 *>(acts);
     const size_t slab = (size_t)B * H * W * kC;
     bf16 *zb = act + slab * (size_t)(keep ? layers - 1 : 2);   // z as the first layer sees it
-    pack_weights_kernel<<<dim3((9 * kC * kC + 255) / 256, layers), 256, 0, s>>>(N, pk);
-    edge_out32_kernel<float, true, false, bf16><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-        EdgeArgs{B, H, W, dilation[0], 1}, z, pk, bias[0], nullptr, 1, act, zb, 1);
+    launch_chained(pack_weights_kernel, dim3((9 * kC * kC + 255) / 256, layers), 256, 0, s, N, pk);
+    launch_chained(edge_out32_kernel<float, true, false, bf16>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation[0], 1}, z, pk, bias[0], nullptr, 1, act, zb, 1);
     cudaError_t e = cudaGetLastError();
     auto at = [&](int k) { return act + slab * (size_t)(keep ? k : (k & 1)); };   // layer k's activations
     for (int k = 1; k < layers - 1 && e == cudaSuccess; ++k)
         e = launch_conv32(B, H, W, dilation[k], ConvArgs{1, kWPacked, pk + pack_at(layers, k), bias[k], nullptr}, at(k - 1),
                           at(k), s);
     if (e == cudaSuccess) {
-        edge_in32_kernel<bf16, false><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-            EdgeArgs{B, H, W, dilation[layers - 1], 1}, at(layers - 2), pk + pack_at(layers, layers - 1), bias[layers - 1],
+        launch_chained(edge_in32_kernel<bf16, false>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation[layers - 1], 1}, at(layers - 2), pk + pack_at(layers, layers - 1), bias[layers - 1],
             0, 0, nullptr, z, out, 1);
         e = cudaGetLastError();
     }
@@ -1078,10 +1076,8 @@ sp_status sp_convnet_bwd(int32_t B, int32_t H, int32_t W, int32_t layers, const 
     cudaError_t e = cudaMemsetAsync(dparam, 0, sizeof(float) * (size_t)(db(L) + 1 - dparam), s);
     if (e != cudaSuccess) return record_error(SP_ECUDA, cudaGetErrorString(e));
     // last layer: g FP32; the gradient of the activations below gated and in BF16
-    edge_wgrad_kernel<bf16, float, true><<<edge_blocks(B, H, W, 2), kEdgeThreads, 0, s>>>(
-        EdgeArgs{B, H, W, dilation[L], -1}, act + slab * (size_t)(L - 1), g, dw(L), db(L), 1);
-    edge_out32_kernel<float, false, true, bf16><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-        EdgeArgs{B, H, W, dilation[L], -1}, g, pk + pack_at(layers, L), nullptr, act + slab * (size_t)(L - 1), 0, gk[0], nullptr, 1);
+    launch_chained(edge_wgrad_kernel<bf16, float, true>, edge_blocks(B, H, W, 2), kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation[L], -1}, act + slab * (size_t)(L - 1), g, dw(L), db(L), 1);
+    launch_chained(edge_out32_kernel<float, false, true, bf16>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation[L], -1}, g, pk + pack_at(layers, L), nullptr, act + slab * (size_t)(L - 1), 0, gk[0], nullptr, 1);
     e = cudaGetLastError();
     int cur = 0;
     for (int k = L - 1; k >= 1 && e == cudaSuccess; --k) {
@@ -1093,11 +1089,9 @@ sp_status sp_convnet_bwd(int32_t B, int32_t H, int32_t W, int32_t layers, const 
         cur ^= 1;
     }
     if (e == cudaSuccess) {
-        edge_wgrad_kernel<bf16, bf16, false><<<edge_blocks(B, H, W, 2), kEdgeThreads, 0, s>>>(
-            EdgeArgs{B, H, W, dilation[0], 1}, gk[cur], act + slab * (size_t)L, dw(0), db(0), 1);
+        launch_chained(edge_wgrad_kernel<bf16, bf16, false>, edge_blocks(B, H, W, 2), kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation[0], 1}, gk[cur], act + slab * (size_t)L, dw(0), db(0), 1);
         if (dx)
-            edge_in32_kernel<bf16, true><<<edge_blocks(B, H, W, 8), kEdgeThreads, 0, s>>>(
-                EdgeArgs{B, H, W, dilation[0], -1}, gk[cur], pk, nullptr, 0, 1, nullptr, nullptr, dx, 1);
+            launch_chained(edge_in32_kernel<bf16, true>, edge_blocks(B, H, W, 8), kEdgeThreads, 0, s, EdgeArgs{B, H, W, dilation[0], -1}, gk[cur], pk, nullptr, 0, 1, nullptr, nullptr, dx, 1);
         e = cudaGetLastError();
     }
     return e == cudaSuccess ? SP_OK : record_error(SP_ECUDA, cudaGetErrorString(e));

@@ -511,6 +511,7 @@ template <int DEG>
 __global__ void __launch_bounds__(kSetupThreads) setup_kernel(GridDev g, LinesDev L, LineHdr *hdr, float *tabs, float *rec,
                                                               int64_t M)
 {
+    chain_begin();
     const int64_t r0 = (int64_t)blockIdx.x * kSetupThreads, r = r0 + threadIdx.x;
     // parallel and fan beams: the views of the block's lines (at most one per thread)
     __shared__ ViewGeo geo[kSetupThreads];
@@ -1236,7 +1237,12 @@ cudaError_t launch_setup(const GridDev &g, const LinesDev &L, LineHdr *hdr, floa
 {
     if (L.m <= 0) return cudaSuccess;
     if (!center_records(g)) rec = nullptr;
-    SPX_DISPATCH(g.kdeg, setup_kernel, blocks_for(L.m, kSetupThreads), kSetupThreads, s, g, L, hdr, tabs, rec, L.m);
+    switch (g.kdeg) {
+    case 0: launch_chained(setup_kernel<0>, blocks_for(L.m, kSetupThreads), kSetupThreads, 0, s, g, L, hdr, tabs, rec, L.m); break;
+    case 1: launch_chained(setup_kernel<1>, blocks_for(L.m, kSetupThreads), kSetupThreads, 0, s, g, L, hdr, tabs, rec, L.m); break;
+    case 2: launch_chained(setup_kernel<2>, blocks_for(L.m, kSetupThreads), kSetupThreads, 0, s, g, L, hdr, tabs, rec, L.m); break;
+    default: launch_chained(setup_kernel<3>, blocks_for(L.m, kSetupThreads), kSetupThreads, 0, s, g, L, hdr, tabs, rec, L.m); break;
+    }
     return cudaGetLastError();
 }
 

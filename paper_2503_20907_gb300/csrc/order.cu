@@ -42,6 +42,7 @@ size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 __global__ void order_keys_kernel(GridDev g, const LineHdr *__restrict__ hdr, int m, int D,
                                   unsigned *__restrict__ keys, int *__restrict__ vals)
 {
+    chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const LineHdr H = hdr[i];
@@ -71,6 +72,7 @@ __global__ void order_keys_kernel(GridDev g, const LineHdr *__restrict__ hdr, in
 __global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const unsigned *__restrict__ keys, int m,
                                                                    int shift, int *__restrict__ counts, int nb)
 {
+    chain_begin();
     __shared__ int hist[kDigits];
     for (int d = threadIdx.x; d < kDigits; d += kSortThreads) hist[d] = 0;
     __syncthreads();
@@ -112,6 +114,7 @@ __device__ __forceinline__ int block_scan(int v, int *wsum, int &total)
 __global__ void __launch_bounds__(kSortThreads) radix_scan_kernel(int *__restrict__ counts, int *__restrict__ totals,
                                                                   int nb)
 {
+    chain_begin();
     __shared__ int wsum[kSortWarps];
     int *row = counts + (size_t)blockIdx.x * nb;
     int run = 0;
@@ -137,6 +140,7 @@ __global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const unsig
                                                                      const int *__restrict__ counts,
                                                                      const int *__restrict__ totals, int nb)
 {
+    chain_begin();
     __shared__ int wcnt[kSortWarps][kDigits];
     __shared__ int wsum[kSortWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -230,16 +234,16 @@ cudaError_t launch_line_order(const GridDev &g, const LinesDev &L, const LineHdr
     int D = (int)std::lround(std::sqrt((double)m / (32.0 * std::sqrt(2.0))));
     D = D < 1 ? 1 : (D > 1023 ? 1023 : D);
     OrderArea o = carve(area, m);
-    order_keys_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(g, hdr, mi, D, o.keysA, o.valsB);
+    launch_chained(order_keys_kernel, (unsigned)((m + 255) / 256), 256, 0, s, g, hdr, mi, D, o.keysA, o.valsB);
     cudaError_t e = cudaGetLastError();
     // an odd number of passes from valsB: the order ends in o.order
     unsigned *ka = o.keysA, *kb = o.keysB;
     int *va = o.valsB, *vb = o.order;
     for (int pass = 0; pass < kPasses && e == cudaSuccess; ++pass) {
         const int shift = kDigitBits * pass;
-        radix_count_kernel<<<nb, kSortThreads, 0, s>>>(ka, mi, shift, o.counts, nb);
-        radix_scan_kernel<<<kDigits, kSortThreads, 0, s>>>(o.counts, o.totals, nb);
-        radix_scatter_kernel<<<nb, kSortThreads, 0, s>>>(ka, va, kb, vb, mi, shift, o.counts, o.totals, nb);
+        launch_chained(radix_count_kernel, nb, kSortThreads, 0, s, ka, mi, shift, o.counts, nb);
+        launch_chained(radix_scan_kernel, kDigits, kSortThreads, 0, s, o.counts, o.totals, nb);
+        launch_chained(radix_scatter_kernel, nb, kSortThreads, 0, s, ka, va, kb, vb, mi, shift, o.counts, o.totals, nb);
         e = cudaGetLastError();
         unsigned *tk = ka; ka = kb; kb = tk;
         int *tv = va; va = vb; vb = tv;

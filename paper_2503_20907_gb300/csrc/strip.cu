@@ -224,6 +224,7 @@ template <int KIND>
 __global__ void row_record_kernel(const LineHdr *__restrict__ hdr, const float *__restrict__ center, int per_table,
                                   int64_t m, longlong2 *__restrict__ out)
 {
+    chain_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     const LineHdr H = hdr[i];
@@ -984,6 +985,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
 template <int KIND, bool ADJ, int FM = kFmAll>
 __global__ void __launch_bounds__(kThreads, kCtas) strip_kernel(const __grid_constant__ StripArgs A, unsigned *defer)
 {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     const bool ran = strip_chunk<KIND, ADJ, FM>(smem, A, (int)blockIdx.x);
     if (FM == kFmFixed && !ran && threadIdx.x == 0) defer[2 + atomicAdd(defer, 1u)] = blockIdx.x;
@@ -994,6 +996,7 @@ __global__ void __launch_bounds__(kThreads, kCtas) strip_kernel(const __grid_con
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, kCtas) strip_float_kernel(const __grid_constant__ StripArgs A, unsigned *defer)
 {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned cur;
     const unsigned n = defer[0];
@@ -1037,6 +1040,7 @@ __global__ void __launch_bounds__(kThreads, kCtas)
 strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total, unsigned long long *counter,
                    long long *defer, unsigned long long *defer_n)
 {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long cur;
     for (;;) {
@@ -1057,6 +1061,7 @@ __global__ void __launch_bounds__(kThreads, kCtas)
 strip_queue_float_kernel(const StripJob *__restrict__ jobs, int njobs, const long long *__restrict__ defer,
                          const unsigned long long *__restrict__ defer_n, unsigned long long *counter)
 {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long cur;
     const unsigned long long n = *defer_n;
@@ -1084,19 +1089,18 @@ cudaError_t launch_queue_t(bool adj, const StripJob *jobs, int njobs, int64_t to
             e = cudaFuncSetAttribute(strip_queue_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemBytes);
         if (e != cudaSuccess) return e;
-        strip_queue_kernel<KIND, true><<<(unsigned)grid, kThreads, kSmemBytes, s>>>(jobs, njobs, (long long)total,
+        launch_chained(strip_queue_kernel<KIND, true>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs, (long long)total,
                                                                                   counter, defer, counter + 1);
         e = cudaGetLastError();
         // the deferred chunks are few (non-finite or extreme sinogram values): a small grid
         if (e == cudaSuccess)
-            strip_queue_float_kernel<KIND><<<(unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s>>>(
-                jobs, njobs, defer, counter + 1, counter + 2);
+            launch_chained(strip_queue_float_kernel<KIND>, (unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s, jobs, njobs, defer, counter + 1, counter + 2);
         return e == cudaSuccess ? cudaGetLastError() : e;
     }
     e = cudaFuncSetAttribute(strip_queue_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    strip_queue_kernel<KIND, false><<<(unsigned)grid, kThreads, kSmemBytes, s>>>(jobs, njobs, (long long)total, counter,
+    launch_chained(strip_queue_kernel<KIND, false>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs, (long long)total, counter,
                                                                                nullptr, nullptr);
     return cudaGetLastError();
 }
@@ -1106,6 +1110,7 @@ cudaError_t launch_queue_t(bool adj, const StripJob *jobs, int njobs, int64_t to
 __global__ void stage_images_kernel(const float *__restrict__ in, float *__restrict__ plain, float *__restrict__ trans,
                                     int nx, int ny)
 {
+    chain_begin();
     __shared__ float tile[32][33];
     const int bx = blockIdx.x * 32, by = blockIdx.y * 32, ldx = image_ld(nx), ldy = image_ld(ny);
     for (int y = threadIdx.y; y < 32; y += 8) {
@@ -1125,6 +1130,7 @@ __global__ void stage_images_kernel(const float *__restrict__ in, float *__restr
 __global__ void join_images_kernel(const float *__restrict__ plain, const float *__restrict__ trans, float *__restrict__ out,
                                    int nx, int ny)
 {
+    chain_begin();
     __shared__ float tile[32][33];
     const int bi = blockIdx.x * 32, bj = blockIdx.y * 32, ldx = image_ld(nx), ldy = image_ld(ny);
     for (int y = threadIdx.y; y < 32; y += 8) {
@@ -1169,14 +1175,14 @@ StripArgs make_args(const GridDev &g, const LinesDev &L, const LineHdr *hdr, con
 cudaError_t launch_images(const StripArgs &A, const float *img, cudaStream_t s)
 {
     const dim3 tb(32, 8), tg((A.g.nx + 31) / 32, (image_ld(A.g.ny) + 31) / 32);
-    stage_images_kernel<<<tg, tb, 0, s>>>(img, A.src[0] == img ? nullptr : A.dst[0], A.dst[1], A.g.nx, A.g.ny);
+    launch_chained(stage_images_kernel, tg, tb, 0, s, img, A.src[0] == img ? nullptr : A.dst[0], A.dst[1], A.g.nx, A.g.ny);
     return cudaGetLastError();
 }
 
 cudaError_t launch_join(const StripArgs &A, float *out, cudaStream_t s)
 {
     const dim3 tb(32, 8), tg((A.g.nx + 31) / 32, (A.g.ny + 31) / 32);
-    join_images_kernel<<<tg, tb, 0, s>>>(A.dst[0], A.dst[1], out, A.g.nx, A.g.ny);
+    launch_chained(join_images_kernel, tg, tb, 0, s, A.dst[0], A.dst[1], out, A.g.nx, A.g.ny);
     return cudaGetLastError();
 }
 
@@ -1188,7 +1194,7 @@ cudaError_t launch_strip_t(const StripArgs &A, bool adj, unsigned *defer, cudaSt
     if (!adj) {
         e = cudaFuncSetAttribute(strip_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (e != cudaSuccess) return e;
-        strip_kernel<KIND, false><<<grid, kThreads, kSmemBytes, s>>>(A, nullptr);
+        launch_chained(strip_kernel<KIND, false>, grid, kThreads, kSmemBytes, s, A, nullptr);
         return cudaGetLastError();
     }
     // fixed-point chunks, then (a small second launch) the chunks they
@@ -1200,10 +1206,10 @@ cudaError_t launch_strip_t(const StripArgs &A, bool adj, unsigned *defer, cudaSt
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    strip_kernel<KIND, true, kFmFixed><<<grid, kThreads, kSmemBytes, s>>>(A, defer);
+    launch_chained(strip_kernel<KIND, true, kFmFixed>, grid, kThreads, kSmemBytes, s, A, defer);
     e = cudaGetLastError();
     if (e == cudaSuccess)
-        strip_float_kernel<KIND><<<grid < (unsigned)sms ? grid : (unsigned)sms, kThreads, kSmemBytes, s>>>(A, defer);
+        launch_chained(strip_float_kernel<KIND>, grid < (unsigned)sms ? grid : (unsigned)sms, kThreads, kSmemBytes, s, A, defer);
     return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
@@ -1304,10 +1310,10 @@ cudaError_t launch_row_records(const GridDev &g, const LinesDev &L, const LineHd
     const unsigned nb = (unsigned)((L.m + 255) / 256);
     const int per = L.kind == SP_LINES_PARALLEL ? L.n_det : 1;
     switch (strip_kind(g)) {
-    case 1: row_record_kernel<1><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
-    case 2: row_record_kernel<2><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
-    case 3: row_record_kernel<3><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
-    case kKindBox: row_record_kernel<kKindBox><<<nb, 256, 0, s>>>(hdr, center, per, L.m, rec); break;
+    case 1: launch_chained(row_record_kernel<1>, nb, 256, 0, s, hdr, center, per, L.m, rec); break;
+    case 2: launch_chained(row_record_kernel<2>, nb, 256, 0, s, hdr, center, per, L.m, rec); break;
+    case 3: launch_chained(row_record_kernel<3>, nb, 256, 0, s, hdr, center, per, L.m, rec); break;
+    case kKindBox: launch_chained(row_record_kernel<kKindBox>, nb, 256, 0, s, hdr, center, per, L.m, rec); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
