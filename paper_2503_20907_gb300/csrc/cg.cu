@@ -43,8 +43,8 @@ __device__ __forceinline__ double block_sum(double v, double *sh)
 
 // <a, a> in FP64 (partial sums per block, then the last block to finish adds
 // them in block order and updates the CG scalars according to `role`).
-__global__ void __launch_bounds__(kDotThreads) dot_kernel(const float *__restrict__ a, int64_t n,
-                                                          double *__restrict__ partial, CgScalars *sc,
+__global__ void __launch_bounds__(kDotThreads) dot_kernel(const float *a, int64_t n,
+                                                          double *partial, CgScalars *sc,
                                                           int role, double *hist, int k)
 {
     chain_begin();
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kDotThreads) dot_kernel(const float *__restric
 }
 
 // r = b - q
-__global__ void residual_kernel(const float *__restrict__ b, const float *__restrict__ q, float *__restrict__ r,
+__global__ void residual_kernel(const float *b, const float *q, float *r,
                                 int64_t m)
 {
     chain_begin();
@@ -95,9 +95,9 @@ __global__ void residual_kernel(const float *__restrict__ b, const float *__rest
 }
 
 // x += alpha p (n values), r -= alpha q (m values)
-__global__ void update_xr_kernel(float *__restrict__ x, const float *__restrict__ p, int64_t n,
-                                 float *__restrict__ r, const float *__restrict__ q, int64_t m,
-                                 const CgScalars *__restrict__ sc)
+__global__ void update_xr_kernel(float *x, const float *p, int64_t n,
+                                 float *r, const float *q, int64_t m,
+                                 const CgScalars *sc)
 {
     chain_begin();
     const float alpha = (float)sc->alpha;
@@ -109,8 +109,8 @@ __global__ void update_xr_kernel(float *__restrict__ x, const float *__restrict_
 }
 
 // p = s + beta p
-__global__ void update_p_kernel(float *__restrict__ p, const float *__restrict__ s, int64_t n,
-                                const CgScalars *__restrict__ sc)
+__global__ void update_p_kernel(float *p, const float *s, int64_t n,
+                                const CgScalars *sc)
 {
     chain_begin();
     const float beta = (float)sc->beta;

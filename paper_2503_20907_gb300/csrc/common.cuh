@@ -113,9 +113,11 @@ static_assert(sizeof(LineHdr) == 64, "LineHdr layout");
 // launched by launch_chained may be set up on the device while the kernel before
 // it in the stream still runs its last blocks; chain_begin() waits until that
 // one has completed and its results are visible, so nothing else changes for
-// either (no kernel touches global memory before it).  That saves 1 to 2 us
-// between two kernels of a stream: 1230 -> 1153 us for the 51 launches of four
-// CGLS steps at 256 x 256, 51 -> 45 us for the eight of two one-shot calls.
+// either (no kernel touches global memory before it).  Such kernels read memory
+// by plain loads: __restrict__ parameters and __ldg make loads read-only, which
+// the compiler may move above the wait.  That saves 1 to 2 us between two
+// kernels of a stream: 1230 -> 1153 us for the 51 launches of four CGLS steps at
+// 256 x 256, 51 -> 45 us for the eight of two one-shot calls.
 __device__ __forceinline__ void chain_begin()
 {
     asm volatile("griddepcontrol.launch_dependents;");

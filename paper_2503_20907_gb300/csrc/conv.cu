@@ -146,11 +146,11 @@ __device__ __forceinline__ bool tap_at(const EdgeArgs &a, INNER, int tap, int h,
 // layer (W [9][32], sign = -1).  S: bf16 or float; ROUND: s rounded to BF16 and
 // kept so in sb.  Results BF16 or FP32; relu clamps, gate masks where gate <= 0.
 template <typename S, bool ROUND, bool GRAD, typename OUT>
-__global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, const S *__restrict__ s,
-                                                                  const bf16 *__restrict__ wt,
-                                                                  const float *__restrict__ bias,
-                                                                  const bf16 *__restrict__ gate, int relu,
-                                                                  OUT *__restrict__ y, bf16 *__restrict__ sb, int vec)
+__global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, const S *s,
+                                                                  const bf16 *wt,
+                                                                  const float *bias,
+                                                                  const bf16 *gate, int relu,
+                                                                  OUT *y, bf16 *sb, int vec)
 {
     chain_begin();
     const int c0 = (threadIdx.x & 3) * 8;
@@ -205,11 +205,11 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 // layer (W [32][9], sign = -1; rounded to BF16 when `round`).  add (may be
 // NULL) is added to the result.
 template <typename V, bool GRAD>
-__global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, const V *__restrict__ v,
-                                                                 const bf16 *__restrict__ wt,
-                                                                 const float *__restrict__ bias, int relu, int round,
-                                                                 const bf16 *__restrict__ gate,
-                                                                 const float *__restrict__ add, float *__restrict__ y,
+__global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, const V *v,
+                                                                 const bf16 *wt,
+                                                                 const float *bias, int relu, int round,
+                                                                 const bf16 *gate,
+                                                                 const float *add, float *y,
                                                                  int vec)
 {
     chain_begin();
@@ -249,9 +249,9 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, con
 // s = g, sign = -1 (the pixel of g that sees x[p] through the tap), dw [9][32],
 // dbias = sum s.  One partial sum per block is added to dw and dbias.
 template <typename V, typename S, bool OUT1>
-__global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, const V *__restrict__ v,
-                                                                  const S *__restrict__ s, float *__restrict__ dw,
-                                                                  float *__restrict__ db, int vec)
+__global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, const V *v,
+                                                                  const S *s, float *dw,
+                                                                  float *db, int vec)
 {
     chain_begin();
     __shared__ float part[9 * kC + kC];
@@ -313,7 +313,7 @@ unsigned edge_blocks(int B, int H, int W, int per_sm)
 
 // ------------------------------------------------------------------ weights
 // W'[i, 2-ky, 2-kx, o] = W[o, ky, kx, i] (the input gradient as a forward convolution)
-__global__ void flip_weights_kernel(const bf16 *__restrict__ w, bf16 *__restrict__ wf, int cin, int cout)
+__global__ void flip_weights_kernel(const bf16 *w, bf16 *wf, int cin, int cout)
 {
     chain_begin();
     const int n = cout * 9 * cin;
@@ -340,7 +340,7 @@ __host__ __device__ constexpr size_t pack_at(int n, int k)   // first element of
     return k == 0 ? 0 : (size_t)kPackEdge + (size_t)(k - 1) * kPackInner;
 }
 
-__global__ void pack_weights_kernel(NetWeights N, bf16 *__restrict__ pack)
+__global__ void pack_weights_kernel(NetWeights N, bf16 *pack)
 {
     chain_begin();
     const int k = blockIdx.y;
@@ -524,7 +524,7 @@ constexpr int kTileRow5 = 4 * kTileGroup5;
 // image) at dst and, unless NULL, again at copy: 16 bytes per copy, FP32 input
 // rounded to BF16 on the way.
 template <typename IN>
-__device__ __forceinline__ void stage_row(const ChainArgs &a, const IN *__restrict__ x, int64_t b, int h, int w,
+__device__ __forceinline__ void stage_row(const ChainArgs &a, const IN *x, int64_t b, int h, int w,
                                           int pixels, int group, unsigned char *dst, unsigned char *copy)
 {
     const bool rin = (unsigned)h < (unsigned)a.H;
@@ -587,8 +587,8 @@ struct ConvArgs {
 // wait is bounded; when MMAs do not complete, the rest of the unit is NaN and
 // the block still frees its tensor memory.
 template <typename IN, typename OUT>
-__global__ void __launch_bounds__(kThreads5) conv32_tc05_kernel(ChainArgs ch, ConvArgs a, const IN *__restrict__ x,
-                                                          OUT *__restrict__ y)
+__global__ void __launch_bounds__(kThreads5) conv32_tc05_kernel(ChainArgs ch, ConvArgs a, const IN *x,
+                                                          OUT *y)
 {
     chain_begin();
     extern __shared__ __align__(128) unsigned char sm5[];
@@ -720,9 +720,9 @@ constexpr uint32_t kWgCols5 = 128;                     // 3 x 32 columns, as a p
 constexpr int kWgCtas5 = 2;                            // CTAs per SM
 
 template <typename G>
-__global__ void __launch_bounds__(kThreads5) conv32_wgrad_tc05_kernel(ChainArgs ch, const bf16 *__restrict__ x,
-                                                                const G *__restrict__ g, float *__restrict__ dw,
-                                                                float *__restrict__ db)
+__global__ void __launch_bounds__(kThreads5) conv32_wgrad_tc05_kernel(ChainArgs ch, const bf16 *x,
+                                                                const G *g, float *dw,
+                                                                float *db)
 {
     chain_begin();
     extern __shared__ __align__(128) unsigned char smw[];

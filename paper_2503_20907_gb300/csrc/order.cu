@@ -39,8 +39,8 @@ constexpr unsigned kKeyEmpty = (1u << (kDigitBits * kPasses)) - 1;   // above ev
 
 size_t al(size_t v) { return (v + 255) & ~(size_t)255; }
 
-__global__ void order_keys_kernel(GridDev g, const LineHdr *__restrict__ hdr, int m, int D,
-                                  unsigned *__restrict__ keys, int *__restrict__ vals)
+__global__ void order_keys_kernel(GridDev g, const LineHdr *hdr, int m, int D,
+                                  unsigned *keys, int *vals)
 {
     chain_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -69,8 +69,8 @@ __global__ void order_keys_kernel(GridDev g, const LineHdr *__restrict__ hdr, in
 }
 
 // counts[d * nb + b] = keys of block b whose digit is d.
-__global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const unsigned *__restrict__ keys, int m,
-                                                                   int shift, int *__restrict__ counts, int nb)
+__global__ void __launch_bounds__(kSortThreads) radix_count_kernel(const unsigned *keys, int m,
+                                                                   int shift, int *counts, int nb)
 {
     chain_begin();
     __shared__ int hist[kDigits];
@@ -111,7 +111,7 @@ __device__ __forceinline__ int block_scan(int v, int *wsum, int &total)
 
 // Block d: exclusive prefix sum of the counts of digit d over the blocks, in
 // place, and their total.
-__global__ void __launch_bounds__(kSortThreads) radix_scan_kernel(int *__restrict__ counts, int *__restrict__ totals,
+__global__ void __launch_bounds__(kSortThreads) radix_scan_kernel(int *counts, int *totals,
                                                                   int nb)
 {
     chain_begin();
@@ -133,12 +133,12 @@ __global__ void __launch_bounds__(kSortThreads) radix_scan_kernel(int *__restric
 // consecutive keys; a key's place among equal digits is (earlier blocks, from
 // the scanned counts) + (earlier warps of the block) + (earlier rounds of its
 // warp) + (lower lanes of its round).
-__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const unsigned *__restrict__ kin,
-                                                                     const int *__restrict__ vin,
-                                                                     unsigned *__restrict__ kout,
-                                                                     int *__restrict__ vout, int m, int shift,
-                                                                     const int *__restrict__ counts,
-                                                                     const int *__restrict__ totals, int nb)
+__global__ void __launch_bounds__(kSortThreads) radix_scatter_kernel(const unsigned *kin,
+                                                                     const int *vin,
+                                                                     unsigned *kout,
+                                                                     int *vout, int m, int shift,
+                                                                     const int *counts,
+                                                                     const int *totals, int nb)
 {
     chain_begin();
     __shared__ int wcnt[kSortWarps][kDigits];

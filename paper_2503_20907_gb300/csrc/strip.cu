@@ -221,8 +221,8 @@ __device__ __forceinline__ void row_stepping(const LineHdr &H, float b, long lon
 // The row records a plan keeps: every line's position in row 0 and its step,
 // from which all its rows follow (degree >= 1).
 template <int KIND>
-__global__ void row_record_kernel(const LineHdr *__restrict__ hdr, const float *__restrict__ center, int per_table,
-                                  int64_t m, longlong2 *__restrict__ out)
+__global__ void row_record_kernel(const LineHdr *hdr, const float *center, int per_table,
+                                  int64_t m, longlong2 *out)
 {
     chain_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -503,7 +503,7 @@ __device__ __forceinline__ void walk_blocks(const Rows &R, const LaneLine &ln, c
 // footprint is a rectangle with edges on nodes, each taking the midpoint value
 // on both sides (so a row has one more candidate): straight from or to global
 // memory.  Such lines occur only at views exactly along an axis.
-__device__ __noinline__ float axis_row0(const LineHdr &H, int r, const float *__restrict__ src, float *dst, int Nq, int ld,
+__device__ __noinline__ float axis_row0(const LineHdr &H, int r, const float *src, float *dst, int Nq, int ld,
                                         float hp, bool adj)
 {
     const float inv_a = 1.0f / H.a;
@@ -514,7 +514,7 @@ __device__ __noinline__ float axis_row0(const LineHdr &H, int r, const float *__
         if ((unsigned)q >= (unsigned)Nq) continue;
         const float phi = e.tie ? 0.5f * inv_a : inv_a;
         if (adj) atomicAdd(dst + (size_t)r * ld + q, hp * phi);
-        else acc = __fmaf_rn(__ldg(src + (size_t)r * ld + q), phi, acc);
+        else acc = __fmaf_rn(src[(size_t)r * ld + q], phi, acc);
     }
     return acc;
 }
@@ -654,7 +654,7 @@ __device__ __forceinline__ int run_lead(int n) { return KIND >= 1 && KIND <= 3 ?
 // coefficient there must not enter.
 template <int DEG>
 __device__ __noinline__ float exact_line(const LineHdr &H, const float *rec, long long Y0, long long step, float w_sup,
-                                         const float *__restrict__ src, int Nq, int ld)
+                                         const float *src, int Nq, int ld)
 {
     constexpr int m = DEG + 1, NC = 2 * DEG + 2;
     constexpr float c = m % 2 == 0 ? 0.5f : 0.f;
@@ -680,7 +680,7 @@ __device__ __noinline__ float exact_line(const LineHdr &H, const float *rec, lon
                 const float *J = rec + kCenterJump + 8 * k + 2 * j;
                 phi = __fmaf_rn(same ? J[0] + J[1] : J[0] - J[1], z[k], phi);
             }
-            pair_add(hi, lo, __ldg(src + (size_t)r * ld + q) * phi);
+            pair_add(hi, lo, src[(size_t)r * ld + q] * phi);
         }
     }
     return isfinite(lo) ? hi + lo : hi;
@@ -770,7 +770,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
     // and lane l's line in every warp (directions: one per view for parallel
     // beams, else one per line)
     const int64_t line0 = (int64_t)v * nd + j0;
-    const int my_line = lane < nl ? (L.order ? __ldg(L.order + line0 + lane) : (int)(line0 + lane)) : 0;
+    const int my_line = lane < nl ? (L.order ? L.order[line0 + lane] : (int)(line0 + lane)) : 0;
     const bool shared_dir = L.kind == SP_LINES_PARALLEL;
 
     // The adjoint's values, and the chunk's fixed-point scale (a power of two;
@@ -800,11 +800,11 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
         const int src = __shfl_sync(0xffffffffu, my_line, (threadIdx.x >> 2) & 31);
         if ((int)threadIdx.x < nl * 4)
             reinterpret_cast<int4 *>(hdr_s)[threadIdx.x] =
-                __ldg(reinterpret_cast<const int4 *>(A.hdr + src) + (threadIdx.x & 3));
+                reinterpret_cast<const int4 *>(A.hdr + src)[threadIdx.x & 3];
     }
     float my_b = 0.f;
     if constexpr (kCenter) {
-        my_b = __ldg(A.center + (shared_dir ? (int64_t)v : (int64_t)my_line) * kCenterFloats + kCenterB);
+        my_b = A.center[(shared_dir ? (int64_t)v : (int64_t)my_line) * kCenterFloats + kCenterB];
         const int nt = shared_dir ? 1 : nl;
         constexpr int kCh = kCenterFloats / 4;
         const unsigned ba = (unsigned)__cvta_generic_to_shared(rec_s);
@@ -827,7 +827,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
         mine_vert = (H.flags & kVert) != 0;
         if (mine) {
             if (A.rec) {
-                const longlong2 t = __ldg(A.rec + my_line);
+                const longlong2 t = A.rec[my_line];
                 my_W = t.x;
                 my_step = t.y;
             } else {
@@ -1024,7 +1024,7 @@ struct StripJob {
 // (count *defer_n) for strip_queue_float_kernel, as the per-instance adjoint
 // does with its second launch.  (One kernel per degree: a kernel holding all
 // three degrees spilled over a hundred bytes per thread.)
-__device__ __forceinline__ const StripJob *queue_job(const StripJob *__restrict__ jobs, int njobs, long long c)
+__device__ __forceinline__ const StripJob *queue_job(const StripJob *jobs, int njobs, long long c)
 {
     int lo = 0, hi = njobs - 1;   // last job whose first chunk is <= c
     while (lo < hi) {
@@ -1037,7 +1037,7 @@ __device__ __forceinline__ const StripJob *queue_job(const StripJob *__restrict_
 
 template <int KIND, bool ADJ>
 __global__ void __launch_bounds__(kThreads, kCtas)
-strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total, unsigned long long *counter,
+strip_queue_kernel(const StripJob *jobs, int njobs, long long total, unsigned long long *counter,
                    long long *defer, unsigned long long *defer_n)
 {
     chain_begin();
@@ -1058,8 +1058,8 @@ strip_queue_kernel(const StripJob *__restrict__ jobs, int njobs, long long total
 // The deferred adjoint chunks (float strip accumulators), persistent likewise.
 template <int KIND>
 __global__ void __launch_bounds__(kThreads, kCtas)
-strip_queue_float_kernel(const StripJob *__restrict__ jobs, int njobs, const long long *__restrict__ defer,
-                         const unsigned long long *__restrict__ defer_n, unsigned long long *counter)
+strip_queue_float_kernel(const StripJob *jobs, int njobs, const long long *defer,
+                         const unsigned long long *defer_n, unsigned long long *counter)
 {
     chain_begin();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1089,25 +1089,26 @@ cudaError_t launch_queue_t(bool adj, const StripJob *jobs, int njobs, int64_t to
             e = cudaFuncSetAttribute(strip_queue_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemBytes);
         if (e != cudaSuccess) return e;
-        launch_chained(strip_queue_kernel<KIND, true>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs, (long long)total,
-                                                                                  counter, defer, counter + 1);
+        launch_chained(strip_queue_kernel<KIND, true>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs,
+                       (long long)total, counter, defer, counter + 1);
         e = cudaGetLastError();
         // the deferred chunks are few (non-finite or extreme sinogram values): a small grid
         if (e == cudaSuccess)
-            launch_chained(strip_queue_float_kernel<KIND>, (unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s, jobs, njobs, defer, counter + 1, counter + 2);
+            launch_chained(strip_queue_float_kernel<KIND>, (unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s,
+                           jobs, njobs, defer, counter + 1, counter + 2);
         return e == cudaSuccess ? cudaGetLastError() : e;
     }
     e = cudaFuncSetAttribute(strip_queue_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    launch_chained(strip_queue_kernel<KIND, false>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs, (long long)total, counter,
-                                                                               nullptr, nullptr);
+    launch_chained(strip_queue_kernel<KIND, false>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs, (long long)total,
+                   counter, nullptr, nullptr);
     return cudaGetLastError();
 }
 
 // The forward's images: the coefficients transposed, and (plain not NULL) as
 // stored, with rows padded by zeros to a multiple of 4.
-__global__ void stage_images_kernel(const float *__restrict__ in, float *__restrict__ plain, float *__restrict__ trans,
+__global__ void stage_images_kernel(const float *in, float *plain, float *trans,
                                     int nx, int ny)
 {
     chain_begin();
@@ -1127,7 +1128,7 @@ __global__ void stage_images_kernel(const float *__restrict__ in, float *__restr
 }
 
 // out[j][i] = plain[j][i] + trans[i][j] (padded rows in, plain rows out)
-__global__ void join_images_kernel(const float *__restrict__ plain, const float *__restrict__ trans, float *__restrict__ out,
+__global__ void join_images_kernel(const float *plain, const float *trans, float *out,
                                    int nx, int ny)
 {
     chain_begin();
