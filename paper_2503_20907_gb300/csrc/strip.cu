@@ -269,6 +269,8 @@ struct SplineRows {
     static constexpr int m = DEG + 1, NC = 2 * DEG + 2, NH = NC / 2;
     static constexpr bool kMid = m % 2 == 1;       // a candidate at v itself
     static constexpr int kKnots = DEG == 1 ? 1 : 2;
+    // the inner knots leave the fourth pair (degree 2: counting the middle one) alone
+    static constexpr __device__ int first_knot(int j) { return j + (kMid ? 1 : 0) == 3 ? 1 : 0; }
     f2 C[J][NH];            // (even, odd) coefficients, by powers of v^2
     f2 K[J][kKnots];        // jumps: half their sum and half their difference
     float cm[NH], km[kKnots];   // the middle candidate
@@ -289,7 +291,7 @@ struct SplineRows {
                 if (k + 1 < NH) C[j][k + 1] = FIX ? f2mul(t.y, sc2) : t.y;
             }
 #pragma unroll
-            for (int q = 0; q < kKnots; ++q) {
+            for (int q = first_knot(j); q < kKnots; ++q) {
                 const f2 t = *reinterpret_cast<const f2 *>(ln.rec + kCenterJump + 8 * q + 2 * (j + (kMid ? 1 : 0)));
                 K[j][q] = FIX ? f2mul(t, sc2) : t;
             }
@@ -341,7 +343,7 @@ struct SplineRows {
             // larger columns takes their sum, its mirror image the difference
             f2 eo = f2pack(e, v * o);
 #pragma unroll
-            for (int q = 0; q < kKnots; ++q) eo = f2fma(zz[q], K[j][q], eo);
+            for (int q = first_knot(j); q < kKnots; ++q) eo = f2fma(zz[q], K[j][q], eo);
             f2unpack(eo, e, o);
             put(sp, J + (kMid ? 1 : 0) + j, J - 1 - j, __fadd_rn(e, o), __fsub_rn(e, o), ca[j], v, acc);
         }
