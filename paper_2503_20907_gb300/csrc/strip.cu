@@ -65,8 +65,8 @@
 // integer reduction costs about what a plain shared store does on this GPU,
 // a float one four to six times more.  Each chunk takes the power of two S
 // that puts its largest contribution h |p| phi (phi <= sqrt(2) < 1.5 for
-// every basis here) at 2^21 or less; a pair then adds round(S h p phi) to its
-// node, at most 2^26 in magnitude after 32 lines, and the flush adds the
+// every basis here) at 2^22 or less; a pair then adds round(S h p phi) to its
+// node, at most 2^27 in magnitude after 32 lines, and the flush adds the
 // sums times 1/S (exact) to the image.  Adding M = 1.5 2^23 does the rounding:
 // the result lies in [2^23, 2^24) where floats are the integers, and its bits
 // minus M's bits are round(S h p phi).  Per pair that is an error of about
@@ -170,7 +170,7 @@ constexpr float kFixMagic = 12582912.0f;
 constexpr int kFixMagicBits = 0x4B400000;
 // Largest contribution of a chunk after scaling, and the bound on phi used
 // to choose the scale.
-constexpr float kFixMax = 2097152.0f;   // 2^21
+constexpr float kFixMax = 4194304.0f;   // 2^22
 constexpr float kPhiBound = 1.5f;
 
 // Which chunks an adjoint call runs (strip_chunk's FM).
