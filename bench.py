@@ -34,11 +34,11 @@ METRIC = "Mrays/s fwd+adj at 512² cubic fan-beam (% roofline); learned-vs-cold 
 UNIT = "Mrays/s"
 WORKLOAD = "fan512_cubic"
 FP32_LANES_PER_SM = 128
-KERNELS_PER_STEP = 6   # line setup with tables (one fused kernel), transpose + forward strip, adjoint strip (fixed-point chunks, then float chunks) + transposed add
+KERNELS_PER_STEP = 6   # line setup with centre records, image copies + forward strip, adjoint strip (fixed-point chunks, then float chunks) + join of the images
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum, one ncu
 # capture of these kernel versions on this workload); set to None whenever the
 # kernels change until they are captured again.
-TRAFFIC = {}   # cleared: the strip kernels changed
+TRAFFIC = {"fan512_cubic": {"spline_fwd": 153478400, "spline_adj": 154919424}}
 CG_ITERS = 100
 CG_MAX_ITERS = 400   # cap of the run to the tolerance
 CG_TOL = 1e-4

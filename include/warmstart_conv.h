@@ -1,6 +1,7 @@
 /*
  * warmstart_conv.h -- 3x3 convolution layers of the learned warm start for
- * the conjugate-gradient reconstruction (part of libspline_project.so).
+ * the conjugate-gradient reconstruction, and the whole network in one call
+ * (part of libspline_project.so).
  *
  * No counterpart in the paper: the network maps the backprojection A^T y to
  * an initial guess of the coefficients (it does not change the projector).
@@ -25,8 +26,8 @@ extern "C" {
 
 /* Forward: y BF16 [B][H][W][cout] (FP32 [B][H][W] when cout = 1); relu != 0
  * clamps at 0 after the bias.  32 -> 32 runs on the fifth-generation tensor
- * cores (tcgen05.mma, BF16 inputs, FP32 accumulators in tensor memory; 128
- * pixels of a row per CTA); 1 -> 32 and 32 -> 1 on the CUDA cores. */
+ * cores (tcgen05.mma, BF16 inputs, FP32 accumulators in tensor memory; tiles
+ * of 128 pixels of a row); 1 -> 32 and 32 -> 1 on the CUDA cores. */
 sp_status sp_conv3x3_fwd(int32_t B, int32_t H, int32_t W, int32_t cin, int32_t cout,
                          int32_t dilation, const void *x, const void *w, const float *bias, int32_t relu,
                          void *y, void *stream);

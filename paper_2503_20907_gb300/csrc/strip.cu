@@ -52,7 +52,7 @@
 // to accumulate; a row adds about 25 instructions (step, v, z, addresses).  The
 // lanes' strip accesses of one row fall on neighbouring columns, in distinct
 // banks.  Measured at the 512 x 512 cubic fan (552,960 lines), forward and
-// adjoint: 0.82 and 0.88 ms; one polynomial of 7 FMAs per candidate of a base
+// adjoint: 0.80 and 0.86 ms; one polynomial of 7 FMAs per candidate of a base
 // interval plus truncated powers with integer weights 1.19 and 1.28 ms; rows
 // sorted by interval, a lane per candidate and row, 2.18 and 2.35 ms.
 // Four CTAs of four warps per SM: while one CTA waits for its line records,

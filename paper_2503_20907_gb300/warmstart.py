@@ -4,10 +4,11 @@ A small CNN maps the scaled backprojection z = alpha A^T b of noisy data b to
 an initial guess x_0 = z + f(z) of the spline coefficients; CGLS
 (Plan.cgls) then starts from x_0 instead of 0, and plain CGLS from 0 stays
 the fallback.  f has six 3x3 convolution layers (1 -> 32, four 32 -> 32,
-32 -> 1; taps 1, 2, 4, 8, 16, 1 apart) with ReLU between them, BF16 weights and activations and FP32
-accumulation, all in this library's kernels (include/warmstart_conv.h):
-the forward of the inner layers on the tensor cores, the gradients on the
-CUDA cores.  Training data (phantom, sinogram, backprojection) come from the
+32 -> 1; taps 1, 2, 4, 8, 16, 1 apart) with ReLU between them, BF16 weights
+and activations and FP32 accumulation, all in this library's kernels
+(include/warmstart_conv.h), one call per direction: the inner layers and their
+gradients on the tensor cores, the first and the last on the CUDA cores.
+Training data (phantom, sinogram, backprojection) come from the
 library's projector.
 
     python -m paper_2503_20907_gb300.warmstart train --out weights.pt
