@@ -107,10 +107,11 @@ __device__ __forceinline__ float masked(float v, bool on)
 
 // This warp's pixel groups: group k is row k / gw (over B H), columns
 // 8 (k % gw) .. + 7.  Calls f(inner, row, h, w, in) with the lane's pixel; inner
-// (a type) says that all of the group's pixels and their taps are in the image:
-// without a test at each tap their loads are in flight together.
+// (a type) says that all of the group's pixels and their taps are in the image
+// and that vectors are aligned (vec): without a test at each tap their loads are
+// in flight together.
 template <typename F>
-__device__ __forceinline__ void for_pixels(const EdgeArgs &a, F f)
+__device__ __forceinline__ void for_pixels(const EdgeArgs &a, bool vec, F f)
 {
     // the position is carried along: no division per group
     const unsigned gw = (unsigned)(a.W + 7) / 8, step = gridDim.x * (kEdgeThreads / 32);
@@ -121,7 +122,7 @@ __device__ __forceinline__ void for_pixels(const EdgeArgs &a, F f)
     unsigned gi = first - (unsigned)row * gw, h = (unsigned)row % (unsigned)a.H;
     while (row < rows) {
         const int w0 = (int)gi * 8, w = w0 + (int)((threadIdx.x & 31) >> 2);
-        if ((int)h >= a.dil && (int)h + a.dil < a.H && w0 >= a.dil && w0 + 7 + a.dil < a.W)
+        if (vec && (int)h >= a.dil && (int)h + a.dil < a.H && w0 >= a.dil && w0 + 7 + a.dil < a.W)
             f(std::true_type{}, row, (int)h, w, true);
         else
             f(std::false_type{}, row, (int)h, w, w < a.W);
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 #pragma unroll
         for (int t = 0; t < 9; ++t) wr[t][k] = __bfloat162float(GRAD ? wt[t * kC + c0 + k] : wt[(c0 + k) * 9 + t]);
     }
-    for_pixels(a, [&](auto inner, int64_t row, int h, int w, bool in) {
+    for_pixels(a, vec, [&](auto inner, int64_t row, int h, int w, bool in) {
         if (!in) return;
         const int64_t p = row * a.W + w;
         float acc[8];
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
             for (int k = 0; k < 8; ++k) acc[k] = fmaxf(acc[k], 0.f);
         if (gate) {
             float gt[8];
-            load8(gate + p * kC + c0, vec, gt);
+            load8(gate + p * kC + c0, inner.value || vec, gt);
 #pragma unroll
             for (int k = 0; k < 8; ++k)
                 acc[k] = masked<OUT>(acc[k], gt[k] > 0.f);
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
         OUT *o = y + p * kC + c0;
         if constexpr (sizeof(OUT) == 2) {
             *reinterpret_cast<uint4 *>(o) = pack8(acc);
-        } else if (vec) {
+        } else if (inner.value || vec) {
             reinterpret_cast<float4 *>(o)[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
             reinterpret_cast<float4 *>(o)[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
         } else {
@@ -203,9 +204,12 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 // 32 channels in, one out: y[p] = bias + sum_tap sum_c v[p + off(tap), c] w
 // (32 -> 1 forward: W [9][32], sign = 1) or the input gradient of a 1 -> 32
 // layer (W [32][9], sign = -1; rounded to BF16 when `round`).  add (may be
-// NULL) is added to the result.
+// NULL) is added to the result.  The weights come from shared memory (four
+// addresses per warp, no conflicts), which leaves the registers to the loads in
+// flight and 32 warps per SM (72 registers of weights and 16 warps: a training pass
+// over 8 x 256 x 256 pixels took 693 instead of 673 us).
 template <typename V, bool GRAD>
-__global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, const V *v,
+__global__ void __launch_bounds__(kEdgeThreads, 4) edge_in32_kernel(EdgeArgs a, const V *v,
                                                                  const bf16 *wt,
                                                                  const float *bias, int relu, int round,
                                                                  const bf16 *gate,
@@ -214,24 +218,28 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_in32_kernel(EdgeArgs a, con
 {
     chain_begin();
     const int c0 = (threadIdx.x & 3) * 8;
-    float wr[9][8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-#pragma unroll
-        for (int t = 0; t < 9; ++t) wr[t][k] = __bfloat162float(GRAD ? wt[(c0 + k) * 9 + t] : wt[t * kC + c0 + k]);
+    __shared__ __align__(16) float ws[9 * kC];   // [tap][channel]
+    for (int i = threadIdx.x; i < 9 * kC; i += kEdgeThreads)
+        ws[i] = __bfloat162float(GRAD ? wt[(i % kC) * 9 + i / kC] : wt[i]);
+    __syncthreads();
     const float b0 = bias ? bias[0] : 0.f;
-    for_pixels(a, [&](auto inner, int64_t row, int h, int w, bool in) {
+    for_pixels(a, vec, [&](auto inner, int64_t row, int h, int w, bool in) {
         const int64_t p = row * a.W + w;
-        float acc = 0.f;
+        float acc = 0.f, acc1 = 0.f;
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             int64_t off;
             if (!in || !tap_at(a, inner, t, h, w, off)) continue;
-            float f[8];
-            load8(v + (p + off) * kC + c0, vec, f);
+            float f[8], wr[8];
+            load8(v + (p + off) * kC + c0, inner.value || vec, f);
+            load8(ws + t * kC + c0, true, wr);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc = __fmaf_rn(f[k], wr[t][k], acc);
+            for (int k = 0; k < 8; k += 2) {
+                acc = __fmaf_rn(f[k], wr[k], acc);
+                acc1 = __fmaf_rn(f[k + 1], wr[k + 1], acc1);
+            }
         }
+        acc += acc1;
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         acc += __shfl_xor_sync(0xffffffffu, acc, 2);
         if (in && (threadIdx.x & 3) == 0) {
@@ -265,11 +273,11 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, co
 #pragma unroll
         for (int t = 0; t < 9; ++t) acc[t][k] = 0.f;
     }
-    for_pixels(a, [&](auto inner, int64_t row, int h, int w, bool in) {
+    for_pixels(a, vec, [&](auto inner, int64_t row, int h, int w, bool in) {
         if (!in) return;
         const int64_t p = row * a.W + w;
         float f[8];
-        load8(v + p * kC + c0, vec, f);
+        load8(v + p * kC + c0, inner.value || vec, f);
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             int64_t off;
