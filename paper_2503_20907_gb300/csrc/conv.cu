@@ -33,14 +33,17 @@ constexpr int kMaxDil = 16;         // largest dilation of the taps
 
 // ------------------------------------------------------------------ edge layers
 // Four lanes hold a pixel's 32 channels, eight each (an octet: 16 bytes of
-// BF16); a warp takes eight consecutive pixels of an image row at a time.  What
-// an octet needs of the nine taps (weights, or partial weight gradients) stays
-// in 72 registers (16 warps per SM).  The floor is 5 us of HBM (64 bytes per
-// pixel) and 4 us of FMAs (288 per pixel) at 8 x 256 x 256 pixels; measured are
-// 28 us out, 52 us in and 28 and 32 us for the weight gradients, with the issue
-// slots 33 to 50 % busy and the rest load latency.  One thread per pixel or per
-// output instead (2-byte loads, 64 bytes apart, or a block per 16 rows) took 54
-// to 267 us forward and 0.72 and 1.81 ms for the two weight gradients.
+// BF16); a warp takes eight consecutive pixels of an image row at a time.  The
+// weights come from shared memory (four addresses per warp, no conflicts), which
+// leaves the registers to the loads in flight and room for 32 warps per SM; the
+// weight gradients keep an octet's 72 partial sums in registers (16 warps).  The
+// floor is 5 us of HBM (64 bytes per pixel) and 4 us of FMAs (288 per pixel) at
+// 8 x 256 x 256 pixels; measured, one kernel at a time from a cold cache, are 25
+// and 27 us out (32 and 37 us with the weights in registers and 16 warps), 41 us
+// in (61 us) and 35 and 38 us for the weight gradients: load latency and issue
+// slots.  One thread per pixel or per output instead (2-byte loads, 64 bytes
+// apart, or a block per 16 rows) took 54 to 267 us forward and 0.72 and 1.81 ms
+// for the two weight gradients.
 constexpr int kEdgeThreads = 256;
 
 struct EdgeArgs {
@@ -147,7 +150,7 @@ __device__ __forceinline__ bool tap_at(const EdgeArgs &a, INNER, int tap, int h,
 // layer (W [9][32], sign = -1).  S: bf16 or float; ROUND: s rounded to BF16 and
 // kept so in sb.  Results BF16 or FP32; relu clamps, gate masks where gate <= 0.
 template <typename S, bool ROUND, bool GRAD, typename OUT>
-__global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, const S *s,
+__global__ void __launch_bounds__(kEdgeThreads, 4) edge_out32_kernel(EdgeArgs a, const S *s,
                                                                   const bf16 *wt,
                                                                   const float *bias,
                                                                   const bf16 *gate, int relu,
@@ -155,13 +158,13 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 {
     chain_begin();
     const int c0 = (threadIdx.x & 3) * 8;
-    float wr[9][8], br[8];
+    __shared__ __align__(16) float ws[9 * kC];   // [tap][channel]
+    for (int i = threadIdx.x; i < 9 * kC; i += kEdgeThreads)
+        ws[i] = __bfloat162float(GRAD ? wt[i] : wt[(i % kC) * 9 + i / kC]);
+    float br[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        br[k] = bias ? bias[c0 + k] : 0.f;
-#pragma unroll
-        for (int t = 0; t < 9; ++t) wr[t][k] = __bfloat162float(GRAD ? wt[t * kC + c0 + k] : wt[(c0 + k) * 9 + t]);
-    }
+    for (int k = 0; k < 8; ++k) br[k] = bias ? bias[c0 + k] : 0.f;
+    __syncthreads();
     for_pixels(a, vec, [&](auto inner, int64_t row, int h, int w, bool in) {
         if (!in) return;
         const int64_t p = row * a.W + w;
@@ -175,8 +178,10 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
             float v = as_float(s[p + off]);
             if (ROUND) v = round_bf16(v);
             if (ROUND && t == 4 && c0 == 0) sb[p] = __float2bfloat16(v);
+            float wr[8];
+            load8(ws + t * kC + c0, true, wr);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k] = __fmaf_rn(v, wr[t][k], acc[k]);
+            for (int k = 0; k < 8; ++k) acc[k] = __fmaf_rn(v, wr[k], acc[k]);
         }
         if (relu)
 #pragma unroll
@@ -204,10 +209,7 @@ __global__ void __launch_bounds__(kEdgeThreads) edge_out32_kernel(EdgeArgs a, co
 // 32 channels in, one out: y[p] = bias + sum_tap sum_c v[p + off(tap), c] w
 // (32 -> 1 forward: W [9][32], sign = 1) or the input gradient of a 1 -> 32
 // layer (W [32][9], sign = -1; rounded to BF16 when `round`).  add (may be
-// NULL) is added to the result.  The weights come from shared memory (four
-// addresses per warp, no conflicts), which leaves the registers to the loads in
-// flight and 32 warps per SM (72 registers of weights and 16 warps: a training pass
-// over 8 x 256 x 256 pixels took 693 instead of 673 us).
+// NULL) is added to the result.
 template <typename V, bool GRAD>
 __global__ void __launch_bounds__(kEdgeThreads, 4) edge_in32_kernel(EdgeArgs a, const V *v,
                                                                  const bf16 *wt,
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(kEdgeThreads, 4) edge_in32_kernel(EdgeArgs a, 
 // s = g, sign = -1 (the pixel of g that sees x[p] through the tap), dw [9][32],
 // dbias = sum s.  One partial sum per block is added to dw and dbias.
 template <typename V, typename S, bool OUT1>
-__global__ void __launch_bounds__(kEdgeThreads) edge_wgrad_kernel(EdgeArgs a, const V *v,
+__global__ void __launch_bounds__(kEdgeThreads, 2) edge_wgrad_kernel(EdgeArgs a, const V *v,
                                                                   const S *s, float *dw,
                                                                   float *db, int vec)
 {
