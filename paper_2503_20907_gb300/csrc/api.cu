@@ -369,9 +369,14 @@ struct sp_plan {
     int device;
     void *mem;
     LineData D;
-    // the footprint tables are built (else their heads only); some projection
-    // has read them, so that every prepare builds them
+    // Footprint tables.  tables: built since the last prepare (else their heads
+    // only); tables_used: some path reads them, so that every prepare from then
+    // on builds them; bare_capture: a captured prepare left them out, so that any
+    // replay of its graph may make them stale; tables_capture: the last capture
+    // (its id) whose prepare builds them, 0 for none.
     mutable bool tables, tables_used;
+    bool bare_capture;
+    mutable unsigned long long tables_capture;
     longlong2 *rec;    // row records written by prepare (NULL: none)
     bool prepared;
     void *cg_ws;       // CGLS vectors and scalars, allocated on first use
@@ -403,37 +408,51 @@ bool plan_alloc_records(sp_plan *p)
     return true;
 }
 
-// The plan's footprint tables, built on the first projection after a prepare
-// whose path reads them.  In a stream that is being captured they become part
-// of the capture, every time: nothing has run yet that a later call could rely
-// on.
-cudaError_t plan_tables(const sp_plan *p, cudaStream_t s)
+// The id of the capture that s is part of, 0 if it is not being captured.
+cudaError_t capture_of(cudaStream_t s, unsigned long long *id)
 {
-    p->tables_used = true;
-    if (p->tables) return cudaSuccess;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(s, &cap);
-    if (e == cudaSuccess) e = spx::launch_tables(p->g, p->L, p->D.tabs, table_count(p->L), s);
-    if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone) p->tables = true;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    *id = 0;
+    unsigned long long n = 0;
+    const cudaError_t e = cudaStreamGetCaptureInfo(s, &st, &n);
+    if (e == cudaSuccess && st == cudaStreamCaptureStatusActive) *id = n;
     return e;
 }
 
-cudaError_t plan_fwd(const sp_plan *p, const float *coef, float *sino, cudaStream_t s, int path)
+// The plan's footprint tables, built on the first projection after a prepare
+// whose path reads them.  In a stream that is being captured they become part
+// of the graph, unless a prepare of the same graph builds them: nothing has run
+// yet that a later call could rely on.  Where a graph with a prepare that left
+// them out may be replayed at any time, every projection builds them.
+cudaError_t plan_tables(const sp_plan *p, cudaStream_t s)
+{
+    p->tables_used = true;
+    if (p->tables && !p->bare_capture) return cudaSuccess;
+    unsigned long long cap;
+    cudaError_t e = capture_of(s, &cap);
+    if (e != cudaSuccess || (cap && cap == p->tables_capture)) return e;
+    e = spx::launch_tables(p->g, p->L, p->D.tabs, table_count(p->L), s);
+    if (e == cudaSuccess && !cap) p->tables = true;
+    return e;
+}
+
+// One projection of a plan; rec: its row records, or NULL.
+cudaError_t plan_fwd(const sp_plan *p, const float *coef, float *sino, cudaStream_t s, int path, const longlong2 *rec)
 {
     if (path_needs_tables(p->g, p->L, p->D.extra, path)) {
         const cudaError_t e = plan_tables(p, s);
         if (e != cudaSuccess) return e;
     }
-    return run_fwd(p->g, p->L, p->D, coef, sino, s, path, p->rec);
+    return run_fwd(p->g, p->L, p->D, coef, sino, s, path, rec);
 }
 
-cudaError_t plan_adj(const sp_plan *p, const float *sino, float *coef_out, cudaStream_t s, int path)
+cudaError_t plan_adj(const sp_plan *p, const float *sino, float *coef_out, cudaStream_t s, int path, const longlong2 *rec)
 {
     if (p->L.m > 0 && path_needs_tables(p->g, p->L, p->D.extra, path)) {
         const cudaError_t e = plan_tables(p, s);
         if (e != cudaSuccess) return e;
     }
-    return run_adj(p->g, p->L, p->D, sino, coef_out, s, path, p->rec);
+    return run_adj(p->g, p->L, p->D, sino, coef_out, s, path, rec);
 }
 
 sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan, bool keep_records)
@@ -471,7 +490,8 @@ sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan
     p->D.tabs = mem ? reinterpret_cast<float *>(w + hb) : nullptr;
     p->D.extra = (mem && xb) ? w + hb + tb : nullptr;
     p->D.center = (mem && cb) ? reinterpret_cast<float *>(w + hb + tb + xb) : nullptr;
-    p->tables = p->tables_used = false;
+    p->tables = p->tables_used = p->bare_capture = false;
+    p->tables_capture = 0;
     p->L.order = static_cast<const int *>(order_area(g, L, p->D.extra));   // written by prepare
     p->prepared = false;
     p->cg_ws = nullptr;
@@ -520,14 +540,22 @@ sp_status spline_plan_prepare(sp_plan *plan, void *stream)
     if (!plan) return fail(SP_EINVAL, "plan is NULL");
     if (plan->L.m == 0) { plan->prepared = true; return SP_OK; }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    unsigned long long cap = 0;
+    cudaError_t e = capture_of(s, &cap);
+    if (e == cudaSuccess) e = spx::launch_setup(plan->g, plan->L, plan->D.hdr, plan->D.tabs, plan->D.center, s);
     // the footprint tables only where a path that is set or was taken reads
     // them (else they wait for one)
-    cudaError_t e = spx::launch_setup(plan->g, plan->L, plan->D.hdr, plan->D.tabs, plan->D.center, s);
-    plan->tables = false;
-    if (e == cudaSuccess &&
-        (plan->tables_used || path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_fwd) ||
-         path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_adj)))
-        e = plan_tables(plan, s);
+    if (plan->tables_used || path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_fwd) ||
+        path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_adj)) {
+        if (e == cudaSuccess) e = spx::launch_tables(plan->g, plan->L, plan->D.tabs, table_count(plan->L), s);
+        plan->tables_used = true;
+        if (cap) plan->tables_capture = cap;
+        else plan->tables = e == cudaSuccess;
+    } else if (cap) {
+        plan->bare_capture = true;
+    } else {
+        plan->tables = false;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "line setup and footprint tables");
     if (plan->L.order) {
         e = spx::launch_line_order(plan->g, plan->L, plan->D.hdr, const_cast<int *>(plan->L.order), s);
@@ -548,7 +576,7 @@ sp_status spline_plan_fwd(const sp_plan *plan, const float *coef, float *sino, v
     if (!plan->prepared) return fail(SP_EINVAL, "plan not prepared");
     if (plan->L.m == 0) return SP_OK;
     if (!coef || !sino) return fail(SP_EINVAL, "coef/sino pointers are NULL");
-    cudaError_t e = plan_fwd(plan, coef, sino, static_cast<cudaStream_t>(stream), plan->path_fwd);
+    cudaError_t e = plan_fwd(plan, coef, sino, static_cast<cudaStream_t>(stream), plan->path_fwd, plan->rec);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "forward projection");
 }
 
@@ -559,7 +587,7 @@ sp_status spline_plan_adj(const sp_plan *plan, const float *sino, float *coef_ou
     if (!plan->prepared) return fail(SP_EINVAL, "plan not prepared");
     if (!coef_out) return fail(SP_EINVAL, "coef_out pointer is NULL");
     if (plan->L.m > 0 && !sino) return fail(SP_EINVAL, "sino pointer is NULL");
-    cudaError_t e = plan_adj(plan, sino, coef_out, static_cast<cudaStream_t>(stream), plan->path_adj);
+    cudaError_t e = plan_adj(plan, sino, coef_out, static_cast<cudaStream_t>(stream), plan->path_adj, plan->rec);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "adjoint projection");
 }
 
@@ -567,12 +595,12 @@ namespace {
 cudaError_t plan_fwd_cb(void *ctx, const float *coef, float *sino, cudaStream_t s)
 {
     const sp_plan *p = static_cast<const sp_plan *>(ctx);
-    return plan_fwd(p, coef, sino, s, p->path_fwd);
+    return plan_fwd(p, coef, sino, s, p->path_fwd, p->rec);
 }
 cudaError_t plan_adj_cb(void *ctx, const float *sino, float *coef_out, cudaStream_t s)
 {
     const sp_plan *p = static_cast<const sp_plan *>(ctx);
-    return plan_adj(p, sino, coef_out, s, p->path_adj);
+    return plan_adj(p, sino, coef_out, s, p->path_adj, p->rec);
 }
 }  // namespace
 
@@ -674,9 +702,9 @@ sp_status spline_plan_autotune(sp_plan *plan, const float *coef, const float *si
         for (int k = 0; k < (gather ? 5 : 4) && e == cudaSuccess; ++k) {
             const int path = k == 4 ? kPathGather : ((k & 1) ? kPathGeneral : kPathStrip);
             if (k < 2)
-                e = time_runs([&] { return plan_fwd(plan, coef, tmp_s, s, path); }, 3, s, &t[k]);
+                e = time_runs([&] { return plan_fwd(plan, coef, tmp_s, s, path, plan->rec); }, 3, s, &t[k]);
             else
-                e = time_runs([&] { return plan_adj(plan, sino, tmp_c, s, path); }, 3, s, &t[k]);
+                e = time_runs([&] { return plan_adj(plan, sino, tmp_c, s, path, plan->rec); }, 3, s, &t[k]);
         }
         cudaError_t e2 = cudaStreamSynchronize(s);
         if (tmp_s) cudaFree(tmp_s);
@@ -851,7 +879,8 @@ cudaError_t upload_jobs(sp_batch *b, int d, In in, Out outp, std::vector<char> &
     e = cudaDeviceSynchronize();
     for (size_t i = 0; i < b->plans.size() && e == cudaSuccess; ++i) {
         const sp_plan *p = b->plans[i];
-        if (p->L.m > 0 && path_needs_tables(p->g, p->L, p->D.extra, d ? p->path_adj : p->path_fwd)) e = plan_tables(p, b->cap);
+        if (p->L.m > 0 && !p->bare_capture && path_needs_tables(p->g, p->L, p->D.extra, d ? p->path_adj : p->path_fwd))
+            e = plan_tables(p, b->cap);
     }
     const int64_t c0 = all;
     b->chunks[d] = c0;
@@ -959,7 +988,7 @@ sp_status spline_batch_fwd(sp_batch *batch, const float *const *coef, float *con
         [&](size_t i, cudaStream_t s) {
             const sp_plan *p = batch->plans[i];
             if (p->L.m == 0 || queued[i]) return cudaSuccess;
-            return run_fwd(p->g, p->L, p->D, coef[i], sino[i], s, p->path_fwd);
+            return plan_fwd(p, coef[i], sino[i], s, p->path_fwd, nullptr);
         },
         [&] { return upload_jobs(batch, 0, coef, sino, queued); },
         [&](cudaStream_t s) { return run_queue(batch, 0, coef, nullptr, s); });
@@ -984,7 +1013,7 @@ sp_status spline_batch_adj(sp_batch *batch, const float *const *sino, float *con
         [&](size_t i, cudaStream_t s) {
             const sp_plan *p = batch->plans[i];
             if (queued[i]) return cudaSuccess;
-            return run_adj(p->g, p->L, p->D, sino[i], coef_out[i], s, p->path_adj);
+            return plan_adj(p, sino[i], coef_out[i], s, p->path_adj, nullptr);
         },
         [&] { return upload_jobs(batch, 1, sino, coef_out, queued); },
         [&](cudaStream_t s) { return run_queue(batch, 1, nullptr, coef_out, s); });
