@@ -190,6 +190,7 @@ bool path_needs_tables(const spx::GridDev &g, const spx::LinesDev &L, void *extr
 cudaError_t run_fwd(const spx::GridDev &g, const spx::LinesDev &L, const LineData &D, const float *coef, float *sino,
                     cudaStream_t s, int path = kPathAuto, const longlong2 *rec = nullptr)
 {
+    if (L.m == 0) return cudaSuccess;
     if (use_strip(g, L, D.extra, path))
         return spx::launch_fwd_strip(g, L, D.hdr, D.center, D.tabs, coef, D.extra, sino, s, rec);
     return spx::launch_fwd(g, D.hdr, D.tabs, L.m, coef, sino, s);
@@ -199,6 +200,7 @@ cudaError_t run_fwd(const spx::GridDev &g, const spx::LinesDev &L, const LineDat
 cudaError_t run_adj(const spx::GridDev &g, const spx::LinesDev &L, const LineData &D, const float *sino, float *coef_out,
                     cudaStream_t s, int path = kPathAuto, const longlong2 *rec = nullptr)
 {
+    if (L.m == 0) return cudaMemsetAsync(coef_out, 0, sizeof(float) * (size_t)g.nx * (size_t)g.ny, s);
     if (path == kPathGather && spx::gather_supported(g, L))
         return spx::launch_adj_gather(g, L, D.hdr, D.tabs, sino, coef_out, s);
     if (use_strip(g, L, D.extra, path))

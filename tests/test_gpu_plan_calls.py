@@ -88,3 +88,33 @@ def test_a_graph_of_prepare_and_projections(paths):
         # eager projections of the plan that the graph prepared
         assert torch.equal(plan.fwd(coef), want[0]) and _close(plan.adj(p), want[1])
     plan.close()
+
+
+@pytest.mark.parametrize("paths", [(0, 0), (1, 1), (2, 2)])
+@pytest.mark.parametrize("degree", [0, 3])
+def test_empty_line_lists(degree, paths):
+    view, grid, lines, coef, p = _case(degree)
+    none = sp.Lines.theta_y(torch.empty(0, device=DEV), torch.empty(0, device=DEV))
+    plan = sp.Plan(grid, none)
+    plan.set_paths(*paths)
+    empty = torch.empty(0, device=DEV)
+    assert plan.fwd(coef).numel() == 0
+    assert torch.equal(plan.adj(empty, torch.full_like(coef, 7.0)), torch.zeros_like(coef))
+    x, gamma = plan.cgls(empty, 2, x0=coef)
+    assert torch.equal(x, coef) and not gamma.any()
+    plan.close()
+
+
+@pytest.mark.parametrize("degree", [0, 3])
+def test_a_batch_with_an_empty_line_list(degree):
+    view, grid, lines, coef, p = _case(degree)
+    none = sp.Lines.points(torch.empty(0, 2, device=DEV), torch.empty(0, 2, device=DEV))
+    empty = torch.empty(0, device=DEV)
+    batch = sp.Batch([grid, grid, grid], [lines, none, lines])
+    want = _fresh(grid, lines, coef, p, (0, 0))
+    out = batch.fwd([coef] * 3)
+    back = batch.adj([p, empty, p], [torch.full_like(coef, 7.0) for _ in range(3)])
+    assert torch.equal(out[0], want[0]) and out[1].numel() == 0 and torch.equal(out[2], want[0])
+    assert _close(back[0], want[1]) and _close(back[2], want[1])
+    assert torch.equal(back[1], torch.zeros_like(coef))
+    batch.close()
