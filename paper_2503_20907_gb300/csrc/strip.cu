@@ -967,7 +967,8 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
                 pair_add(hi, lo, t.x);
                 lo += t.y;
             }
-            float sum = hi + lo;
+            // (an infinite sum leaves no finite remainder)
+            float sum = isfinite(lo) ? hi + lo : hi;
             if constexpr (kCenter) {
                 if (mine && !isfinite(sum)) {
                     const int axis = mine_vert ? 0 : 1, Nq = mine_vert ? g.nx : g.ny;
