@@ -275,7 +275,12 @@ struct SplineRows {
     f2 K[J][kKnots];        // jumps: half their sum and half their difference
     float cm[NH], km[kKnots];   // the middle candidate
     float beta[2], ua, ha;
-    float hp, ca[J], w_sup;     // float adjoint: factor, (j + c) a, half-width of the support
+    float hp;                   // float adjoint: factor
+    // The candidates of pair j lie in the support where v < end[j] and -v <
+    // end[j], w - (j + c) a.  Only the outermost pair can leave it, and in lines
+    // that share a warp with wider ones the one before.
+    float end[J];
+    static constexpr int kTail = DEG == 1 || J == DEG ? J - 1 : J - 2;
 
     __device__ __forceinline__ void load(const LaneLine &ln)
     {
@@ -295,7 +300,7 @@ struct SplineRows {
                 const f2 t = *reinterpret_cast<const f2 *>(ln.rec + kCenterJump + 8 * q + 2 * (j + (kMid ? 1 : 0)));
                 K[j][q] = FIX ? f2mul(t, sc2) : t;
             }
-            ca[j] = ((float)j + (kMid ? 1.f : 0.5f)) * ln.a;
+            end[j] = ln.w_sup - ((float)j + (kMid ? 1.f : 0.5f)) * ln.a;
         }
         if constexpr (kMid) {
 #pragma unroll
@@ -308,7 +313,6 @@ struct SplineRows {
         ua = ln.ua;
         ha = 0.5f * ln.a;
         hp = ln.hp;
-        w_sup = ln.w_sup;
     }
 
     // One row at strip address sp (the run's first column).
@@ -345,7 +349,7 @@ struct SplineRows {
 #pragma unroll
             for (int q = first_knot(j); q < kKnots; ++q) eo = f2fma(zz[q], K[j][q], eo);
             f2unpack(eo, e, o);
-            put(sp, J + (kMid ? 1 : 0) + j, J - 1 - j, __fadd_rn(e, o), __fsub_rn(e, o), ca[j], v, acc);
+            put(sp, J + (kMid ? 1 : 0) + j, J - 1 - j, __fadd_rn(e, o), __fsub_rn(e, o), j, v, acc);
         }
         if constexpr (kMid) {
             float e = cm[NH - 1];
@@ -364,18 +368,25 @@ struct SplineRows {
         }
     }
 
-    __device__ __forceinline__ void put(float *sp, int ip, int im, float p, float q, float c, float v, f2 &acc) const
+    // Adds the pair j: p at column ip and q at column im.  Beyond the support
+    // the polynomials leave their rounding (up to 2e-8) where phi is 0: the
+    // forward does not read nodes there, so that a line does not see what it does
+    // not meet (whatever the size of the coefficient), and the fixed-point strip
+    // rounds such values to 0.
+    __device__ __forceinline__ void put(float *sp, int ip, int im, float p, float q, int j, float v, f2 &acc) const
     {
         if constexpr (ADJ && FIX) {
             f2unpack(f2add(f2pack(p, q), f2pack(kFixMagic, kFixMagic)), p, q);
             red_shared_u32(reinterpret_cast<int *>(sp) + ip, __float_as_int(p) - kFixMagicBits);
             red_shared_u32(reinterpret_cast<int *>(sp) + im, __float_as_int(q) - kFixMagicBits);
         } else if constexpr (ADJ) {
-            // (values here may be non-finite: only candidates in the support)
-            if (c + v <= w_sup) red_shared(sp + ip, hp * p);
-            if (c - v <= w_sup) red_shared(sp + im, hp * q);
+            if (v < end[j]) red_shared(sp + ip, hp * p);
+            if (-v < end[j]) red_shared(sp + im, hp * q);
         } else {
-            acc = f2fma(f2pack(sp[ip], sp[im]), f2pack(p, q), acc);
+            float x = 0.f, y = 0.f;
+            if (j < kTail || v < end[j]) x = sp[ip];
+            if (j < kTail || -v < end[j]) y = sp[im];
+            acc = f2fma(f2pack(x, y), f2pack(p, q), acc);
         }
     }
 };
@@ -650,44 +661,6 @@ __device__ __forceinline__ int run_columns(const LineHdr &H, float b)
 template <int KIND>
 __device__ __forceinline__ int run_lead(int n) { return KIND >= 1 && KIND <= 3 ? n / 2 : 0; }
 
-// One line's sum over the nodes in its support only, from global memory (FP32,
-// by one thread): lines whose sum is not finite are taken again with this, as
-// the run of a row may reach nodes beyond the support, which a non-finite
-// coefficient there must not enter.
-template <int DEG>
-__device__ __noinline__ float exact_line(const LineHdr &H, const float *rec, long long Y0, long long step, float w_sup,
-                                         const float *src, int Nq, int ld)
-{
-    constexpr int m = DEG + 1, NC = 2 * DEG + 2;
-    constexpr float c = m % 2 == 0 ? 0.5f : 0.f;
-    const float a = H.a;
-    float hi = 0.f, lo = 0.f;
-    for (int r = H.r_begin; r < H.r_end; ++r) {
-        const long long Y = Y0 + r * step;
-        const float v = __fmaf_rn((float)(unsigned)Y, a * 2.3283064365386963e-10f, -0.5f * a), w = fabsf(v);
-        float z[2];
-        for (int q = 0; q < 2; ++q) {
-            const float d = fmaxf(w - rec[kCenterBeta + q], 0.f);
-            z[q] = d;
-            for (int k = 0; k < DEG; ++k) z[q] *= d * d;
-        }
-        for (int kk = -4; kk < 4; ++kk) {
-            const int q = H.q_ref - (int)(Y >> 32) + kk, j = kk >= 0 ? kk : (m % 2 == 0 ? -kk - 1 : -kk);
-            if ((unsigned)q >= (unsigned)Nq || j > 3 || !(fabsf(((float)kk + c) * a + v) < w_sup)) continue;
-            const bool same = (kk >= 0) == (v >= 0.f) || (m % 2 == 1 && kk == 0);
-            const float x = same ? w : -w;
-            float phi = rec[8 * j + NC - 1];
-            for (int k = NC - 2; k >= 0; --k) phi = __fmaf_rn(phi, x, rec[8 * j + k]);
-            for (int k = 0; k < 2; ++k) {
-                const float *J = rec + kCenterJump + 8 * k + 2 * j;
-                phi = __fmaf_rn(same ? J[0] + J[1] : J[0] - J[1], z[k], phi);
-            }
-            pair_add(hi, lo, src[(size_t)r * ld + q] * phi);
-        }
-    }
-    return isfinite(lo) ? hi + lo : hi;
-}
-
 // Adds the accumulated strip into the image by 16-byte reductions.
 __device__ __forceinline__ void strip_flush(const Strip &st, int S0, const Image &im, bool fixed, float finv)
 {
@@ -895,7 +868,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
             ln.q_first = H.q_ref - lead;
             ln.a = H.a;
             ln.ua = H.a * (F == 32 ? 2.3283064365386963e-10f : 3.5527136788005009e-15f);
-            ln.w_sup = 0.5f * H.two_w * 1.000001f;   // (a bound for rounding)
+            ln.w_sup = 0.5f * H.two_w;
             const float hp_raw = ADJ ? g.h * __shfl_sync(0xffffffffu, pv, lj) : 0.f;
             ln.hp = hp_raw * fscale;
             ln.rec = rec_s + (shared_dir ? 0 : lj) * kCenterFloats;
@@ -968,15 +941,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
                 lo += t.y;
             }
             // (an infinite sum leaves no finite remainder)
-            float sum = isfinite(lo) ? hi + lo : hi;
-            if constexpr (kCenter) {
-                if (mine && !isfinite(sum)) {
-                    const int axis = mine_vert ? 0 : 1, Nq = mine_vert ? g.nx : g.ny;
-                    sum = exact_line<KIND>(hdr_s[lane], rec_s + (shared_dir ? 0 : lane) * kCenterFloats, my_W, my_step,
-                                           0.5f * hdr_s[lane].two_w, A.src[axis], Nq, image_ld(Nq));
-                }
-            }
-            A.sino[my_line] = g.h * sum;
+            A.sino[my_line] = g.h * (isfinite(lo) ? hi + lo : hi);
         }
     }
     return true;

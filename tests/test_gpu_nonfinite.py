@@ -56,3 +56,30 @@ def test_sums_that_overflow(degree, basis, path):
         got = plan.fwd(torch.full((N, N), sign * 3e38, device=DEV)).cpu().numpy()
         assert np.all(got[length > 1.5] == sign * np.inf)
     plan.close()
+
+
+@pytest.mark.parametrize("path", [0, 1, 2])
+@pytest.mark.parametrize("degree,basis", [(0, 0), (1, 0), (2, 0), (3, 0), (1, 1)])
+def test_a_line_sees_only_the_nodes_it_meets(degree, basis, path):
+    # a coefficient of any size leaves every line that does not meet it as it
+    # is, bit for bit; a line that misses the support of every basis gives 0
+    og, grid = oracle.Grid(N, N, degree, 1.0, basis=basis), sp.Grid(N, N, degree, 1.0, basis=basis)
+    for kind in ("parallel", "list"):
+        lines, th, yy = _scan(kind)
+        plan = sp.Plan(grid, lines)
+        plan.set_paths(path, 0)
+        coef = torch.rand((N, N), device=DEV, generator=torch.Generator(DEV).manual_seed(2)) + 0.5
+        missed = oracle.forward(og, np.ones((N, N)), th, yy) == 0.0
+        got = plan.fwd(coef).cpu().numpy()
+        assert missed.sum() > 20 and np.all(got[missed] == 0.0) and np.all(got[~missed] >= 0.0)
+        for j, i in ((21, 17), (0, 0), (39, 20)):
+            mask = np.zeros((N, N))
+            mask[j, i] = 1.0
+            clear = oracle.forward(og, mask, th, yy) == 0.0
+            c = coef.clone()
+            c[j, i] = 0.0
+            without = plan.fwd(c).cpu().numpy()
+            for big in (1e30, np.inf if path != 2 else 1e38):
+                c[j, i] = big
+                assert np.array_equal(plan.fwd(c).cpu().numpy()[clear], without[clear])
+        plan.close()
