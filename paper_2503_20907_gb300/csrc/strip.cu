@@ -61,7 +61,7 @@
 // (80 registers) 0.95 and 0.98 ms, five of four warps (96 registers) 0.93 and
 // 0.92 ms.
 //
-// The adjoint accumulates its strip in 32-bit fixed point: a shared-memory
+// The adjoint (degree 0 apart) accumulates its strip in 32-bit fixed point: a shared-memory
 // integer reduction costs about what a plain shared store does on this GPU,
 // a float one four to six times more.  Each chunk takes the power of two S
 // that puts its largest contribution h |p| phi (phi <= sqrt(2) < 1.5 for
@@ -173,8 +173,14 @@ constexpr int kFixMagicBits = 0x4B400000;
 constexpr float kFixMax = 4194304.0f;   // 2^22
 constexpr float kPhiBound = 1.5f;
 
-// Which chunks an adjoint call runs (strip_chunk's FM).
+// Which chunks an adjoint call runs (strip_chunk's FM).  Degree 0 has float
+// strips only: its pixels belong to few lines, and where those are far below the
+// chunk's largest, fixed point would leave them fewer bits than FP32 sums have.
+// (Parallel beams, 501 x 501 pixels, 367 x 751 lines: 332 us, in fixed point 274,
+// with the general kernel's global additions 625.)
 enum FixMode { kFmAll = 0, kFmFixed = 1, kFmFloat = 2 };
+template <int KIND>
+__host__ __device__ constexpr int adj_mode() { return KIND == 0 ? kFmFloat : kFmFixed; }
 
 __device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool in = true)
 {
@@ -532,7 +538,7 @@ __device__ __noinline__ float axis_row0(const LineHdr &H, int r, const float *sr
     return acc;
 }
 
-template <bool ADJ, bool FIX>
+template <bool ADJ>
 struct PixelRows {
     static constexpr int F = kFrac0;
     // c0 + c1 t of candidates 0 and 1 in the intervals 0 and 1 (candidate 1
@@ -554,13 +560,6 @@ struct PixelRows {
         c1[0][1] = -slope;
         c0[1][0] = top;
         c1[1][0] = c0[1][1] = c1[1][1] = 0.f;
-        if constexpr (FIX) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                c0[k >> 1][k & 1] = __fmaf_rn(c0[k >> 1][k & 1], ln.hp, kFixMagic);
-                c1[k >> 1][k & 1] *= ln.hp;
-            }
-        }
         const float s = b > 0.f ? b : a;
         const float q1 = s * top;
         const float r = __fmaf_rn(-q1, a, s) * top;
@@ -577,10 +576,7 @@ struct PixelRows {
         const float t = (float)(x - (up ? S1 : 0ull) + 1ull) * ua;
         const float p0 = __fmaf_rn(up ? c1[1][0] : c1[0][0], t, up ? c0[1][0] : c0[0][0]);
         const float p1 = __fmaf_rn(up ? c1[1][1] : c1[0][1], t, up ? c0[1][1] : c0[0][1]);
-        if constexpr (FIX) {
-            red_shared_u32(reinterpret_cast<int *>(sp), __float_as_int(p0) - kFixMagicBits);
-            if (on_last) red_shared_u32(reinterpret_cast<int *>(sp) + 1, __float_as_int(p1) - kFixMagicBits);
-        } else if constexpr (ADJ) {
+        if constexpr (ADJ) {
             red_shared(sp, hp * p0);
             if (on_last) red_shared(sp + 1, hp * p1);
         } else {
@@ -619,7 +615,7 @@ __device__ __forceinline__ void strip_line(int n, const LaneLine &ln, const Line
             return;
         }
         const float b = fabsf(H.rho_hi + H.rho_lo);
-        PixelRows<ADJ, FIX> R;
+        PixelRows<ADJ> R;
         R.load(ln, b < 1e-30f ? 0.f : b, H.a_corr);
         walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
     } else if constexpr (KIND == kKindBox) {
@@ -754,18 +750,20 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
     float pv = 0.f, fscale = 1.f, finv = 1.f;
     if constexpr (ADJ) {
         if (lane < nl) pv = A.sino[my_line];
-        // (bits of non-negative floats order like the floats; non-finite ones on top)
-        const unsigned pm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(pv)));
-        const float top = kPhiBound * g.h * __uint_as_float(pm);   // largest |h p phi| of the chunk
-        // (an all-zero chunk counts as fixed point: its lines are skipped)
-        const bool fix = pm < 0x7f800000u && (top == 0.f || (top >= 1e-20f && top <= 1e20f));
-        if (fix != FIX) return false;   // left to the other launch
-        if (FIX && top > 0.f) {
-            int e;
-            frexpf(kFixMax / top, &e);   // kFixMax / top in [2^(e-1), 2^e)
-            e -= 1;                      // S = 2^e <= kFixMax / top
-            fscale = ldexpf(1.f, e);
-            finv = ldexpf(1.f, -e);
+        if constexpr (adj_mode<KIND>() == kFmFixed) {
+            // (bits of non-negative floats order like the floats; non-finite ones on top)
+            const unsigned pm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(pv)));
+            const float top = kPhiBound * g.h * __uint_as_float(pm);   // largest |h p phi| of the chunk
+            // (an all-zero chunk counts as fixed point: its lines are skipped)
+            const bool fix = pm < 0x7f800000u && (top == 0.f || (top >= 1e-20f && top <= 1e20f));
+            if (fix != FIX) return false;   // left to the other launch
+            if (FIX && top > 0.f) {
+                int e;
+                frexpf(kFixMax / top, &e);   // kFixMax / top in [2^(e-1), 2^e)
+                e -= 1;                      // S = 2^e <= kFixMax / top
+                fscale = ldexpf(1.f, e);
+                finv = ldexpf(1.f, -e);
+            }
         }
     }
 
@@ -1018,8 +1016,9 @@ strip_queue_kernel(const StripJob *jobs, int njobs, long long total, unsigned lo
         const long long c = cur;
         if (c >= total) break;
         const StripJob *J = queue_job(jobs, njobs, c);
-        const bool ran = strip_chunk<KIND, ADJ, ADJ ? kFmFixed : kFmAll>(smem, J->A, (int)(c - J->chunk0));
-        if (ADJ && !ran && threadIdx.x == 0) defer[atomicAdd(defer_n, 1ull)] = c;
+        constexpr int FM = ADJ ? adj_mode<KIND>() : kFmAll;
+        const bool ran = strip_chunk<KIND, ADJ, FM>(smem, J->A, (int)(c - J->chunk0));
+        if (FM == kFmFixed && !ran && threadIdx.x == 0) defer[atomicAdd(defer_n, 1ull)] = c;
     }
 }
 
@@ -1053,18 +1052,21 @@ cudaError_t launch_queue_t(bool adj, const StripJob *jobs, int njobs, int64_t to
     if (adj) {
         e = cudaFuncSetAttribute(strip_queue_kernel<KIND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(strip_queue_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kSmemBytes);
         if (e != cudaSuccess) return e;
         launch_chained(strip_queue_kernel<KIND, true>, (unsigned)grid, kThreads, kSmemBytes, s, jobs, njobs,
                        (long long)total, counter, defer, counter + 1);
         e = cudaGetLastError();
-        // the deferred chunks are few (non-finite or extreme sinogram values): a small grid
-        if (e == cudaSuccess)
+        if constexpr (adj_mode<KIND>() == kFmFixed) {
+            // the deferred chunks are few (non-finite or extreme sinogram values): a small grid
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(strip_queue_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSmemBytes);
+            if (e != cudaSuccess) return e;
             launch_chained(strip_queue_float_kernel<KIND>, (unsigned)(grid < sms ? grid : sms), kThreads, kSmemBytes, s,
                            jobs, njobs, defer, counter + 1, counter + 2);
-        return e == cudaSuccess ? cudaGetLastError() : e;
+            e = cudaGetLastError();
+        }
+        return e;
     }
     e = cudaFuncSetAttribute(strip_queue_kernel<KIND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
@@ -1166,20 +1168,23 @@ cudaError_t launch_strip_t(const StripArgs &A, bool adj, unsigned *defer, cudaSt
         launch_chained(strip_kernel<KIND, false>, grid, kThreads, kSmemBytes, s, A, nullptr);
         return cudaGetLastError();
     }
-    // fixed-point chunks, then (a small second launch) the chunks they
-    // deferred to float strips
-    e = cudaFuncSetAttribute(strip_kernel<KIND, true, kFmFixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(strip_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    int dev = 0, sms = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    constexpr int FM = adj_mode<KIND>();
+    e = cudaFuncSetAttribute(strip_kernel<KIND, true, FM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
     if (e != cudaSuccess) return e;
-    launch_chained(strip_kernel<KIND, true, kFmFixed>, grid, kThreads, kSmemBytes, s, A, defer);
+    launch_chained(strip_kernel<KIND, true, FM>, grid, kThreads, kSmemBytes, s, A, defer);
     e = cudaGetLastError();
-    if (e == cudaSuccess)
+    if constexpr (FM == kFmFixed) {
+        // a small second launch for the chunks deferred to float strips
+        int dev = 0, sms = 0;
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(strip_float_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
         launch_chained(strip_float_kernel<KIND>, grid < (unsigned)sms ? grid : (unsigned)sms, kThreads, kSmemBytes, s, A, defer);
-    return e == cudaSuccess ? cudaGetLastError() : e;
+        e = cudaGetLastError();
+    }
+    return e;
 }
 
 cudaError_t launch_strip(const StripArgs &A, bool adj, unsigned *defer, cudaStream_t s)
