@@ -518,26 +518,6 @@ __device__ __forceinline__ void walk_blocks(const Rows &R, const LaneLine &ln, c
 // Degree 0 has at most two candidates per row and two intervals; its lanes
 // select the (linear) polynomials.  Its footprint can have ramps far narrower
 // than one float ulp of u, so W carries 48 fractional bits.
-// One row of a degree-0 line exactly along an axis (kDeg0Axis), whose
-// footprint is a rectangle with edges on nodes, each taking the midpoint value
-// on both sides (so a row has one more candidate): straight from or to global
-// memory.  Such lines occur only at views exactly along an axis.
-__device__ __noinline__ float axis_row0(const LineHdr &H, int r, const float *src, float *dst, int Nq, int ld,
-                                        float hp, bool adj)
-{
-    const float inv_a = 1.0f / H.a;
-    float s0[1] = {H.a};   // b = 0: one interval
-    float acc = 0.f;
-    const RowEval e = row_eval<0>(H, s0, inv_a, r);
-    for (int q = e.tie ? e.q0 - 1 : e.q0; q <= e.q0; ++q) {
-        if ((unsigned)q >= (unsigned)Nq) continue;
-        const float phi = e.tie ? 0.5f * inv_a : inv_a;
-        if (adj) atomicAdd(dst + (size_t)r * ld + q, hp * phi);
-        else acc = __fmaf_rn(src[(size_t)r * ld + q], phi, acc);
-    }
-    return acc;
-}
-
 template <bool ADJ>
 struct PixelRows {
     static constexpr int F = kFrac0;
@@ -567,6 +547,21 @@ struct PixelRows {
         ua = ln.ua;
         hp = ln.hp;
         has_last = ln.has_last;
+    }
+
+    // A line exactly along an axis (kDeg0Axis): all rows alike, the footprint a
+    // rectangle; where its edges fall on two nodes (tie), the midpoint value on
+    // both.  (4 views of 512 x 512 pixels, one of them along an axis: forward 27
+    // us; with such rows walked one by one in global memory 87.)
+    __device__ __forceinline__ void load_axis(const LaneLine &ln, bool tie)
+    {
+        const float top = 1.0f / ln.a;
+        c0[0][0] = c0[0][1] = tie ? 0.5f * top : top;
+        c0[1][0] = c0[1][1] = c1[0][0] = c1[0][1] = c1[1][0] = c1[1][1] = 0.f;
+        S1 = 1ull << kFrac0;   // interval 0 throughout
+        ua = ln.ua;
+        hp = ln.hp;
+        has_last = tie;
     }
 
     __device__ __forceinline__ void row(long long W, float *sp, f2 &acc) const
@@ -602,22 +597,21 @@ struct Image {
 // the warp's runs.
 template <int KIND, bool ADJ, bool FIX>
 __device__ __forceinline__ void strip_line(int n, const LaneLine &ln, const LineHdr &H, const float *tab, const Strip &st,
-                                           int S0, int b0, int b1, const Image &im, float hp_raw, float &hi, float &lo)
+                                           int b0, int b1, float &hi, float &lo)
 {
     if constexpr (KIND == 0) {
-        if (H.flags & kDeg0Axis) {
-            for (int b = b0; b < b1; ++b) {
-                float acc = 0.f;
-                for (int r = max(S0 + b * kRowBlock, H.r_begin); r < min(S0 + (b + 1) * kRowBlock, H.r_end); ++r)
-                    acc += axis_row0(H, r, im.src, im.dst, im.Nq, im.ld, hp_raw, ADJ);
-                pair_add(hi, lo, acc);
-            }
-            return;
-        }
-        const float b = fabsf(H.rho_hi + H.rho_lo);
         PixelRows<ADJ> R;
-        R.load(ln, b < 1e-30f ? 0.f : b, H.a_corr);
-        walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo);
+        LaneLine l = ln;
+        if (H.flags & kDeg0Axis) {
+            const float s0[1] = {H.a};   // b = 0: one interval
+            const RowEval e = row_eval<0>(H, s0, 1.0f / H.a, H.r_begin);
+            R.load_axis(ln, e.tie);
+            l.q_first = (e.tie ? e.q0 - 1 : e.q0) + (int)(ln.W0 >> kFrac0);
+        } else {
+            const float b = fabsf(H.rho_hi + H.rho_lo);
+            R.load(ln, b < 1e-30f ? 0.f : b, H.a_corr);
+        }
+        walk_blocks(R, l, st, b0, b1, ADJ, hi, lo);
     } else if constexpr (KIND == kKindBox) {
         switch (n) {
         case 6: { BoxRows<6, ADJ, FIX> R; R.load(ln, tab); walk_blocks(R, ln, st, b0, b1, ADJ, hi, lo); break; }
@@ -867,8 +861,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
             ln.a = H.a;
             ln.ua = H.a * (F == 32 ? 2.3283064365386963e-10f : 3.5527136788005009e-15f);
             ln.w_sup = 0.5f * H.two_w;
-            const float hp_raw = ADJ ? g.h * __shfl_sync(0xffffffffu, pv, lj) : 0.f;
-            ln.hp = hp_raw * fscale;
+            ln.hp = ADJ ? g.h * __shfl_sync(0xffffffffu, pv, lj) * fscale : 0.f;
             ln.rec = rec_s + (shared_dir ? 0 : lj) * kCenterFloats;
             ln.has_last = __shfl_sync(0xffffffffu, my_n, lj) >= n && H.K >= n;
             {
@@ -907,7 +900,7 @@ __device__ __forceinline__ bool strip_chunk(unsigned char *smem, const StripArgs
                 const int nb = st.rows / kRowBlock, unit = warp * parts + lane / len, units = kWarps * parts;
                 const int b0 = nb * unit / units, b1 = on ? nb * (unit + 1) / units : b0;
                 ln.W0 = W_row0 + S0 * ln.Wstep;
-                strip_line<KIND, ADJ, FIX>(n, ln, H, tab, st, S0, b0, b1, im, hp_raw, hi, lo);
+                strip_line<KIND, ADJ, FIX>(n, ln, H, tab, st, b0, b1, hi, lo);
                 if constexpr (ADJ) {
                     __syncthreads();
                     strip_flush(st, S0, im, FIX, finv);
