@@ -161,14 +161,46 @@ void *order_area(const spx::GridDev &g, const spx::LinesDev &L, void *extra)
     return static_cast<char *>(extra) + image_list_bytes(g, L);
 }
 
-// Kernel paths: strip kernels (kPathAuto too) or the general warp-per-line
-// kernels.
+// Degree 0 on the automatic path: whether the strip kernels are the faster ones.
+// A strip costs per row and 32 lines about as much as its window is wide, and a
+// call three more launches; a line alone costs the general kernels per row the
+// same in any company.  Measured, strip / general, forward and adjoint:
+//   parallel beam, 360 views: bins 1 pixel apart 0.64 and 0.58 at 512^2 pixels,
+//     0.77 and 0.56 at 256^2; 2 apart 0.80 and 0.72 at 512^2; 4 apart 1.10, 1.09;
+//     8 apart 1.69, 1.78.  Hence at most 3 apart (fan beams: at the grid's centre).
+//   fewer lines, 1 apart: 11,520 at 256^2 1.07 and 0.97, 3,072 at 512^2 1.28 and
+//     1.87, 23,040 at 512^2 0.81 and 0.77; 34,560 at 64^2 1.11 and 0.56.  Hence
+//     16,384 lines, and in the forward, which gains less, 2^23 lines times rows.
+//   chunks are filled by a view's bins: at most a quarter of their lines missing.
+//   random lists (neighbours in the sorted order are 13.5 N / sqrt(m) columns
+//     apart over 32 lines, see order.cu): forward 0.84 at 30,000 lines and 512^2
+//     (40 columns), 1.60 at 10,000 (69), 1.22 at 30,000 and 1024^2 (80): at most 48
+//     columns.  Their adjoint 1.2 to 1.5 (lanes that add to one pixel): never.
+bool pixels_on_strips(const spx::GridDev &g, const spx::LinesDev &L, bool adj)
+{
+    const double m = (double)L.m, N = (double)(g.nx > g.ny ? g.nx : g.ny);
+    if (!adj && m * N < 8388608.0) return false;
+    if (spx::strip_needs_order(L)) return !adj && 13.5 * 13.5 * N * N <= 48.0 * 48.0 * m;
+    double apart = std::fabs((double)L.ddet) / g.h;
+    if (L.kind == SP_LINES_FAN) apart *= (double)L.dso / ((double)L.dso + (double)L.dod);
+    return m >= 16384.0 && apart <= 3.0 && 32.0 * (double)spx::strip_chunk_count(L) <= 1.25 * m;
+}
+
+// Kernel paths: strip kernels (kPathAuto where they are the faster ones: always
+// for degree >= 1 and the box-spline) or the general warp-per-line kernels.
 // kPathGather (adjoint only): the pixel-driven gather where it applies.
 enum KernelPath { kPathAuto = 0, kPathStrip = 1, kPathGeneral = 2, kPathGather = 3 };
 
-bool use_strip(const spx::GridDev &g, const spx::LinesDev &L, void *extra, int path)
+bool strip_path(const spx::GridDev &g, const spx::LinesDev &L, int path, bool adj)
 {
-    return extra && spx::strip_supported(g, L) && (path == kPathStrip || path == kPathAuto);
+    return spx::strip_supported(g, L) &&
+           (path == kPathStrip || (path == kPathAuto && (g.kdeg >= 1 || pixels_on_strips(g, L, adj))));
+}
+
+// The same of a plan or call with this scratch for them (NULL: none).
+bool use_strip(const spx::GridDev &g, const spx::LinesDev &L, const void *extra, int path, bool adj)
+{
+    return extra && strip_path(g, L, path, adj);
 }
 
 // What line setup leaves behind for one (grid, lines) pair.
@@ -181,9 +213,9 @@ struct LineData {
 
 // Whether a path reads the footprint tables (beyond their heads): all but the
 // strip kernels on B-splines.
-bool path_needs_tables(const spx::GridDev &g, const spx::LinesDev &L, void *extra, int path)
+bool path_needs_tables(const spx::GridDev &g, const spx::LinesDev &L, const void *extra, int path, bool adj)
 {
-    return g.basis != SP_BASIS_BSPLINE || !use_strip(g, L, extra, path);
+    return g.basis != SP_BASIS_BSPLINE || !use_strip(g, L, extra, path, adj);
 }
 
 // Forward projection (rec: the plan's row records, or NULL).
@@ -191,7 +223,7 @@ cudaError_t run_fwd(const spx::GridDev &g, const spx::LinesDev &L, const LineDat
                     cudaStream_t s, int path = kPathAuto, const longlong2 *rec = nullptr)
 {
     if (L.m == 0) return cudaSuccess;
-    if (use_strip(g, L, D.extra, path))
+    if (use_strip(g, L, D.extra, path, false))
         return spx::launch_fwd_strip(g, L, D.hdr, D.center, D.tabs, coef, D.extra, sino, s, rec);
     return spx::launch_fwd(g, D.hdr, D.tabs, L.m, coef, sino, s);
 }
@@ -203,7 +235,7 @@ cudaError_t run_adj(const spx::GridDev &g, const spx::LinesDev &L, const LineDat
     if (L.m == 0) return cudaMemsetAsync(coef_out, 0, sizeof(float) * (size_t)g.nx * (size_t)g.ny, s);
     if (path == kPathGather && spx::gather_supported(g, L))
         return spx::launch_adj_gather(g, L, D.hdr, D.tabs, sino, coef_out, s);
-    if (use_strip(g, L, D.extra, path))
+    if (use_strip(g, L, D.extra, path, true))
         return spx::launch_adj_strip(g, L, D.hdr, D.center, D.tabs, sino, D.extra, coef_out, s, rec);
     return spx::launch_adj(g, D.hdr, D.tabs, L.m, sino, coef_out, s);
 }
@@ -225,15 +257,19 @@ size_t rec_bytes_wanted(const spx::GridDev &g, const spx::LinesDev &L)
     return (size_t)L.m * sizeof(longlong2);
 }
 
-// Line setup of a one-shot call in the cached workspace: with `project` for the
-// strip kernels (and the chunk order of free lists), else the footprint tables.
-sp_status prepare(const spx::GridDev &g, spx::LinesDev &L, cudaStream_t s, bool project, LineData *D)
+// Line setup of a one-shot call in the cached workspace, with what its kernels
+// read: the strip kernels' records (and the chunk order of free lists) or the
+// footprint tables.
+enum Call { kCallFwd, kCallAdj, kCallVisited };
+
+sp_status prepare(const spx::GridDev &g, spx::LinesDev &L, cudaStream_t s, Call call, LineData *D)
 {
     const int64_t nt = table_count(L);
     const size_t hb = align_up(sizeof(spx::LineHdr) * (size_t)L.m);
-    const size_t xb = project ? align_up(extra_bytes(g, L)) : 0;
-    const size_t cb = project ? center_bytes(g, nt) : 0;
-    const bool tables = !project || g.basis != SP_BASIS_BSPLINE || xb == 0;
+    const bool strip = call != kCallVisited && strip_path(g, L, kPathAuto, call == kCallAdj);
+    const size_t xb = strip ? align_up(extra_bytes(g, L)) : 0;
+    const size_t cb = strip ? center_bytes(g, nt) : 0;
+    const bool tables = !strip || g.basis != SP_BASIS_BSPLINE;
     const size_t tb = tables ? align_up(sizeof(float) * (size_t)spx::kTabFloats * (size_t)nt) : 0;
     void *ws = nullptr;
     sp_status st = workspace(hb + xb + cb + tb + 256, &ws);
@@ -285,7 +321,7 @@ sp_status spline_project_fwd(const sp_grid *grid, const float *coef, const sp_li
     if (!coef || !sino) return fail(SP_EINVAL, "coef/sino pointers are NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     LineData D;
-    if ((st = prepare(g, L, s, true, &D)) != SP_OK) return st;
+    if ((st = prepare(g, L, s, kCallFwd, &D)) != SP_OK) return st;
     cudaError_t e = run_fwd(g, L, D, coef, sino, s);
     if (e != cudaSuccess) return cuda_fail(e, "forward projection");
     return SP_OK;
@@ -308,7 +344,7 @@ sp_status spline_project_adj(const sp_grid *grid, const float *sino, const sp_li
         return e == cudaSuccess ? SP_OK : cuda_fail(e, "cudaMemsetAsync");
     }
     LineData D;
-    if ((st = prepare(g, L, s, true, &D)) != SP_OK) return st;
+    if ((st = prepare(g, L, s, kCallAdj, &D)) != SP_OK) return st;
     cudaError_t e = run_adj(g, L, D, sino, coef_out, s);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint projection");
     return SP_OK;
@@ -360,7 +396,7 @@ sp_status spline_visited(const sp_grid *grid, const sp_lines *lines, int32_t *co
     if (!counts) return fail(SP_EINVAL, "counts pointer is NULL");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     LineData D;
-    if ((st = prepare(g, L, s, false, &D)) != SP_OK) return st;
+    if ((st = prepare(g, L, s, kCallVisited, &D)) != SP_OK) return st;
     cudaError_t e = spx::launch_visited(g, D.hdr, D.tabs, L.m, counts, offsets, nodes, s);
     return e == cudaSuccess ? SP_OK : cuda_fail(e, "visited set");
 }
@@ -441,7 +477,7 @@ cudaError_t plan_tables(const sp_plan *p, cudaStream_t s)
 // One projection of a plan; rec: its row records, or NULL.
 cudaError_t plan_fwd(const sp_plan *p, const float *coef, float *sino, cudaStream_t s, int path, const longlong2 *rec)
 {
-    if (path_needs_tables(p->g, p->L, p->D.extra, path)) {
+    if (path_needs_tables(p->g, p->L, p->D.extra, path, false)) {
         const cudaError_t e = plan_tables(p, s);
         if (e != cudaSuccess) return e;
     }
@@ -450,7 +486,7 @@ cudaError_t plan_fwd(const sp_plan *p, const float *coef, float *sino, cudaStrea
 
 cudaError_t plan_adj(const sp_plan *p, const float *sino, float *coef_out, cudaStream_t s, int path, const longlong2 *rec)
 {
-    if (p->L.m > 0 && path_needs_tables(p->g, p->L, p->D.extra, path)) {
+    if (p->L.m > 0 && path_needs_tables(p->g, p->L, p->D.extra, path, true)) {
         const cudaError_t e = plan_tables(p, s);
         if (e != cudaSuccess) return e;
     }
@@ -547,8 +583,8 @@ sp_status spline_plan_prepare(sp_plan *plan, void *stream)
     if (e == cudaSuccess) e = spx::launch_setup(plan->g, plan->L, plan->D.hdr, plan->D.tabs, plan->D.center, s);
     // the footprint tables only where a path that is set or was taken reads
     // them (else they wait for one)
-    if (plan->tables_used || path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_fwd) ||
-        path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_adj)) {
+    if (plan->tables_used || path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_fwd, false) ||
+        path_needs_tables(plan->g, plan->L, plan->D.extra, plan->path_adj, true)) {
         if (e == cudaSuccess) e = spx::launch_tables(plan->g, plan->L, plan->D.tabs, table_count(plan->L), s);
         plan->tables_used = true;
         if (cap) plan->tables_capture = cap;
@@ -844,7 +880,7 @@ cudaError_t run_graph(sp_batch *b, GraphCache &gc, const std::vector<const void 
 bool in_queue(const sp_plan *p, int d)
 {
     const int path = d ? p->path_adj : p->path_fwd;
-    if (p->L.m == 0 || !use_strip(p->g, p->L, p->D.extra, path)) return false;
+    if (p->L.m == 0 || !use_strip(p->g, p->L, p->D.extra, path, d == 1)) return false;
     return p->g.kdeg >= 1 || path == kPathStrip;
 }
 
@@ -881,7 +917,7 @@ cudaError_t upload_jobs(sp_batch *b, int d, In in, Out outp, std::vector<char> &
     e = cudaDeviceSynchronize();
     for (size_t i = 0; i < b->plans.size() && e == cudaSuccess; ++i) {
         const sp_plan *p = b->plans[i];
-        if (p->L.m > 0 && !p->bare_capture && path_needs_tables(p->g, p->L, p->D.extra, d ? p->path_adj : p->path_fwd))
+        if (p->L.m > 0 && !p->bare_capture && path_needs_tables(p->g, p->L, p->D.extra, d ? p->path_adj : p->path_fwd, d == 1))
             e = plan_tables(p, b->cap);
     }
     const int64_t c0 = all;
