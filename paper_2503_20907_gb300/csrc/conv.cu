@@ -99,6 +99,14 @@ __device__ __forceinline__ float as_float(bf16 v) { return __bfloat162float(v); 
 __device__ __forceinline__ float as_float(float v) { return v; }
 __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16(v)); }
 
+// The ReLU: a NaN stays one (fmaxf would take it to 0).
+__device__ __forceinline__ float relu_of(float v)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 // The ReLU's mask: a factor of 0 or 1 on the BF16 gradients of the network
 // (non-finite values stay non-finite), a selection on the FP32 results.
 template <typename OUT>
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(kEdgeThreads, 4) edge_out32_kernel(EdgeArgs a,
         }
         if (relu)
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k] = fmaxf(acc[k], 0.f);
+            for (int k = 0; k < 8; ++k) acc[k] = relu_of(acc[k]);
         if (gate) {
             float gt[8];
             load8(gate + p * kC + c0, inner.value || vec, gt);
@@ -246,7 +254,7 @@ __global__ void __launch_bounds__(kEdgeThreads, 4) edge_in32_kernel(EdgeArgs a, 
         acc += __shfl_xor_sync(0xffffffffu, acc, 2);
         if (in && (threadIdx.x & 3) == 0) {
             acc += b0;
-            if (relu) acc = fmaxf(acc, 0.f);
+            if (relu) acc = relu_of(acc);
             if (gate && !(__bfloat162float(gate[p]) > 0.f)) acc = 0.f;
             if (round) acc = round_bf16(acc);
             y[p] = add ? add[p] + acc : acc;
@@ -571,7 +579,7 @@ __device__ __forceinline__ void stage_row(const ChainArgs &a, const IN *x, int64
 //   weights wb[kc][n][8]: K = tap 32 + input channel in groups kc of 8,
 //          n the output channel; LBO = 32 * 16 B, SBO = 128 B.
 //
-// Three CTAs of 128 threads per SM, each with its weights, a ring of five rows
+// Three CTAs of 160 threads per SM, each with its weights, a ring of five rows
 // and two accumulators: while the tensor cores work on a tile, the block stores
 // the one before and copies the row two tiles ahead.  Bound by the latency of a
 // tile's chain (copies, MMAs, read-back, stores; 64 bytes in and out per pixel
@@ -687,10 +695,10 @@ __global__ void __launch_bounds__(kThreads5) conv32_tc05_kernel(ChainArgs ch, Co
                 load8(bias_s + o, true, bv);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    float v = good ? __uint_as_float(acc[o + j]) + bv[j] : bad;
-                    if (a.relu) v = fmaxf(v, 0.f);
+                    float v = __uint_as_float(acc[o + j]) + bv[j];
+                    if (a.relu) v = relu_of(v);
                     if (a.gate) v = masked<OUT>(v, gt[j] > 0.f);
-                    f[j] = v;
+                    f[j] = good ? v : bad;
                 }
                 if constexpr (sizeof(OUT) == 2) {
                     *reinterpret_cast<uint4 *>(y + off + o) = pack8(f);
