@@ -622,16 +622,15 @@ __global__ void __launch_bounds__(kThreads5) conv32_tc05_kernel(ChainArgs ch, Co
     // weights: wb[kc][n][8] = W[n][kc 8 .. kc 8 + 7] (W is [n][tap][i], K = tap 32 + i);
     // flipped for the input gradient: n = i, K = tap' 32 + o, W[o][8 - tap'][i]
     for (int i = threadIdx.x; i < 36 * kC; i += kThreads5) {
-        if (a.form == kWPacked) {
-            cp16(s_u32(wsb + i * 16), a.w + (size_t)i * 8, true);
+        const int kc = i / kC, n = i - kc * kC;
+        if (a.form != kWFlip) {
+            cp16(s_u32(wsb + i * 16), a.w + (a.form == kWPacked ? (size_t)i * 8 : (size_t)n * 9 * kC + kc * 8), true);
             continue;
         }
-        const int kc = i / kC, n = i - kc * kC;
         __align__(16) bf16 e[8];
         const int tp = kc >> 2, c0 = (kc & 3) * 8;
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            e[j] = a.form == kWFlip ? a.w[((size_t)(c0 + j) * 9 + (8 - tp)) * kC + n] : a.w[(size_t)n * 9 * kC + kc * 8 + j];
+        for (int j = 0; j < 8; ++j) e[j] = a.w[((size_t)(c0 + j) * 9 + (8 - tp)) * kC + n];
         *reinterpret_cast<uint4 *>(wsb + i * 16) = *reinterpret_cast<const uint4 *>(e);
     }
     if (threadIdx.x < kC) bias_s[threadIdx.x] = a.bias ? a.bias[threadIdx.x] : 0.f;
