@@ -431,7 +431,7 @@ bool plan_alloc_records(sp_plan *p)
 {
     if (p->rec) return true;
     const size_t rb = rec_bytes_wanted(p->g, p->L);
-    if (rb == 0) return false;
+    if (rb == 0 || !p->D.extra) return false;
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || rb > fr / 4 || rb > kRecMaxBytes) {
         cudaGetLastError();
@@ -513,6 +513,14 @@ sp_status plan_create(const sp_grid *grid, const sp_lines *lines, sp_plan **plan
     void *mem = nullptr;
     if (hb + tb + xb + cb > 0) {
         e = cudaMalloc(&mem, hb + tb + xb + cb);
+        if (e == cudaErrorMemoryAllocation) {
+            // the line records and tables alone do for the general kernels (of
+            // about 1,600 bytes per line with its own direction 200 are the strip
+            // kernels')
+            cudaGetLastError();
+            xb = cb = 0;
+            e = cudaMalloc(&mem, hb + tb);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(SP_ENOMEM, std::string("plan allocation failed: ") + cudaGetErrorString(e));
