@@ -161,12 +161,19 @@ sp_status spline_visited(const sp_grid *grid, const sp_lines *lines, int32_t *co
                          const int64_t *offsets, int32_t *nodes, void *stream);
 
 /*
- * Plans.  A plan keeps the per-line records and footprint tables of one
- * (grid, lines) pair in its own device memory, so that repeated projections
+ * Plans.  A plan keeps the per-line records and the footprints of one
+ * (grid, lines) pair in its own device memory (about 1.6 KB per line, or per
+ * view of parallel beams and 64 bytes per line), so that repeated projections
  * (iterative reconstruction, autograd) skip the setup.  The steps of one pass
  * of the projector are then separate calls:
- *   spline_plan_prepare  line setup (eq. rayparam) and footprint tables
- *                        (Prop. 1, eq. xsa), for THETA_Y and POINTS lists
+ *   spline_plan_prepare  line setup (eq. rayparam) and footprints (Prop. 1, eq.
+ *                        xsa): centre records for the strip kernels on
+ *                        B-splines of degree >= 1; footprint tables where a
+ *                        kernel path (spline_plan_set_paths) reads them that is
+ *                        set or was taken before, else with the first projection
+ *                        that does (or, where a prepare without them was
+ *                        captured into a graph, with every such projection);
+ *                        for THETA_Y and POINTS lists
  *                        the strip kernels' line order, and, where the plan keeps
  *                        them, the row records: where each line's rows start
  *                        in their runs of nodes and how that moves from row to
@@ -182,7 +189,9 @@ sp_status spline_visited(const sp_grid *grid, const sp_lines *lines, int32_t *co
  * the descriptors but enqueues no work; the device arrays that `lines` points
  * to must stay valid until the last spline_plan_prepare on the plan has run.
  * A plan is used on the device that was current at creation.  Calls on one
- * plan must be ordered (same stream, or synchronised).
+ * plan must be ordered (same stream, or synchronised).  Where device memory does
+ * not hold the strip kernels' part of the plan (200 bytes per line and the image
+ * copies), the plan is created without it and runs on the general kernels.
  */
 typedef struct sp_plan sp_plan;
 
@@ -217,12 +226,16 @@ sp_status spline_plan_cgls(sp_plan *plan, const float *b, float *x, int32_t iter
                            double *gamma_hist, void *stream);
 /*
  * Kernel choice of a plan, per direction: 0 = automatic (the strip kernels
- * for degree >= 1, else the general kernels; THETA_Y and POINTS lists reach
+ * for degree >= 1; for degree 0 by the number of lines and their spacing: the
+ * strip kernels for beams of at least 16,384 lines with bins at most 3 nodes
+ * apart, in the forward also for long dense lists, else the general kernels;
+ * THETA_Y and POINTS lists reach
  * the strip kernels through an order that prepare sorts them into: by major
  * axis, direction and offset, so that 32 consecutive lines are nearly
  * parallel neighbours),
  * 1 = strip kernels where they apply (ray-driven: the adjoint scatters into
- * shared-memory strips), 2 = general kernels (warp per line; the adjoint
+ * shared-memory strips, in 32-bit fixed point relative to the largest of 32
+ * neighbouring values for degree >= 1, in FP32 for degree 0), 2 = general kernels (warp per line; the adjoint
  * scatters with global atomics), and for the adjoint only 3 = pixel-driven
  * gather (thread per node over every view, no atomics; PARALLEL and FAN
  * lines of degree >= 1, else as 0).  All give the same results within
@@ -257,7 +270,7 @@ sp_status spline_plan_autotune(sp_plan *plan, const float *coef, const float *si
  *   spline_batch_create   count >= 1 instances from grids[count], lines[count]
  *                         (each as spline_plan_create; all pointers of
  *                         lines must stay valid while the batch is prepared)
- *   spline_batch_prepare  line setup and tables of every instance
+ *   spline_batch_prepare  spline_plan_prepare of every instance
  *   spline_batch_fwd      sino[i] = A_i coef[i] for every i; coef and sino
  *                         are HOST arrays of count DEVICE pointers
  *   spline_batch_adj      coef_out[i] = A_i^T sino[i]

@@ -25,7 +25,7 @@ extern "C" {
 #endif
 
 /* Forward: y BF16 [B][H][W][cout] (FP32 [B][H][W] when cout = 1); relu != 0
- * clamps at 0 after the bias.  32 -> 32 runs on the fifth-generation tensor
+ * clamps at 0 after the bias (a NaN stays NaN).  32 -> 32 runs on the fifth-generation tensor
  * cores (tcgen05.mma, BF16 inputs, FP32 accumulators in tensor memory; tiles
  * of 128 pixels of a row); 1 -> 32 and 32 -> 1 on the CUDA cores. */
 sp_status sp_conv3x3_fwd(int32_t B, int32_t H, int32_t W, int32_t cin, int32_t cout,
@@ -49,8 +49,9 @@ sp_status sp_conv3x3_bwd_data(int32_t B, int32_t H, int32_t W, int32_t cin, int3
  * tensor memory, one atomic add per entry and block, so the order of the
  * blocks' partial sums may vary between runs; dbias from g in FP32); the
  * others on the CUDA cores in FP32.  Returns SP_EINVAL for unsupported
- * channels, a dilation outside 1..16, NULL pointers, or (32 -> 32) x or g
- * not 16-byte aligned. */
+ * channels, a dilation outside 1..16, NULL pointers, (32 -> 32) x or g not
+ * 16-byte aligned, or (1 -> 32, 32 -> 1) rows of more than 204,800 bytes,
+ * counted as 4 W cout + 6 (W + 2 d) cin: 1,042 pixels for 32 -> 1 with d = 1. */
 sp_status sp_conv3x3_bwd_weight(int32_t B, int32_t H, int32_t W, int32_t cin, int32_t cout,
                                 int32_t dilation, const void *x, const float *g, float *dw, float *dbias,
                                 void *stream);
@@ -79,7 +80,7 @@ sp_status sp_conv3x3_flip_weights(int32_t cin, int32_t cout, const void *w, void
  * gradient through f (rounded to BF16, as z was; the one through z is g).  work
  * BF16: two slabs of scratch.  Gradients between layers are BF16, those of the
  * last layer's output FP32; sums are FP32, over blocks by atomic adds (their
- * order may vary between runs).
+ * order may vary between runs).  Image widths as in sp_conv3x3_bwd_weight.
  */
 int64_t sp_convnet_pack_elems(int32_t layers);
 sp_status sp_convnet_fwd(int32_t B, int32_t H, int32_t W, int32_t layers, const int32_t *dilation,

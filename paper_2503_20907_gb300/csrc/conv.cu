@@ -321,6 +321,8 @@ __global__ void __launch_bounds__(kEdgeThreads, 2) edge_wgrad_kernel(EdgeArgs a,
         atomicAdd(k < 9 * kC ? dw + k : db + (k - 9 * kC), part[k]);
 }
 
+// Blocks of an edge kernel: all that are resident at once on this GPU's 152 SMs
+// (twice as many forward, whose blocks are short), or one per eight pixel groups.
 unsigned edge_blocks(int B, int H, int W, int per_sm)
 {
     const int64_t groups = (int64_t)B * H * ((W + 7) / 8);
@@ -894,8 +896,9 @@ cudaError_t launch_wgrad32(int B, int H, int W, int dil, const bf16 *x, const G 
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// The weight gradient of the 1 -> 32 and 32 -> 1 layers has always been limited
-// to rows of this many bytes.
+// Rows that the entry points of the weight gradient of the 1 -> 32 and 32 -> 1
+// layers refuse (warmstart_conv.h): a limit of the interface, whose first kernels
+// staged whole rows in shared memory; the present ones hold none.
 bool edge_too_wide(int W, int cin, int cout, int dil)
 {
     return sizeof(float) * (size_t)W * cout + sizeof(bf16) * 3 * (size_t)(W + 2 * dil) * cin > 200 * 1024;

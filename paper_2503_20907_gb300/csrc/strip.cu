@@ -45,32 +45,34 @@
 // (two-sum), so that a line's value does not depend on how its blocks were
 // spread over warps and lanes, i.e. on the lines it shares a chunk with.
 //
-// What bounds it: the issue slots (about 70 instructions per row and warp at
-// n = 3, 62 % of the slots filled) and the FMA pipe (54 % busy).  A pair of
+// What bounds it: the issue slots (about 75 instructions per row and warp
+// forward and 80 in the adjoint at n = 3, 64 % of the slots filled) and the FMA
+// pipe (54 and 52 % busy).  A pair of
 // candidates takes 3 packed FMAs (n = 3) for the even and odd parts, one
 // multiply and two additions to join them, 2 packed FMAs for the jumps and one
 // to accumulate; a row adds about 25 instructions (step, v, z, addresses).  The
 // lanes' strip accesses of one row fall on neighbouring columns, in distinct
 // banks.  Measured at the 512 x 512 cubic fan (552,960 lines), forward and
-// adjoint: 0.80 and 0.86 ms; one polynomial of 7 FMAs per candidate of a base
+// adjoint: 0.83 and 0.86 ms (the forward 0.80 without the tests of its outermost
+// candidates); one polynomial of 7 FMAs per candidate of a base
 // interval plus truncated powers with integer weights 1.19 and 1.28 ms; rows
 // sorted by interval, a lane per candidate and row, 2.18 and 2.35 ms.
 // Four CTAs of four warps per SM: while one CTA waits for its line records,
 // its strip or its flush, three others compute; two CTAs of eight warps with
 // strips of twice the height took 0.91 and 0.99 ms, three CTAs of eight warps
 // (80 registers) 0.95 and 0.98 ms, five of four warps (96 registers) 0.93 and
-// 0.92 ms.
+// 0.92 ms, against 0.80 and 0.86.
 //
-// The adjoint (degree 0 apart) accumulates its strip in 32-bit fixed point: a shared-memory
-// integer reduction costs about what a plain shared store does on this GPU,
-// a float one four to six times more.  Each chunk takes the power of two S
+// The adjoint of degree >= 1 accumulates its strip in 32-bit fixed point: a
+// shared-memory integer reduction costs about what a plain shared store does on
+// this GPU, a float one four to six times more.  Each chunk takes the power of two S
 // that puts its largest contribution h |p| phi (phi <= sqrt(2) < 1.5 for
 // every basis here) at 2^22 or less; a pair then adds round(S h p phi) to its
 // node, at most 2^27 in magnitude after 32 lines, and the flush adds the
 // sums times 1/S (exact) to the image.  Adding M = 1.5 2^23 does the rounding:
 // the result lies in [2^23, 2^24) where floats are the integers, and its bits
 // minus M's bits are round(S h p phi).  Per pair that is an error of about
-// half a unit, 1/S <= 1.5 h max|p| 2^-21 = 7e-7 h max|p|.
+// half a unit, 1/S <= 1.5 h max|p| 2^-21 = 7e-7 h max|p|.  Degree 0 adds floats.
 #include <climits>
 #include <cfloat>
 
