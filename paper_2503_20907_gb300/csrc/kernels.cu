@@ -622,22 +622,27 @@ __device__ void build_table_half(float a, float b, float *out, float *sm, int l,
             tab[tab_poly(0, i) + e] = kBPiece[n][i][e] * sc;
         }
     } else {
-        // breakpoints p a + q b, ranked (ties by p, then q)
+        // breakpoints p a + q b, ranked (ties by p, then q) by their exact values in
+        // units of 2^-47 (a and b >= kBMin > 2^-24 are multiples): rounded values of
+        // breakpoints less than an ulp apart, as at b/a = 1/2, came in the wrong
+        // order, and the piece that then stood last lacked a derivative's jump
         constexpr int NB = (m + 1) * (m + 1);
         constexpr int NI = (NB + G - 1) / G;   // breakpoints per lane: l and l + 16
+        constexpr float kUnit = 140737488355328.f;   // 2^47
+        const long long A = __float2ll_rn(a * kUnit), B = __float2ll_rn(b * kUnit);
         // all values in the scratch of the pieces (filled later), read back
-        // four at a time; ties go by index, which orders (p, q) lexicographically
-        float *vr = P;
+        // two at a time; ties go by index, which orders (p, q) lexicographically
+        long long *vr = reinterpret_cast<long long *>(P);
         int p[NI], q[NI];
-        float v[NI];
+        long long v[NI];
 #pragma unroll
         for (int it = 0; it < NI; ++it) {
             const int idx = l + G * it;
-            p[it] = 0; q[it] = 0; v[it] = 0.f;
+            p[it] = 0; q[it] = 0; v[it] = 0;
             if (idx < NB) {
                 p[it] = idx / (m + 1);
                 q[it] = idx - p[it] * (m + 1);
-                v[it] = __fmaf_rn((float)p[it], a, (float)q[it] * b);
+                v[it] = p[it] * A + q[it] * B;
                 vr[idx] = v[it];
             }
         }
@@ -646,12 +651,12 @@ __device__ void build_table_half(float a, float b, float *out, float *sm, int l,
 #pragma unroll
         for (int it = 0; it < NI; ++it) rank[it] = 0;
 #pragma unroll
-        for (int j4 = 0; j4 < (NB + 3) / 4; ++j4) {
-            const float4 w4 = reinterpret_cast<const float4 *>(vr)[j4];
-            const float vj[4] = {w4.x, w4.y, w4.z, w4.w};
+        for (int j2 = 0; j2 < (NB + 1) / 2; ++j2) {
+            const longlong2 w2 = reinterpret_cast<const longlong2 *>(vr)[j2];
+            const long long vj[2] = {w2.x, w2.y};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = 4 * j4 + u;
+            for (int u = 0; u < 2; ++u) {
+                const int j = 2 * j2 + u;
                 if (j < NB)
 #pragma unroll
                     for (int it = 0; it < NI; ++it)
@@ -661,7 +666,7 @@ __device__ void build_table_half(float a, float b, float *out, float *sm, int l,
         __syncwarp(gmask);
 #pragma unroll
         for (int it = 0; it < NI; ++it)
-            if (l + G * it < NB) { bv[rank[it]] = v[it]; bpq[rank[it]] = p[it] | (q[it] << 8); }
+            if (l + G * it < NB) bpq[rank[it]] = p[it] | (q[it] << 8);
         __syncwarp(gmask);
         // pieces that start at or before the centre w: the leading sorted run
         // (the last breakpoint, at 2w, is always beyond it)
@@ -696,12 +701,16 @@ __device__ void build_table_half(float a, float b, float *out, float *sm, int l,
                     if (q0 >= m) continue;
                     piece = q0; tau = 0.f;
                 } else {
-                    const float vv = __fmaf_rn((float)(p0 - pp), a, (float)q0 * b);
-                    if (vv < 0.f) continue;
-                    const float t = __fdiv_rn(vv, b);   // exact when vv is a multiple of b
-                    piece = (int)floorf(t);
-                    if (piece < 0 || piece >= m) continue;
-                    tau = t - (float)piece;
+                    // the piece of the B-spline of b that starts at or before this
+                    // breakpoint, by the exact values as in the ranking
+                    long long left = (p0 - pp) * A + q0 * B;
+                    if (left < 0) continue;
+                    piece = 0;
+#pragma unroll
+                    for (int k = 0; k < m; ++k)
+                        if (left >= B) { left -= B; ++piece; }
+                    if (piece >= m) continue;
+                    tau = __fdiv_rn((float)left, (float)B);
                 }
                 float D[n + 1];
                 bspline_piece_derivs<n>(piece, tau, binv, D);
