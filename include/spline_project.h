@@ -238,7 +238,8 @@ sp_status spline_plan_cgls(sp_plan *plan, const float *b, float *x, int32_t iter
  * neighbouring values for degree >= 1, in FP32 for degree 0), 2 = general kernels (warp per line; the adjoint
  * scatters with global atomics), and for the adjoint only 3 = pixel-driven
  * gather (thread per node over every view, no atomics; PARALLEL and FAN
- * lines and B-splines of degree >= 1, else as 2).  All give the same results within
+ * lines with ddet != 0, for FAN the whole grid in front of the source at every
+ * angle, and B-splines of degree >= 1; else as 2).  All give the same results within
  * rounding (no paper counterpart: this is an implementation choice).
  */
 sp_status spline_plan_set_paths(sp_plan *plan, int32_t fwd_path, int32_t adj_path);

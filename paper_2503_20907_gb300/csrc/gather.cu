@@ -21,6 +21,7 @@
 // search.  spline_plan_autotune times both and keeps the faster.
 #include <cfloat>
 #include <climits>
+#include <cmath>
 
 #include "common.cuh"
 
@@ -182,7 +183,14 @@ __global__ void __launch_bounds__(kThreads) gather_adj_kernel(GridDev g, LinesDe
 
 bool gather_supported(const GridDev &g, const LinesDev &L)
 {
-    return (L.kind == SP_LINES_PARALLEL || L.kind == SP_LINES_FAN) && g.kdeg >= 1 && g.basis == SP_BASIS_BSPLINE;
+    if ((L.kind != SP_LINES_PARALLEL && L.kind != SP_LINES_FAN) || g.kdeg < 1 || g.basis != SP_BASIS_BSPLINE) return false;
+    if (L.ddet == 0.f) return false;   // bins that coincide have no order
+    if (L.kind == SP_LINES_PARALLEL) return true;
+    // lines go on behind the source: a node's lines are neighbours in the fan
+    // only where all tiles, widened as above, lie in front of it at every angle
+    const double marg = ((double)(g.kdeg + 1) * 0.7072 + 1.0) + kTile;
+    const double x = std::fabs((double)g.cx) + (0.5 * g.nx + marg) * g.h, y = std::fabs((double)g.cy) + (0.5 * g.ny + marg) * g.h;
+    return (double)L.dso > std::sqrt(x * x + y * y);
 }
 
 cudaError_t launch_adj_gather(const GridDev &g, const LinesDev &L, const LineHdr *hdr, const float *tabs,
