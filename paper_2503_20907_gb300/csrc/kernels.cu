@@ -586,6 +586,13 @@ __device__ __forceinline__ float sym_diff(int dp, int dq, float a, float b, floa
     return __fmaf_rn((float)dp, a, __fmaf_rn((float)dq, b, extra));
 }
 
+// Slot l of a B-spline table's head, s its interval end: what the line setup left
+// there for the builder stays, so that a table can be built again from its head.
+__device__ __forceinline__ float head_slot(int l, float a, float b, float s)
+{
+    return l == kTabA ? a : l == kTabB ? b : l == kTabMode ? (float)kModeBspline : s;
+}
+
 // Build the footprint table of one direction (see common.cuh), degree N, on
 // one half-warp: l is the lane within the half (0..15) and gmask the half's
 // lanes.  sm is the half's shared scratch of kBuildScratch floats; the table
@@ -614,7 +621,7 @@ __device__ void build_table_half(float a, float b, float *out, float *sm, int l,
     const float ainv = 1.0f / a;
     if (b == 0.f) {
         // Dirac factor (Prop. 1): phi(u) = beta^n(u/a)/a on the a-knots.
-        if (l < kTabHead) tab[l] = l == kTabA ? a : (l == kTabB ? 0.f : (l < m ? a : FLT_MAX));
+        if (l < kTabHead) tab[l] = head_slot(l, a, 0.f, l < m ? a : FLT_MAX);
         if (l < m * (n + 1)) {
             const int i = l / (n + 1), e = l - i * (n + 1);
             float sc = ainv;
@@ -779,7 +786,7 @@ __device__ void build_table_half(float a, float b, float *out, float *sm, int l,
         if (l >= 1 && l <= m) { sv[srank] = rq; sq[srank] = l; sf[srank] = fq; }
         if (l == 0) { sv[0] = 0.f; sq[0] = 0; sf[0] = 0; }
         __syncwarp(gmask);
-        if (l < kTabHead) tab[l] = l == kTabA ? a : (l == kTabB ? b : (l < m ? sv[l + 1] : FLT_MAX));
+        if (l < kTabHead) tab[l] = head_slot(l, a, b, l < m ? sv[l + 1] : FLT_MAX);
         const int K = slots_of(m, a, b, two_w);
         // entry e = (sigma, candidate) = (e / 8, e % 8), two sigmas per pass
 #pragma unroll

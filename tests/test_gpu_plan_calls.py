@@ -42,12 +42,13 @@ def _capture(f):
     return graph
 
 
+@pytest.mark.parametrize("degree", [1, 2, 3])
 @pytest.mark.parametrize("paths", [(2, 2), (2, 3)])
 @pytest.mark.parametrize("warm", [False, True])
-def test_projections_after_a_replayed_prepare(paths, warm):
+def test_projections_after_a_replayed_prepare(paths, warm, degree):
     # the prepare is captured on the strip kernels' path (no footprint tables)
     # and replayed when the plan has gone over to kernels that read them
-    view, grid, lines, coef, p = _case()
+    view, grid, lines, coef, p = _case(degree)
     plan = sp.Plan(grid, lines, prepare=warm)
     graph = _capture(plan.prepare)
     graph.replay()
@@ -60,15 +61,17 @@ def test_projections_after_a_replayed_prepare(paths, warm):
         graph.replay()
         want = _fresh(grid, lines, coef, p, paths)
         assert not _close(first, want[0])
-        assert torch.equal(plan.fwd(coef), want[0]) and _close(plan.adj(p), want[1])
+        for _ in range(2):               # (each builds the tables again)
+            assert torch.equal(plan.fwd(coef), want[0]) and _close(plan.adj(p), want[1])
     plan.prepare()                       # and an ordinary prepare again
     assert torch.equal(plan.fwd(coef), want[0]) and _close(plan.adj(p), want[1])
     plan.close()
 
 
+@pytest.mark.parametrize("degree", [0, 2, 3])
 @pytest.mark.parametrize("paths", [(0, 0), (2, 2), (2, 3)])
-def test_a_graph_of_prepare_and_projections(paths):
-    view, grid, lines, coef, p = _case()
+def test_a_graph_of_prepare_and_projections(paths, degree):
+    view, grid, lines, coef, p = _case(degree)
     plan = sp.Plan(grid, lines)
     plan.set_paths(*paths)
     sino, back = torch.empty(lines.m, device=DEV), torch.empty(grid.ny, grid.nx, device=DEV)
@@ -86,6 +89,25 @@ def test_a_graph_of_prepare_and_projections(paths):
         want = _fresh(grid, lines, coef, p, paths)
         assert torch.equal(sino, want[0]) and _close(back, want[1])
         # eager projections of the plan that the graph prepared
+        assert torch.equal(plan.fwd(coef), want[0]) and _close(plan.adj(p), want[1])
+    plan.close()
+
+
+@pytest.mark.parametrize("degree,basis", [(1, 0), (2, 0), (3, 0), (1, 1)])
+def test_a_captured_projection_replayed(degree, basis):
+    # captured before any projection of its path has run: the graph builds the
+    # tables, at every replay
+    view, _, lines, coef, p = _case(degree)
+    grid = sp.Grid(coef.shape[1], coef.shape[0], degree, 1.0, basis=basis)
+    want = _fresh(grid, lines, coef, p, (2, 2))
+    plan = sp.Plan(grid, lines)
+    plan.set_paths(2, 2)
+    sino = torch.empty(lines.m, device=DEV)
+    graph = _capture(lambda: plan.fwd(coef, sino))
+    for _ in range(3):
+        sino.zero_()
+        graph.replay()
+        assert torch.equal(sino, want[0])
         assert torch.equal(plan.fwd(coef), want[0]) and _close(plan.adj(p), want[1])
     plan.close()
 
