@@ -188,20 +188,28 @@ __device__ __forceinline__ float row_start(const LineHdr &H, float inv_a, int r,
 
 // Degree 0 near an axis has footprint ramps of width b, which can be far
 // narrower than one float ulp of u.  For that degree u_0 is carried as an
-// unevaluated sum hi + lo.
+// unevaluated sum hi + lo of U0, the row's and the column's part (each product
+// exact, their sum not: rho's last bits lie far below a's).
 struct U0DF {
     float hi, lo;
 };
 
+// s + err = a + b exactly.
+__device__ __forceinline__ float two_sum(float a, float b, float &err)
+{
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+
 __device__ __forceinline__ U0DF row_u0_df(const LineHdr &H, int dr, int k)
 {
     float fr = (float)dr, fk = (float)k;
-    float big = __fsub_rn(__fmul_rn(fr, H.rho_hi), __fmul_rn(fk, H.a_hi));   // exact
     float small = __fadd_rn(__fmaf_rn(fr, H.rho_lo, __fmul_rn(-fk, H.a_lo)), H.U0_lo);
-    float s = __fadd_rn(H.U0, big);                                             // two-sum
-    float bb = __fsub_rn(s, H.U0);
-    float err = __fadd_rn(__fsub_rn(H.U0, __fsub_rn(s, bb)), __fsub_rn(big, bb));
-    float lo = __fadd_rn(err, small);
+    float e1, e2;
+    const float c = two_sum(H.U0, -__fmul_rn(fk, H.a_hi), e1);
+    const float s = two_sum(c, __fmul_rn(fr, H.rho_hi), e2);
+    float lo = __fadd_rn(__fadd_rn(e1, e2), small);
     float hi = __fadd_rn(s, lo);
     lo = __fsub_rn(lo, __fsub_rn(hi, s));
     return U0DF{hi, lo};
