@@ -227,8 +227,8 @@ sp_status spline_plan_cgls(sp_plan *plan, const float *b, float *x, int32_t iter
 /*
  * Kernel choice of a plan, per direction: 0 = automatic (the strip kernels
  * for degree >= 1; for degree 0 by the number of lines and their spacing: the
- * strip kernels for beams of at least 16,384 lines with bins at most 3 nodes
- * apart, in the forward also for long dense lists, else the general kernels;
+ * strip kernels for beams of at least 16,384 lines with bins at most 3 (adjoint:
+ * 2) nodes apart, in the forward also for long dense lists, else the general kernels;
  * THETA_Y and POINTS lists reach
  * the strip kernels through an order that prepare sorts them into: by major
  * axis, direction and offset, so that 32 consecutive lines are nearly

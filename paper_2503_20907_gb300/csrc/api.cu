@@ -165,17 +165,19 @@ void *order_area(const spx::GridDev &g, const spx::LinesDev &L, void *extra)
 // A strip costs per row and 32 lines about as much as its window is wide, and a
 // call three more launches; a line alone costs the general kernels per row the
 // same in any company.  Measured, strip / general, forward and adjoint:
-//   parallel beam, 360 views: bins 1 pixel apart 0.64 and 0.58 at 512^2 pixels,
-//     0.77 and 0.56 at 256^2; 2 apart 0.80 and 0.72 at 512^2; 4 apart 1.10, 1.09;
-//     8 apart 1.69, 1.78.  Hence at most 3 apart (fan beams: at the grid's centre).
-//   fewer lines, 1 apart: 11,520 at 256^2 1.07 and 0.97, 3,072 at 512^2 1.28 and
-//     1.87, 23,040 at 512^2 0.81 and 0.77; 34,560 at 64^2 1.11 and 0.56.  Hence
-//     16,384 lines, and in the forward, which gains less, 2^23 lines times rows.
+//   parallel beam, 360 views: bins 1 pixel apart 0.60 and 0.73 at 512^2 pixels,
+//     0.72 and 0.68 at 256^2; 2 apart 0.75 and 0.91 at 512^2; 4 apart 1.05, 1.31;
+//     8 apart 1.63, 2.09.  Hence at most 3 apart forward, 2 in the adjoint (fan
+//     beams: at the grid's centre).
+//   fewer lines, 1 apart: 11,520 at 256^2 1.08 and 1.09, 3,072 at 512^2 1.25 and
+//     1.97, 23,040 at 512^2 0.80 and 0.90; 34,560 at 64^2 1.09 and 0.66.  Hence
+//     16,384 lines, and in the forward, which gains less on small grids, 2^23 lines
+//     times rows.
 //   chunks are filled by a view's bins: at most a quarter of their lines missing.
 //   random lists (neighbours in the sorted order are 13.5 N / sqrt(m) columns
-//     apart over 32 lines, see order.cu): forward 0.84 at 30,000 lines and 512^2
-//     (40 columns), 1.60 at 10,000 (69), 1.22 at 30,000 and 1024^2 (80): at most 48
-//     columns.  Their adjoint 1.2 to 1.5 (lanes that add to one pixel): never.
+//     apart over 32 lines, see order.cu): forward 0.81 at 30,000 lines and 512^2
+//     (40 columns), 1.53 at 10,000 (69), 1.17 at 30,000 and 1024^2 (80): at most 48
+//     columns.  Their adjoint 1.0 to 2.3 (lanes that add to one pixel): never.
 bool pixels_on_strips(const spx::GridDev &g, const spx::LinesDev &L, bool adj)
 {
     const double m = (double)L.m, N = (double)(g.nx > g.ny ? g.nx : g.ny);
@@ -183,7 +185,7 @@ bool pixels_on_strips(const spx::GridDev &g, const spx::LinesDev &L, bool adj)
     if (spx::strip_needs_order(L)) return !adj && 13.5 * 13.5 * N * N <= 48.0 * 48.0 * m;
     double apart = std::fabs((double)L.ddet) / g.h;
     if (L.kind == SP_LINES_FAN) apart *= (double)L.dso / ((double)L.dso + (double)L.dod);
-    return m >= 16384.0 && apart <= 3.0 && 32.0 * (double)spx::strip_chunk_count(L) <= 1.25 * m;
+    return m >= 16384.0 && apart <= (adj ? 2.0 : 3.0) && 32.0 * (double)spx::strip_chunk_count(L) <= 1.25 * m;
 }
 
 // Kernel paths: strip kernels (kPathAuto where they are the faster ones: always

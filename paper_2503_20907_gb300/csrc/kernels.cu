@@ -1060,7 +1060,7 @@ __device__ __forceinline__ void walk_line(const LineHdr &H, const float *tab, co
 // candidates beyond the support are left out, so that coefficients and values
 // that are not finite do not reach across it.  (The forward still loads them:
 // with loads that wait for phi 512 x 512 pixels and 300 lines took 24 us instead
-// of 21; the adjoint saves the additions, 770 -> 536 us at 256 x 256 pixels and
+// of 21; the adjoint saves the additions, 770 -> 615 us at 256 x 256 pixels and
 // 552,960 lines.)
 template <int DEG>
 __device__ __forceinline__ bool in_support(float phi) { return DEG > 0 || phi != 0.f; }

@@ -179,7 +179,7 @@ constexpr float kPhiBound = 1.5f;
 // strips only: its pixels belong to few lines, and where those are far below the
 // chunk's largest, fixed point would leave them fewer bits than FP32 sums have.
 // (Parallel beams, 501 x 501 pixels, 367 x 751 lines: 332 us, in fixed point 274,
-// with the general kernel's global additions 625.)
+// with the general kernel's global additions 488.)
 enum FixMode { kFmAll = 0, kFmFixed = 1, kFmFloat = 2 };
 template <int KIND>
 __host__ __device__ constexpr int adj_mode() { return KIND == 0 ? kFmFloat : kFmFixed; }

@@ -32,7 +32,8 @@ CASES = [   # grid, lines, forward and adjoint on the strip kernels
     ((64, 64), lambda: _beam("parallel", 64, 30, 96, 1.0), False, False),
     ((64, 64), lambda: _beam("parallel", 64, 180, 96, 1.0), False, True),
     ((300, 512), lambda: _beam("parallel", 512, 30, 768, 1.0), True, True),
-    ((512, 512), lambda: _beam("fan", 512, 60, 512, 4.4), True, True),
+    ((512, 512), lambda: _beam("fan", 512, 60, 512, 2.9), True, True),
+    ((512, 512), lambda: _beam("fan", 512, 60, 512, 4.4), True, False),
     ((512, 512), lambda: _beam("fan", 512, 60, 512, 4.6), False, False),
     ((512, 512), lambda: _beam("parallel", 512, 300, 96, 4.0), False, False),
     ((512, 512), lambda: _beam("parallel", 512, 700, 33, 1.0), False, False),
